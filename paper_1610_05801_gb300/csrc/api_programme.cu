@@ -53,6 +53,7 @@ int derive_programme(const phtl_params& p, const double* V, const double* p0, in
             if (!(std::fabs(x) < 1.0)) return PHTL_E_UNSTABLE;
             T.phis = eta > 0.0 ? std::asin(x) : kPi - std::asin(x);
             T.sinphis = std::sin(T.phis);
+            T.uphis = phase_turns(T.phis);
             const double K = T.etaC * T.A * k * std::cos(T.phis);
             if (!(K > 0.0 && K < 4.0)) return PHTL_E_UNSTABLE;
         }

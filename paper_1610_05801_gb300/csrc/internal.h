@@ -22,6 +22,69 @@ inline void split_df(double v, float& hi, float& lo)
     lo = static_cast<float>(v - static_cast<double>(hi));
 }
 
+// k / 2 pi for the integer phase of the FP64 sines: K 2^(958 - cn), K with its top bit set
+// (64 significant bits).  cn = kNoPhaseScale (no integer phase) where k is zero or so large or
+// small that the exponent arithmetic of the device would leave the range of a double.
+struct PhaseScale {
+    uint64_t K;
+    int32_t cn;
+    int32_t pad_;
+};
+constexpr int32_t kNoPhaseScale = -(1 << 20);
+
+// 1 / 2 pi 2^130, rounded down (binary digits of 2 / pi, A2F983 6E4E44 ...)
+constexpr uint64_t kInvTwoPiHi = 0xA2F9836E4E441529ull, kInvTwoPiLo = 0xFC2757D1F534DDC0ull;
+
+// x / 2 pi = v 2^(x's exponent - 2): the 128-bit product of x's 53-bit significand (top bit of
+// m at 63) and the digits above.
+inline unsigned __int128 over_two_pi(uint64_t m)
+{
+    return static_cast<unsigned __int128>(m) * kInvTwoPiHi +
+           ((static_cast<unsigned __int128>(m) * kInvTwoPiLo) >> 64);
+}
+
+inline PhaseScale phase_scale(double k)
+{
+    PhaseScale r{0, kNoPhaseScale, 0};
+    int e = 0;
+    const double f = std::frexp(k, &e);  // k = f 2^e, f in [1/2, 1)
+    if (!(f >= 0.5 && std::isfinite(k))) return r;
+    unsigned __int128 v = over_two_pi(static_cast<uint64_t>(std::ldexp(f, 53)) << 11);  // k / 2 pi = v 2^(e - 130)
+    int x = e - 2;                                                                        // = (v 2^-128) 2^x
+    if (!(v >> 127)) {
+        v <<= 1;
+        --x;
+    }
+    uint64_t K = static_cast<uint64_t>(v >> 64);
+    if ((v >> 63) & 1) ++K;   // round to nearest; a carry out of the top bit cannot occur for
+    if (K == 0) return r;     // a 53-bit k times these digits, and would disable the path
+    const int cn = 1022 - x;
+    if (cn < 900 || cn > 1900) return r;
+    r.K = K;
+    r.cn = cn;
+    return r;
+}
+
+// phi / 2 pi modulo 1 in 2^-64 turns (|phi| < 2^40; larger phases are the caller's to keep off)
+inline uint64_t phase_turns(double phi)
+{
+    int e = 0;
+    const double f = std::frexp(std::fabs(phi), &e);
+    if (f == 0.0) return 0;
+    const unsigned __int128 v = over_two_pi(static_cast<uint64_t>(std::ldexp(f, 53)) << 11);
+    const int s = 130 - e - 64;  // |phi| / 2 pi = v 2^(e - 130); in units of 2^-64: v >> s
+    uint64_t u = 0;
+    if (s >= 128) u = 0;
+    else if (s > 0) u = static_cast<uint64_t>((v >> s) + ((v >> (s - 1)) & 1));
+    return phi < 0.0 ? 0 - u : u;
+}
+
+// The phase scale of sin(k z + phi): none where |phi| is beyond phase_turns().
+inline PhaseScale integer_phase(double k, double phi)
+{
+    return std::fabs(phi) < 1e5 ? phase_scale(k) : PhaseScale{0, kNoPhaseScale, 0};
+}
+
 // Per-stage coefficients of one turn of the longitudinal map (Sec. 1.1.2 schemes),
 // pre-multiplied on the host in FP64:
 //   drift stage i:  z <- z - dc[i] * delta           dc[i] = w_i * eta * C
@@ -49,6 +112,8 @@ struct MapConsts {
     float mx_hi[4], mx_lo[4], my_hi[4], my_lo[4];
     int32_t linear;  // rf_linear flag
     float k2opi;     // k * 2/pi rounded to FP32 (quadrant estimate of the fused FP64 sine)
+    PhaseScale kap;  // k / 2 pi and phi_s / 2 pi of the integer phase
+    uint64_t uphis;
     // widened map: nonlinear slippage eta(d) = eta0 + eta1 d + eta2 d^2 and chromaticity
     int32_t general;             // eta1, eta2 or a chromaticity nonzero: general turn loop
     int32_t chroma_x, chroma_y;  // xi != 0 in that plane
@@ -66,6 +131,8 @@ struct MapConsts {
     int32_t pad3_;
     double kw2[3];
     double k2, phi2, sinphi2, lin2;
+    PhaseScale kap2;
+    uint64_t uphi2;
     float kw2_hi[3], kw2_lo[3];
     float k2_hi, k2_lo, phi2_hi, phi2_lo, sinphi2_hi, sinphi2_lo, lin2_hi, lin2_lo;
 };
@@ -108,8 +175,9 @@ struct RampTurn {
     double w_ec[2];
     double w_lf[3];
     double w_r4[7];
+    uint64_t uphis;  // phi_s,n / 2 pi in 2^-64 turns
 };
-static_assert(sizeof(RampTurn) == 192, "RampTurn is 192 bytes");
+static_assert(sizeof(RampTurn) == 200, "RampTurn is 200 bytes");
 
 // Slicing grid and strength of the collective (wake) step.
 struct CollArgs {

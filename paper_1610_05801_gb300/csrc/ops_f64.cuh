@@ -46,8 +46,8 @@ template <bool ZS>
 __device__ __forceinline__ double rf_force(const MapConsts& c, double z)
 {
     if (c.linear) return c.lin * z;
-    if (ZS) return sin_kz(c.k, c.k2opi, z);
-    return sin_f64(fma(c.k, z, c.phis)) - c.sinphis;
+    if (ZS) return sin_kz(c.k, c.k2opi, c.kap, z);
+    return sin_kz_phi(c.k, c.kap, z, c.phis, c.uphis) - c.sinphis;
 }
 
 __device__ __forceinline__ void drift(double (&z)[P], const double (&d)[P], double dc)
@@ -132,7 +132,7 @@ __device__ __forceinline__ void drift_nl(double (&z)[P], const double (&d)[P], d
 __device__ __forceinline__ double rf_force2(const MapConsts& c, double z)
 {
     if (c.linear) return c.lin2 * z;
-    return sin_f64(fma(c.k2, z, c.phi2)) - c.sinphi2;
+    return sin_kz_phi(c.k2, c.kap2, z, c.phi2, c.uphi2) - c.sinphi2;
 }
 
 // Kick of the widened map: the main RF system, then the second one when `dual` (a

@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include "dfloat.cuh"
+#include "internal.h"
 
 namespace phtl {
 namespace detail {
@@ -52,6 +53,88 @@ __host__ __device__ constexpr double kC(int i)
 constexpr double kTwoPi = 6.283185307179586;
 
 __device__ __forceinline__ double sc_coef(bool odd, double s, double c) { return odd ? c : s; }
+
+// ---- sines on the integer pipe ---------------------------------------------------------
+//
+// An FP64 instruction takes the FP64 pipe half a clock per lane (2 per clock per SM), as long
+// as 64 issue slots of the other pipes, so a kick's sine costs less as ~90 integer
+// instructions than as 11 FP64 ones.  The phase is a 64-bit binary fraction of a turn (its
+// overflow is the reduction modulo 2 pi, and no fold is ever rounded), the sine one unsigned
+// fixed-point polynomial
+//     sin(pi V) = V p(rho),   rho = (2 V)^2 in [0, 1],   V in [0, 1/2] half turns,
+// p of degree 8 (Chebyshev interpolation at 60 digits, gen_sin_coeffs.py --fixed; error 2e-19
+// of p): the upper five steps in 64 bits, the three last terms (below 1.2e-7) in 32.  The
+// result is normalised and rounded to FP64 once: |error| <= 0.66 2^-53 over the range, where
+// the FP64 polynomial has about 1.
+
+// High 64 bits of a 128-bit product, short of it by at most 2 (the low product and the carry
+// of the low halves are left out).
+__device__ __forceinline__ uint64_t mulhi_trunc(uint64_t a, uint64_t b)
+{
+    const uint32_t a1 = static_cast<uint32_t>(a >> 32), a0 = static_cast<uint32_t>(a);
+    const uint32_t b1 = static_cast<uint32_t>(b >> 32), b0 = static_cast<uint32_t>(b);
+    return static_cast<uint64_t>(a1) * b1 + __umulhi(a1, b0) + __umulhi(a0, b1);
+}
+
+// 64-bit shifts whose amount saturates (0 for 64 and more), as the hardware's do.
+__device__ __forceinline__ uint64_t shr_sat(uint64_t a, uint32_t n)
+{
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
+    return r;
+}
+__device__ __forceinline__ uint64_t shl_sat(uint64_t a, uint32_t n)
+{
+    uint64_t r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
+    return r;
+}
+
+// The significand of a normal double with its leading one at bit 63.
+__device__ __forceinline__ uint64_t mantissa64(double x)
+{
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+    return (static_cast<uint64_t>(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
+}
+
+// p(rho) 2^62, rho = R^2 2^-128 (see above): R = 2 V.
+__device__ __forceinline__ uint64_t sin_poly_fixed(uint64_t R)
+{
+    const uint64_t T = mulhi_trunc(R, R);
+    const uint32_t t = static_cast<uint32_t>(T >> 32);
+    uint32_t q = 0x02DEF59Bu - __umulhi(t, 0x00067519u);          // c7, c8 (2^55)
+    q = 0xF479B3AFu - __umulhi(t, q);                              // c6
+    uint64_t p = 0x00001E3074DFAF88ull - ((static_cast<uint64_t>(t) * q) >> 25);  // c5 (2^62)
+    p = 0x000541E0D2154615ull - mulhi_trunc(T, p);
+    p = 0x009969667313E42Full - mulhi_trunc(T, p);
+    p = 0x0A335E33BAD53E48ull - mulhi_trunc(T, p);
+    p = 0x52AEF39896F94915ull - mulhi_trunc(T, p);
+    return 0xC90FDAA22168C232ull - mulhi_trunc(T, p);              // pi
+}
+
+// S 2^(-62 - x) as a double with the sign bit of `sign`, rounded to nearest (ties up).
+__device__ __forceinline__ double fixed_to_double(uint64_t S, int x, uint32_t sign)
+{
+    if (static_cast<uint32_t>(S >> 32) == 0u) {  // near a zero of the sine: at most 32 bits left
+        if (S == 0) return __hiloint2double(static_cast<int>(sign & 0x80000000u), 0);
+        S <<= 32;
+        x += 32;
+    }
+    const int c = __clz(static_cast<int>(S >> 32));
+    const uint64_t N = shl_sat(S, static_cast<uint32_t>(c));   // leading one at bit 63
+    const uint64_t r = (N >> 11) + ((N >> 10) & 1u);            // the leading one adds 1 to the exponent
+    const uint32_t hi = static_cast<uint32_t>(r >> 32) + (static_cast<uint32_t>(1023 - c - x) << 20);
+    return __hiloint2double(static_cast<int>(hi | (sign & 0x80000000u)), static_cast<int>(static_cast<uint32_t>(r)));
+}
+
+// sin(2 pi U) of a phase U in 2^-64 turns; `flip`: its top bit flips the sign.
+__device__ __forceinline__ double sin_turns_fixed(uint64_t U, uint32_t flip)
+{
+    const uint64_t s = static_cast<uint64_t>(static_cast<int64_t>(U << 1) >> 63);
+    const uint64_t V = (U << 1) ^ s;                              // folded into [0, 1/2] half turns
+    return fixed_to_double(mulhi_trunc(V, sin_poly_fixed((U << 2) ^ s)), 0,
+                           static_cast<uint32_t>(U >> 32) ^ flip);
+}
 
 // sin(q pi/2 + r) for |r| <= pi/4 (a hair more when q came out one off), given the low
 // bits qi of q.
@@ -107,11 +190,9 @@ __device__ __forceinline__ double neg_q_h(int q)
 
 }  // namespace detail
 
-// sin(k z); k2opi = k * 2/pi rounded to FP32.  The fused form holds for |k z| up to ~1e5
-// (the quadrant q below 2^16): it covers the bucket and the particles that leave it for
-// ~1e6 turns, so a warp does not split between two sine paths when one of its particles
-// drifts away.  Beyond, and for Inf and NaN: sin_f64(k * z).
-__device__ __forceinline__ double sin_kz(double k, float k2opi, double z)
+// sin(k z) in FP64 arithmetic; k2opi = k * 2/pi rounded to FP32.  The fused form holds for
+// |k z| up to ~1e5 (the quadrant q below 2^16).  Beyond, and for Inf and NaN: sin_f64(k * z).
+static __device__ __noinline__ double sin_kz_wide(double k, float k2opi, double z)
 {
     using namespace detail;
     const float xq = __fmul_rn(split_bits(z).h, k2opi);   // ~ k z * 2/pi
@@ -125,39 +206,67 @@ __device__ __forceinline__ double sin_kz(double k, float k2opi, double z)
     return sin_quadrant(r, qi);
 }
 
-// sin and cos of 2 pi a, a in turns (the chromatic phase advance).  Quarter-turn
-// reduction a = n/4 + f: f = a - n/4 is exact (Sterbenz; n from FP32, so |f| may exceed
-// 1/8 by a hair), r = 2 pi f is rounded once, then both polynomials of sin_quadrant on r
-// and the quadrant's swap and signs as integer selects.  19 FP64 operations for the pair.
-// |a| >= 2^20 turns falls back to CUDA's sin and cos.
+static __device__ __noinline__ double sin_wide(double x) { return sin_f64(x); }
+
+// sin(k z) of a phase below one turn: k / 2 pi = kap.K 2^(958 - kap.cn), so that with the
+// significand M and the biased exponent e of z the phase is (M K 2^-64) 2^(-64 - n) turns,
+// n = cn - e.  Below a quarter turn (n >= 2) the product keeps all its 64 bits as the last
+// factor, so the result is as exact relative to itself as to 1 however small z is.  A whole
+// turn or more (a particle that has left the bucket), |k z| below 2^-800, Inf and NaN take
+// the FP64 form; z = 0 (also the unused lanes of a ragged bunch) is returned as it is.
+__device__ __forceinline__ double sin_kz(double k, float k2opi, PhaseScale kap, double z)
+{
+    using namespace detail;
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(z));
+    const uint32_t n = static_cast<uint32_t>(kap.cn - static_cast<int>((hi >> 20) & 0x7ffu));
+    if (n > 800u) return z == 0.0 ? z : sin_kz_wide(k, k2opi, z);
+    const uint64_t p = mulhi_trunc(mantissa64(z), kap.K);
+    const uint64_t U = shr_sat(p, n);
+    const uint64_t s = static_cast<uint64_t>(static_cast<int64_t>(U << 1) >> 63);
+    const bool small = n >= 2u;
+    const uint64_t Q = small ? p : (U << 1) ^ s;
+    return fixed_to_double(mulhi_trunc(Q, sin_poly_fixed((U << 2) ^ s)), small ? static_cast<int>(n) - 1 : 0,
+                           hi ^ static_cast<uint32_t>(U >> 32));
+}
+
+// sin(k z + phi), phi in FP64 and as uphi in 2^-64 turns: the phases are added as fractions
+// of a turn, without rounding.
+__device__ __forceinline__ double sin_kz_phi(double k, PhaseScale kap, double z, double phi, uint64_t uphi)
+{
+    using namespace detail;
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(z));
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    const int n = kap.cn - static_cast<int>(e);
+    if (n < 0 || e == 0u) {
+        if (z != 0.0) return sin_wide(fma(k, z, phi));
+        return sin_turns_fixed(uphi, 0u);
+    }
+    const uint64_t U = shr_sat(mulhi_trunc(mantissa64(z), kap.K), static_cast<uint32_t>(n));
+    return sin_turns_fixed(static_cast<int>(hi) < 0 ? uphi - U : uphi + U, 0u);
+}
+
+// sin and cos of 2 pi a, a in turns (the chromatic phase advance): the fraction of a as 2^-64
+// turns, exact, and two fixed-point sines a quarter turn apart.  |a| >= 2^20 turns, Inf and
+// NaN fall back to CUDA's sin and cos.
+static __device__ __noinline__ void sincos_turns_wide(double a, double& s, double& c)
+{
+    s = sin(detail::kTwoPi * a);
+    c = cos(detail::kTwoPi * a);
+}
+
 __device__ __forceinline__ void sincos_turns(double a, double& s, double& c)
 {
     using namespace detail;
-    const float af = split_bits(a).h;
-    if (!(fabsf(af) < 1048576.0f)) {
-        s = sin(kTwoPi * a);
-        c = cos(kTwoPi * a);
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(a));
+    const int n = 1022 - static_cast<int>((hi >> 20) & 0x7ffu);  // |a| = M 2^(-64 - n)
+    if (n < -20) {
+        sincos_turns_wide(a, s, c);
         return;
     }
-    const float tf = __fmaf_rn(af, 4.0f, kMagic);
-    const int ni = __float_as_int(tf);                       // n mod 2^22
-    const float nf = __fsub_rn(tf, kMagic);
-    const double r = (a - widen_float_bits(__fmul_rn(nf, 0.25f))) * kTwoPi;
-    const double r2 = r * r;
-    double ps = kS(0), pc = kC(0);
-#pragma unroll
-    for (int i = 1; i < 6; ++i) {
-        ps = fma(ps, r2, kS(i));
-        pc = fma(pc, r2, kC(i));
-    }
-    const double sr = fma(r * r2, ps, r);
-    const double cr = fma(r2 * r2, pc, fma(-0.5, r2, 1.0));
-    const bool swap = (ni & 1) != 0;
-    // n mod 4 = 0: (sr, cr); 1: (cr, -sr); 2: (-sr, -cr); 3: (-cr, sr)
-    s = __longlong_as_double(__double_as_longlong(swap ? cr : sr) ^
-                             (static_cast<long long>(ni & 2) << 62));
-    c = __longlong_as_double(__double_as_longlong(swap ? sr : cr) ^
-                             (static_cast<long long>((ni + 1) & 2) << 62));
+    const uint64_t M = mantissa64(a);
+    const uint64_t U = n >= 0 ? shr_sat(M, static_cast<uint32_t>(n)) : shl_sat(M, static_cast<uint32_t>(-n));
+    s = sin_turns_fixed(U, hi);
+    c = sin_turns_fixed(U + 0x4000000000000000ull, 0u);
 }
 
 }  // namespace phtl

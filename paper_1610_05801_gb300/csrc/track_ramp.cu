@@ -5,7 +5,7 @@
 // The same persistent structure as the fixed-machine kernels (Sec. 2.3: turn loop inside
 // the kernel, state in registers, grid-stride over particle chunks), but each turn reads
 // its constants -- eta_n C, A_n, phi_s,n, sin(phi_s,n), r_n = p0_n / p0_{n+1} -- from a
-// device table that the host derived in FP64 (192 bytes per turn, the same address for
+// device table that the host derived in FP64 (200 bytes per turn, the same address for
 // every thread, so the loads are L1 broadcasts).  The next turn's phase constants are
 // loaded while the current turn computes.  After the turn's stages and the transverse
 // rotation, delta and the slopes x', y' are re-expressed against the next turn's reference
@@ -29,6 +29,7 @@ using namespace f64;
 
 struct Turn {
     double phis, sinphis, lin, r;
+    uint64_t uphis;
 };
 
 __device__ __forceinline__ Turn load_turn(const RampTurn* __restrict__ p)
@@ -38,6 +39,7 @@ __device__ __forceinline__ Turn load_turn(const RampTurn* __restrict__ p)
     t.sinphis = __ldg(&p->sinphis);
     t.lin = __ldg(&p->lin);
     t.r = __ldg(&p->r);
+    t.uphis = __ldg(reinterpret_cast<const unsigned long long*>(&p->uphis));
     return t;
 }
 
@@ -56,7 +58,7 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
 {
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        const double f = c.linear ? T.lin * z[p] : sin_f64(fma(c.k, z[p], T.phis)) - T.sinphis;
+        const double f = c.linear ? T.lin * z[p] : sin_kz_phi(c.k, c.kap, z[p], T.phis, T.uphis) - T.sinphis;
         d[p] = fma(kw, f, d[p]);
     }
 }
