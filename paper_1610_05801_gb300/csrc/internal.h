@@ -22,8 +22,7 @@ inline void split_df(double v, float& hi, float& lo)
     lo = static_cast<float>(v - static_cast<double>(hi));
 }
 
-// k / 2 pi for the integer phase of the FP64 sines: K 2^(958 - cn), K with its top bit set
-// (64 significant bits).  cn = kNoPhaseScale (no integer phase) where k is zero or so large or
+// k / 2 pi for the integer phase of the FP64 sines: K 2^(959 - cn), K in [2^62, 2^63).  cn = kNoPhaseScale (no integer phase) where k is zero or so large or
 // small that the exponent arithmetic of the device would leave the range of a double.
 struct PhaseScale {
     uint64_t K;
@@ -55,11 +54,10 @@ inline PhaseScale phase_scale(double k)
         v <<= 1;
         --x;
     }
-    uint64_t K = static_cast<uint64_t>(v >> 64);
-    if ((v >> 63) & 1) ++K;   // round to nearest; a carry out of the top bit cannot occur for
-    if (K == 0) return r;     // a 53-bit k times these digits, and would disable the path
+    const uint64_t K = static_cast<uint64_t>(v >> 65) + (static_cast<uint64_t>(v >> 64) & 1);  // rounded
     const int cn = 1022 - x;
-    if (cn < 900 || cn > 1900) return r;
+    // K = 2^63 (a carry out of the rounding) does not fit the device's products
+    if ((K >> 63) || cn < 900 || cn > 1900) return r;
     r.K = K;
     r.cn = cn;
     return r;

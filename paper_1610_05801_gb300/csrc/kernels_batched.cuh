@@ -50,14 +50,14 @@ __device__ __forceinline__ void run_f64_zs(double (&z)[f64::P], double (&d)[f64:
     int64_t row = g0 / J.stride + 1;
     double g1[4], g2[4];
     if (GEN) f64::slip_stages<SCHEME>(c, g1, g2);
+    f64::TurnWeights w{};
+    if (!GEN) w = f64::turn_weights<SCHEME, true>(J.dc, J.kw, c);
     for (int t = 0; t < nt; ++t) {
         if (GEN) {
             f64::long_turn_nl<SCHEME, ZS>(z, d, c, J.dc, J.kw, J.kw2, g1, g2, c.dual_rf != 0);
             f64::transverse_gen(x, xp, y, yp, d, hx, hy, c);
         } else {
-            f64::long_turn<SCHEME, ZS>(z, d, c, J.dc, J.kw);
-            if (hx) f64::rotate(x, xp, c.mx, c.shx, c.shear_x != 0);
-            if (hy) f64::rotate(y, yp, c.my, c.shy, c.shear_y != 0);
+            f64::long_turn<SCHEME, ZS>(z, d, c, w, f64::RotateBeside<SCHEME>{x, xp, y, yp, hx, hy, c, w});
         }
         if (MON && J.mon) {
             if (--until == 0) {

@@ -32,7 +32,7 @@ using namespace f64;
 template <int SCHEME, bool TRANS, bool MON, bool ZS, bool GEN, bool DUAL>
 __device__ __forceinline__ void turns(double (&z)[P], double (&d)[P], double (&x)[P],
                                       double (&xp)[P], double (&y)[P], double (&yp)[P], bool hx,
-                                      bool hy, float cnt, const MapConsts& c,
+                                      bool hy, float cnt, const MapConsts& c, const TurnWeights& w,
                                       const MonitorArgs& m, int nturns, double* smem, int& parity)
 {
     int64_t until = m.until, row = m.row;
@@ -43,11 +43,10 @@ __device__ __forceinline__ void turns(double (&z)[P], double (&d)[P], double (&x
             long_turn_nl<SCHEME, ZS>(z, d, c, c.dc, c.kw, c.kw2, g1, g2, DUAL);
             if (TRANS) transverse_gen(x, xp, y, yp, d, hx, hy, c);
         } else {
-            long_turn<SCHEME, ZS>(z, d, c, c.dc, c.kw);
-            if (TRANS) {
-                if (hx) rotate(x, xp, c.mx, c.shx, c.shear_x != 0);
-                if (hy) rotate(y, yp, c.my, c.shy, c.shear_y != 0);
-            }
+            if (TRANS)
+                long_turn<SCHEME, ZS>(z, d, c, w, RotateBeside<SCHEME>{x, xp, y, yp, hx, hy, c, w});
+            else
+                long_turn<SCHEME, ZS>(z, d, c, w, NoSideWork{});
         }
         if (MON && m.rows) {
             if (--until == 0) {
@@ -93,6 +92,8 @@ __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
     const int64_t chunk = static_cast<int64_t>(blockDim.x) * P;
     const int64_t nchunks = (L.n + chunk - 1) / chunk;
     int parity = 0;
+    TurnWeights w{};
+    if (!GEN) w = turn_weights<SCHEME, TRANS>(c.dc, c.kw, c);
 
     for (int64_t ci = blockIdx.x; ci < nchunks; ci += gridDim.x) {
         const int64_t base = ci * chunk + static_cast<int64_t>(threadIdx.x) * P;
@@ -117,10 +118,10 @@ __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
             parity ^= 1;
         }
         if (c.phis_zero)
-            turns<SCHEME, TRANS, MON, true, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, m,
+            turns<SCHEME, TRANS, MON, true, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
                                                        L.nturns, smem, parity);
         else
-            turns<SCHEME, TRANS, MON, false, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, m,
+            turns<SCHEME, TRANS, MON, false, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
                                                         L.nturns, smem, parity);
         store2(gz, base, L.n, vec, z);
         store2(gd, base, L.n, vec, d);

@@ -45,6 +45,30 @@ __device__ __forceinline__ double warp_reduce_scatter(double (&f)[NF], int lane)
     return v;
 }
 
+// The same for 64-bit integer partial sums (exact, so the order of the additions is free).
+template <int NF>
+__device__ __forceinline__ int64_t warp_reduce_scatter_int(int64_t (&f)[NF], int lane)
+{
+    static_assert(NF == 8 || NF == 16, "NF must be 8 or 16");
+#pragma unroll
+    for (int o = 16; o >= (NF == 16 ? 2 : 4); o >>= 1) {
+        const int h = (NF == 16) ? (o >> 1) : (o >> 2);
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < NF / 2; ++i) {
+            if (i < h) {
+                const int64_t send = upper ? f[i] : f[i + h];
+                const int64_t keep = upper ? f[i + h] : f[i];
+                f[i] = keep + __shfl_xor_sync(kFullMask, static_cast<long long>(send), o);
+            }
+        }
+    }
+    int64_t v = f[0];
+    if (NF == 8) v += __shfl_xor_sync(kFullMask, static_cast<long long>(v), 2);
+    v += __shfl_xor_sync(kFullMask, static_cast<long long>(v), 1);
+    return v;
+}
+
 // Block-level reduction + atomics into monitor row `row`.
 // smem: 2 * (blockDim.x / 32) * 16 doubles.  nvalid: number of leading fields of the
 // row that may be nonzero (6 = longitudinal only, 16 = with transverse planes).

@@ -39,15 +39,77 @@ constexpr int min_blocks_256()
     return SCHEME == PHTL_RUTH4 ? PHTL_F64_MIN_BLOCKS_256_RUTH4 : PHTL_F64_MIN_BLOCKS_256;
 }
 
-// ZS: phi_s == 0 (stationary bucket): the force is sin(k z), with the phase product fused
-// into the sine's reduction and no subtraction (the kernels choose the instantiation
-// once, outside the turn loop).
-template <bool ZS>
-__device__ __forceinline__ double rf_force(const MapConsts& c, double z)
+// A launch constant held in a register.  An FP64 FMA whose operands all lie in registers takes
+// the pipe 0.50 clocks per lane and SM, one with an operand in the constant bank 0.59 (also
+// DADD and DMUL; measured), so the persistent kernels move the weights of their turn loop to
+// registers.  Through a shuffle, which the compiler does not fold back into the operand.
+__device__ __forceinline__ double in_register(double v)
 {
-    if (c.linear) return c.lin * z;
-    if (ZS) return sin_kz(c.k, c.k2opi, c.kap, z);
-    return sin_kz_phi(c.k, c.kap, z, c.phis, c.uphis) - c.sinphis;
+    return __hiloint2double(__shfl_sync(kFullMask, __double2hiint(v), 0),
+                            __shfl_sync(kFullMask, __double2loint(v), 0));
+}
+
+// Weights of the linear map's turn loop (drifts, kicks, shears of the two planes).
+struct TurnWeights {
+    double dc[4], kw[3], shx[2], shy[2];
+};
+
+template <int SCHEME, bool TRANS>
+__device__ __forceinline__ TurnWeights turn_weights(const double* dc, const double* kw, const MapConsts& c)
+{
+    constexpr int kStages = SCHEME == PHTL_RUTH4 ? 3 : 1;  // kicks; drifts: one more but for Euler-Cromer
+    TurnWeights w{};
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+        if (j < kStages) w.kw[j] = in_register(kw[j]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (i < (SCHEME == PHTL_EULER_CROMER ? 1 : kStages + 1)) w.dc[i] = in_register(-dc[i]);
+    if (TRANS) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            w.shx[i] = in_register(c.shx[i]);
+            w.shy[i] = in_register(c.shy[i]);
+        }
+    }
+    return w;
+}
+
+// Work that a turn runs beside the sines of its kick j, in the same stretch of code without a
+// branch: the sines occupy the integer pipe and the transverse push the FP64 pipe.
+struct NoSideWork {
+    __device__ __forceinline__ void operator()(int) const {}
+};
+
+// The force of the main RF system per unit weight, sin(phi_s + k z) - sin(phi_s) or lin z in
+// rf_linear mode, of the thread's P particles.  ZS: phi_s == 0 (stationary bucket), the force
+// is sin(k z) alone (the kernels choose the instantiation once, outside the turn loop).
+template <bool ZS, class Side>
+__device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[P], double (&f)[P],
+                                         const Side& side, int j)
+{
+    if (c.linear) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) f[p] = c.lin * z[p];
+        side(j);
+        return;
+    }
+    bool ok[P], all = true;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        f[p] = ZS ? sin_kz_fixed(c.kap, z[p], ok[p]) : sin_kz_phi_fixed(c.kap, z[p], c.uphis, ok[p]);
+        all = all && ok[p];
+    }
+    side(j);
+    if (!all) {
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            if (!ok[p]) f[p] = ZS ? sin_kz_rest(c.k, c.k2opi, z[p]) : sin_wide(fma(c.k, z[p], c.phis));
+    }
+    if (!ZS) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) f[p] -= c.sinphis;
+    }
 }
 
 __device__ __forceinline__ void drift(double (&z)[P], const double (&d)[P], double dc)
@@ -56,36 +118,45 @@ __device__ __forceinline__ void drift(double (&z)[P], const double (&d)[P], doub
     for (int p = 0; p < P; ++p) z[p] = fma(-dc, d[p], z[p]);
 }
 
-template <bool ZS>
-__device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], double kw,
-                                     const MapConsts& c)
+// The same with the weight negated beforehand.
+__device__ __forceinline__ void drift_neg(double (&z)[P], const double (&d)[P], double ndc)
 {
 #pragma unroll
-    for (int p = 0; p < P; ++p) d[p] = fma(kw, rf_force<ZS>(c, z[p]), d[p]);
+    for (int p = 0; p < P; ++p) z[p] = fma(ndc, d[p], z[p]);
+}
+
+template <bool ZS, class Side>
+__device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], double kw,
+                                     const MapConsts& c, const Side& side, int j)
+{
+    double f[P];
+    rf_force<ZS>(c, z, f, side, j);
+#pragma unroll
+    for (int p = 0; p < P; ++p) d[p] = fma(kw, f[p], d[p]);
 }
 
 // One turn of the scheme; stage order as in Sec. 1.1.2's readings (see phtl.h).
-// dc, kw: the drift and kick weights of this bunch's scheme (w_i eta C, w_j A); the
-// single-bunch kernel passes c.dc, c.kw, the batched kernel the job table's copies.
-template <int SCHEME, bool ZS>
+// w: the drift (negated) and kick weights of this bunch's scheme, -w_i eta C and w_j A.
+// side: work beside the kicks' sines that touches neither z nor delta.
+template <int SCHEME, bool ZS, class Side>
 __device__ __forceinline__ void long_turn(double (&z)[P], double (&d)[P], const MapConsts& c,
-                                          const double* dc, const double* kw)
+                                          const TurnWeights& w, const Side& side)
 {
     if (SCHEME == PHTL_EULER_CROMER) {
-        kick<ZS>(z, d, kw[0], c);
-        drift(z, d, dc[0]);
+        kick<ZS>(z, d, w.kw[0], c, side, 0);
+        drift_neg(z, d, w.dc[0]);
     } else if (SCHEME == PHTL_LEAPFROG) {
-        drift(z, d, dc[0]);
-        kick<ZS>(z, d, kw[0], c);
-        drift(z, d, dc[1]);
+        drift_neg(z, d, w.dc[0]);
+        kick<ZS>(z, d, w.kw[0], c, side, 0);
+        drift_neg(z, d, w.dc[1]);
     } else {
-        drift(z, d, dc[0]);
-        kick<ZS>(z, d, kw[0], c);
-        drift(z, d, dc[1]);
-        kick<ZS>(z, d, kw[1], c);
-        drift(z, d, dc[2]);
-        kick<ZS>(z, d, kw[2], c);
-        drift(z, d, dc[3]);
+        drift_neg(z, d, w.dc[0]);
+        kick<ZS>(z, d, w.kw[0], c, side, 0);
+        drift_neg(z, d, w.dc[1]);
+        kick<ZS>(z, d, w.kw[1], c, side, 1);
+        drift_neg(z, d, w.dc[2]);
+        kick<ZS>(z, d, w.kw[2], c, side, 2);
+        drift_neg(z, d, w.dc[3]);
     }
 }
 
@@ -112,6 +183,24 @@ __device__ __forceinline__ void rotate(double (&u)[P], double (&v)[P], const dou
     }
 }
 
+// The linear map's transverse push as the side work of a turn's kicks: both planes beside the
+// only kick, or x beside Ruth4's first and y beside its second.
+template <int SCHEME>
+struct RotateBeside {
+    double (&x)[P];
+    double (&xp)[P];
+    double (&y)[P];
+    double (&yp)[P];
+    bool hx, hy;
+    const MapConsts& c;
+    const TurnWeights& w;
+    __device__ __forceinline__ void operator()(int j) const
+    {
+        if (j == 0 && hx) rotate(x, xp, c.mx, w.shx, c.shear_x != 0);
+        if (j == (SCHEME == PHTL_RUTH4 ? 1 : 0) && hy) rotate(y, yp, c.my, w.shy, c.shear_y != 0);
+    }
+};
+
 // ---- widened map: nonlinear slippage and chromaticity -------------------------------
 
 // Drift with the slippage expansion: z -= (dc + g1 d + g2 d^2) d for this stage's
@@ -129,10 +218,26 @@ __device__ __forceinline__ void drift_nl(double (&z)[P], const double (&d)[P], d
 
 // Force of the second RF system (double RF) per unit weight: sin(phi2 + k2 z) - sin(phi2),
 // or cos(phi2) k2 z in rf_linear mode.
-__device__ __forceinline__ double rf_force2(const MapConsts& c, double z)
+__device__ __forceinline__ void rf_force2(const MapConsts& c, const double (&z)[P], double (&f)[P])
 {
-    if (c.linear) return c.lin2 * z;
-    return sin_kz_phi(c.k2, c.kap2, z, c.phi2, c.uphi2) - c.sinphi2;
+    if (c.linear) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) f[p] = c.lin2 * z[p];
+        return;
+    }
+    bool ok[P], all = true;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        f[p] = sin_kz_phi_fixed(c.kap2, z[p], c.uphi2, ok[p]);
+        all = all && ok[p];
+    }
+    if (!all) {
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            if (!ok[p]) f[p] = sin_wide(fma(c.k2, z[p], c.phi2));
+    }
+#pragma unroll
+    for (int p = 0; p < P; ++p) f[p] -= c.sinphi2;
 }
 
 // Kick of the widened map: the main RF system, then the second one when `dual` (a
@@ -142,10 +247,12 @@ template <bool ZS>
 __device__ __forceinline__ void kick_gen(const double (&z)[P], double (&d)[P], double kw, double kw2,
                                          const MapConsts& c, bool dual)
 {
+    kick<ZS>(z, d, kw, c, NoSideWork{}, 0);
+    if (dual) {
+        double f[P];
+        rf_force2(c, z, f);
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        d[p] = fma(kw, rf_force<ZS>(c, z[p]), d[p]);
-        if (dual) d[p] = fma(kw2, rf_force2(c, z[p]), d[p]);
+        for (int p = 0; p < P; ++p) d[p] = fma(kw2, f[p], d[p]);
     }
 }
 
@@ -153,18 +260,27 @@ __device__ __forceinline__ void kick_gen(const double (&z)[P], double (&d)[P], d
 // dz/dn = -eta(d) C d = -(dc + g1 d + g2 d^2) d and dd/dn = kw F1(z) + kw2 F2(z), with
 // dc = eta0 C, g1 = eta1 C, g2 = eta2 C, kw = A, kw2 = A2.
 template <bool ZS>
-__device__ __forceinline__ void rk4_rhs(double z, double d, const MapConsts& c, double dc, double g1,
-                                        double g2, double kw, double kw2, bool dual, double& fz,
-                                        double& fd)
+__device__ __forceinline__ void rk4_rhs(const double (&z)[P], const double (&d)[P], const MapConsts& c,
+                                        double dc, double g1, double g2, double kw, double kw2, bool dual,
+                                        double (&fz)[P], double (&fd)[P])
 {
     // the products are rounded on their own (__dmul_rn): the stage arguments and the
     // weighted sum reuse them, and an FMA contraction chosen differently where `dual` is a
     // compile-time constant than where it is not would break the bitwise agreement of the
     // single-bunch and batched kernels
-    const double e = fma(fma(g2, d, g1), d, dc);
-    fz = -__dmul_rn(e, d);
-    fd = __dmul_rn(kw, rf_force<ZS>(c, z));
-    if (dual) fd = fma(kw2, rf_force2(c, z), fd);
+    double f[P];
+    rf_force<ZS>(c, z, f, NoSideWork{}, 0);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const double e = fma(fma(g2, d[p], g1), d[p], dc);
+        fz[p] = -__dmul_rn(e, d[p]);
+        fd[p] = __dmul_rn(kw, f[p]);
+    }
+    if (dual) {
+        rf_force2(c, z, f);
+#pragma unroll
+        for (int p = 0; p < P; ++p) fd[p] = fma(kw2, f[p], fd[p]);
+    }
 }
 
 // One classic RK4 step of one turn: k1 at the start, k2 and k3 at the half step from k1
@@ -175,15 +291,30 @@ __device__ __forceinline__ void rk4_turn(double (&z)[P], double (&d)[P], const M
                                          bool dual)
 {
     constexpr double kSixth = 1.0 / 6.0;
+    double k1z[P], k1d[P], k2z[P], k2d[P], k3z[P], k3d[P], k4z[P], k4d[P], a[P], b[P];
+    rk4_rhs<ZS>(z, d, c, dc, g1, g2, kw, kw2, dual, k1z, k1d);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        double k1z, k1d, k2z, k2d, k3z, k3d, k4z, k4d;
-        rk4_rhs<ZS>(z[p], d[p], c, dc, g1, g2, kw, kw2, dual, k1z, k1d);
-        rk4_rhs<ZS>(fma(0.5, k1z, z[p]), fma(0.5, k1d, d[p]), c, dc, g1, g2, kw, kw2, dual, k2z, k2d);
-        rk4_rhs<ZS>(fma(0.5, k2z, z[p]), fma(0.5, k2d, d[p]), c, dc, g1, g2, kw, kw2, dual, k3z, k3d);
-        rk4_rhs<ZS>(__dadd_rn(z[p], k3z), __dadd_rn(d[p], k3d), c, dc, g1, g2, kw, kw2, dual, k4z, k4d);
-        z[p] = fma(fma(2.0, __dadd_rn(k2z, k3z), __dadd_rn(k1z, k4z)), kSixth, z[p]);
-        d[p] = fma(fma(2.0, __dadd_rn(k2d, k3d), __dadd_rn(k1d, k4d)), kSixth, d[p]);
+        a[p] = fma(0.5, k1z[p], z[p]);
+        b[p] = fma(0.5, k1d[p], d[p]);
+    }
+    rk4_rhs<ZS>(a, b, c, dc, g1, g2, kw, kw2, dual, k2z, k2d);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        a[p] = fma(0.5, k2z[p], z[p]);
+        b[p] = fma(0.5, k2d[p], d[p]);
+    }
+    rk4_rhs<ZS>(a, b, c, dc, g1, g2, kw, kw2, dual, k3z, k3d);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        a[p] = __dadd_rn(z[p], k3z[p]);
+        b[p] = __dadd_rn(d[p], k3d[p]);
+    }
+    rk4_rhs<ZS>(a, b, c, dc, g1, g2, kw, kw2, dual, k4z, k4d);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        z[p] = fma(fma(2.0, __dadd_rn(k2z[p], k3z[p]), __dadd_rn(k1z[p], k4z[p])), kSixth, z[p]);
+        d[p] = fma(fma(2.0, __dadd_rn(k2d[p], k3d[p]), __dadd_rn(k1d[p], k4d[p])), kSixth, d[p]);
     }
 }
 
@@ -256,32 +387,103 @@ __device__ __forceinline__ void transverse_gen(double (&x)[P], double (&xp)[P], 
     }
 }
 
-// Per-thread moment contributions of one plane (a, b): sum a, sum b, sum a^2, sum b^2,
-// sum ab over this thread's P particles, as double-float pairs.  The doubles are split
-// into float pairs with integer operations and the products formed with the exact FP32
-// product error, so the sums keep ~47 bits without using the FP64 pipe.
-__device__ __forceinline__ void pair_sums_df(const double (&a)[P], const double (&b)[P], DF2* f)
+// ---- moments: exact integer sums per warp ------------------------------------------------
+//
+// A coordinate's values are brought to the warp's common exponent E (the largest biased
+// exponent among its lanes, at least 128 so that a zero's significand shifts out) as 57-bit
+// integers X, a = X 2^(E + kMomentShift - 1086): no bit of a value within 2^-4 of the largest
+// is lost.  The sums of X, X^2 and X Y over the thread's particles and the warp's lanes are
+// 64-bit integer additions, and each is converted to FP64 once.  The squares are products of
+// the magnitudes rounded down, so a single particle's variance does not come out positive.
+//
+// The double-float sums before these took ~590 instructions per particle and record with both
+// planes (bit splits, TwoSum and Fast2Sum in every addition); these take ~240.
+constexpr int kMomentShift = P <= 2 ? 7 : 8;     // P 32 values of X add up below 2^63
+constexpr int kMomentProductBits = P <= 2 ? 6 : 7;  // fraction bits kept of X Y 2^-64
+
+struct PlaneExponents {
+    int a, b;  // the warp's exponents of the plane's two coordinates
+};
+
+// High words without the sign: ordered as the magnitudes are.
+__device__ __forceinline__ int warp_exponent(const double (&a)[P])
 {
-    DF2 ap = split_bits(a[0]), bp = split_bits(b[0]);
-    f[0] = ap;
-    f[1] = bp;
-    f[2] = df_mul(ap, ap);
-    f[3] = df_mul(bp, bp);
-    f[4] = df_mul(ap, bp);
+    unsigned m = 0u;
 #pragma unroll
-    for (int p = 1; p < P; ++p) {
-        ap = split_bits(a[p]);
-        bp = split_bits(b[p]);
-        f[0] = df_add(f[0], ap);
-        f[1] = df_add(f[1], bp);
-        f[2] = df_add(f[2], df_mul(ap, ap));
-        f[3] = df_add(f[3], df_mul(bp, bp));
-        f[4] = df_add(f[4], df_mul(ap, bp));
+    for (int p = 0; p < P; ++p) m = max(m, static_cast<unsigned>(__double2hiint(a[p])) & 0x7fffffffu);
+    return max(static_cast<int>(__reduce_max_sync(kFullMask, m) >> 20), 128);
+}
+
+// |a| in units of 2^(E + kMomentShift - 1086), and the sign as a mask.
+__device__ __forceinline__ uint64_t moment_magnitude(double a, int E, uint32_t& neg)
+{
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(a));
+    neg = static_cast<uint32_t>(static_cast<int32_t>(hi) >> 31);
+    return detail::shr_sat(detail::mantissa64(a),
+                           static_cast<uint32_t>(E + kMomentShift) - ((hi >> 20) & 0x7ffu));
+}
+
+__device__ __forceinline__ int64_t moment_signed(uint64_t X, uint32_t neg)
+{
+    const uint64_t m = static_cast<uint64_t>(neg) << 32 | neg;
+    return static_cast<int64_t>((X ^ m) - m);
+}
+
+// Sums of one plane (a, b) over the thread's particles: a, b (units of X), a^2, b^2 and ab
+// (units of X Y 2^(kMomentProductBits - 64)).
+__device__ __forceinline__ void pair_sums_fixed(const double (&a)[P], const double (&b)[P],
+                                                PlaneExponents E, int64_t* f)
+{
+    uint64_t aa = 0, aac = 0, bb = 0, bbc = 0;
+    int64_t ab = 0, abc = 0;
+    f[0] = f[1] = 0;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        uint32_t na, nb;
+        const uint64_t A = moment_magnitude(a[p], E.a, na), B = moment_magnitude(b[p], E.b, nb);
+        const uint32_t a1 = static_cast<uint32_t>(A >> 32), a0 = static_cast<uint32_t>(A);
+        const uint32_t b1 = static_cast<uint32_t>(B >> 32), b0 = static_cast<uint32_t>(B);
+        aa += static_cast<uint64_t>(a1) * a1;     // A^2 = aa 2^64 + 2 aac 2^32 + (below 2^64)
+        aac += static_cast<uint64_t>(a1) * a0;
+        bb += static_cast<uint64_t>(b1) * b1;
+        bbc += static_cast<uint64_t>(b1) * b0;
+        const int64_t As = moment_signed(A, na), Bs = moment_signed(B, nb);
+        f[0] += As;
+        f[1] += Bs;
+        const int32_t as1 = static_cast<int32_t>(As >> 32), bs1 = static_cast<int32_t>(Bs >> 32);
+        const int32_t ah = static_cast<int32_t>(static_cast<uint32_t>(As) >> 1);
+        const int32_t bh = static_cast<int32_t>(static_cast<uint32_t>(Bs) >> 1);
+        ab += static_cast<int64_t>(as1) * bs1;    // A B = ab 2^64 + abc 2^33 + ...
+        abc += static_cast<int64_t>(as1) * bh;
+        abc += static_cast<int64_t>(bs1) * ah;
     }
+    constexpr int q = kMomentProductBits;
+    f[2] = static_cast<int64_t>((aa << q) + (aac >> (31 - q)));
+    f[3] = static_cast<int64_t>((bb << q) + (bbc >> (31 - q)));
+    f[4] = (ab << q) + (abc >> (31 - q));
+}
+
+// S 2^x in FP64, rounded to nearest; beyond its range 0 or Inf.
+__device__ __forceinline__ double scaled_to_double(int64_t S, int x)
+{
+    const uint64_t a = static_cast<uint64_t>(S < 0 ? -S : S);
+    const int c = __clzll(static_cast<long long>(a));
+    const uint64_t N = detail::shl_sat(a, static_cast<uint32_t>(c));
+    const uint64_t r = (N >> 11) + ((N >> 10) & 1u);
+    const int e = 1085 - c + x;  // biased exponent less the leading one of r
+    uint32_t hi = static_cast<uint32_t>(r >> 32) + (static_cast<uint32_t>(e) << 20);
+    uint32_t lo = static_cast<uint32_t>(r);
+    if (a == 0 || e < 0) hi = lo = 0u;
+    if (e > 2045 && a != 0) {
+        hi = 0x7ff00000u;
+        lo = 0u;
+    }
+    return __hiloint2double(static_cast<int>(hi | (static_cast<uint32_t>(S >> 32) & 0x80000000u)),
+                            static_cast<int>(lo));
 }
 
 // Add this block's moment sums of the current turn into monitor row `row`.
-// smem: 2 * (blockDim.x / 32) * 16 DF2.
+// smem: 2 * (blockDim.x / 32) * 16 doubles.
 template <bool TRANS>
 __device__ __forceinline__ void record(const double (&z)[P], const double (&d)[P],
                                        const double (&x)[P], const double (&xp)[P],
@@ -290,28 +492,57 @@ __device__ __forceinline__ void record(const double (&z)[P], const double (&d)[P
                                        double* rows, int64_t row)
 {
     constexpr int NF = TRANS ? 16 : 8;
-    const DF2 zero{0.0f, 0.0f};
-    DF2 f[NF];
-    f[0] = DF2{cnt, 0.0f};  // 0..P: exact
-    pair_sums_df(z, d, f + 1);
+    constexpr int kShift = TRANS ? 1 : 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int field = lane >> kShift;  // the field whose total this lane ends up with
+    int64_t f[NF];
+    f[0] = static_cast<int64_t>(static_cast<int>(cnt));
+    PlaneExponents E{warp_exponent(z), warp_exponent(d)}, Ef = E;
+    int k = field - 1;                 // 0..4: a, b, a^2, b^2, ab of the plane Ef
+    pair_sums_fixed(z, d, E, f + 1);
     if constexpr (TRANS) {
         if (hx) {
-            pair_sums_df(x, xp, f + 6);
+            E = PlaneExponents{warp_exponent(x), warp_exponent(xp)};
+            pair_sums_fixed(x, xp, E, f + 6);
+            if (field >= 6 && field < 11) Ef = E;
         } else {
 #pragma unroll
-            for (int j = 6; j < 11; ++j) f[j] = zero;
+            for (int j = 6; j < 11; ++j) f[j] = 0;
         }
         if (hy) {
-            pair_sums_df(y, yp, f + 11);
+            E = PlaneExponents{warp_exponent(y), warp_exponent(yp)};
+            pair_sums_fixed(y, yp, E, f + 11);
+            if (field >= 11) Ef = E;
         } else {
 #pragma unroll
-            for (int j = 11; j < 16; ++j) f[j] = zero;
+            for (int j = 11; j < 16; ++j) f[j] = 0;
         }
+        k -= field >= 11 ? 10 : (field >= 6 ? 5 : 0);
     } else {
-        f[6] = zero;
-        f[7] = zero;
+        f[6] = f[7] = 0;
     }
-    block_record_df<NF>(f, reinterpret_cast<DF2*>(smem), parity, rows, row, TRANS ? 16 : 6);
+    const int64_t total = warp_reduce_scatter_int<NF>(f, lane);
+    double v;
+    if (field == 0) {
+        v = static_cast<double>(static_cast<int>(total));
+    } else {
+        // units: X of a plane's coordinate 2^(E + kMomentShift - 1086), products of two such
+        // less the 64 - kMomentProductBits bits taken off
+        const int e1 = k == 1 || k == 3 ? Ef.b : Ef.a;
+        const int e2 = k == 3 || k == 4 ? Ef.b : Ef.a;
+        v = scaled_to_double(total, k < 2 ? e1 + kMomentShift - 1086
+                                          : e1 + e2 + 2 * (kMomentShift - 1086) + 64 - kMomentProductBits);
+        // Inf or NaN among the warp's values
+        if (e1 == 2047 || (k >= 2 && e2 == 2047)) v = __hiloint2double(0x7ff80000, 0);
+    }
+    double* buf = smem + parity * (nwarps * 16);
+    if ((lane & ((1 << kShift) - 1)) == 0) buf[warp * 16 + field] = v;
+    __syncthreads();
+    if (warp == 0 && lane < (TRANS ? 16 : 6)) {
+        double s = buf[lane];
+        for (int w = 1; w < nwarps; ++w) s += buf[w * 16 + lane];
+        atomicAdd(rows + row * PHTL_MON_FIELDS + lane, s);
+    }
 }
 
 // 128-bit accesses only where the host allowed them (vec) AND the address really is

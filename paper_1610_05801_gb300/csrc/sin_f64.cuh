@@ -57,15 +57,18 @@ __device__ __forceinline__ double sc_coef(bool odd, double s, double c) { return
 // ---- sines on the integer pipe ---------------------------------------------------------
 //
 // An FP64 instruction takes the FP64 pipe half a clock per lane (2 per clock per SM), as long
-// as 64 issue slots of the other pipes, so a kick's sine costs less as ~90 integer
-// instructions than as 11 FP64 ones.  The phase is a 64-bit binary fraction of a turn (its
-// overflow is the reduction modulo 2 pi, and no fold is ever rounded), the sine one unsigned
-// fixed-point polynomial
+// as 64 issue slots of the other pipes, so a kick's sine costs less as ~80 integer
+// instructions than as 11 FP64 ones.  The phase is a 64-bit binary fraction (its overflow is
+// the reduction modulo 2 pi, and no fold is ever rounded), the sine one unsigned fixed-point
+// polynomial
 //     sin(pi V) = V p(rho),   rho = (2 V)^2 in [0, 1],   V in [0, 1/2] half turns,
 // p of degree 8 (Chebyshev interpolation at 60 digits, gen_sin_coeffs.py --fixed; error 2e-19
 // of p): the upper five steps in 64 bits, the three last terms (below 1.2e-7) in 32.  The
-// result is normalised and rounded to FP64 once: |error| <= 0.66 2^-53 over the range, where
+// result is normalised and rounded to FP64 once: |error| <= 0.7 2^-53 over the range, where
 // the FP64 polynomial has about 1.
+//
+// The multiplications bound it: a 32 x 32 product, high half or wide, issues at 32 lanes per
+// clock per SM (against 64 for shifts and logic, 128 for adds), and there are 26 of them.
 
 // High 64 bits of a 128-bit product, short of it by at most 2 (the low product and the carry
 // of the low halves are left out).
@@ -74,6 +77,14 @@ __device__ __forceinline__ uint64_t mulhi_trunc(uint64_t a, uint64_t b)
     const uint32_t a1 = static_cast<uint32_t>(a >> 32), a0 = static_cast<uint32_t>(a);
     const uint32_t b1 = static_cast<uint32_t>(b >> 32), b0 = static_cast<uint32_t>(b);
     return static_cast<uint64_t>(a1) * b1 + __umulhi(a1, b0) + __umulhi(a0, b1);
+}
+
+// The same for a, b < 2^63: the two cross terms add up in 32 bits.
+__device__ __forceinline__ uint64_t mulhi_trunc63(uint64_t a, uint64_t b)
+{
+    const uint32_t a1 = static_cast<uint32_t>(a >> 32), a0 = static_cast<uint32_t>(a);
+    const uint32_t b1 = static_cast<uint32_t>(b >> 32), b0 = static_cast<uint32_t>(b);
+    return static_cast<uint64_t>(a1) * b1 + (__umulhi(a1, b0) + __umulhi(a0, b1));
 }
 
 // 64-bit shifts whose amount saturates (0 for 64 and more), as the hardware's do.
@@ -97,43 +108,58 @@ __device__ __forceinline__ uint64_t mantissa64(double x)
     return (static_cast<uint64_t>(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
 }
 
-// p(rho) 2^62, rho = R^2 2^-128 (see above): R = 2 V.
-__device__ __forceinline__ uint64_t sin_poly_fixed(uint64_t R)
+// A phase in half turns (2^-64) folded to [0, 1/2]: sin(pi V) = sin(pi (1 - V)).
+__device__ __forceinline__ uint64_t fold_half_turn(uint64_t V)
 {
-    const uint64_t T = mulhi_trunc(R, R);
-    const uint32_t t = static_cast<uint32_t>(T >> 32);
-    uint32_t q = 0x02DEF59Bu - __umulhi(t, 0x00067519u);          // c7, c8 (2^55)
-    q = 0xF479B3AFu - __umulhi(t, q);                              // c6
-    uint64_t p = 0x00001E3074DFAF88ull - ((static_cast<uint64_t>(t) * q) >> 25);  // c5 (2^62)
-    p = 0x000541E0D2154615ull - mulhi_trunc(T, p);
-    p = 0x009969667313E42Full - mulhi_trunc(T, p);
-    p = 0x0A335E33BAD53E48ull - mulhi_trunc(T, p);
-    p = 0x52AEF39896F94915ull - mulhi_trunc(T, p);
-    return 0xC90FDAA22168C232ull - mulhi_trunc(T, p);              // pi
+    const uint32_t s = static_cast<uint32_t>(static_cast<int32_t>(V >> 32) >> 31);
+    return V ^ (static_cast<uint64_t>(s) << 32 | s);
 }
 
-// S 2^(-62 - x) as a double with the sign bit of `sign`, rounded to nearest (ties up).
+// p(rho) 2^60 of V in [0, 1/2] half turns (2^-64).  rho is kept as 2^62 rho = hi64(V V), so
+// each 64-bit Horner step comes down by four in scale: c5 at 2^70, ..., pi at 2^60.
+__device__ __forceinline__ uint64_t sin_poly_fixed(uint64_t V)
+{
+    const uint64_t T = mulhi_trunc63(V, V);
+    const uint32_t t = static_cast<uint32_t>(T >> 30);             // rho 2^32
+    uint32_t q = 0x02DEF59Bu - __umulhi(t, 0x00067519u);          // c7 and c8 (2^55)
+    q = 0xF479B3AFu - __umulhi(t, q);                              // c6
+    uint64_t p = 0x001E3074DFAF87AFull - ((static_cast<uint64_t>(t) * q) >> 17);  // c5 (2^70)
+    p = 0x015078348551853Bull - mulhi_trunc63(T, p);
+    p = 0x09969667313E42F1ull - mulhi_trunc63(T, p);
+    p = 0x28CD78CEEB54F91Eull - mulhi_trunc63(T, p);
+    p = 0x52AEF39896F94915ull - mulhi_trunc63(T, p);
+    return 0x3243F6A8885A308Cull - mulhi_trunc63(T, p);            // pi
+}
+
+// S 2^(-60 - x) as a double with the sign bit of `sign`, rounded to nearest (ties up), for
+// S >= 2^32.
 __device__ __forceinline__ double fixed_to_double(uint64_t S, int x, uint32_t sign)
 {
-    if (static_cast<uint32_t>(S >> 32) == 0u) {  // near a zero of the sine: at most 32 bits left
-        if (S == 0) return __hiloint2double(static_cast<int>(sign & 0x80000000u), 0);
-        S <<= 32;
-        x += 32;
-    }
     const int c = __clz(static_cast<int>(S >> 32));
     const uint64_t N = shl_sat(S, static_cast<uint32_t>(c));   // leading one at bit 63
     const uint64_t r = (N >> 11) + ((N >> 10) & 1u);            // the leading one adds 1 to the exponent
-    const uint32_t hi = static_cast<uint32_t>(r >> 32) + (static_cast<uint32_t>(1023 - c - x) << 20);
+    const uint32_t hi = static_cast<uint32_t>(r >> 32) + (static_cast<uint32_t>(1025 - c - x) << 20);
     return __hiloint2double(static_cast<int>(hi | (sign & 0x80000000u)), static_cast<int>(static_cast<uint32_t>(r)));
 }
 
-// sin(2 pi U) of a phase U in 2^-64 turns; `flip`: its top bit flips the sign.
-__device__ __forceinline__ double sin_turns_fixed(uint64_t U, uint32_t flip)
+// sin(2 pi U), U in 2^-64 turns, with the sign flipped where bit 31 of `flip` is set.  ok is
+// cleared within 2^-31 of a zero, where the result does not fill the significand.
+__device__ __forceinline__ double sin_turns_fixed(uint64_t U, uint32_t flip, bool& ok)
 {
-    const uint64_t s = static_cast<uint64_t>(static_cast<int64_t>(U << 1) >> 63);
-    const uint64_t V = (U << 1) ^ s;                              // folded into [0, 1/2] half turns
-    return fixed_to_double(mulhi_trunc(V, sin_poly_fixed((U << 2) ^ s)), 0,
-                           static_cast<uint32_t>(U >> 32) ^ flip);
+    const uint64_t V = fold_half_turn(U << 1);
+    const uint64_t S = mulhi_trunc63(V, sin_poly_fixed(V));
+    ok = ok && (S >> 32) != 0u;
+    return fixed_to_double(S, 0, static_cast<uint32_t>(U >> 32) ^ flip);
+}
+
+// The same with every U valid: 0 at a zero of the sine, fewer significant bits next to one.
+__device__ __forceinline__ double sin_turns_any(uint64_t U, uint32_t flip)
+{
+    const uint64_t V = fold_half_turn(U << 1);
+    const uint64_t S = mulhi_trunc63(V, sin_poly_fixed(V));
+    const bool low = (S >> 32) == 0u;
+    const double r = fixed_to_double(low ? S << 32 : S, low ? 32 : 0, static_cast<uint32_t>(U >> 32) ^ flip);
+    return S == 0u ? 0.0 : r;
 }
 
 // sin(q pi/2 + r) for |r| <= pi/4 (a hair more when q came out one off), given the low
@@ -208,41 +234,47 @@ static __device__ __noinline__ double sin_kz_wide(double k, float k2opi, double 
 
 static __device__ __noinline__ double sin_wide(double x) { return sin_f64(x); }
 
-// sin(k z) of a phase below one turn: k / 2 pi = kap.K 2^(958 - kap.cn), so that with the
-// significand M and the biased exponent e of z the phase is (M K 2^-64) 2^(-64 - n) turns,
-// n = cn - e.  Below a quarter turn (n >= 2) the product keeps all its 64 bits as the last
-// factor, so the result is as exact relative to itself as to 1 however small z is.  A whole
-// turn or more (a particle that has left the bucket), |k z| below 2^-800, Inf and NaN take
-// the FP64 form; z = 0 (also the unused lanes of a ragged bunch) is returned as it is.
-__device__ __forceinline__ double sin_kz(double k, float k2opi, PhaseScale kap, double z)
+// The kicks take the integer sine of all their particles first, without a branch in between
+// (the particles' chains and the FP64 work beside them overlap), and then mend the few that
+// it does not cover: `ok` is cleared for those.
+
+// sin(k z) of a phase below one turn: k / 2 pi = kap.K 2^(959 - kap.cn), so that with the
+// significand M and the biased exponent e of z the phase is (M K 2^-64) 2^(-63 - n) turns,
+// n = cn - e (n >= 0 for every phase below half a turn).  Below a quarter turn (n >= 2) the product keeps all its bits as the last
+// factor, so the result is as exact relative to itself as to 1 however small z is.  Not
+// covered: z = 0, n < 0 (a particle that has left the bucket), |k z| below 2^-800, a phase within 1e-9 of a half turn, Inf and NaN.
+__device__ __forceinline__ double sin_kz_fixed(PhaseScale kap, double z, bool& ok)
 {
     using namespace detail;
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(z));
     const uint32_t n = static_cast<uint32_t>(kap.cn - static_cast<int>((hi >> 20) & 0x7ffu));
-    if (n > 800u) return z == 0.0 ? z : sin_kz_wide(k, k2opi, z);
     const uint64_t p = mulhi_trunc(mantissa64(z), kap.K);
-    const uint64_t U = shr_sat(p, n);
-    const uint64_t s = static_cast<uint64_t>(static_cast<int64_t>(U << 1) >> 63);
+    const uint64_t W = shr_sat(p, n);                             // 2^-63 turns
+    const uint64_t V = fold_half_turn(W << 2);
     const bool small = n >= 2u;
-    const uint64_t Q = small ? p : (U << 1) ^ s;
-    return fixed_to_double(mulhi_trunc(Q, sin_poly_fixed((U << 2) ^ s)), small ? static_cast<int>(n) - 1 : 0,
-                           hi ^ static_cast<uint32_t>(U >> 32));
+    const uint64_t S = mulhi_trunc63(small ? p : V, sin_poly_fixed(V));
+    ok = n <= 800u && (S >> 32) != 0u;
+    return fixed_to_double(S, small ? static_cast<int>(n) - 2 : 0, hi ^ static_cast<uint32_t>(W >> 31));
 }
 
-// sin(k z + phi), phi in FP64 and as uphi in 2^-64 turns: the phases are added as fractions
-// of a turn, without rounding.
-__device__ __forceinline__ double sin_kz_phi(double k, PhaseScale kap, double z, double phi, uint64_t uphi)
+// sin(k z) where sin_kz_fixed does not cover it.
+__device__ __forceinline__ double sin_kz_rest(double k, float k2opi, double z)
+{
+    return z == 0.0 ? z : sin_kz_wide(k, k2opi, z);
+}
+
+// sin(k z + phi), phi as uphi in 2^-64 turns: the phases are added as fractions of a turn,
+// without rounding.  Not covered: n < -1 (never below one turn of k z), a denormal z, a total phase within
+// 1e-9 of a half turn, Inf and NaN.
+__device__ __forceinline__ double sin_kz_phi_fixed(PhaseScale kap, double z, uint64_t uphi, bool& ok)
 {
     using namespace detail;
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(z));
     const uint32_t e = (hi >> 20) & 0x7ffu;
-    const int n = kap.cn - static_cast<int>(e);
-    if (n < 0 || e == 0u) {
-        if (z != 0.0) return sin_wide(fma(k, z, phi));
-        return sin_turns_fixed(uphi, 0u);
-    }
-    const uint64_t U = shr_sat(mulhi_trunc(mantissa64(z), kap.K), static_cast<uint32_t>(n));
-    return sin_turns_fixed(static_cast<int>(hi) < 0 ? uphi - U : uphi + U, 0u);
+    const uint32_t n1 = static_cast<uint32_t>(kap.cn + 1 - static_cast<int>(e));  // n + 1: from n = -1 on
+    const uint64_t U = shr_sat(mulhi_trunc(mantissa64(z), kap.K), n1) << 2;
+    ok = n1 <= 2047u && (e != 0u || z == 0.0);
+    return sin_turns_fixed(static_cast<int>(hi) < 0 ? uphi - U : uphi + U, 0u, ok);
 }
 
 // sin and cos of 2 pi a, a in turns (the chromatic phase advance): the fraction of a as 2^-64
@@ -265,8 +297,8 @@ __device__ __forceinline__ void sincos_turns(double a, double& s, double& c)
     }
     const uint64_t M = mantissa64(a);
     const uint64_t U = n >= 0 ? shr_sat(M, static_cast<uint32_t>(n)) : shl_sat(M, static_cast<uint32_t>(-n));
-    s = sin_turns_fixed(U, hi);
-    c = sin_turns_fixed(U + 0x4000000000000000ull, 0u);
+    s = sin_turns_any(U, hi);
+    c = sin_turns_any(U + 0x4000000000000000ull, 0u);
 }
 
 }  // namespace phtl

@@ -81,6 +81,9 @@ __global__ void __launch_bounds__(256, 3)
     int parity = 0;
     double g1[4], g2[4];
     if (GEN) slip_stages<S>(c, g1, g2);
+    // one turn a launch: the weights stay in the constant bank
+    const TurnWeights w{{-c.dc[0], -c.dc[1], -c.dc[2], -c.dc[3]}, {c.kw[0], c.kw[1], c.kw[2]},
+                        {c.shx[0], c.shx[1]}, {c.shy[0], c.shy[1]}};
     const int ns_hi = __double2hiint(static_cast<double>(A.nslices));
     for (int64_t ci = blockIdx.x; ci < nchunks; ci += gridDim.x) {
         const int64_t base = ci * chunk + static_cast<int64_t>(threadIdx.x) * P;
@@ -116,10 +119,9 @@ __global__ void __launch_bounds__(256, 3)
                 else long_turn_nl<S, false>(z, d, c, c.dc, c.kw, c.kw2, g1, g2, c.dual_rf != 0);
                 transverse_gen(x, xp, y, yp, d, hx, hy, c);
             } else {
-                if (c.phis_zero) long_turn<S, true>(z, d, c, c.dc, c.kw);
-                else long_turn<S, false>(z, d, c, c.dc, c.kw);
-                if (hx) rotate(x, xp, c.mx, c.shx, c.shear_x != 0);
-                if (hy) rotate(y, yp, c.my, c.shy, c.shear_y != 0);
+                const RotateBeside<S> side{x, xp, y, yp, hx, hy, c, w};
+                if (c.phis_zero) long_turn<S, true>(z, d, c, w, side);
+                else long_turn<S, false>(z, d, c, w, side);
             }
         }
         if (counts) {

@@ -85,7 +85,11 @@ __global__ void k_eval_sin_kz(double k, float k2opi, PhaseScale kap, const doubl
 {
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        y[i] = sin_kz(k, k2opi, kap, z[i]);
+    {
+        bool ok;
+        const double s = sin_kz_fixed(kap, z[i], ok);
+        y[i] = ok ? s : sin_kz_rest(k, k2opi, z[i]);
+    }
 }
 
 int eval_grid(int64_t n, int block)

@@ -53,34 +53,53 @@ __device__ __forceinline__ const double* stage_weights(const RampTurn* __restric
 }
 
 // delta += kw (sin(phi_s,n + k z) - sin(phi_s,n)), kw this stage's weight times A_n
+template <class Side>
 __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], double kw,
-                                     const Turn& T, const MapConsts& c)
+                                     const Turn& T, const MapConsts& c, const Side& side, int j)
 {
+    double f[P];
+    bool ok[P], all = true;
+    if (c.linear) {
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        const double f = c.linear ? T.lin * z[p] : sin_kz_phi(c.k, c.kap, z[p], T.phis, T.uphis) - T.sinphis;
-        d[p] = fma(kw, f, d[p]);
+        for (int p = 0; p < P; ++p) f[p] = T.lin * z[p];
+        side(j);
+    } else {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            f[p] = sin_kz_phi_fixed(c.kap, z[p], T.uphis, ok[p]);
+            all = all && ok[p];
+        }
+        side(j);
+        if (!all) {
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                if (!ok[p]) f[p] = sin_wide(fma(c.k, z[p], T.phis));
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p) f[p] -= T.sinphis;
     }
+#pragma unroll
+    for (int p = 0; p < P; ++p) d[p] = fma(kw, f[p], d[p]);
 }
 
-template <int S>
+template <int S, class Side>
 __device__ __forceinline__ void turn(double (&z)[P], double (&d)[P], const Turn& T, const MapConsts& c,
-                                     const double* __restrict__ w)
+                                     const double* __restrict__ w, const Side& side)
 {
     if (S == PHTL_EULER_CROMER) {
-        kick(z, d, __ldg(w + 1), T, c);
+        kick(z, d, __ldg(w + 1), T, c, side, 0);
         drift(z, d, __ldg(w + 0));
     } else if (S == PHTL_LEAPFROG) {
         drift(z, d, __ldg(w + 0));
-        kick(z, d, __ldg(w + 2), T, c);
+        kick(z, d, __ldg(w + 2), T, c, side, 0);
         drift(z, d, __ldg(w + 1));
     } else {
         drift(z, d, __ldg(w + 0));
-        kick(z, d, __ldg(w + 4), T, c);
+        kick(z, d, __ldg(w + 4), T, c, side, 0);
         drift(z, d, __ldg(w + 1));
-        kick(z, d, __ldg(w + 5), T, c);
+        kick(z, d, __ldg(w + 5), T, c, side, 1);
         drift(z, d, __ldg(w + 2));
-        kick(z, d, __ldg(w + 6), T, c);
+        kick(z, d, __ldg(w + 6), T, c, side, 2);
         drift(z, d, __ldg(w + 3));
     }
 }
@@ -99,6 +118,12 @@ __global__ void __launch_bounds__(256, 2)
     const int64_t chunk = static_cast<int64_t>(blockDim.x) * P;
     const int64_t nchunks = (L.n + chunk - 1) / chunk;
     int parity = 0;
+    TurnWeights tw{};  // the shears; the stage weights come from the table
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        tw.shx[i] = in_register(c.shx[i]);
+        tw.shy[i] = in_register(c.shy[i]);
+    }
     for (int64_t ci = blockIdx.x; ci < nchunks; ci += gridDim.x) {
         const int64_t base = ci * chunk + static_cast<int64_t>(threadIdx.x) * P;
         double z[P], d[P], x[P], xp[P], y[P], yp[P];
@@ -126,9 +151,7 @@ __global__ void __launch_bounds__(256, 2)
         for (int t = 0; t < L.nturns; ++t) {
             // the next turn's constants, loaded while this turn computes
             const Turn Tn = load_turn(prog + turn0 + (t + 1 < L.nturns ? t + 1 : t));
-            turn<S>(z, d, T, c, stage_weights<S>(prog + turn0 + t));
-            if (hx) rotate(x, xp, c.mx, c.shx, c.shear_x != 0);
-            if (hy) rotate(y, yp, c.my, c.shy, c.shear_y != 0);
+            turn<S>(z, d, T, c, stage_weights<S>(prog + turn0 + t), RotateBeside<S>{x, xp, y, yp, hx, hy, c, tw});
 #pragma unroll
             for (int p = 0; p < P; ++p) {
                 d[p] = T.r * d[p];
