@@ -132,11 +132,13 @@ int derive(const phtl_params& p, phtl_derived& d, MapConsts (&mc)[4])
         c.k2opi = static_cast<float>(d.k * (2.0 / kPi));
         c.kap = integer_phase(d.k, p.phi_s_rad);
         c.uphis = phase_turns(p.phi_s_rad);
+        c.kq = quarter_phase(d.k, p.phi_s_rad);
+        c.kq2 = quarter_phase(k2, p.phi2_rad);
         c.phis = p.phi_s_rad;
         c.sinphis = d.sin_phis;
         c.lin = d.cos_phis * d.k;
         c.linear = p.rf_linear != 0;
-        c.phis_zero = p.phi_s_rad == 0.0 ? 1 : 0;
+        c.phis_zero = p.phi_s_rad == 0.0 && !p.rf_linear ? 1 : 0;
         for (int i = 0; i < 4; ++i) {
             c.mx[i] = d.mx[i];
             c.my[i] = d.my[i];
@@ -160,6 +162,11 @@ int derive(const phtl_params& p, phtl_derived& d, MapConsts (&mc)[4])
         c.by = p.beta_y_m;
         c.ibx = 1.0 / p.beta_x_m;
         c.iby = 1.0 / p.beta_y_m;
+        c.chx = chroma_plane(c.qx, p.xi_x, p.beta_x_m);
+        c.chy = chroma_plane(c.qy, p.xi_y, p.beta_y_m);
+        c.slip = p.eta1 != 0.0 || p.eta2 != 0.0 ? 1 : 0;
+        c.phi2_zero = p.phi2_rad == 0.0 ? 1 : 0;
+        c.plain = c.phis_zero && !c.slip && (!dual || c.phi2_zero) ? 1 : 0;
         c.chroma_x = p.xi_x != 0.0 ? 1 : 0;
         c.chroma_y = p.xi_y != 0.0 ? 1 : 0;
         // second RF system

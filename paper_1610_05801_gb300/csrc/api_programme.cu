@@ -54,6 +54,9 @@ int derive_programme(const phtl_params& p, const double* V, const double* p0, in
             T.phis = eta > 0.0 ? std::asin(x) : kPi - std::asin(x);
             T.sinphis = std::sin(T.phis);
             T.uphis = phase_turns(T.phis);
+            const QuarterPhase q = quarter_phase(0.0, T.phis);
+            T.phq_h = q.ph;
+            T.phq_l = q.pl;
             const double K = T.etaC * T.A * k * std::cos(T.phis);
             if (!(K > 0.0 && K < 4.0)) return PHTL_E_UNSTABLE;
         }

@@ -1,5 +1,6 @@
 """Fit the polynomial coefficients of the library's FP64 sine (sin_f64.cuh) and, with
---f32, of the FP32 sine of the FP32-compensated kick (ops_f32c.cuh).
+--f32, of the FP32 sine of the FP32-compensated kick (ops_f32c.cuh); with --fixed, the
+integers of the fixed-point sine sin(pi V) = V p(rho), rho = (2 V)^2 in [0, 1] (sin_f64.cuh).
 
 Method (textbook): after Cody-Waite reduction x = q pi/2 + r, |r| <= pi/4,
     sin r = r + r^3 S(r^2),          S(t) ~ (sin(sqrt t) - sqrt t) / t^(3/2)
@@ -62,8 +63,29 @@ def check_f32(sc, cc):
     return sc32, cc32, float(ws), float(wc)
 
 
+def fixed():
+    """p(rho) of degree 8 at the binary scales of sin_poly_fixed: c_k 2^(60 + 2 k) in 64 bits up
+    to c5, c_k 2^55 in 32 bits beyond."""
+    mp.mp.dps = 60
+
+    def p(rho):
+        v = mp.sqrt(rho) / 2
+        return mp.sin(mp.pi * v) / v
+
+    c, err = mp.chebyfit(p, [mp.mpf(10) ** -40, 1], 9, error=True)
+    c = [abs(v) for v in reversed(c)]  # signs alternate
+    return ([int(mp.nint(c[k] * mp.mpf(2) ** (60 + 2 * k))) for k in range(6)],
+            [int(mp.nint(c[k] * mp.mpf(2) ** 55)) for k in (6, 7, 8)], float(err))
+
+
 if __name__ == "__main__":
     import sys
+
+    if "--fixed" in sys.argv:
+        wide, narrow, err = fixed()
+        print("// c0..c5 (2^60, 2^62, ... 2^70):", ", ".join("0x%016X" % v for v in wide))
+        print("// c6..c8 (2^55):", ", ".join("0x%08X" % v for v in narrow), "(fit error %.2e)" % err)
+        sys.exit(0)
 
     if "--f32" in sys.argv:
         # the FP32 sine of the FP32-compensated kick: degree 2 in t for both S and C

@@ -83,6 +83,72 @@ inline PhaseScale integer_phase(double k, double phi)
     return std::fabs(phi) < 1e5 ? phase_scale(k) : PhaseScale{0, kNoPhaseScale, 0};
 }
 
+// A factor of the integer phases and sines by its magnitude, K 2^(e - 63) with K in
+// [2^62, 2^63); e = kNoFactor where it is zero or beyond 2^+-200 (the FP64 form is taken).
+struct FixedFactor {
+    uint64_t K;
+    int32_t e;
+    int32_t neg;
+};
+constexpr int32_t kNoFactor = 1 << 20;
+
+inline FixedFactor fixed_factor(double v)
+{
+    FixedFactor r{0, kNoFactor, v < 0.0 ? 1 : 0};
+    int e = 0;
+    const double f = std::frexp(std::fabs(v), &e);
+    if (!(f >= 0.5 && std::isfinite(v)) || e < -200 || e > 200) return r;
+    r.K = static_cast<uint64_t>(std::ldexp(f, 53)) << 10;
+    r.e = e;
+    return r;
+}
+
+// Chromatic plane: 2^-64 turns per unit of delta, the phase advance at delta = 0, beta, 1/beta.
+struct ChromaPlane {
+    FixedFactor xi, b, ib;
+    uint64_t uq;
+    int32_t on;  // all of them in range
+    int32_t pad_;
+};
+
+inline ChromaPlane chroma_plane(double q, double xi, double beta)
+{
+    ChromaPlane c{fixed_factor(xi), fixed_factor(beta), fixed_factor(1.0 / beta), 0, 0, 0};
+    // q in [0, 1): its fraction of 2^64, exact down to q of 2^-12 and rounded below
+    c.uq = static_cast<uint64_t>(std::ldexp(q, 63)) << 1;
+    c.on = xi != 0.0 && c.xi.e != kNoFactor && c.b.e != kNoFactor && c.ib.e != kNoFactor;
+    return c;
+}
+
+// k and phi in quarter turns for the double-float sine of the FP32 kernels: k 2/pi as three
+// floats (72 bits), phi 2/pi as two, reduced modulo a whole turn.
+struct QuarterPhase {
+    float kh, km, kl;
+    float ph, pl;
+};
+
+inline void over_half_pi(double v, double& hi, double& lo)  // v 2/pi = hi + lo
+{
+    constexpr double h = 0.63661977236758138, l = -3.9357353350364970e-17;
+    hi = v * h;
+    lo = std::fma(v, h, -hi) + v * l;
+}
+
+inline QuarterPhase quarter_phase(double k, double phi)
+{
+    QuarterPhase q;
+    double hi, lo;
+    over_half_pi(k, hi, lo);
+    q.kh = static_cast<float>(hi);
+    const double rest = (hi - static_cast<double>(q.kh)) + lo;
+    q.km = static_cast<float>(rest);
+    q.kl = static_cast<float>(rest - static_cast<double>(q.km));
+    over_half_pi(phi, hi, lo);
+    const double n = 4.0 * std::nearbyint(hi * 0.25);
+    split_df((hi - n) + lo, q.ph, q.pl);
+    return q;
+}
+
 // Per-stage coefficients of one turn of the longitudinal map (Sec. 1.1.2 schemes),
 // pre-multiplied on the host in FP64:
 //   drift stage i:  z <- z - dc[i] * delta           dc[i] = w_i * eta * C
@@ -102,10 +168,11 @@ struct MapConsts {
     // p = beta tan(mu/2), q = -sin(mu)/beta (shear_* = 0: use the matrix instead)
     double shx[2], shy[2];
     int32_t shear_x, shear_y;
-    int32_t phis_zero;  // phi_s == 0: the kick is sin(k z), with k z fused into the sine's reduction
+    int32_t phis_zero;  // phi_s == 0 and not rf_linear: the kick is sin(k z)
     // double-float (FP32 pair) copies for the FP32 paths: value = hi + lo
     float dc_hi[4], dc_lo[4];
     float kw_hi[3], kw_lo[3];
+    QuarterPhase kq, kq2;  // both RF systems' phases in quarter turns
     float k_hi, k_lo, phis_hi, phis_lo, sinphis_hi, sinphis_lo, lin_hi, lin_lo;
     float mx_hi[4], mx_lo[4], my_hi[4], my_lo[4];
     int32_t linear;  // rf_linear flag
@@ -115,18 +182,21 @@ struct MapConsts {
     // widened map: nonlinear slippage eta(d) = eta0 + eta1 d + eta2 d^2 and chromaticity
     int32_t general;             // eta1, eta2 or a chromaticity nonzero: general turn loop
     int32_t chroma_x, chroma_y;  // xi != 0 in that plane
-    int32_t pad2_;
+    int32_t slip;                // eta1 or eta2 nonzero
     double eta1C, eta2C;         // eta1 C, eta2 C
     double qx, qy;               // frac(Q): the phase advance in turns
     double xi_x, xi_y;           // chromaticities dQ/d delta
     double bx, by, ibx, iby;     // beta and 1/beta of the chromatic rotations
+    ChromaPlane chx, chy;        // the same for the integer sines of the FP64 kernels
     float eta1C_hi, eta1C_lo, eta2C_hi, eta2C_lo;
     float qx_hi, qx_lo, qy_hi, qy_lo, xi_x_hi, xi_x_lo, xi_y_hi, xi_y_lo;
     float bx_hi, bx_lo, by_hi, by_lo, ibx_hi, ibx_lo, iby_hi, iby_lo;
     // second RF system (double RF): stage j adds kw2[j] * (sin(phi2 + k2 z) - sin(phi2)),
     // kw2[j] = w_j * A2 (lin2 z in rf_linear mode)
     int32_t dual_rf;
-    int32_t pad3_;
+    int32_t phi2_zero;
+    int32_t plain;  // phis_zero, phi2 = 0 where there is a second system, no slippage expansion
+    int32_t pad4_;
     double kw2[3];
     double k2, phi2, sinphi2, lin2;
     PhaseScale kap2;
@@ -173,9 +243,10 @@ struct RampTurn {
     double w_ec[2];
     double w_lf[3];
     double w_r4[7];
-    uint64_t uphis;  // phi_s,n / 2 pi in 2^-64 turns
+    uint64_t uphis;      // phi_s,n / 2 pi in 2^-64 turns
+    float phq_h, phq_l;  // phi_s,n in quarter turns, modulo a whole turn
 };
-static_assert(sizeof(RampTurn) == 200, "RampTurn is 200 bytes");
+static_assert(sizeof(RampTurn) == 208, "RampTurn is 208 bytes");
 
 // Slicing grid and strength of the collective (wake) step.
 struct CollArgs {

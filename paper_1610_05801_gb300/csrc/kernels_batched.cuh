@@ -38,8 +38,8 @@ __device__ __forceinline__ int find_job(const JobDesc* __restrict__ jobs, int nj
 }
 
 // ---------------------------------------------------------------------------------- FP64
-template <int SCHEME, bool MON, bool ZS, bool GEN>
-__device__ __forceinline__ void run_f64_zs(double (&z)[f64::P], double (&d)[f64::P],
+template <int SCHEME, bool MON, int MODE, bool GEN>
+__device__ __forceinline__ void run_f64_mode(double (&z)[f64::P], double (&d)[f64::P],
                                         double (&x)[f64::P], double (&xp)[f64::P],
                                         double (&y)[f64::P], double (&yp)[f64::P], bool hx,
                                         bool hy, const MapConsts& c, const JobDesc& J,
@@ -48,16 +48,16 @@ __device__ __forceinline__ void run_f64_zs(double (&z)[f64::P], double (&d)[f64:
     const int64_t g0 = t0 + J.turn_offset;  // turns done before this launch
     int64_t until = J.stride - (g0 % J.stride);
     int64_t row = g0 / J.stride + 1;
-    double g1[4], g2[4];
-    if (GEN) f64::slip_stages<SCHEME>(c, g1, g2);
+    f64::GeneralWeights gw{};
+    if (GEN) gw = f64::general_weights<SCHEME>(J.dc, J.kw, J.kw2, c);
     f64::TurnWeights w{};
     if (!GEN) w = f64::turn_weights<SCHEME, true>(J.dc, J.kw, c);
     for (int t = 0; t < nt; ++t) {
         if (GEN) {
-            f64::long_turn_nl<SCHEME, ZS>(z, d, c, J.dc, J.kw, J.kw2, g1, g2, c.dual_rf != 0);
-            f64::transverse_gen(x, xp, y, yp, d, hx, hy, c);
+            f64::long_turn_nl<SCHEME, MODE>(z, d, c, gw, c.dual_rf != 0);
+            f64::transverse_gen(x, xp, y, yp, d, hx, hy, c, gw);
         } else {
-            f64::long_turn<SCHEME, ZS>(z, d, c, w, f64::RotateBeside<SCHEME>{x, xp, y, yp, hx, hy, c, w});
+            f64::long_turn<SCHEME, MODE>(z, d, c, w, f64::RotateBeside<SCHEME>{x, xp, y, yp, hx, hy, c, w});
         }
         if (MON && J.mon) {
             if (--until == 0) {
@@ -81,10 +81,15 @@ __device__ __forceinline__ void run_f64(double (&z)[f64::P], double (&d)[f64::P]
                                         bool hy, const MapConsts& c, const JobDesc& J,
                                         float cnt, int64_t t0, int nt, double* smem, int& parity)
 {
-    if (c.phis_zero)
-        run_f64_zs<SCHEME, MON, true, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+    if (GEN && c.plain)
+        run_f64_mode<SCHEME, MON, f64::kRfPlain, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem,
+                                                      parity);
+    else if (c.phis_zero)
+        run_f64_mode<SCHEME, MON, f64::kRfZero, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem,
+                                                     parity);
     else
-        run_f64_zs<SCHEME, MON, false, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+        run_f64_mode<SCHEME, MON, f64::kRfGeneral, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem,
+                                                        parity);
 }
 
 // GEN: the widened map (separate kernels chosen on the host; built with MON = true, the

@@ -11,8 +11,11 @@
 // shares were measured slower: the ragged warp at the end of every share costs more
 // than the lone extra chunk some blocks run in the last round.)
 //
-// On GB300 the FP64 pipe retires 2 DFMA per clock per SM (1/64 of FP32), so this
-// kernel is FP64-pipe bound: every FP64 operation per particle-turn counts.
+// On GB300 the FP64 pipe retires 2 DFMA per clock per SM (1/64 of FP32).  The turn keeps only
+// the updates of the state there (leap-frog 3 FMAs, each plane 3); the sines and the moment
+// sums run on the integer pipe beside it.  Leap-frog without planes: 83 % of the FP64 pipe, 1.8
+// clocks per particle-turn and SM (14 FP64 instructions and 7.9 clocks with the sine in FP64);
+// with both planes and moments every turn 70 %, 57 % of the integer (ALU) pipe, 7.1 clocks (12.5).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -29,24 +32,24 @@ using namespace f64;
 // The turn loop of one particle chunk (state in registers throughout).  GEN: the widened
 // map (slippage expansion, chromaticity, RK4), DUAL: with the second RF system; both
 // chosen once per launch.
-template <int SCHEME, bool TRANS, bool MON, bool ZS, bool GEN, bool DUAL>
+template <int SCHEME, bool TRANS, bool MON, int MODE, bool GEN, bool DUAL>
 __device__ __forceinline__ void turns(double (&z)[P], double (&d)[P], double (&x)[P],
                                       double (&xp)[P], double (&y)[P], double (&yp)[P], bool hx,
                                       bool hy, float cnt, const MapConsts& c, const TurnWeights& w,
                                       const MonitorArgs& m, int nturns, double* smem, int& parity)
 {
     int64_t until = m.until, row = m.row;
-    double g1[4], g2[4];
-    if (GEN) slip_stages<SCHEME>(c, g1, g2);
+    GeneralWeights gw{};
+    if (GEN) gw = general_weights<SCHEME>(c.dc, c.kw, c.kw2, c);
     for (int t = 0; t < nturns; ++t) {
         if (GEN) {
-            long_turn_nl<SCHEME, ZS>(z, d, c, c.dc, c.kw, c.kw2, g1, g2, DUAL);
-            if (TRANS) transverse_gen(x, xp, y, yp, d, hx, hy, c);
+            long_turn_nl<SCHEME, MODE>(z, d, c, gw, DUAL);
+            if (TRANS) transverse_gen(x, xp, y, yp, d, hx, hy, c, gw);
         } else {
             if (TRANS)
-                long_turn<SCHEME, ZS>(z, d, c, w, RotateBeside<SCHEME>{x, xp, y, yp, hx, hy, c, w});
+                long_turn<SCHEME, MODE>(z, d, c, w, RotateBeside<SCHEME>{x, xp, y, yp, hx, hy, c, w});
             else
-                long_turn<SCHEME, ZS>(z, d, c, w, NoSideWork{});
+                long_turn<SCHEME, MODE>(z, d, c, w, NoSideWork{});
         }
         if (MON && m.rows) {
             if (--until == 0) {
@@ -70,7 +73,7 @@ __device__ __forceinline__ void turns(double (&z)[P], double (&d)[P], double (&x
     __launch_bounds__(256) __maxnreg__((S) == PHTL_RUTH4 && !(G) ? PHTL_F64_RUTH4_MAXNREG : ((G) ? 128 : 80))
 #else
 #ifndef PHTL_F64_GEN_MIN_BLOCKS
-#define PHTL_F64_GEN_MIN_BLOCKS 2
+#define PHTL_F64_GEN_MIN_BLOCKS 3  // widened leap-frog 11 %, double-RF RK4 6 % faster than at 2
 #endif
 #define PHTL_F64_BOUNDS(S, G) __launch_bounds__(256, (G) ? PHTL_F64_GEN_MIN_BLOCKS : min_blocks_256<S>())
 #endif
@@ -117,12 +120,15 @@ __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
             record<TRANS>(z, d, x, xp, y, yp, cnt, hx, hy, smem, parity, m.rows, 0);
             parity ^= 1;
         }
-        if (c.phis_zero)
-            turns<SCHEME, TRANS, MON, true, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
-                                                       L.nturns, smem, parity);
+        if (GEN && c.plain)
+            turns<SCHEME, TRANS, MON, kRfPlain, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
+                                                           L.nturns, smem, parity);
+        else if (c.phis_zero)
+            turns<SCHEME, TRANS, MON, kRfZero, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
+                                                          L.nturns, smem, parity);
         else
-            turns<SCHEME, TRANS, MON, false, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
-                                                        L.nturns, smem, parity);
+            turns<SCHEME, TRANS, MON, kRfGeneral, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
+                                                             L.nturns, smem, parity);
         store2(gz, base, L.n, vec, z);
         store2(gd, base, L.n, vec, d);
         if (hx) {

@@ -22,17 +22,19 @@ constexpr int P = PHTL_F64_PARTICLES_PER_THREAD;
 static_assert(P % 2 == 0, "P must be even (128-bit loads of two doubles)");
 
 // Minimum resident 256-thread blocks per SM asked of the compiler (caps registers at
-// 65536 / (256 * this)): the FP64 kernels hide the FP64 pipe's latency with warps.
-// Euler-Cromer and leap-frog run faster with 3 (80 registers, 24 warps per SM); Ruth4,
-// with three kicks per turn in flight, with 2 (measured on GB300).
+// 65536 / (256 * this)): the FP64 kernels hide the latency of the FP64 pipe and of the sine's
+// integer chain with warps.  3 (80 registers, 24 warps) for all of them: Ruth4 with both planes
+// and moments took 11 % longer at 2, Euler-Cromer and leap-frog 3 to 17 % longer at 4 (spills).
 #ifndef PHTL_F64_MIN_BLOCKS_256
 #define PHTL_F64_MIN_BLOCKS_256 3
 #endif
 #ifndef PHTL_F64_MIN_BLOCKS_256_RUTH4
-#define PHTL_F64_MIN_BLOCKS_256_RUTH4 2
+#define PHTL_F64_MIN_BLOCKS_256_RUTH4 3
 #endif
-// The batched kernel holds all three schemes; at 3 it would spill.
-constexpr int kBatchedMinBlocks256 = 2;
+#ifndef PHTL_F64_BATCHED_MIN_BLOCKS
+#define PHTL_F64_BATCHED_MIN_BLOCKS 3  // mixed batch 2 % faster than at 2
+#endif
+constexpr int kBatchedMinBlocks256 = PHTL_F64_BATCHED_MIN_BLOCKS;
 template <int SCHEME>
 constexpr int min_blocks_256()
 {
@@ -75,6 +77,16 @@ __device__ __forceinline__ TurnWeights turn_weights(const double* dc, const doub
     return w;
 }
 
+// a b for the rf_linear branches: out of line, or the compiler issues the product with every
+// kick under a predicate (an FP64 instruction, half a clock of the pipe, even when it is off).
+static __device__ __noinline__ double branch_product(double a, double b) { return a * b; }
+
+// What the turn loop's code leaves out, chosen once per launch:
+//   kRfGeneral  any phi_s, rf_linear;
+//   kRfZero     phi_s = 0 with the sine force: the kick is sin(k z), no subtraction;
+//   kRfPlain    kRfZero, a second RF system (if any) with phi2 = 0, no slippage expansion.
+enum RfMode { kRfGeneral = 0, kRfZero = 1, kRfPlain = 2 };
+
 // Work that a turn runs beside the sines of its kick j, in the same stretch of code without a
 // branch: the sines occupy the integer pipe and the transverse push the FP64 pipe.
 struct NoSideWork {
@@ -82,55 +94,50 @@ struct NoSideWork {
 };
 
 // The force of the main RF system per unit weight, sin(phi_s + k z) - sin(phi_s) or lin z in
-// rf_linear mode, of the thread's P particles.  ZS: phi_s == 0 (stationary bucket), the force
-// is sin(k z) alone (the kernels choose the instantiation once, outside the turn loop).
-template <bool ZS, class Side>
+// rf_linear mode, of the thread's P particles.
+template <int MODE, class Side>
 __device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[P], double (&f)[P],
                                          const Side& side, int j)
 {
-    if (c.linear) {
+    if (MODE == kRfGeneral && c.linear) {
 #pragma unroll
-        for (int p = 0; p < P; ++p) f[p] = c.lin * z[p];
+        for (int p = 0; p < P; ++p) f[p] = branch_product(c.lin, z[p]);
         side(j);
         return;
     }
     bool ok[P], all = true;
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        f[p] = ZS ? sin_kz_fixed(c.kap, z[p], ok[p]) : sin_kz_phi_fixed(c.kap, z[p], c.uphis, ok[p]);
+        f[p] = MODE != kRfGeneral ? sin_kz_fixed(c.kap, z[p], ok[p])
+                                  : sin_kz_phi_fixed(c.kap, z[p], c.uphis, ok[p]);
         all = all && ok[p];
     }
     side(j);
     if (!all) {
 #pragma unroll
         for (int p = 0; p < P; ++p)
-            if (!ok[p]) f[p] = ZS ? sin_kz_rest(c.k, c.k2opi, z[p]) : sin_wide(fma(c.k, z[p], c.phis));
+            if (!ok[p])
+                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.k2opi, z[p]) : sin_phi_rest(c.k, z[p], c.phis);
     }
-    if (!ZS) {
+    if (MODE == kRfGeneral) {
 #pragma unroll
         for (int p = 0; p < P; ++p) f[p] -= c.sinphis;
     }
 }
 
-__device__ __forceinline__ void drift(double (&z)[P], const double (&d)[P], double dc)
-{
-#pragma unroll
-    for (int p = 0; p < P; ++p) z[p] = fma(-dc, d[p], z[p]);
-}
-
-// The same with the weight negated beforehand.
+// Linear drift, ndc = -w eta C.
 __device__ __forceinline__ void drift_neg(double (&z)[P], const double (&d)[P], double ndc)
 {
 #pragma unroll
     for (int p = 0; p < P; ++p) z[p] = fma(ndc, d[p], z[p]);
 }
 
-template <bool ZS, class Side>
+template <int MODE, class Side>
 __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], double kw,
                                      const MapConsts& c, const Side& side, int j)
 {
     double f[P];
-    rf_force<ZS>(c, z, f, side, j);
+    rf_force<MODE>(c, z, f, side, j);
 #pragma unroll
     for (int p = 0; p < P; ++p) d[p] = fma(kw, f[p], d[p]);
 }
@@ -138,24 +145,24 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
 // One turn of the scheme; stage order as in Sec. 1.1.2's readings (see phtl.h).
 // w: the drift (negated) and kick weights of this bunch's scheme, -w_i eta C and w_j A.
 // side: work beside the kicks' sines that touches neither z nor delta.
-template <int SCHEME, bool ZS, class Side>
+template <int SCHEME, int MODE, class Side>
 __device__ __forceinline__ void long_turn(double (&z)[P], double (&d)[P], const MapConsts& c,
                                           const TurnWeights& w, const Side& side)
 {
     if (SCHEME == PHTL_EULER_CROMER) {
-        kick<ZS>(z, d, w.kw[0], c, side, 0);
+        kick<MODE>(z, d, w.kw[0], c, side, 0);
         drift_neg(z, d, w.dc[0]);
     } else if (SCHEME == PHTL_LEAPFROG) {
         drift_neg(z, d, w.dc[0]);
-        kick<ZS>(z, d, w.kw[0], c, side, 0);
+        kick<MODE>(z, d, w.kw[0], c, side, 0);
         drift_neg(z, d, w.dc[1]);
     } else {
         drift_neg(z, d, w.dc[0]);
-        kick<ZS>(z, d, w.kw[0], c, side, 0);
+        kick<MODE>(z, d, w.kw[0], c, side, 0);
         drift_neg(z, d, w.dc[1]);
-        kick<ZS>(z, d, w.kw[1], c, side, 1);
+        kick<MODE>(z, d, w.kw[1], c, side, 1);
         drift_neg(z, d, w.dc[2]);
-        kick<ZS>(z, d, w.kw[2], c, side, 2);
+        kick<MODE>(z, d, w.kw[2], c, side, 2);
         drift_neg(z, d, w.dc[3]);
     }
 }
@@ -203,170 +210,231 @@ struct RotateBeside {
 
 // ---- widened map: nonlinear slippage and chromaticity -------------------------------
 
-// Drift with the slippage expansion: z -= (dc + g1 d + g2 d^2) d for this stage's
-// w eta(d) C, i.e. dc = w eta0 C, g1 = w eta1 C, g2 = w eta2 C.  With g1 = g2 = 0 it
-// is bitwise the linear drift.
-__device__ __forceinline__ void drift_nl(double (&z)[P], const double (&d)[P], double dc,
-                                         double g1, double g2)
+// Weights of the general turn loop: the drifts and their slippage terms negated (-w_i eta0 C,
+// -w_i eta1 C, -w_i eta2 C), the kicks of both RF systems, the shears of planes without
+// chromaticity, and the constants with which sums and products are formed as FMAs of registers
+// (a + b = fma(a, 1, b) and a b = fma(a, b, -0) exactly; see in_register).
+struct GeneralWeights {
+    double dc[4], g1[4], g2[4], kw[3], kw2[3], shx[2], shy[2];
+    double one, mzero, half, two, sixth;
+};
+
+template <int SCHEME>
+__device__ __forceinline__ GeneralWeights general_weights(const double* dc, const double* kw,
+                                                          const double* kw2, const MapConsts& c)
 {
+    GeneralWeights w{};
+    constexpr int kKicks = SCHEME == PHTL_RUTH4 ? 3 : 1;
+    constexpr int kDrifts = SCHEME == PHTL_RUTH4 ? 4 : (SCHEME == PHTL_LEAPFROG ? 2 : 1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (i < kDrifts) {
+            w.dc[i] = in_register(-dc[i]);
+            w.g1[i] = -(drift_weight(SCHEME, i) * c.eta1C);
+            w.g2[i] = -(drift_weight(SCHEME, i) * c.eta2C);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        if (j < kKicks) {
+            w.kw[j] = in_register(kw[j]);
+            w.kw2[j] = in_register(kw2[j]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        w.shx[i] = in_register(c.shx[i]);
+        w.shy[i] = in_register(c.shy[i]);
+    }
+    w.one = in_register(1.0);
+    w.mzero = in_register(-0.0);
+    w.half = in_register(0.5);
+    w.two = in_register(2.0);
+    w.sixth = in_register(1.0 / 6.0);
+    return w;
+}
+
+// Drift with the slippage expansion: z -= (dc + g1 d + g2 d^2) d for this stage's
+// w eta(d) C (weights negated, see GeneralWeights).  Without the expansion the linear drift.
+template <int MODE>
+__device__ __forceinline__ void drift_nl(double (&z)[P], const double (&d)[P], const GeneralWeights& w, int i)
+{
+    if (MODE == kRfPlain) {
+        drift_neg(z, d, w.dc[i]);
+        return;
+    }
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        const double e = fma(fma(g2, d[p], g1), d[p], dc);
-        z[p] = fma(-e, d[p], z[p]);
+        const double e = fma(fma(w.g2[i], d[p], w.g1[i]), d[p], w.dc[i]);
+        z[p] = fma(e, d[p], z[p]);
     }
 }
 
-// Force of the second RF system (double RF) per unit weight: sin(phi2 + k2 z) - sin(phi2),
-// or cos(phi2) k2 z in rf_linear mode.
-__device__ __forceinline__ void rf_force2(const MapConsts& c, const double (&z)[P], double (&f)[P])
+// Forces of both RF systems per unit weight: f of the main one (as rf_force) and, when `dual`, g of
+// the second, sin(phi2 + k2 z) - sin(phi2) or cos(phi2) k2 z in rf_linear mode.  The sines of both
+// run together, before the particles they do not cover are mended.
+// `dual`: a compile-time constant in the single-bunch kernels, which have a variant without the
+// second system; the batched kernels pass the ring's flag.
+template <int MODE>
+__device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[P], double (&f)[P],
+                                          double (&g)[P], bool dual)
 {
-    if (c.linear) {
-#pragma unroll
-        for (int p = 0; p < P; ++p) f[p] = c.lin2 * z[p];
+    if (!dual) {
+        rf_force<MODE>(c, z, f, NoSideWork{}, 0);
         return;
     }
-    bool ok[P], all = true;
+    if (MODE == kRfGeneral && c.linear) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            f[p] = branch_product(c.lin, z[p]);
+            g[p] = branch_product(c.lin2, z[p]);
+        }
+        return;
+    }
+    bool ok[P], ok2[P], all = true;
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        f[p] = sin_kz_phi_fixed(c.kap2, z[p], c.uphi2, ok[p]);
-        all = all && ok[p];
+        f[p] = MODE != kRfGeneral ? sin_kz_fixed(c.kap, z[p], ok[p])
+                                  : sin_kz_phi_fixed(c.kap, z[p], c.uphis, ok[p]);
+        g[p] = sin_kz_phi_fixed(c.kap2, z[p], c.uphi2, ok2[p]);
+        all = all && ok[p] && ok2[p];
     }
     if (!all) {
 #pragma unroll
-        for (int p = 0; p < P; ++p)
-            if (!ok[p]) f[p] = sin_wide(fma(c.k2, z[p], c.phi2));
+        for (int p = 0; p < P; ++p) {
+            if (!ok[p])
+                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.k2opi, z[p]) : sin_phi_rest(c.k, z[p], c.phis);
+            if (!ok2[p]) g[p] = sin_phi_rest(c.k2, z[p], c.phi2);
+        }
     }
 #pragma unroll
-    for (int p = 0; p < P; ++p) f[p] -= c.sinphi2;
+    for (int p = 0; p < P; ++p) {
+        if (MODE == kRfGeneral) f[p] -= c.sinphis;
+        if (MODE != kRfPlain) g[p] -= c.sinphi2;
+    }
 }
 
-// Kick of the widened map: the main RF system, then the second one when `dual` (a
-// compile-time constant in the single-bunch kernels, which have a variant without the
-// second system; the batched kernels pass the ring's flag) -- kw2: this stage's w_j A2.
-template <bool ZS>
+// Kick of the widened map: the main RF system, then the second one when `dual` -- kw2: this
+// stage's w_j A2.
+template <int MODE>
 __device__ __forceinline__ void kick_gen(const double (&z)[P], double (&d)[P], double kw, double kw2,
                                          const MapConsts& c, bool dual)
 {
-    kick<ZS>(z, d, kw, c, NoSideWork{}, 0);
-    if (dual) {
-        double f[P];
-        rf_force2(c, z, f);
+    double f[P], g[P];
+    rf_forces<MODE>(c, z, f, g, dual);
 #pragma unroll
-        for (int p = 0; p < P; ++p) d[p] = fma(kw2, f[p], d[p]);
+    for (int p = 0; p < P; ++p) {
+        d[p] = fma(kw, f[p], d[p]);
+        if (dual) d[p] = fma(kw2, g[p], d[p]);
     }
 }
 
 // Right-hand side of the smooth motion per turn (classic RK4's derivative):
 // dz/dn = -eta(d) C d = -(dc + g1 d + g2 d^2) d and dd/dn = kw F1(z) + kw2 F2(z), with
 // dc = eta0 C, g1 = eta1 C, g2 = eta2 C, kw = A, kw2 = A2.
-template <bool ZS>
+template <int MODE>
 __device__ __forceinline__ void rk4_rhs(const double (&z)[P], const double (&d)[P], const MapConsts& c,
-                                        double dc, double g1, double g2, double kw, double kw2, bool dual,
-                                        double (&fz)[P], double (&fd)[P])
+                                        const GeneralWeights& w, bool dual, double (&fz)[P],
+                                        double (&fd)[P])
 {
-    // the products are rounded on their own (__dmul_rn): the stage arguments and the
-    // weighted sum reuse them, and an FMA contraction chosen differently where `dual` is a
-    // compile-time constant than where it is not would break the bitwise agreement of the
-    // single-bunch and batched kernels
-    double f[P];
-    rf_force<ZS>(c, z, f, NoSideWork{}, 0);
+    // the products are rounded on their own: the stage arguments and the weighted sum reuse
+    // them, and an FMA contraction chosen differently where `dual` is a compile-time constant
+    // than where it is not would break the bitwise agreement of the single-bunch and batched
+    // kernels
+    double f[P], g[P];
+    rf_forces<MODE>(c, z, f, g, dual);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        const double e = fma(fma(g2, d[p], g1), d[p], dc);
-        fz[p] = -__dmul_rn(e, d[p]);
-        fd[p] = __dmul_rn(kw, f[p]);
-    }
-    if (dual) {
-        rf_force2(c, z, f);
-#pragma unroll
-        for (int p = 0; p < P; ++p) fd[p] = fma(kw2, f[p], fd[p]);
+        const double e = MODE == kRfPlain ? w.dc[0] : fma(fma(w.g2[0], d[p], w.g1[0]), d[p], w.dc[0]);
+        fz[p] = __fma_rn(e, d[p], w.mzero);
+        fd[p] = __fma_rn(w.kw[0], f[p], w.mzero);
+        if (dual) fd[p] = fma(w.kw2[0], g[p], fd[p]);
     }
 }
 
 // One classic RK4 step of one turn: k1 at the start, k2 and k3 at the half step from k1
 // and k2, k4 at the full step from k3, and the weighted sum (k1 + 2 k2 + 2 k3 + k4) / 6.
-template <bool ZS>
+template <int MODE>
 __device__ __forceinline__ void rk4_turn(double (&z)[P], double (&d)[P], const MapConsts& c,
-                                         double dc, double kw, double kw2, double g1, double g2,
-                                         bool dual)
+                                         const GeneralWeights& w, bool dual)
 {
-    constexpr double kSixth = 1.0 / 6.0;
     double k1z[P], k1d[P], k2z[P], k2d[P], k3z[P], k3d[P], k4z[P], k4d[P], a[P], b[P];
-    rk4_rhs<ZS>(z, d, c, dc, g1, g2, kw, kw2, dual, k1z, k1d);
+    rk4_rhs<MODE>(z, d, c, w, dual, k1z, k1d);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        a[p] = fma(0.5, k1z[p], z[p]);
-        b[p] = fma(0.5, k1d[p], d[p]);
+        a[p] = fma(w.half, k1z[p], z[p]);
+        b[p] = fma(w.half, k1d[p], d[p]);
     }
-    rk4_rhs<ZS>(a, b, c, dc, g1, g2, kw, kw2, dual, k2z, k2d);
+    rk4_rhs<MODE>(a, b, c, w, dual, k2z, k2d);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        a[p] = fma(0.5, k2z[p], z[p]);
-        b[p] = fma(0.5, k2d[p], d[p]);
+        a[p] = fma(w.half, k2z[p], z[p]);
+        b[p] = fma(w.half, k2d[p], d[p]);
     }
-    rk4_rhs<ZS>(a, b, c, dc, g1, g2, kw, kw2, dual, k3z, k3d);
+    rk4_rhs<MODE>(a, b, c, w, dual, k3z, k3d);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        a[p] = __dadd_rn(z[p], k3z[p]);
-        b[p] = __dadd_rn(d[p], k3d[p]);
+        a[p] = __fma_rn(k3z[p], w.one, z[p]);
+        b[p] = __fma_rn(k3d[p], w.one, d[p]);
     }
-    rk4_rhs<ZS>(a, b, c, dc, g1, g2, kw, kw2, dual, k4z, k4d);
+    rk4_rhs<MODE>(a, b, c, w, dual, k4z, k4d);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        z[p] = fma(fma(2.0, __dadd_rn(k2z[p], k3z[p]), __dadd_rn(k1z[p], k4z[p])), kSixth, z[p]);
-        d[p] = fma(fma(2.0, __dadd_rn(k2d[p], k3d[p]), __dadd_rn(k1d[p], k4d[p])), kSixth, d[p]);
+        const double sz = fma(w.two, __fma_rn(k2z[p], w.one, k3z[p]), __fma_rn(k1z[p], w.one, k4z[p]));
+        const double sd = fma(w.two, __fma_rn(k2d[p], w.one, k3d[p]), __fma_rn(k1d[p], w.one, k4d[p]));
+        z[p] = fma(sz, w.sixth, z[p]);
+        d[p] = fma(sd, w.sixth, d[p]);
     }
 }
 
-// One turn of the scheme with the slippage expansion (g1[i], g2[i]: stage i's w_i eta1 C,
-// w_i eta2 C) and the second RF system (kw2[j]: stage j's w_j A2).
-template <int SCHEME, bool ZS>
+// One turn of the scheme with the slippage expansion and the second RF system.
+template <int SCHEME, int MODE>
 __device__ __forceinline__ void long_turn_nl(double (&z)[P], double (&d)[P], const MapConsts& c,
-                                             const double* dc, const double* kw, const double* kw2,
-                                             const double (&g1)[4], const double (&g2)[4], bool dual)
+                                             const GeneralWeights& w, bool dual)
 {
     if (SCHEME == PHTL_RK4) {
-        rk4_turn<ZS>(z, d, c, dc[0], kw[0], kw2[0], g1[0], g2[0], dual);
+        rk4_turn<MODE>(z, d, c, w, dual);
     } else if (SCHEME == PHTL_EULER_CROMER) {
-        kick_gen<ZS>(z, d, kw[0], kw2[0], c, dual);
-        drift_nl(z, d, dc[0], g1[0], g2[0]);
+        kick_gen<MODE>(z, d, w.kw[0], w.kw2[0], c, dual);
+        drift_nl<MODE>(z, d, w, 0);
     } else if (SCHEME == PHTL_LEAPFROG) {
-        drift_nl(z, d, dc[0], g1[0], g2[0]);
-        kick_gen<ZS>(z, d, kw[0], kw2[0], c, dual);
-        drift_nl(z, d, dc[1], g1[1], g2[1]);
+        drift_nl<MODE>(z, d, w, 0);
+        kick_gen<MODE>(z, d, w.kw[0], w.kw2[0], c, dual);
+        drift_nl<MODE>(z, d, w, 1);
     } else {
-        drift_nl(z, d, dc[0], g1[0], g2[0]);
-        kick_gen<ZS>(z, d, kw[0], kw2[0], c, dual);
-        drift_nl(z, d, dc[1], g1[1], g2[1]);
-        kick_gen<ZS>(z, d, kw[1], kw2[1], c, dual);
-        drift_nl(z, d, dc[2], g1[2], g2[2]);
-        kick_gen<ZS>(z, d, kw[2], kw2[2], c, dual);
-        drift_nl(z, d, dc[3], g1[3], g2[3]);
-    }
-}
-
-// Stage constants g1, g2 of the slippage expansion for this scheme (loop-invariant).
-template <int SCHEME>
-__device__ __forceinline__ void slip_stages(const MapConsts& c, double (&g1)[4], double (&g2)[4])
-{
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        g1[i] = drift_weight(SCHEME, i) * c.eta1C;
-        g2[i] = drift_weight(SCHEME, i) * c.eta2C;
+        drift_nl<MODE>(z, d, w, 0);
+        kick_gen<MODE>(z, d, w.kw[0], w.kw2[0], c, dual);
+        drift_nl<MODE>(z, d, w, 1);
+        kick_gen<MODE>(z, d, w.kw[1], w.kw2[1], c, dual);
+        drift_nl<MODE>(z, d, w, 2);
+        kick_gen<MODE>(z, d, w.kw[2], w.kw2[2], c, dual);
+        drift_nl<MODE>(z, d, w, 3);
     }
 }
 
 // Chromatic rotation of one plane: each particle turns by 2 pi (q + xi d) with its own d
 // (after the turn's longitudinal step).
 __device__ __forceinline__ void rotate_chroma(double (&u)[P], double (&v)[P], const double (&d)[P],
-                                              double q, double xi, double b, double ib)
+                                              const ChromaPlane& h, double q, double xi, double b,
+                                              double ib, double mzero)
 {
+    double sb[P], sib[P], cs[P];
+    bool ok[P], all = h.on != 0;
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        double sn, cs;
-        sincos_turns(fma(xi, d[p], q), sn, cs);
-        const double un = fma(b * sn, v[p], cs * u[p]);
-        const double vn = fma(-(sn * ib), u[p], cs * v[p]);
+        chroma_fixed(h, d[p], sb[p], sib[p], cs[p], ok[p]);
+        ok[p] = ok[p] && h.on != 0;
+        all = all && ok[p];
+    }
+    if (!all) {
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            if (!ok[p]) chroma_rest(q, xi, b, ib, d[p], sb[p], sib[p], cs[p]);
+    }
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const double un = fma(sb[p], v[p], __fma_rn(cs[p], u[p], mzero));
+        const double vn = fma(-sib[p], u[p], __fma_rn(cs[p], v[p], mzero));
         u[p] = un;
         v[p] = vn;
     }
@@ -375,31 +443,32 @@ __device__ __forceinline__ void rotate_chroma(double (&u)[P], double (&v)[P], co
 // The transverse step of the general loop: chromatic where xi != 0, else the one matrix.
 __device__ __forceinline__ void transverse_gen(double (&x)[P], double (&xp)[P], double (&y)[P],
                                                double (&yp)[P], const double (&d)[P], bool hx,
-                                               bool hy, const MapConsts& c)
+                                               bool hy, const MapConsts& c, const GeneralWeights& w)
 {
     if (hx) {
-        if (c.chroma_x) rotate_chroma(x, xp, d, c.qx, c.xi_x, c.bx, c.ibx);
-        else rotate(x, xp, c.mx, c.shx, c.shear_x != 0);
+        if (c.chroma_x) rotate_chroma(x, xp, d, c.chx, c.qx, c.xi_x, c.bx, c.ibx, w.mzero);
+        else rotate(x, xp, c.mx, w.shx, c.shear_x != 0);
     }
     if (hy) {
-        if (c.chroma_y) rotate_chroma(y, yp, d, c.qy, c.xi_y, c.by, c.iby);
-        else rotate(y, yp, c.my, c.shy, c.shear_y != 0);
+        if (c.chroma_y) rotate_chroma(y, yp, d, c.chy, c.qy, c.xi_y, c.by, c.iby, w.mzero);
+        else rotate(y, yp, c.my, w.shy, c.shear_y != 0);
     }
 }
 
 // ---- moments: exact integer sums per warp ------------------------------------------------
 //
 // A coordinate's values are brought to the warp's common exponent E (the largest biased
-// exponent among its lanes, at least 128 so that a zero's significand shifts out) as 57-bit
-// integers X, a = X 2^(E + kMomentShift - 1086): no bit of a value within 2^-4 of the largest
-// is lost.  The sums of X, X^2 and X Y over the thread's particles and the warp's lanes are
-// 64-bit integer additions, and each is converted to FP64 once.  The squares are products of
-// the magnitudes rounded down, so a single particle's variance does not come out positive.
+// exponent among its lanes) as 61-bit integers X, a = X 2^(E + kMomentShift - 1086): no bit of a
+// value within 2^-8 of the largest is lost.  The thread adds X, X^2 and X Y over its particles,
+// the warp the threads' sums as 64-bit integers, and each total is converted to FP64 once: sums
+// keep 2^-55 of the warp's largest term.  The squares are products of the magnitudes rounded
+// down, so a single particle's variance does not come out positive.
 //
 // The double-float sums before these took ~590 instructions per particle and record with both
-// planes (bit splits, TwoSum and Fast2Sum in every addition); these take ~240.
-constexpr int kMomentShift = P <= 2 ? 7 : 8;     // P 32 values of X add up below 2^63
-constexpr int kMomentProductBits = P <= 2 ? 6 : 7;  // fraction bits kept of X Y 2^-64
+// planes (bit splits, TwoSum and Fast2Sum in every addition); these take ~390.
+constexpr int kMomentShift = P <= 2 ? 3 : 4;  // P X below 2^62
+constexpr int kSumDrop = 4;                   // the warp adds (sum of X) 2^-4 ...
+constexpr int kProductDrop = 65;              // ... and (sum of X Y) 2^-65, below 2^63
 
 struct PlaneExponents {
     int a, b;  // the warp's exponents of the plane's two coordinates
@@ -411,7 +480,7 @@ __device__ __forceinline__ int warp_exponent(const double (&a)[P])
     unsigned m = 0u;
 #pragma unroll
     for (int p = 0; p < P; ++p) m = max(m, static_cast<unsigned>(__double2hiint(a[p])) & 0x7fffffffu);
-    return max(static_cast<int>(__reduce_max_sync(kFullMask, m) >> 20), 128);
+    return static_cast<int>(__reduce_max_sync(kFullMask, m) >> 20);
 }
 
 // |a| in units of 2^(E + kMomentShift - 1086), and the sign as a mask.
@@ -419,8 +488,8 @@ __device__ __forceinline__ uint64_t moment_magnitude(double a, int E, uint32_t& 
 {
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(a));
     neg = static_cast<uint32_t>(static_cast<int32_t>(hi) >> 31);
-    return detail::shr_sat(detail::mantissa64(a),
-                           static_cast<uint32_t>(E + kMomentShift) - ((hi >> 20) & 0x7ffu));
+    const uint32_t e = (hi >> 20) & 0x7ffu;  // 0: zero (or subnormal) has no leading one, shift it out
+    return detail::shr_sat(detail::mantissa64(a), e != 0u ? static_cast<uint32_t>(E + kMomentShift) - e : 64u);
 }
 
 __device__ __forceinline__ int64_t moment_signed(uint64_t X, uint32_t neg)
@@ -429,14 +498,14 @@ __device__ __forceinline__ int64_t moment_signed(uint64_t X, uint32_t neg)
     return static_cast<int64_t>((X ^ m) - m);
 }
 
-// Sums of one plane (a, b) over the thread's particles: a, b (units of X), a^2, b^2 and ab
-// (units of X Y 2^(kMomentProductBits - 64)).
+// Sums of one plane (a, b) over the thread's particles: a, b (in 2^kSumDrop X), a^2, b^2 and ab
+// (in 2^kProductDrop X Y).
 __device__ __forceinline__ void pair_sums_fixed(const double (&a)[P], const double (&b)[P],
                                                 PlaneExponents E, int64_t* f)
 {
     uint64_t aa = 0, aac = 0, bb = 0, bbc = 0;
     int64_t ab = 0, abc = 0;
-    f[0] = f[1] = 0;
+    int64_t sa = 0, sb = 0;
 #pragma unroll
     for (int p = 0; p < P; ++p) {
         uint32_t na, nb;
@@ -448,8 +517,8 @@ __device__ __forceinline__ void pair_sums_fixed(const double (&a)[P], const doub
         bb += static_cast<uint64_t>(b1) * b1;
         bbc += static_cast<uint64_t>(b1) * b0;
         const int64_t As = moment_signed(A, na), Bs = moment_signed(B, nb);
-        f[0] += As;
-        f[1] += Bs;
+        sa += As;
+        sb += Bs;
         const int32_t as1 = static_cast<int32_t>(As >> 32), bs1 = static_cast<int32_t>(Bs >> 32);
         const int32_t ah = static_cast<int32_t>(static_cast<uint32_t>(As) >> 1);
         const int32_t bh = static_cast<int32_t>(static_cast<uint32_t>(Bs) >> 1);
@@ -457,23 +526,30 @@ __device__ __forceinline__ void pair_sums_fixed(const double (&a)[P], const doub
         abc += static_cast<int64_t>(as1) * bh;
         abc += static_cast<int64_t>(bs1) * ah;
     }
-    constexpr int q = kMomentProductBits;
-    f[2] = static_cast<int64_t>((aa << q) + (aac >> (31 - q)));
-    f[3] = static_cast<int64_t>((bb << q) + (bbc >> (31 - q)));
-    f[4] = (ab << q) + (abc >> (31 - q));
+    f[0] = sa >> kSumDrop;
+    f[1] = sb >> kSumDrop;
+    f[2] = static_cast<int64_t>((aa >> 1) + (aac >> 32));
+    f[3] = static_cast<int64_t>((bb >> 1) + (bbc >> 32));
+    f[4] = (ab >> 1) + (abc >> 32);
 }
 
-// S 2^x in FP64, rounded to nearest; beyond its range 0 or Inf.
-__device__ __forceinline__ double scaled_to_double(int64_t S, int x)
+// S 2^x in FP64, rounded to nearest or (nearest = 0, and below the normal range) truncated;
+// above the range Inf.  Integer instructions: a conversion to FP64 takes the FP64 pipe.
+__device__ __forceinline__ double scaled_to_double(int64_t S, int x, uint32_t nearest)
 {
     const uint64_t a = static_cast<uint64_t>(S < 0 ? -S : S);
     const int c = __clzll(static_cast<long long>(a));
     const uint64_t N = detail::shl_sat(a, static_cast<uint32_t>(c));
-    const uint64_t r = (N >> 11) + ((N >> 10) & 1u);
+    const uint64_t r = (N >> 11) + (static_cast<uint32_t>(N >> 10) & nearest);
     const int e = 1085 - c + x;  // biased exponent less the leading one of r
     uint32_t hi = static_cast<uint32_t>(r >> 32) + (static_cast<uint32_t>(e) << 20);
     uint32_t lo = static_cast<uint32_t>(r);
-    if (a == 0 || e < 0) hi = lo = 0u;
+    if (e < 0) {
+        const uint64_t sub = detail::shr_sat(N, static_cast<uint32_t>(11 - e));
+        hi = static_cast<uint32_t>(sub >> 32);
+        lo = static_cast<uint32_t>(sub);
+    }
+    if (a == 0) hi = lo = 0u;
     if (e > 2045 && a != 0) {
         hi = 0x7ff00000u;
         lo = 0u;
@@ -522,19 +598,16 @@ __device__ __forceinline__ void record(const double (&z)[P], const double (&d)[P
         f[6] = f[7] = 0;
     }
     const int64_t total = warp_reduce_scatter_int<NF>(f, lane);
-    double v;
-    if (field == 0) {
-        v = static_cast<double>(static_cast<int>(total));
-    } else {
-        // units: X of a plane's coordinate 2^(E + kMomentShift - 1086), products of two such
-        // less the 64 - kMomentProductBits bits taken off
-        const int e1 = k == 1 || k == 3 ? Ef.b : Ef.a;
-        const int e2 = k == 3 || k == 4 ? Ef.b : Ef.a;
-        v = scaled_to_double(total, k < 2 ? e1 + kMomentShift - 1086
-                                          : e1 + e2 + 2 * (kMomentShift - 1086) + 64 - kMomentProductBits);
-        // Inf or NaN among the warp's values
-        if (e1 == 2047 || (k >= 2 && e2 == 2047)) v = __hiloint2double(0x7ff80000, 0);
-    }
+    // the unit of X is 2^(E + kMomentShift - 1086); field 0 counts
+    const int e1 = k == 1 || k == 3 ? Ef.b : Ef.a;
+    const int e2 = k == 3 || k == 4 ? Ef.b : Ef.a;
+    const int ex = field == 0 ? 0
+                   : k < 2    ? e1 + kMomentShift - 1086 + kSumDrop
+                              : e1 + e2 + 2 * (kMomentShift - 1086) + kProductDrop;
+    // squares truncated once more: a single particle's variance stays at or below zero
+    double v = scaled_to_double(total, ex, k == 2 || k == 3 ? 0u : 1u);
+    // Inf or NaN among the warp's values
+    if (field != 0 && (e1 == 2047 || (k >= 2 && e2 == 2047))) v = __hiloint2double(0x7ff80000, 0);
     double* buf = smem + parity * (nwarps * 16);
     if ((lane & ((1 << kShift) - 1)) == 0) buf[warp * 16 + field] = v;
     __syncthreads();

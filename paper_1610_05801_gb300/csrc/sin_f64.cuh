@@ -1,7 +1,8 @@
-// FP64 sine of the FP64 kick, written for the scarce FP64 pipe of GB300 (2 DFMA per
-// clock per SM).
+// Sines of the FP64 kernels, written for the scarce FP64 pipe of GB300 (2 DFMA per clock per
+// SM): on the integer pipe for every phase in and around the bucket (second part of this file),
+// in FP64 arithmetic for what lies outside it.
 //
-// Method: Cody-Waite argument reduction x = q pi/2 + r (Cody & Waite, "Software Manual
+// The FP64 form: Cody-Waite argument reduction x = q pi/2 + r (Cody & Waite, "Software Manual
 // for the Elementary Functions", 1980), done with fused multiply-adds so a two-part
 // pi/2 suffices, then one polynomial on |r| <= pi/4 whose coefficient set (sine or
 // cosine) is selected per lane by the quadrant parity:
@@ -13,12 +14,10 @@
 // Accuracy: a few ulp on |x| <= 1e5 (checked against CUDA's sin and mpmath in the
 // tests through phtl_eval_sin).
 //
-// sin_kz(k, z) = sin(k z) is the kick's phase for phi_s = 0 with the product folded into
-// the reduction: r = (k z - q H) - q L with H = 3217/2048 (12 significant bits, so q H is
-// an integer times 2^-11, formed exactly for |q| < 2^16) and L = pi/2 - H rounded to FP64.
-// The first step is one FMA on the exact k z, the second one FMA, so the phase costs no
-// separate FP64 operation and r is rounded relative to itself rather than to k z: 11 FP64
-// operations for sin(k z), against 12 for the phase product followed by sin_f64.
+// sin_kz_rest(k, z) = sin(k z) folds the product into the reduction: r = (k z - q H) - q L with
+// H = 3217/2048 (12 significant bits, so q H is an integer times 2^-11, formed exactly for
+// |q| < 2^16) and L = pi/2 - H rounded to FP64, so r is rounded relative to itself rather than to
+// k z.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -218,9 +217,12 @@ __device__ __forceinline__ double neg_q_h(int q)
 
 // sin(k z) in FP64 arithmetic; k2opi = k * 2/pi rounded to FP32.  The fused form holds for
 // |k z| up to ~1e5 (the quadrant q below 2^16).  Beyond, and for Inf and NaN: sin_f64(k * z).
-static __device__ __noinline__ double sin_kz_wide(double k, float k2opi, double z)
+// z = 0 (also the unused lanes of a ragged bunch) is returned as it is.  Out of line, as
+// sin_phi_rest: none of their FP64 instructions may be hoisted into the kicks.
+static __device__ __noinline__ double sin_kz_rest(double k, float k2opi, double z)
 {
     using namespace detail;
+    if ((__double2hiint(z) << 1 | __double2loint(z)) == 0) return z;
     const float xq = __fmul_rn(split_bits(z).h, k2opi);   // ~ k z * 2/pi
     if (!(fabsf(xq) < 65536.0f)) return sin_f64(k * z);
     const float tf = __fadd_rn(xq, kMagic);
@@ -232,7 +234,11 @@ static __device__ __noinline__ double sin_kz_wide(double k, float k2opi, double 
     return sin_quadrant(r, qi);
 }
 
-static __device__ __noinline__ double sin_wide(double x) { return sin_f64(x); }
+// sin(k z + phi) in FP64 arithmetic.
+static __device__ __noinline__ double sin_phi_rest(double k, double z, double phi)
+{
+    return sin_f64(fma(k, z, phi));
+}
 
 // The kicks take the integer sine of all their particles first, without a branch in between
 // (the particles' chains and the FP64 work beside them overlap), and then mend the few that
@@ -257,12 +263,6 @@ __device__ __forceinline__ double sin_kz_fixed(PhaseScale kap, double z, bool& o
     return fixed_to_double(S, small ? static_cast<int>(n) - 2 : 0, hi ^ static_cast<uint32_t>(W >> 31));
 }
 
-// sin(k z) where sin_kz_fixed does not cover it.
-__device__ __forceinline__ double sin_kz_rest(double k, float k2opi, double z)
-{
-    return z == 0.0 ? z : sin_kz_wide(k, k2opi, z);
-}
-
 // sin(k z + phi), phi as uphi in 2^-64 turns: the phases are added as fractions of a turn,
 // without rounding.  Not covered: n < -1 (never below one turn of k z), a denormal z, a total phase within
 // 1e-9 of a half turn, Inf and NaN.
@@ -273,7 +273,7 @@ __device__ __forceinline__ double sin_kz_phi_fixed(PhaseScale kap, double z, uin
     const uint32_t e = (hi >> 20) & 0x7ffu;
     const uint32_t n1 = static_cast<uint32_t>(kap.cn + 1 - static_cast<int>(e));  // n + 1: from n = -1 on
     const uint64_t U = shr_sat(mulhi_trunc(mantissa64(z), kap.K), n1) << 2;
-    ok = n1 <= 2047u && (e != 0u || z == 0.0);
+    ok = n1 <= 2047u && (e != 0u || (hi << 1 | static_cast<uint32_t>(__double2loint(z))) == 0u);
     return sin_turns_fixed(static_cast<int>(hi) < 0 ? uphi - U : uphi + U, 0u, ok);
 }
 
@@ -298,6 +298,39 @@ __device__ __forceinline__ void sincos_turns(double a, double& s, double& c)
     const uint64_t M = mantissa64(a);
     const uint64_t U = n >= 0 ? shr_sat(M, static_cast<uint32_t>(n)) : shl_sat(M, static_cast<uint32_t>(-n));
     s = sin_turns_any(U, hi);
+    c = sin_turns_any(U + 0x4000000000000000ull, 0u);
+}
+
+// The chromatic rotation's sine times beta, sine over beta and cosine of 2 pi (q + xi d):
+// the phase as a sum of 2^-64 turns and the products with beta and 1/beta on the fixed-point
+// sine, so each is rounded once and no FP64 instruction is used.
+static __device__ __noinline__ void chroma_rest(double q, double xi, double beta, double ibeta, double d,
+                                                double& sb, double& sib, double& c)
+{
+    double s;
+    sincos_turns(fma(xi, d, q), s, c);
+    sb = beta * s;
+    sib = s * ibeta;
+}
+
+__device__ __forceinline__ void chroma_fixed(const ChromaPlane& w, double d, double& sb, double& sib,
+                                             double& c, bool& ok)
+{
+    using namespace detail;
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(d));
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    // |xi d| = hi64(M K) 2^(e + xi.e - 1021) in 2^-64 turns; a turn or more is not covered
+    const uint32_t n = static_cast<uint32_t>(1022 - w.xi.e - static_cast<int>(e));
+    const uint64_t A = shr_sat(mulhi_trunc(mantissa64(d), w.xi.K), n) << 1;
+    ok = n <= 2047u && (e != 0u || (hi << 1 | static_cast<uint32_t>(__double2loint(d))) == 0u);
+    const uint64_t U = ((hi >> 31) ^ static_cast<uint32_t>(w.xi.neg)) != 0u ? w.uq - A : w.uq + A;
+    const uint64_t V = fold_half_turn(U << 1);
+    const uint64_t S = mulhi_trunc63(V, sin_poly_fixed(V));
+    const uint32_t sign = static_cast<uint32_t>(U >> 32);
+    const uint64_t Sb = mulhi_trunc63(S, w.b.K), Si = mulhi_trunc63(S, w.ib.K);
+    ok = ok && (Sb >> 32) != 0u && (Si >> 32) != 0u;
+    sb = fixed_to_double(Sb, -1 - w.b.e, sign);  // Sb 2^(b.e - 59)
+    sib = fixed_to_double(Si, -1 - w.ib.e, sign);
     c = sin_turns_any(U + 0x4000000000000000ull, 0u);
 }
 

@@ -5,7 +5,7 @@
 // The same persistent structure as the fixed-machine kernels (Sec. 2.3: turn loop inside
 // the kernel, state in registers, grid-stride over particle chunks), but each turn reads
 // its constants -- eta_n C, A_n, phi_s,n, sin(phi_s,n), r_n = p0_n / p0_{n+1} -- from a
-// device table that the host derived in FP64 (200 bytes per turn, the same address for
+// device table that the host derived in FP64 (208 bytes per turn, the same address for
 // every thread, so the loads are L1 broadcasts).  The next turn's phase constants are
 // loaded while the current turn computes.  After the turn's stages and the transverse
 // rotation, delta and the slopes x', y' are re-expressed against the next turn's reference
@@ -52,6 +52,13 @@ __device__ __forceinline__ const double* stage_weights(const RampTurn* __restric
     return S == PHTL_EULER_CROMER ? e->w_ec : (S == PHTL_LEAPFROG ? e->w_lf : e->w_r4);
 }
 
+// z -= dc delta
+__device__ __forceinline__ void drift(double (&z)[P], const double (&d)[P], double dc)
+{
+#pragma unroll
+    for (int p = 0; p < P; ++p) z[p] = fma(-dc, d[p], z[p]);
+}
+
 // delta += kw (sin(phi_s,n + k z) - sin(phi_s,n)), kw this stage's weight times A_n
 template <class Side>
 __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], double kw,
@@ -61,7 +68,7 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
     bool ok[P], all = true;
     if (c.linear) {
 #pragma unroll
-        for (int p = 0; p < P; ++p) f[p] = T.lin * z[p];
+        for (int p = 0; p < P; ++p) f[p] = branch_product(T.lin, z[p]);
         side(j);
     } else {
 #pragma unroll
@@ -73,7 +80,7 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
         if (!all) {
 #pragma unroll
             for (int p = 0; p < P; ++p)
-                if (!ok[p]) f[p] = sin_wide(fma(c.k, z[p], T.phis));
+                if (!ok[p]) f[p] = sin_phi_rest(c.k, z[p], T.phis);
         }
 #pragma unroll
         for (int p = 0; p < P; ++p) f[p] -= T.sinphis;
@@ -104,8 +111,11 @@ __device__ __forceinline__ void turn(double (&z)[P], double (&d)[P], const Turn&
     }
 }
 
+#ifndef PHTL_F64_RAMP_MIN_BLOCKS
+#define PHTL_F64_RAMP_MIN_BLOCKS 3  // 8 % faster than at 2 (leap-frog, both planes, moments)
+#endif
 template <int S>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, PHTL_F64_RAMP_MIN_BLOCKS)
     k_ramp_f64(LaunchDesc L, MapConsts c, MonitorArgs m, const RampTurn* __restrict__ prog, int64_t turn0)
 {
     if (L.go && *L.go == 0) return;  // the call was cancelled before this launch
