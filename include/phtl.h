@@ -88,10 +88,10 @@ enum { PHTL_EULER_CROMER = 0, PHTL_LEAPFROG = 1, PHTL_RUTH4 = 2, PHTL_RK4 = 3 };
  *               hi[i] + comp[i].  Increments are double-float products of the FP64
  *               coefficients (split into hi + lo floats) and the pair, added with
  *               TwoSum and renormalised with Fast2Sum.  The RF phase argument is formed
- *               in FP64 from hi + comp; the sine is the library's double-float sine
- *               (~4e-12 absolute on the bucket).
- *  PHTL_F32CD : as PHTL_F32C, but the phase argument is formed in double-float (FP32
- *               pair) arithmetic instead of FP64 (no FP64 instruction on the path).
+ *               in quarter turns from hi + comp and k 2/pi in three floats, reduced exactly
+ *               and kept to 2^-47; the sine is the library's double-float sine (~2e-12
+ *               absolute on the bucket).  No FP64 instruction on the path.
+ *  PHTL_F32CD : the same arithmetic as PHTL_F32C (kept as a type of its own).
  *  PHTL_F32CS : FP32 increments (coefficients split into hi + lo, TwoSum accumulation),
  *               the phase rounded to FP32 and the SFU's sine (__sinf, absolute error
  *               ~2^-21 on [-pi, pi]): fastest, least accurate over long horizons.    */

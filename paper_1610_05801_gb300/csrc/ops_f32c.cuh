@@ -16,23 +16,18 @@ namespace f32c {
 constexpr int P = 4;
 
 // Register budgets of the FP32-compensated kernels, as resident 256-thread blocks per SM asked
-// of the compiler.  The kernels are issue-bound with few resident warps (116-160 registers:
-// 12-16 warps per SM), so more blocks per SM (fewer registers, some spill) pays where it was
-// measured to (1e6 particles, transverse planes, a monitor row every turn):
-//   - linear map: 4 blocks (at most 64 registers: 32 warps) for FP32C (+3.8 % over 3 blocks,
-//     all three schemes); 3 blocks (at most 85 registers) for FP32CS (-2.5 % at 4) and the Ruth4
-//     FP32CD kernel (-7 % at 4); the FP32CD Euler-Cromer and leap-frog kernels ran slower at 3
-//     and keep the compiler's choice (1);
-//   - widened map and RK4 / double RF (general kernels): 3 blocks for FP32C (-4 % time over the
-//     three symplectic schemes, -34 % for RK4 on the double-RF ring), FP32CS (-29 %) and FP32CD
-//     RK4 (-24 %); 2 blocks (at most 128 registers) for the FP32CD symplectic schemes (-2 %;
-//     3 blocks was 1 % slower than the compiler's choice);
-//   - batched kernels: 3 blocks (the batched FP32C kernel spills 2 KB a thread at 64 registers
-//     for +1.2 %); the widened map's batched kernels (16 bunches of 2.5e5 particles, 500
-//     turns): 2 blocks for FP32C and FP32CD (FP32CD leap-frog -17 %, Ruth4 -47 %), 3 for FP32CS
-//     (-37 %);
-//   - ramp programme: 3 blocks for FP32C (-6.6 %), the compiler's choice for FP32CD and FP32CS
-//     (track_ramp.cu).
+// of the compiler, or as registers (PHTL_F32C and PHTL_F32CD run the PHTL_F32CD kernels, but for
+// the collective step).  The kernels are issue-bound; four particles' sines in
+// flight want registers more than the SM wants warps (1e6 particles and the benchmark's cases):
+//   - linear map: 2 blocks (at most 128 registers) for FP32C and FP32CD (leap-frog 3.7 % faster
+//     than at 64 or 80 registers, Ruth4 with planes and moments 4 %); 3 for FP32CS;
+//   - widened map and RK4 / double RF (general kernels): 2 blocks for FP32C and FP32CD (widened
+//     leap-frog 5 % faster than at 3, RK4 on the double-RF ring 20 %), 3 for FP32CS;
+//   - batched kernels: 96 registers for FP32C and FP32CD (64 bunches, moments every turn: 7 %
+//     faster than at 80 or 128, 13 % than at 64; without launch bounds beside the cap, with which
+//     the compiler spills 288 bytes instead of 32 and the gain is lost), 80 for FP32CS; the widened
+//     map's: 128 for FP32C and FP32CD, 80 for FP32CS;
+//   - ramp programme: the compiler's choice (track_ramp.cu).
 // Build options PHTL_F32C_GEN_MIN_BLOCKS, PHTL_F32C_GEN_BATCHED_MIN_BLOCKS (general kernels) and
 // PHTL_F32C_MAXNREG (one register cap for all of them) override these, for measuring.
 constexpr int f32c_general_min_blocks(int scheme, int dtype)
@@ -40,32 +35,28 @@ constexpr int f32c_general_min_blocks(int scheme, int dtype)
 #ifdef PHTL_F32C_GEN_MIN_BLOCKS
     return (void)scheme, (void)dtype, PHTL_F32C_GEN_MIN_BLOCKS;
 #else
-    return dtype == PHTL_F32CD && scheme != PHTL_RK4 ? 2 : 3;
+    return (void)scheme, dtype == PHTL_F32CS ? 3 : 2;
 #endif
 }
 constexpr int f32c_track_min_blocks(int scheme, int dtype, bool general)
 {
-    return general ? f32c_general_min_blocks(scheme, dtype)
-                   : dtype == PHTL_F32C ? 4 : (dtype == PHTL_F32CD && scheme != PHTL_RUTH4 ? 1 : 3);
+    return general ? f32c_general_min_blocks(scheme, dtype) : (dtype == PHTL_F32CS ? 3 : 2);
 }
-constexpr int f32c_batched_min_blocks(int dtype, bool general)
+constexpr int f32c_batched_registers(int dtype, bool general)
 {
 #ifdef PHTL_F32C_GEN_BATCHED_MIN_BLOCKS
-    return general ? ((void)dtype, PHTL_F32C_GEN_BATCHED_MIN_BLOCKS) : 3;
-#else
-    return general ? (dtype == PHTL_F32CS ? 3 : 2) : 3;
+    if (general) return 65536 / (256 * PHTL_F32C_GEN_BATCHED_MIN_BLOCKS) / 8 * 8;
 #endif
+    return dtype == PHTL_F32CS ? 80 : (general ? 128 : 96);
 }
 #ifdef PHTL_F32C_MAXNREG
 #define PHTL_F32C_RAMP_BOUNDS(S, DT) __maxnreg__(PHTL_F32C_MAXNREG)
-#define PHTL_F32C_RAMP_BOUNDS_C __maxnreg__(PHTL_F32C_MAXNREG)
 #define PHTL_F32C_TRACK_BOUNDS(S, DT, G) __maxnreg__(PHTL_F32C_MAXNREG)
 #define PHTL_F32C_BATCHED_BOUNDS(DT, G) __maxnreg__(PHTL_F32C_MAXNREG)
 #else
 #define PHTL_F32C_RAMP_BOUNDS(S, DT) __launch_bounds__(256)
-#define PHTL_F32C_RAMP_BOUNDS_C __launch_bounds__(256, 3)
 #define PHTL_F32C_TRACK_BOUNDS(S, DT, G) __launch_bounds__(256, f32c::f32c_track_min_blocks(S, DT, G))
-#define PHTL_F32C_BATCHED_BOUNDS(DT, G) __launch_bounds__(256, f32c::f32c_batched_min_blocks(DT, G))
+#define PHTL_F32C_BATCHED_BOUNDS(DT, G) __maxnreg__(f32c::f32c_batched_registers(DT, G))
 #endif
 constexpr float kTwoPiHi = 6.28318548202514648438f;     // float(2 pi)
 constexpr float kTwoPiLo = -1.74845553146951715e-07f;    // 2 pi - kTwoPiHi
@@ -145,26 +136,12 @@ __device__ __forceinline__ void acc2(DF& a, DF2 inc)
 
 __device__ __forceinline__ double widen_bits(float f) { return widen_float_bits(f); }
 
-// Phase argument phi = phi_s + k z as a double-float pair.  PHTL_F32C forms it in FP64 from
-// hi + comp (exact in double) with one DFMA and splits it with the phase forms of the
-// integer widening and split; PHTL_F32CD in double-float arithmetic.
+// Phase argument phi = phi_s + k z as a double-float pair, in radians (for the SFU sine).
 // ZS: phi_s == 0, so the phase is k z alone (chosen once, outside the turn loop).
-template <int DT, bool ZS>
+template <bool ZS>
 __device__ __forceinline__ DF2 phase_df(const MapConsts& c, const DF& z)
 {
-    if (DT == PHTL_F32C) {
-        const double zd = widen_float_phase(z.hi) + widen_float_phase(z.c);
-        return split_phase(ZS ? c.k * zd : fma(c.k, zd, c.phis));
-    }
     const DF2 kz = df_mul(DF2{c.k_hi, c.k_lo}, as2(z));
-#ifdef PHTL_F32CD_PHASE_F32
-    // build option, for the accuracy comparison of the FP32 variants: the PHTL_F32CD phase
-    // rounded to one float (double-float state, increments and sine otherwise)
-    if (DT == PHTL_F32CD) {
-        const DF2 ph = ZS ? kz : df_add(kz, DF2{c.phis_hi, c.phis_lo});
-        return DF2{__fadd_rn(ph.h, ph.l), 0.0f};
-    }
-#endif
     return ZS ? kz : df_add(kz, DF2{c.phis_hi, c.phis_lo});
 }
 
@@ -174,33 +151,48 @@ struct DFC {
     __host__ __device__ constexpr DFC(double v) : h(static_cast<float>(v)), l(static_cast<float>(v - static_cast<double>(static_cast<float>(v)))) {}
 };
 
-// Double-float sine, absolute error ~1e-12 on the kick's range (a per-kick force error
-// far below what moves a particle's phase measurably in 1e6 turns).
-// Reduction x = q pi/2 + r with pi/2 = P1 + P2 + P3: q P1 is formed exactly (two_prod),
-// x.h - q P1 exactly as a TwoSum pair (its low part is zero whenever Sterbenz applies), and
-// the small remainder (x.l - e1 - q P2 - q P3, each ~1e-7) is summed in FP32 and
-// renormalised.  Then on |r| <= pi/4 one polynomial chosen per lane by the
-// quadrant parity, sin r = r + r^3 S(r^2), cos r = 1 - r^2/2 + r^4 C(r^2), with the
-// coefficients of the FP64 sine (sin_f64.cuh): the two leading Horner steps in
-// double-float, the four trailing terms (|t^2 S_2| <= 8e-5, |t^2 C_2| <= 1e-5) in FP32.
+// Double-float sine of k z + phi, absolute error ~1e-12 on the kick's range (a per-kick force
+// error far below what moves a particle's phase measurably in 1e6 turns).
+// The phase is formed in quarter turns, where its reduction is a subtraction of an integer: the
+// head product k.kh z.h less the nearest integer q is exact, and the product's error and the
+// cross terms (k in 72 bits) follow as one float, 2^-47 of the phase; r = pi/2 times that pair.
+// Then on |r| <= pi/4 one polynomial chosen per lane by the quadrant parity,
+// sin r = r + r^3 S(r^2), cos r = 1 - r^2/2 + r^4 C(r^2), with the coefficients of the FP64
+// sine (sin_f64.cuh): the two leading Horner steps in double-float, the four trailing terms
+// (|t^2 S_2| <= 8e-5, |t^2 C_2| <= 1e-5) in FP32: they set the accuracy (1.7e-13 rms).
 // Every double-float addition after the reduction adds a smaller term to a larger one
 // (Horner constant vs product, r vs r^3 S, 1 - t/2 vs r^4 C), so it uses Fast2Sum on the
-// heads.  |x| >= 1e4 falls back to the FP64 sine.
-__device__ __forceinline__ DF2 sin_df(DF2 x)
+// heads, and neither products nor these sums are renormalised before the next operation (the
+// result is not either).  73 operations, where the radian form (FP64 or double-float phase,
+// Cody-Waite reduction, renormalised pairs) took 135.
+// ok is cleared at 6366 quarter turns (1e4 radians) and more, for Inf and NaN.
+template <bool ZS>
+__device__ __forceinline__ DF2 sin_quarter_df(const QuarterPhase& k, float ph, float pl, DF2 z, bool& ok)
 {
-    if (!(fabsf(x.h) < 1.0e4f)) return split_bits(sin_f64(widen_bits(x.h) + widen_bits(x.l)));
+    float p = __fmul_rn(z.h, k.kh);
+    float c = __fmaf_rn(z.h, k.kh, -p);
+    c = __fmaf_rn(z.h, k.kl, c);
+    c = __fmaf_rn(z.h, k.km, c);
+    c = __fmaf_rn(z.l, k.kh, c);
+    if (!ZS) {
+        const DF2 s = df_two_sum(p, ph);
+        p = s.h;
+        c = __fadd_rn(__fadd_rn(c, pl), s.l);
+    }
+    ok = fabsf(p) < 6366.0f;
     const float magic = 12582912.0f;
-    const float t0 = __fmaf_rn(x.h, 0.6366197466850281f, magic);
-    const float q = __fsub_rn(t0, magic);
+    const float t0 = __fadd_rn(p, magic);
     const int qi = __float_as_int(t0);
-    const float p1 = __fmul_rn(q, 1.5707963705062866f);
-    const float e1 = __fmaf_rn(q, 1.5707963705062866f, -p1);
-    const DF2 hd = df_two_sum(x.h, -p1);  // exact as a pair (Sterbenz makes hd.l ~0)
-    float rest = __fadd_rn(__fsub_rn(x.l, e1), hd.l);
-    rest = __fmaf_rn(-q, -4.371138828673793e-08f, rest);
-    rest = __fmaf_rn(-q, -1.7151245100058819e-15f, rest);
-    const DF2 r = df_fast_two_sum(hd.h, rest);
-    const DF2 t = df_mul(r, r);
+    const float f = __fsub_rn(p, __fsub_rn(t0, magic));
+    // r = (f + c) pi/2, pi/2 = 1.57079637 - 4.37113883e-8 - 1.71512451e-15
+    const float rp = __fmul_rn(f, 1.5707963705062866f);
+    float re = __fmaf_rn(f, 1.5707963705062866f, -rp);
+    re = __fmaf_rn(f, -1.7151245100058819e-15f, re);
+    re = __fmaf_rn(f, -4.371138828673793e-08f, re);
+    const DF2 r = df_fast_two_sum(rp, __fmaf_rn(c, 1.5707963705062866f, re));
+    DF2 t;
+    t.h = __fmul_rn(r.h, r.h);
+    t.l = __fmaf_rn(__fadd_rn(r.h, r.h), r.l, __fmaf_rn(r.h, r.h, -t.h));
     const bool odd = (qi & 1) != 0;
     // trailing terms in FP32: C_5..C_2 / S_5..S_2
     float tail = odd ? -1.1382632425521717e-11f : 1.5918129294866608e-10f;
@@ -210,12 +202,31 @@ __device__ __forceinline__ DF2 sin_df(DF2 x)
     // leading Horner steps in double-float
     constexpr DFC s1(0.008333333333330948), s0(-0.16666666666666666);
     constexpr DFC c1(-0.0013888888888887398), c0(0.041666666666666664);
-    DF2 u = df_add_dominant(odd ? DF2{c1.h, c1.l} : DF2{s1.h, s1.l}, df_mul_f(t, tail));
-    u = df_add_dominant(odd ? DF2{c0.h, c0.l} : DF2{s0.h, s0.l}, df_mul(t, u));
-    const DF2 m = df_mul(odd ? t : r, t);                                  // r^3 or r^4
-    const DF2 a = odd ? df_add_dominant(DF2{1.0f, 0.0f}, DF2{-0.5f * t.h, -0.5f * t.l}) : r;
-    const DF2 res = df_add_dominant(a, df_mul(m, u));
+    const float tp = __fmul_rn(t.h, tail);
+    DF2 u = df_add_dominant_raw(odd ? DF2{c1.h, c1.l} : DF2{s1.h, s1.l},
+                                DF2{tp, __fmaf_rn(t.l, tail, __fmaf_rn(t.h, tail, -tp))});
+    u = df_add_dominant_raw(odd ? DF2{c0.h, c0.l} : DF2{s0.h, s0.l}, df_mul_raw(t, u));
+    const DF2 m = df_mul_raw(odd ? t : r, t);                              // r^3 or r^4
+    // 1 - t/2: the head's rounding error is exact
+    const float oh = __fmaf_rn(-0.5f, t.h, 1.0f);
+    const float ol = __fmaf_rn(-0.5f, t.l, __fmaf_rn(-0.5f, t.h, __fsub_rn(1.0f, oh)));
+    const DF2 res = df_add_dominant_raw(odd ? DF2{oh, ol} : r, df_mul_raw(m, u));
     return df_xor_sign(res, static_cast<unsigned>(qi & 2) << 30);      // quadrants 2, 3: -res
+}
+
+// sin(k z + phi) where sin_quarter_df does not cover it, in FP64.
+static __device__ __noinline__ DF2 sin_quarter_rest(double k, double phi, DF2 z)
+{
+    return split_bits(sin_f64(fma(k, widen_bits(z.h) + widen_bits(z.l), phi)));
+}
+
+// Double-float sine of a pair in radians (diagnostics).
+__device__ __forceinline__ DF2 sin_df(DF2 x)
+{
+    constexpr QuarterPhase one{0.636619746685028076f, 2.5682552973194106e-08f, 2.93709547963155499e-16f, 0.0f, 0.0f};
+    bool ok;
+    const DF2 s = sin_quarter_df<true>(one, 0.0f, 0.0f, x, ok);
+    return ok ? s : sin_quarter_rest(1.0, 0.0, x);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -233,7 +244,7 @@ __device__ __forceinline__ float phase_f(const MapConsts& c, const DF& z)
     const DF2 p2 = split_bits(ph);
     return __fadd_rn(p2.h, p2.l);
 #else
-    const DF2 ph = phase_df<PHTL_F32CD, ZS>(c, z);
+    const DF2 ph = phase_df<ZS>(c, z);
     return __fadd_rn(ph.h, ph.l);
 #endif
 }
@@ -252,15 +263,40 @@ __device__ __forceinline__ float sin_sfu(float x)
 }
 
 // ---------------------------------------------------------------------------------------
+// Force of one RF system per unit weight of the thread's particles, sin(phi + k z) - sin(phi)
+// (ZS: phi == 0, no subtraction), in double-float: q, (ph, pl): the phase in quarter turns, k64
+// and phi64 for particles the quarter-turn form does not cover.  All sines first, so that the
+// particles' chains interleave.
+template <bool ZS, int N>
+__device__ __forceinline__ void force_df(const QuarterPhase& q, float ph, float pl, double k64, double phi64,
+                                         DF2 minus_sin_phi, const DF2 (&z)[N], DF2 (&f)[N])
+{
+    bool ok[N], all = true;
+#pragma unroll
+    for (int p = 0; p < N; ++p) {
+        f[p] = sin_quarter_df<ZS>(q, ph, pl, z[p], ok[p]);
+        all = all && ok[p];
+    }
+    if (!all) {
+#pragma unroll
+        for (int p = 0; p < N; ++p)
+            if (!ok[p]) f[p] = sin_quarter_rest(k64, ZS ? 0.0 : phi64, z[p]);
+    }
+    if (!ZS) {
+#pragma unroll
+        for (int p = 0; p < N; ++p) f[p] = df_add(f[p], minus_sin_phi);
+    }
+}
+
 // kick: delta += kw * (sin(phi) - sin(phi_s)), kw = kh + kl (the FP64 weight as a pair);
 // ZS: phi_s == 0, no subtraction
 template <int DT, bool ZS>
 __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], float kh, float kl,
                                      const MapConsts& c)
 {
+    if (DT == PHTL_F32CS) {
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        if (DT == PHTL_F32CS) {
+        for (int p = 0; p < P; ++p) {
             float f;
             if (c.linear) {
                 f = c.lin_hi * (z[p].hi + z[p].c);
@@ -269,17 +305,20 @@ __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], float kh, flo
                 if (!ZS) f -= c.sinphis_hi;
             }
             acc(d[p], __fmaf_rn(kh, f, __fmul_rn(kl, f)));
-        } else {
-            DF2 f;
-            if (c.linear) {
-                f = df_mul(DF2{c.lin_hi, c.lin_lo}, as2(z[p]));
-            } else {
-                f = sin_df(phase_df<DT, ZS>(c, z[p]));
-                if (!ZS) f = df_add(f, DF2{-c.sinphis_hi, -c.sinphis_lo});
-            }
-            acc2(d[p], df_mul(DF2{kh, kl}, f));
         }
+        return;
     }
+    DF2 f[P], zz[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) zz[p] = as2(z[p]);
+    if (c.linear) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) f[p] = df_mul(DF2{c.lin_hi, c.lin_lo}, zz[p]);
+    } else {
+        force_df<ZS>(c.kq, c.kq.ph, c.kq.pl, c.k, c.phis, DF2{-c.sinphis_hi, -c.sinphis_lo}, zz, f);
+    }
+#pragma unroll
+    for (int p = 0; p < P; ++p) acc2(d[p], df_mul_raw(DF2{kh, kl}, f[p]));
 }
 
 // drift: z -= dc * delta, dc = dh + dl
@@ -292,7 +331,7 @@ __device__ __forceinline__ void drift(DF (&z)[P], const DF (&d)[P], float dh, fl
             const float inc = __fmaf_rn(dh, d[p].hi, __fmaf_rn(dl, d[p].hi, __fmul_rn(dh, d[p].c)));
             acc(z[p], -inc);
         } else {
-            acc2(z[p], neg2(df_mul(DF2{dh, dl}, as2(d[p]))));
+            acc2(z[p], df_mul_raw(DF2{-dh, -dl}, as2(d[p])));
         }
     }
 }
@@ -339,9 +378,9 @@ __device__ __forceinline__ void drift_nl(DF (&z)[P], const DF (&d)[P], float dh,
             acc(z[p], -inc);
         } else {
             const DF2 dd = as2(d[p]);
-            DF2 e = df_add(df_mul(DF2{g2h, g2l}, dd), DF2{g1h, g1l});
-            e = df_add(df_mul(e, dd), DF2{dh, dl});
-            acc2(z[p], neg2(df_mul(e, dd)));
+            DF2 e = df_add(df_mul_raw(DF2{g2h, g2l}, dd), DF2{g1h, g1l});
+            e = df_add(df_mul_raw(e, dd), DF2{dh, dl});
+            acc2(z[p], neg2(df_mul_raw(e, dd)));
         }
     }
 }
@@ -349,20 +388,18 @@ __device__ __forceinline__ void drift_nl(DF (&z)[P], const DF (&d)[P], float dh,
 // ---- second RF system (double RF) and classic RK4 ----------------------------------
 
 // Force of the second RF system per unit weight, sin(phi2 + k2 z) - sin(phi2) (rf_linear:
-// cos(phi2) k2 z), as a pair: the phase in FP64 for PHTL_F32C, in double-float for
-// PHTL_F32CD, and the double-float sine.
-template <int DT>
-__device__ __forceinline__ DF2 force2_df(const MapConsts& c, DF2 z)
+// cos(phi2) k2 z), as a pair.
+template <int N>
+__device__ __forceinline__ void force2_df(const MapConsts& c, const DF2 (&z)[N], DF2 (&f)[N])
 {
-    if (c.linear) return df_mul(DF2{c.lin2_hi, c.lin2_lo}, z);
-    DF2 ph;
-    if (DT == PHTL_F32C) {
-        const double zd = widen_float_phase(z.h) + widen_float_phase(z.l);
-        ph = split_phase(fma(c.k2, zd, c.phi2));
+    if (c.linear) {
+#pragma unroll
+        for (int p = 0; p < N; ++p) f[p] = df_mul(DF2{c.lin2_hi, c.lin2_lo}, z[p]);
+    } else if (c.phi2_zero) {
+        force_df<true>(c.kq2, 0.0f, 0.0f, c.k2, 0.0, DF2{0.0f, 0.0f}, z, f);
     } else {
-        ph = df_add(df_mul(DF2{c.k2_hi, c.k2_lo}, z), DF2{c.phi2_hi, c.phi2_lo});
+        force_df<false>(c.kq2, c.kq2.ph, c.kq2.pl, c.k2, c.phi2, DF2{-c.sinphi2_hi, -c.sinphi2_lo}, z, f);
     }
-    return df_add(sin_df(ph), DF2{-c.sinphi2_hi, -c.sinphi2_lo});
 }
 
 // The same for PHTL_F32CS: the phase rounded to FP32 and the SFU sine.
@@ -374,12 +411,14 @@ __device__ __forceinline__ float force2_f(const MapConsts& c, DF2 z)
 }
 
 // Force of the main RF system per unit weight at a pair z (the bracket of kick()).
-template <int DT, bool ZS>
+template <bool ZS>
 __device__ __forceinline__ DF2 force1_df(const MapConsts& c, DF2 z)
 {
     if (c.linear) return df_mul(DF2{c.lin_hi, c.lin_lo}, z);
-    const DF2 f = sin_df(phase_df<DT, ZS>(c, DF{z.h, z.l}));
-    return ZS ? f : df_add(f, DF2{-c.sinphis_hi, -c.sinphis_lo});
+    const DF2 zz[1] = {z};
+    DF2 f[1];
+    force_df<ZS>(c.kq, c.kq.ph, c.kq.pl, c.k, c.phis, DF2{-c.sinphis_hi, -c.sinphis_lo}, zz, f);
+    return f[0];
 }
 
 template <bool ZS>
@@ -398,15 +437,20 @@ __device__ __forceinline__ void kick_gen(const DF (&z)[P], DF (&d)[P], float kh,
 {
     kick<DT, ZS>(z, d, kh, kl, c);
     if (!dual) return;
+    if (DT == PHTL_F32CS) {
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        if (DT == PHTL_F32CS) {
+        for (int p = 0; p < P; ++p) {
             const float f = force2_f(c, as2(z[p]));
             acc(d[p], __fmaf_rn(k2h, f, __fmul_rn(k2l, f)));
-        } else {
-            acc2(d[p], df_mul(DF2{k2h, k2l}, force2_df<DT>(c, as2(z[p]))));
         }
+        return;
     }
+    DF2 f[P], zz[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) zz[p] = as2(z[p]);
+    force2_df(c, zz, f);
+#pragma unroll
+    for (int p = 0; p < P; ++p) acc2(d[p], df_mul_raw(DF2{k2h, k2l}, f[p]));
 }
 
 // Right-hand side of the smooth motion per turn as pairs: dz/dn = -(dc + g1 d + g2 d^2) d,
@@ -415,11 +459,19 @@ template <int DT, bool ZS>
 __device__ __forceinline__ void rk4_rhs_df(DF2 z, DF2 d, const MapConsts& c, DF2 dc, DF2 g1, DF2 g2,
                                            DF2 kw, DF2 kw2, bool dual, DF2& fz, DF2& fd)
 {
-    DF2 e = df_add(df_mul(g2, d), g1);
-    e = df_add(df_mul(e, d), dc);
+    DF2 e = dc;
+    if (c.slip) {
+        e = df_add(df_mul_raw(g2, d), g1);
+        e = df_add(df_mul_raw(e, d), dc);
+    }
     fz = neg2(df_mul(e, d));
-    fd = df_mul(kw, force1_df<DT, ZS>(c, z));
-    if (dual) fd = df_add(fd, df_mul(kw2, force2_df<DT>(c, z)));
+    fd = df_mul(kw, force1_df<ZS>(c, z));
+    if (dual) {
+        const DF2 zz[1] = {z};
+        DF2 f[1];
+        force2_df(c, zz, f);
+        fd = df_add(fd, df_mul_raw(kw2, f[0]));
+    }
 }
 
 __device__ __forceinline__ DF2 df_scale2(DF2 a, float s) { return DF2{s * a.h, s * a.l}; }  // s = 2^k: exact
@@ -589,8 +641,8 @@ __device__ __forceinline__ void rotate_chroma(DF (&u)[P], DF (&v)[P], const DF (
             sincos_df_turns(df_add(DF2{qh, ql}, df_mul(DF2{xh, xl}, as2(d[p]))), sn, cs);
             const DF2 bs = df_mul(DF2{bh, bl}, sn);
             const DF2 sib = df_mul(DF2{ibh, ibl}, sn);
-            const DF2 un = df_add(df_mul(cs, as2(u[p])), df_mul(bs, as2(v[p])));
-            const DF2 vn = df_add(df_mul(cs, as2(v[p])), neg2(df_mul(sib, as2(u[p]))));
+            const DF2 un = df_add(df_mul_raw(cs, as2(u[p])), df_mul_raw(bs, as2(v[p])));
+            const DF2 vn = df_add(df_mul_raw(cs, as2(v[p])), neg2(df_mul_raw(sib, as2(u[p]))));
             u[p] = DF{un.h, un.l};
             v[p] = DF{vn.h, vn.l};
         }

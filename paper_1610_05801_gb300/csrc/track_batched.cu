@@ -13,10 +13,8 @@ const void* select_batched(int dtype, bool mon)
     if (dtype == PHTL_F64)
         return mon ? reinterpret_cast<const void*>(&k_batched_f64<true, false>)
                    : reinterpret_cast<const void*>(&k_batched_f64<false, false>);
-    if (dtype == PHTL_F32C)
-        return mon ? reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32C, true, false>)
-                   : reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32C, false, false>);
-    if (dtype == PHTL_F32CD)
+    // PHTL_F32C and PHTL_F32CD are the same arithmetic: one instantiation
+    if (dtype == PHTL_F32C || dtype == PHTL_F32CD)
         return mon ? reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32CD, true, false>)
                    : reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32CD, false, false>);
     if (dtype == PHTL_F32CS)

@@ -18,9 +18,7 @@ const void* general_kernel_single(int scheme, int dtype, bool dual)
 #define PHTL_GEN(S)                                                                          \
     if (scheme == S) {                                                                       \
         if (dtype == PHTL_F64) return reinterpret_cast<const void*>(&kf64::k_track_f64<S, true, true, true>); \
-        if (dtype == PHTL_F32C)                                                              \
-            return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32C, true, true, true>); \
-        if (dtype == PHTL_F32CD)                                                             \
+        if (dtype == PHTL_F32C || dtype == PHTL_F32CD)                                       \
             return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32CD, true, true, true>); \
         if (dtype == PHTL_F32CS)                                                             \
             return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32CS, true, true, true>); \

@@ -13,7 +13,6 @@ namespace phtl {
 const void* general_kernel_batched(int dtype)
 {
     if (dtype == PHTL_F64) return reinterpret_cast<const void*>(&k_batched_f64<true, true>);
-    if (dtype == PHTL_F32C) return reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32C, true, true>);
     return general_kernel_batched_f32(dtype);
 }
 

@@ -15,8 +15,6 @@ template <int S>
 const void* dual_s(int dtype)
 {
     if (dtype == PHTL_F64) return reinterpret_cast<const void*>(&kf64::k_track_f64<S, true, true, true, true>);
-    if (dtype == PHTL_F32C)
-        return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32C, true, true, true, true>);
     return nullptr;
 }
 
@@ -24,7 +22,7 @@ const void* dual_s(int dtype)
 
 const void* general_kernel_single_dual(int scheme, int dtype)
 {
-    if (dtype == PHTL_F32CD || dtype == PHTL_F32CS) return general_kernel_single_dual_f32(scheme, dtype);
+    if (dtype != PHTL_F64) return general_kernel_single_dual_f32(scheme, dtype);
     if (scheme == PHTL_EULER_CROMER) return dual_s<PHTL_EULER_CROMER>(dtype);
     if (scheme == PHTL_LEAPFROG) return dual_s<PHTL_LEAPFROG>(dtype);
     if (scheme == PHTL_RUTH4) return dual_s<PHTL_RUTH4>(dtype);

@@ -198,7 +198,8 @@ using namespace f32c;
 
 struct Turn {
     DF2 etaC, A, phis, sinphis, lin, r;
-    double phis64;  // PHTL_F32C forms the phase in FP64
+    DF2 phq;        // phi_s,n in quarter turns
+    double phis64;  // for the particles that form does not cover
 };
 
 template <int DT>
@@ -211,12 +212,13 @@ __device__ __forceinline__ Turn load_turn(const RampTurn* __restrict__ p)
     t.sinphis = DF2{__ldg(&p->sinphis_h), __ldg(&p->sinphis_l)};
     t.lin = DF2{__ldg(&p->lin_h), __ldg(&p->lin_l)};
     t.r = DF2{__ldg(&p->r_h), __ldg(&p->r_l)};
-    t.phis64 = DT == PHTL_F32C ? __ldg(&p->phis) : 0.0;
+    t.phis64 = __ldg(&p->phis);
+    t.phq = DF2{__ldg(&p->phq_h), __ldg(&p->phq_l)};
     return t;
 }
 
 // kick of weight w (a compile-time constant of the scheme): delta += w A_n (sin(phi_s,n +
-// k z) - sin(phi_s,n)), the phase in FP64 (PHTL_F32C), double-float (PHTL_F32CD) or
+// k z) - sin(phi_s,n)), the phase in double-float quarter turns (PHTL_F32C, PHTL_F32CD) or
 // rounded to FP32 for the SFU sine (PHTL_F32CS)
 template <int DT>
 __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], double w, const Turn& T,
@@ -224,9 +226,9 @@ __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], double w, con
 {
     const DFC wc(w);
     const DF2 kw = df_mul(DF2{wc.h, wc.l}, T.A);
+    if (DT == PHTL_F32CS) {
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        if (DT == PHTL_F32CS) {
+        for (int p = 0; p < P; ++p) {
             float f;
             if (c.linear) {
                 f = T.lin.h * (z[p].hi + z[p].c);
@@ -235,23 +237,21 @@ __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], double w, con
                 f = sin_sfu(__fadd_rn(ph.h, ph.l)) - T.sinphis.h;
             }
             acc(d[p], __fmaf_rn(kw.h, f, __fmul_rn(kw.l, f)));
-        } else {
-            DF2 f;
-            if (c.linear) {
-                f = df_mul(T.lin, as2(z[p]));
-            } else {
-                DF2 ph;
-                if (DT == PHTL_F32C) {
-                    const double zd = widen_float_phase(z[p].hi) + widen_float_phase(z[p].c);
-                    ph = split_phase(fma(c.k, zd, T.phis64));
-                } else {
-                    ph = df_add(df_mul(DF2{c.k_hi, c.k_lo}, as2(z[p])), T.phis);
-                }
-                f = df_add(sin_df(ph), neg2(T.sinphis));
-            }
-            acc2(d[p], df_mul(kw, f));
         }
+        return;
     }
+    DF2 f[P], zz[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) zz[p] = as2(z[p]);
+    if (c.linear) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) f[p] = df_mul(T.lin, zz[p]);
+    } else {
+        force_df<false>(c.kq, T.phq.h, T.phq.l, c.k, T.phis64,
+                        neg2(T.sinphis), zz, f);
+    }
+#pragma unroll
+    for (int p = 0; p < P; ++p) acc2(d[p], df_mul_raw(kw, f[p]));
 }
 
 template <int DT>
@@ -367,21 +367,13 @@ __device__ __forceinline__ void ramp_f32c_body(const LaunchDesc& L, const MapCon
     }
 }
 
-// FP32CD and FP32CS: the compiler's register choice; FP32C: 3 resident 256-thread blocks per SM
-// (80 registers), 6.6 % faster over the three schemes (1e6 particles x 1000 turns, transverse,
-// a monitor row every turn; FP32CD and FP32CS gained nothing at 2 or 3 blocks)
+// The compiler's register choice: 3 resident 256-thread blocks per SM (80 registers) took 8 %
+// longer for FP32C / FP32CD (1e6 particles x 300 turns, leap-frog, both planes, moments every turn)
 template <int S, int DT>
 __global__ void PHTL_F32C_RAMP_BOUNDS(S, DT)
     k_ramp_f32c(LaunchDesc L, MapConsts c, MonitorArgs m, const RampTurn* __restrict__ prog, int64_t turn0)
 {
     ramp_f32c_body<S, DT>(L, c, m, prog, turn0);
-}
-
-template <int S>
-__global__ void PHTL_F32C_RAMP_BOUNDS_C
-    k_ramp_f32c_c(LaunchDesc L, MapConsts c, MonitorArgs m, const RampTurn* __restrict__ prog, int64_t turn0)
-{
-    ramp_f32c_body<S, PHTL_F32C>(L, c, m, prog, turn0);
 }
 
 }  // namespace rf32
@@ -390,8 +382,8 @@ template <int S>
 const void* ramp_kernel_s(int dtype)
 {
     if (dtype == PHTL_F64) return reinterpret_cast<const void*>(&rf64::k_ramp_f64<S>);
-    if (dtype == PHTL_F32C) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c_c<S>);
-    if (dtype == PHTL_F32CD) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32CD>);
+    // PHTL_F32C and PHTL_F32CD are the same arithmetic: one instantiation
+    if (dtype == PHTL_F32C || dtype == PHTL_F32CD) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32CD>);
     if (dtype == PHTL_F32CS) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32CS>);
     return nullptr;
 }
