@@ -169,8 +169,9 @@ int phtl_track_programme(phtl_handle* h, void* z, void* dp, void* x, void* xp, v
         }
     }
     if (n == 0 || (turns == 0 && !mon_rows)) return PHTL_OK;
-    // default block: 96 threads in FP64 (2 % over 128 on 1e6 x 4000 turns), 128 in FP32
-    const int block = h->block > 0 ? h->block : (dtype == PHTL_F64 ? 96 : 128);
+    // default block: 32 threads in FP64 (a block of one warp needs no barrier for its moment sums,
+    // as in phtl_track), 128 in FP32
+    const int block = h->block > 0 ? h->block : (dtype == PHTL_F64 ? 32 : 128);
     const int ppt = particles_per_thread(dtype);
     int64_t tpl = h->tpl > 0 ? h->tpl : auto_turns_per_launch(dtype, integrator, n);
     tpl = std::min<int64_t>(tpl, 1 << 30);

@@ -511,15 +511,21 @@ __device__ __forceinline__ void rk4_turn(DF (&z)[P], DF (&d)[P], const MapConsts
         } else {
             const DF2 dc{dh, dl}, g1{g1h, g1l}, g2{g2h, g2l}, kw{kh, kl}, kw2{k2h, k2l};
             const DF2 z0 = as2(z[p]), d0 = as2(d[p]);
-            DF2 k1z, k1d, k2z, k2d, k3z, k3d, k4z, k4d;
-            rk4_rhs_df<DT, ZS>(z0, d0, c, dc, g1, g2, kw, kw2, dual, k1z, k1d);
-            rk4_rhs_df<DT, ZS>(df_add(z0, df_scale2(k1z, 0.5f)), df_add(d0, df_scale2(k1d, 0.5f)), c,
-                               dc, g1, g2, kw, kw2, dual, k2z, k2d);
-            rk4_rhs_df<DT, ZS>(df_add(z0, df_scale2(k2z, 0.5f)), df_add(d0, df_scale2(k2d, 0.5f)), c,
-                               dc, g1, g2, kw, kw2, dual, k3z, k3d);
-            rk4_rhs_df<DT, ZS>(df_add(z0, k3z), df_add(d0, k3d), c, dc, g1, g2, kw, kw2, dual, k4z, k4d);
-            const DF2 sz = df_add(df_add(k1z, k4z), df_scale2(df_add(k2z, k3z), 2.0f));
-            const DF2 sd = df_add(df_add(k1d, k4d), df_scale2(df_add(k2d, k3d), 2.0f));
+            DF2 a = z0, b = d0, kz, kd, sz{0.0f, 0.0f}, sd{0.0f, 0.0f};
+            // the stages as a loop: in line, the sines of four particles and stages overrun the
+            // instruction cache
+#pragma unroll 1
+            for (int st = 0;; ++st) {
+                rk4_rhs_df<DT, ZS>(a, b, c, dc, g1, g2, kw, kw2, dual, kz, kd);
+                if (st == 3) break;
+                const float cs = st == 0 ? 1.0f : 2.0f, step = st == 2 ? 1.0f : 0.5f;
+                sz = df_add(sz, df_scale2(kz, cs));
+                sd = df_add(sd, df_scale2(kd, cs));
+                a = df_add(z0, df_scale2(kz, step));
+                b = df_add(d0, df_scale2(kd, step));
+            }
+            sz = df_add(sz, kz);
+            sd = df_add(sd, kd);
             acc2(z[p], df_mul(sz, DF2{sixth.h, sixth.l}));
             acc2(d[p], df_mul(sd, DF2{sixth.h, sixth.l}));
         }

@@ -354,36 +354,37 @@ __device__ __forceinline__ void rk4_rhs(const double (&z)[P], const double (&d)[
 
 // One classic RK4 step of one turn: k1 at the start, k2 and k3 at the half step from k1
 // and k2, k4 at the full step from k3, and the weighted sum (k1 + 2 k2 + 2 k3 + k4) / 6.
+// The four stages are a loop that is not unrolled: with the sines of both RF systems in line
+// four times the turn's code did not fit the instruction cache (3.5 stalled cycles for
+// instructions per issue on the double-RF ring).
 template <int MODE>
 __device__ __forceinline__ void rk4_turn(double (&z)[P], double (&d)[P], const MapConsts& c,
                                          const GeneralWeights& w, bool dual)
 {
-    double k1z[P], k1d[P], k2z[P], k2d[P], k3z[P], k3d[P], k4z[P], k4d[P], a[P], b[P];
-    rk4_rhs<MODE>(z, d, c, w, dual, k1z, k1d);
+    double a[P], b[P], kz[P], kd[P], sz[P], sd[P];
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        a[p] = fma(w.half, k1z[p], z[p]);
-        b[p] = fma(w.half, k1d[p], d[p]);
+        a[p] = z[p];
+        b[p] = d[p];
+        sz[p] = sd[p] = 0.0;
     }
-    rk4_rhs<MODE>(a, b, c, w, dual, k2z, k2d);
+#pragma unroll 1
+    for (int st = 0;; ++st) {
+        rk4_rhs<MODE>(a, b, c, w, dual, kz, kd);
+        if (st == 3) break;
+        const double cs = st == 0 ? w.one : w.two, step = st == 2 ? w.one : w.half;
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        a[p] = fma(w.half, k2z[p], z[p]);
-        b[p] = fma(w.half, k2d[p], d[p]);
+        for (int p = 0; p < P; ++p) {
+            sz[p] = fma(cs, kz[p], sz[p]);
+            sd[p] = fma(cs, kd[p], sd[p]);
+            a[p] = fma(step, kz[p], z[p]);
+            b[p] = fma(step, kd[p], d[p]);
+        }
     }
-    rk4_rhs<MODE>(a, b, c, w, dual, k3z, k3d);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        a[p] = __fma_rn(k3z[p], w.one, z[p]);
-        b[p] = __fma_rn(k3d[p], w.one, d[p]);
-    }
-    rk4_rhs<MODE>(a, b, c, w, dual, k4z, k4d);
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-        const double sz = fma(w.two, __fma_rn(k2z[p], w.one, k3z[p]), __fma_rn(k1z[p], w.one, k4z[p]));
-        const double sd = fma(w.two, __fma_rn(k2d[p], w.one, k3d[p]), __fma_rn(k1d[p], w.one, k4d[p]));
-        z[p] = fma(sz, w.sixth, z[p]);
-        d[p] = fma(sd, w.sixth, d[p]);
+        z[p] = fma(__fma_rn(kz[p], w.one, sz[p]), w.sixth, z[p]);
+        d[p] = fma(__fma_rn(kd[p], w.one, sd[p]), w.sixth, d[p]);
     }
 }
 
@@ -608,8 +609,13 @@ __device__ __forceinline__ void record(const double (&z)[P], const double (&d)[P
     double v = scaled_to_double(total, ex, k == 2 || k == 3 ? 0u : 1u);
     // Inf or NaN among the warp's values
     if (field != 0 && (e1 == 2047 || (k >= 2 && e2 == 2047))) v = __hiloint2double(0x7ff80000, 0);
+    const bool owner = (lane & ((1 << kShift) - 1)) == 0;  // one lane of each field's
+    if (nwarps == 1) {
+        if (owner && field < (TRANS ? 16 : 6)) atomicAdd(rows + row * PHTL_MON_FIELDS + field, v);
+        return;
+    }
     double* buf = smem + parity * (nwarps * 16);
-    if ((lane & ((1 << kShift) - 1)) == 0) buf[warp * 16 + field] = v;
+    if (owner) buf[warp * 16 + field] = v;
     __syncthreads();
     if (warp == 0 && lane < (TRANS ? 16 : 6)) {
         double s = buf[lane];
