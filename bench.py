@@ -526,6 +526,8 @@ def run_ours(args, wl_name, wl):
         kname = kname.replace("k_track_", "k_ramp_")
     if wl.get("wake"):
         kname = f"k_coll_turn<{dom}> (one turn + slicing + previous turn's wake kick)"
+    issue_key = (dt, dom, bool(wl["transverse"]), bool(wl["stride"]),
+                 False if map_variant(wl) == "plain" else map_variant(wl))
 
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
@@ -542,11 +544,10 @@ def run_ours(args, wl_name, wl):
                    "l2": "flushed between timed steps (256 MiB write); state 48 MB resident",
                    "parallelism": f"replica per GPU x{ws}",
                    "launch": "per-turn" if wl.get("perturn") else "persistent"},
-        "roofline": roof or (issue_roofline(
-            kname, (dt, dom, bool(wl["transverse"]), bool(wl["stride"]),
-                    False if map_variant(wl) == "plain" else map_variant(wl)),
-            n * tpl / dur_s, clk.get("sm_mhz")) if dt != "f64" else None) or fp64_roofline(
-            kname, dt, dom, wl, n, tpl, dur_s, flops_pt, achieved),
+        "roofline": roof or executed_now(
+            issue_roofline(kname, issue_key, n * tpl / dur_s, clk.get("sm_mhz")) if dt != "f64"
+            else fp64_roofline(kname, dt, dom, wl, n, tpl, dur_s, flops_pt, achieved),
+            issue_key if dt != "f64" else (*issue_key[:4], map_variant(wl)), n * tpl / dur_s),
         "gpu_launches": launches,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "steps": e2e_steps,
@@ -569,7 +570,9 @@ def run_ours(args, wl_name, wl):
 NCU_TRAFFIC_BYTES_PER_PARTICLE = {("f64", "ruth4", True, True): (144.729600e6 + 83.410688e6) / 3e6}
 
 
-# FP64 flops the kernel executes per particle-turn, from the same ncu capture:
+# FP64 flops per particle-turn of the kernels with the sines in FP64 arithmetic, from the same ncu
+# capture (what the present kernels execute is in EXECUTED_NOW below; this count is reported beside it
+# as the work of that form):
 # (2 x DFMA + DMUL + DADD thread instructions per cycle) x cycles / particle-turns, i.e.
 # (2 x 225.068198 + 33.760230 + 0.474220) x 22.946400 ms x 2.044726 GHz / (3e6 x 88).
 # Fewer than the algorithmic count: for phi_s = 0 the kernel skips the phase addition and the
@@ -755,7 +758,8 @@ def _clocked(fn):
     return v, clk
 
 
-# Executed warp-instructions per particle-turn of the FP32-compensated persistent kernels
+# Warp-instructions per particle-turn of the FP32-compensated persistent kernels with the phase in FP64
+# or radians and renormalised products (the present kernels' are in EXECUTED_NOW)
 # (sm__inst_executed.sum / particle-turns of the launch), from one ncu capture per kernel:
 # 2e6 particles x 200 turns per launch, transverse planes, stride-1 monitor (summary:
 # profiles/k_track_f32c_instruction_counts_2e6x200.md); keyed by (dtype, scheme,
@@ -805,6 +809,59 @@ def issue_roofline(kname, key=None, pts=None, sm_mhz=None):
         return out
     ach = per * pts / 1e9
     out.update(achieved=ach, frac=ach / peak, warp_inst_per_particle_turn_ncu=per)
+    return out
+
+
+# What the present kernels execute per particle-turn, from one ncu capture each (1e6 particles x 40
+# turns, both planes, moments every turn; the batches 64 leap-frog bunches of 4.0e6 particles, 200 turns;
+# profiles/executed_counts_1e6x40.md): FP64 flops (2 DFMA + DMUL + DADD thread instructions) of the FP64
+# kernels, warp-instructions of the FP32 ones; keyed as above.
+EXECUTED_NOW = {
+    ("f64", "ruth4", True, True, "plain"): (2 * 520_000_000 + 40_466_944) / 4e7,
+    ("f64", "ruth4", True, True, "widened"): (2 * 920_012_240 + 2_002_720 + 82_000_000) / 4e7,
+    ("f64", "ruth4", True, True, "double_rf"): (2 * 640_000_000 + 42_000_000) / 4e7,
+    ("f64", "rk4", True, True, "double_rf"): (2 * 1_360_000_010 + 80_500_000) / 4e7,
+    ("f64", "ruth4", True, True, "ramp"): (2 * 520_000_010 + 120_000_002 + 120_000_000) / 4e7,
+    ("f64", "leapfrog", False, True, "batched"): (2 * 2_402_150_400 + 41_724_852) / 799_999_200,
+    ("f64", "leapfrog", True, True, "collective"): (2 * 27_000_576 + 3_000_000 + 6_562_512) / 3e6,
+    ("f32cs", "leapfrog", True, True, False): 235314078 / 4e7,
+    ("f32cs", "ruth4", True, True, False): 350447674 / 4e7,
+    ("f32cs", "leapfrog", True, True, "widened"): 273249116 / 4e7,
+    ("f32cs", "ruth4", True, True, "widened"): 400925430 / 4e7,
+    ("f32cs", "rk4", True, True, "double_rf"): 460129668 / 4e7,
+}
+for _dt in ("f32c", "f32cd"):  # one arithmetic, the same kernels
+    EXECUTED_NOW.update({
+        (_dt, "leapfrog", True, True, False): 315765457 / 4e7,
+        (_dt, "ruth4", True, True, False): 593405387 / 4e7,
+        (_dt, "leapfrog", False, True, True): 3912999552 / 799999200,
+        (_dt, "leapfrog", True, True, "widened"): 898412636 / 4e7,
+        (_dt, "ruth4", True, True, "widened"): 1252241904 / 4e7,
+        (_dt, "rk4", True, True, "double_rf"): 1569819738 / 4e7,
+    })
+
+
+def executed_now(r, key, pts):
+    """The roofline r with achieved and frac from what the present kernels execute (EXECUTED_NOW)
+    where a capture of the variant exists; the fraction r had goes to `frac_of_the_earlier_count`
+    (FP64: sines as FP64 work; FP32: instructions of the earlier kernels), which a kernel that
+    does the same work with less can take beyond 1."""
+    per = EXECUTED_NOW.get(key)
+    if per is None or not r:
+        return r
+    issue = r.get("bound") == "issue"
+    achieved = per * pts / (1e9 if issue else 1e12)
+    out = dict(r, frac_of_the_earlier_count=r.get("frac"), achieved=achieved, frac=achieved / r["peak"])
+    if issue:
+        out["warp_inst_per_particle_turn_ncu"] = per
+    else:
+        for k in ("executed_flops_per_particle_turn_ncu", "executed_tflops", "executed_frac"):
+            out.pop(k, None)
+        out.update(executed_flops_per_particle_turn_ncu=per, executed_tflops=achieved,
+                   executed_frac=achieved / r["peak"],
+                   basis="ncu-executed FP64 flops per particle-turn (2 DFMA + DMUL + DADD) of the present "
+                         "kernels x live particle-turns/s; sines, chromatic phases and moment sums run on "
+                         f"the integer pipe; alg_frac counts each sine as {SINE_FLOPS} flops")
     return out
 
 
@@ -895,9 +952,10 @@ def measure_batched(wl, steps, warmup):
         "gpu_launches": launches, "clocks": clk,
     }
     if dt != "f64":
-        out["roofline"] = issue_roofline(f"k_batched_f32c<{dt}, {wl['scheme']}, monitor>",
-                                         (dt, wl["scheme"], False, True, True), value,
-                                         clk.get("sm_mhz"))
+        key = (dt, wl["scheme"], False, True, True)
+        out["roofline"] = executed_now(
+            issue_roofline(f"k_batched_f32c<{dt}, {wl['scheme']}, monitor>", key, value, clk.get("sm_mhz")),
+            key, value)
     else:
         # FP64-pipe roofline at the rate over whole batch runs (many launches per run)
         wlb = dict(wl, transverse=False)
@@ -906,6 +964,7 @@ def measure_batched(wl, steps, warmup):
                           pt * steps, 1, t, fpt, fpt * value / 1e12)
         r.pop("launch_ms", None)
         r.pop("turns_per_launch", None)
+        r = executed_now(r, ("f64", wl["scheme"], False, True, "batched"), value)
         r["basis"] += "; rate over whole batch runs (CUDA events)"
         out["roofline"] = r
     B.close()

@@ -129,7 +129,6 @@ int derive(const phtl_params& p, phtl_derived& d, MapConsts (&mc)[4])
         std::memset(&c, 0, sizeof(c));
         scheme_consts(d, s, c);
         c.k = d.k;
-        c.k2opi = static_cast<float>(d.k * (2.0 / kPi));
         c.kap = integer_phase(d.k, p.phi_s_rad);
         c.uphis = phase_turns(p.phi_s_rad);
         c.kq = quarter_phase(d.k, p.phi_s_rad);

@@ -24,8 +24,10 @@ inline void split_df(double v, float& hi, float& lo)
 
 // k / 2 pi for the integer phase of the FP64 sines: K 2^(959 - cn), K in [2^62, 2^63).  cn = kNoPhaseScale (no integer phase) where k is zero or so large or
 // small that the exponent arithmetic of the device would leave the range of a double.
+// K2: what K leaves of k / 2 pi, in 2^-64 of K's unit.
 struct PhaseScale {
     uint64_t K;
+    int64_t K2;
     int32_t cn;
     int32_t pad_;
 };
@@ -44,7 +46,7 @@ inline unsigned __int128 over_two_pi(uint64_t m)
 
 inline PhaseScale phase_scale(double k)
 {
-    PhaseScale r{0, kNoPhaseScale, 0};
+    PhaseScale r{0, 0, kNoPhaseScale, 0};
     int e = 0;
     const double f = std::frexp(k, &e);  // k = f 2^e, f in [1/2, 1)
     if (!(f >= 0.5 && std::isfinite(k))) return r;
@@ -59,6 +61,7 @@ inline PhaseScale phase_scale(double k)
     // K = 2^63 (a carry out of the rounding) does not fit the device's products
     if ((K >> 63) || cn < 900 || cn > 1900) return r;
     r.K = K;
+    r.K2 = static_cast<int64_t>(static_cast<uint64_t>(v >> 1));  // v less K 2^65, in 2^1: signed
     r.cn = cn;
     return r;
 }
@@ -80,7 +83,7 @@ inline uint64_t phase_turns(double phi)
 // The phase scale of sin(k z + phi): none where |phi| is beyond phase_turns().
 inline PhaseScale integer_phase(double k, double phi)
 {
-    return std::fabs(phi) < 1e5 ? phase_scale(k) : PhaseScale{0, kNoPhaseScale, 0};
+    return std::fabs(phi) < 1e5 ? phase_scale(k) : PhaseScale{0, 0, kNoPhaseScale, 0};
 }
 
 // A factor of the integer phases and sines by its magnitude, K 2^(e - 63) with K in
@@ -176,7 +179,7 @@ struct MapConsts {
     float k_hi, k_lo, phis_hi, phis_lo, sinphis_hi, sinphis_lo, lin_hi, lin_lo;
     float mx_hi[4], mx_lo[4], my_hi[4], my_lo[4];
     int32_t linear;  // rf_linear flag
-    float k2opi;     // k * 2/pi rounded to FP32 (quadrant estimate of the fused FP64 sine)
+    int32_t pad2_;
     PhaseScale kap;  // k / 2 pi and phi_s / 2 pi of the integer phase
     uint64_t uphis;
     // widened map: nonlinear slippage eta(d) = eta0 + eta1 d + eta2 d^2 and chromaticity

@@ -15,7 +15,7 @@
 // the updates of the state there (leap-frog 3 FMAs, each plane 3); the sines and the moment
 // sums run on the integer pipe beside it.  Leap-frog without planes: 83 % of the FP64 pipe, 1.8
 // clocks per particle-turn and SM (14 FP64 instructions and 7.9 clocks with the sine in FP64);
-// with both planes and moments every turn 70 %, 57 % of the integer (ALU) pipe, 7.1 clocks (12.5).
+// with both planes and moments every turn 68 %, 61 % of the integer (ALU) pipe, 6.4 clocks (12.5).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -117,7 +117,7 @@ __device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[P
 #pragma unroll
         for (int p = 0; p < P; ++p)
             if (!ok[p])
-                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.k2opi, z[p]) : sin_phi_rest(c.k, z[p], c.phis);
+                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.uphis);
     }
     if (MODE == kRfGeneral) {
 #pragma unroll
@@ -194,6 +194,7 @@ __device__ __forceinline__ void rotate(double (&u)[P], double (&v)[P], const dou
 // only kick, or x beside Ruth4's first and y beside its second.
 template <int SCHEME>
 struct RotateBeside {
+    static constexpr int kYBeside = SCHEME == PHTL_RUTH4 ? 1 : 0;
     double (&x)[P];
     double (&xp)[P];
     double (&y)[P];
@@ -204,7 +205,7 @@ struct RotateBeside {
     __device__ __forceinline__ void operator()(int j) const
     {
         if (j == 0 && hx) rotate(x, xp, c.mx, w.shx, c.shear_x != 0);
-        if (j == (SCHEME == PHTL_RUTH4 ? 1 : 0) && hy) rotate(y, yp, c.my, w.shy, c.shear_y != 0);
+        if (j == kYBeside && hy) rotate(y, yp, c.my, w.shy, c.shear_y != 0);
     }
 };
 
@@ -217,7 +218,15 @@ struct RotateBeside {
 struct GeneralWeights {
     double dc[4], g1[4], g2[4], kw[3], kw2[3], shx[2], shy[2];
     double one, mzero, half, two, sixth;
+    int zero;  // see integer_copy
 };
+
+// A copy of a double on the integer pipe, zero = 0 in a register the compiler cannot see through:
+// it copies a register pair with a DADD otherwise.
+__device__ __forceinline__ double integer_copy(double v, int zero)
+{
+    return __hiloint2double(__double2hiint(v) ^ zero, __double2loint(v) ^ zero);
+}
 
 template <int SCHEME>
 __device__ __forceinline__ GeneralWeights general_weights(const double* dc, const double* kw,
@@ -230,8 +239,9 @@ __device__ __forceinline__ GeneralWeights general_weights(const double* dc, cons
     for (int i = 0; i < 4; ++i) {
         if (i < kDrifts) {
             w.dc[i] = in_register(-dc[i]);
-            w.g1[i] = -(drift_weight(SCHEME, i) * c.eta1C);
-            w.g2[i] = -(drift_weight(SCHEME, i) * c.eta2C);
+            // (also keeps the compiler from forming the products anew in every turn)
+            w.g1[i] = in_register(-(drift_weight(SCHEME, i) * c.eta1C));
+            w.g2[i] = in_register(-(drift_weight(SCHEME, i) * c.eta2C));
         }
     }
 #pragma unroll
@@ -251,6 +261,7 @@ __device__ __forceinline__ GeneralWeights general_weights(const double* dc, cons
     w.half = in_register(0.5);
     w.two = in_register(2.0);
     w.sixth = in_register(1.0 / 6.0);
+    w.zero = __shfl_sync(kFullMask, 0, 0);
     return w;
 }
 
@@ -303,8 +314,8 @@ __device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[
 #pragma unroll
         for (int p = 0; p < P; ++p) {
             if (!ok[p])
-                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.k2opi, z[p]) : sin_phi_rest(c.k, z[p], c.phis);
-            if (!ok2[p]) g[p] = sin_phi_rest(c.k2, z[p], c.phi2);
+                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.uphis);
+            if (!ok2[p]) g[p] = sin_phi_rest(c.k2, c.kap2, z[p], c.phi2, c.uphi2);
         }
     }
 #pragma unroll
@@ -364,8 +375,8 @@ __device__ __forceinline__ void rk4_turn(double (&z)[P], double (&d)[P], const M
     double a[P], b[P], kz[P], kd[P], sz[P], sd[P];
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        a[p] = z[p];
-        b[p] = d[p];
+        a[p] = integer_copy(z[p], w.zero);
+        b[p] = integer_copy(d[p], w.zero);
         sz[p] = sd[p] = 0.0;
     }
 #pragma unroll 1

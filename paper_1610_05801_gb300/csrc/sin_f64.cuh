@@ -1,6 +1,6 @@
 // Sines of the FP64 kernels, written for the scarce FP64 pipe of GB300 (2 DFMA per clock per
-// SM): on the integer pipe for every phase in and around the bucket (second part of this file),
-// in FP64 arithmetic for what lies outside it.
+// SM): on the integer pipe for every phase k z up to ~1e5 (second part of this file), in FP64
+// arithmetic beyond and for the sine of a double (sin_f64).
 //
 // The FP64 form: Cody-Waite argument reduction x = q pi/2 + r (Cody & Waite, "Software Manual
 // for the Elementary Functions", 1980), done with fused multiply-adds so a two-part
@@ -13,11 +13,6 @@
 // integer pipe.  |x| > 1e5 (far outside any RF bucket) falls back to CUDA's sin().
 // Accuracy: a few ulp on |x| <= 1e5 (checked against CUDA's sin and mpmath in the
 // tests through phtl_eval_sin).
-//
-// sin_kz_rest(k, z) = sin(k z) folds the product into the reduction: r = (k z - q H) - q L with
-// H = 3217/2048 (12 significant bits, so q H is an integer times 2^-11, formed exactly for
-// |q| < 2^16) and L = pi/2 - H rounded to FP64, so r is rounded relative to itself rather than to
-// k z.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -31,8 +26,6 @@ namespace detail {
 constexpr double kTwoOverPi = 0.63661977236758134308;
 constexpr double kPio2Hi = 1.5707963267948966;      // nearest double to pi/2
 constexpr double kPio2Lo = 6.123233995736766e-17;   // pi/2 - kPio2Hi
-constexpr float kPio2H12 = 1.57080078125f;          // 3217 / 2048
-constexpr double kPio2L12 = -4.454455103380769e-06; // pi/2 - 3217/2048
 constexpr float kMagic = 12582912.0f;               // 1.5 * 2^23: rounds to an integer
 
 // sin r = r + r^3 S(r^2), cos r = 1 - r^2/2 + r^4 C(r^2): coefficients of S and C from the
@@ -196,48 +189,42 @@ __device__ __forceinline__ double sin_f64(double x)
     return sin_quadrant(r, qi);
 }
 
-namespace detail {
-
-// -q H = -q 3217 / 2048 as a double, exactly, for |q| < 2^16: the integer product m = q 3217
-// (|m| < 2^28) placed into the significand with integer operations (no FP64 or conversion
-// instruction).  Within |q| < 4096 it equals the FP32 product q H, which is exact there.
-__device__ __forceinline__ double neg_q_h(int q)
-{
-    const int m = -q * 3217;
-    const unsigned a = static_cast<unsigned>(m < 0 ? -m : m);
-    const int p = 31 - __clz(static_cast<int>(a | 1u));            // leading bit of |m|
-    const unsigned long long mant = (static_cast<unsigned long long>(a) << (52 - p)) &
-                                    0x000FFFFFFFFFFFFFull;
-    const unsigned long long bits = (static_cast<unsigned long long>(m < 0 ? 1u : 0u) << 63) |
-                                    (static_cast<unsigned long long>(1023 - 11 + p) << 52) | mant;
-    return a == 0u ? -0.0 : __longlong_as_double(static_cast<long long>(bits));  // q = 0: -0 * H
-}
-
-}  // namespace detail
-
-// sin(k z) in FP64 arithmetic; k2opi = k * 2/pi rounded to FP32.  The fused form holds for
-// |k z| up to ~1e5 (the quadrant q below 2^16).  Beyond, and for Inf and NaN: sin_f64(k * z).
-// z = 0 (also the unused lanes of a ragged bunch) is returned as it is.  Out of line, as
-// sin_phi_rest: none of their FP64 instructions may be hoisted into the kicks.
-static __device__ __noinline__ double sin_kz_rest(double k, float k2opi, double z)
+// The phase k z of up to 2^14 turns (|k z| ~ 1e5) in 2^-64 turns, from the whole product of z's
+// significand and k / 2 pi in 127 bits: within 2^-62 turns however many turns there are.  false:
+// beyond that, |k z| below 2^-800, or a z that is zero, subnormal, Inf or NaN.
+__device__ __forceinline__ bool phase_of_turns(PhaseScale kap, double z, uint64_t& U)
 {
     using namespace detail;
-    if ((__double2hiint(z) << 1 | __double2loint(z)) == 0) return z;
-    const float xq = __fmul_rn(split_bits(z).h, k2opi);   // ~ k z * 2/pi
-    if (!(fabsf(xq) < 65536.0f)) return sin_f64(k * z);
-    const float tf = __fadd_rn(xq, kMagic);
-    const int qi = __float_as_int(tf);
-    const float qf = __fsub_rn(tf, kMagic);
-    const double mqh = neg_q_h(qi - __float_as_int(kMagic));         // -q H, exact
-    double r = fma(k, z, mqh);
-    r = fma(widen_float_bits(qf), -kPio2L12, r);
-    return sin_quadrant(r, qi);
+    const int e = (__double2hiint(z) >> 20) & 0x7ff;
+    const int n = kap.cn - e;
+    if (n < -15 || n > 800 || e == 0) return false;
+    const uint64_t M = mantissa64(z);
+    unsigned __int128 p = static_cast<unsigned __int128>(M) * kap.K;
+    p += static_cast<__int128>(__mul64hi(static_cast<long long>(M >> 1), kap.K2)) * 2;
+    if (n == -15 && (p >> 126) != 0) return false;
+    U = n > 64 ? 0u : static_cast<uint64_t>(p >> (63 + n));
+    return true;
 }
 
-// sin(k z + phi) in FP64 arithmetic.
-static __device__ __noinline__ double sin_phi_rest(double k, double z, double phi)
+// sin(k z) where sin_kz_fixed does not cover it.  z = 0 (also the unused lanes of a ragged bunch)
+// is returned as it is; up to 2^14 turns (particles that have left the bucket, an unbunched beam)
+// the integer form with the longer phase; beyond it, close to zero and for Inf and NaN
+// sin_f64(k * z).  Out of line, as sin_phi_rest: none of their instructions may be hoisted into the
+// kicks.
+static __device__ __noinline__ double sin_kz_rest(double k, PhaseScale kap, double z)
 {
-    return sin_f64(fma(k, z, phi));
+    if ((__double2hiint(z) << 1 | __double2loint(z)) == 0) return z;
+    uint64_t U;
+    if (!phase_of_turns(kap, z, U)) return sin_f64(k * z);
+    return detail::sin_turns_any(U, static_cast<uint32_t>(__double2hiint(z)));
+}
+
+// sin(k z + phi) where sin_kz_phi_fixed does not cover it, likewise.
+static __device__ __noinline__ double sin_phi_rest(double k, PhaseScale kap, double z, double phi, uint64_t uphi)
+{
+    uint64_t U;
+    if (!phase_of_turns(kap, z, U)) return sin_f64(fma(k, z, phi));
+    return detail::sin_turns_any(__double2hiint(z) < 0 ? uphi - U : uphi + U, 0u);
 }
 
 // The kicks take the integer sine of all their particles first, without a branch in between

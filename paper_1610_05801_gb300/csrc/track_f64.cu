@@ -80,7 +80,7 @@ __global__ void k_eval_sin(const double* __restrict__ x, double* __restrict__ y,
     }
 }
 
-__global__ void k_eval_sin_kz(double k, float k2opi, PhaseScale kap, const double* __restrict__ z,
+__global__ void k_eval_sin_kz(double k, PhaseScale kap, const double* __restrict__ z,
                               double* __restrict__ y, int64_t n)
 {
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
@@ -88,7 +88,7 @@ __global__ void k_eval_sin_kz(double k, float k2opi, PhaseScale kap, const doubl
     {
         bool ok;
         const double s = sin_kz_fixed(kap, z[i], ok);
-        y[i] = ok ? s : sin_kz_rest(k, k2opi, z[i]);
+        y[i] = ok ? s : sin_kz_rest(k, kap, z[i]);
     }
 }
 
@@ -130,9 +130,8 @@ extern "C" int phtl_eval_sin_kz(double k, const double* z, double* y, int64_t n,
     }
     if (n == 0) return PHTL_OK;
     const int block = 256;
-    const float k2opi = static_cast<float>(k * (2.0 / 3.14159265358979323846));
     phtl::k_eval_sin_kz<<<phtl::eval_grid(n, block), block, 0, static_cast<cudaStream_t>(stream)>>>(
-        k, k2opi, phtl::phase_scale(k), z, y, n);
+        k, phtl::phase_scale(k), z, y, n);
     if (cudaGetLastError() != cudaSuccess) return PHTL_E_CUDA;
     return PHTL_OK;
 }

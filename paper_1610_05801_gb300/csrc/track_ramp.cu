@@ -32,6 +32,12 @@ struct Turn {
     uint64_t uphis;
 };
 
+// Sums and products as FMAs of registers, a + b = fma(a, 1, b) and a b = fma(a, b, -0) exactly:
+// DADD and DMUL take the FP64 pipe a fifth longer.
+struct Unit {
+    double one, mzero;
+};
+
 __device__ __forceinline__ Turn load_turn(const RampTurn* __restrict__ p)
 {
     Turn t;
@@ -62,7 +68,7 @@ __device__ __forceinline__ void drift(double (&z)[P], const double (&d)[P], doub
 // delta += kw (sin(phi_s,n + k z) - sin(phi_s,n)), kw this stage's weight times A_n
 template <class Side>
 __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], double kw,
-                                     const Turn& T, const MapConsts& c, const Side& side, int j)
+                                     const Turn& T, const MapConsts& c, const Unit& u, const Side& side, int j)
 {
     double f[P];
     bool ok[P], all = true;
@@ -80,10 +86,10 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
         if (!all) {
 #pragma unroll
             for (int p = 0; p < P; ++p)
-                if (!ok[p]) f[p] = sin_phi_rest(c.k, z[p], T.phis);
+                if (!ok[p]) f[p] = sin_phi_rest(c.k, c.kap, z[p], T.phis, T.uphis);
         }
 #pragma unroll
-        for (int p = 0; p < P; ++p) f[p] -= T.sinphis;
+        for (int p = 0; p < P; ++p) f[p] = __fma_rn(f[p], u.one, -T.sinphis);
     }
 #pragma unroll
     for (int p = 0; p < P; ++p) d[p] = fma(kw, f[p], d[p]);
@@ -91,22 +97,22 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
 
 template <int S, class Side>
 __device__ __forceinline__ void turn(double (&z)[P], double (&d)[P], const Turn& T, const MapConsts& c,
-                                     const double* __restrict__ w, const Side& side)
+                                     const double* __restrict__ w, const Unit& u, const Side& side)
 {
     if (S == PHTL_EULER_CROMER) {
-        kick(z, d, __ldg(w + 1), T, c, side, 0);
+        kick(z, d, __ldg(w + 1), T, c, u, side, 0);
         drift(z, d, __ldg(w + 0));
     } else if (S == PHTL_LEAPFROG) {
         drift(z, d, __ldg(w + 0));
-        kick(z, d, __ldg(w + 2), T, c, side, 0);
+        kick(z, d, __ldg(w + 2), T, c, u, side, 0);
         drift(z, d, __ldg(w + 1));
     } else {
         drift(z, d, __ldg(w + 0));
-        kick(z, d, __ldg(w + 4), T, c, side, 0);
+        kick(z, d, __ldg(w + 4), T, c, u, side, 0);
         drift(z, d, __ldg(w + 1));
-        kick(z, d, __ldg(w + 5), T, c, side, 1);
+        kick(z, d, __ldg(w + 5), T, c, u, side, 1);
         drift(z, d, __ldg(w + 2));
-        kick(z, d, __ldg(w + 6), T, c, side, 2);
+        kick(z, d, __ldg(w + 6), T, c, u, side, 2);
         drift(z, d, __ldg(w + 3));
     }
 }
@@ -128,6 +134,7 @@ __global__ void __launch_bounds__(256, PHTL_F64_RAMP_MIN_BLOCKS)
     const int64_t chunk = static_cast<int64_t>(blockDim.x) * P;
     const int64_t nchunks = (L.n + chunk - 1) / chunk;
     int parity = 0;
+    const Unit unit{in_register(1.0), in_register(-0.0)};
     TurnWeights tw{};  // the shears; the stage weights come from the table
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -161,12 +168,12 @@ __global__ void __launch_bounds__(256, PHTL_F64_RAMP_MIN_BLOCKS)
         for (int t = 0; t < L.nturns; ++t) {
             // the next turn's constants, loaded while this turn computes
             const Turn Tn = load_turn(prog + turn0 + (t + 1 < L.nturns ? t + 1 : t));
-            turn<S>(z, d, T, c, stage_weights<S>(prog + turn0 + t), RotateBeside<S>{x, xp, y, yp, hx, hy, c, tw});
+            turn<S>(z, d, T, c, stage_weights<S>(prog + turn0 + t), unit, RotateBeside<S>{x, xp, y, yp, hx, hy, c, tw});
 #pragma unroll
             for (int p = 0; p < P; ++p) {
-                d[p] = T.r * d[p];
-                xp[p] = T.r * xp[p];
-                yp[p] = T.r * yp[p];
+                d[p] = __fma_rn(T.r, d[p], unit.mzero);
+                xp[p] = __fma_rn(T.r, xp[p], unit.mzero);
+                yp[p] = __fma_rn(T.r, yp[p], unit.mzero);
             }
             if (m.rows && --until == 0) {
                 record<true>(z, d, x, xp, y, yp, cnt, hx, hy, smem, parity, m.rows, row);
