@@ -395,14 +395,14 @@ cudaError_t launch_perturn(const LaunchDesc& L, const MapConsts& c, const Monito
 
 int occupancy_perturn(int scheme, bool trans, bool mon, int dtype, int block, int gen)
 {
-    return dtype == PHTL_F64 ? occupancy_f64(scheme, trans, mon, block, gen)
+    return dtype == PHTL_F64 ? occupancy_f64(scheme, trans, mon, block, gen, 0)
                              : occupancy_f32c(scheme, trans, mon, dtype, block, gen);
 }
 
-int occupancy(int dtype, int scheme, bool trans, bool mon, int block, bool perturn, int gen)
+int occupancy(int dtype, int scheme, bool trans, bool mon, int block, bool perturn, int gen, int ppt)
 {
     if (perturn) return occupancy_perturn(scheme, trans, mon, dtype, block, gen);
-    if (dtype == PHTL_F64) return occupancy_f64(scheme, trans, mon, block, gen);
+    if (dtype == PHTL_F64) return occupancy_f64(scheme, trans, mon, block, gen, ppt);
     return occupancy_f32c(scheme, trans, mon, dtype, block, gen);
 }
 
@@ -452,7 +452,9 @@ int enqueue_track(phtl_handle* h, void* const* c, int64_t n, int64_t turns, int 
     // ones (block size made no difference without a monitor), 256 for the per-turn launches
     const int block = h->block > 0 ? h->block : (perturn ? 256 : (dtype == PHTL_F64 ? 32 : 128));
     const int es = dtype == PHTL_F64 ? 8 : 4;
-    const int ppt = particles_per_thread(dtype);
+    const int gen = gen_level(h->mc[integrator]);
+    const int ppt = dtype == PHTL_F64 && !perturn ? f64_particles_per_thread(trans, mon, gen, n, h->nsm)
+                                                  : particles_per_thread(dtype);
     int64_t tpl = perturn ? 1 : (h->tpl > 0 ? h->tpl : auto_turns_per_launch(dtype, integrator, n));
     tpl = std::min<int64_t>(tpl, 1 << 30);
 
@@ -462,8 +464,7 @@ int enqueue_track(phtl_handle* h, void* const* c, int64_t n, int64_t turns, int 
     // FP32C buffers are [hi | comp]: the comp half is 16-byte aligned only if n % 4 == 0
     if (dtype != PHTL_F64 && (n * es) % 16 != 0) vec = false;
 
-    const int occ = occupancy(dtype, integrator, trans, mon, block, perturn,
-                              gen_level(h->mc[integrator]));
+    const int occ = occupancy(dtype, integrator, trans, mon, block, perturn, gen, ppt);
     if (occ <= 0) return PHTL_E_INVALID;
     const int64_t chunk = static_cast<int64_t>(block) * ppt;
     const int64_t nchunks = (n + chunk - 1) / chunk;
@@ -480,6 +481,7 @@ int enqueue_track(phtl_handle* h, void* const* c, int64_t n, int64_t turns, int 
     L.block = block;
     L.grid = std::max(grid, 1);
     L.vec = vec ? 1 : 0;
+    L.ppt = ppt;
     const MapConsts& mc = h->mc[integrator];
     // persistent calls: a cancellation gate in front of every launch (phtl_track_cancel)
     const bool gated = !perturn && h->ctl_dev && h->gate_go && !stream_capturing(s);

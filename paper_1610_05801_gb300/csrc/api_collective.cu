@@ -95,7 +95,10 @@ namespace {
 // Launch shape of the collective kernels for n particles (grid = resident capacity).
 int coll_launch(phtl_handle* h, void* const* c, int64_t n, int integrator, int dtype, LaunchDesc& L)
 {
-    const int block = h->block > 0 ? h->block : 128;
+    // 256 threads in FP64 (us per turn at 128 / 256, leap-frog, both planes, 512 slices: 12.5 / 12.1 at 1e5
+    // particles, 19.8 / 17.8 at 3e5, 25.5 / 26.2 at 6e5, 37.4 / 34.7 at 1e6, 63.4 / 64.5 at 2e6), 128 in
+    // FP32 (25.8 / 26.7 at 1e6, 44.9 / 49.1 at 2e6)
+    const int block = h->block > 0 ? h->block : (dtype == PHTL_F64 ? 256 : 128);
     const int occ = dtype == PHTL_F64 ? occupancy_coll(integrator, h->mc[integrator].general != 0, block,
                                                        h->coll.nslices)
                                       : occupancy_coll_f32(integrator, dtype, h->mc[integrator].general != 0,

@@ -282,7 +282,7 @@ struct LaunchDesc {
     int32_t block;     // threads per block
     int32_t grid;      // blocks
     int32_t vec;       // nonzero: all pointers 16-byte aligned (128-bit loads)
-    int32_t pad_;
+    int32_t ppt;       // FP64 single-bunch kernels: particles per thread (0: f64::P)
     const int* go;     // non-null: the launch runs only if *go != 0 (the call's cancellation
                        // gate, written by the gate kernel launched just before it)
 };
@@ -453,7 +453,9 @@ inline int gen_level(const MapConsts& c) { return c.general ? (c.dual_rf ? 2 : 1
 
 // Resident blocks per SM of a kernel variant at a block size (0 = cannot launch);
 // gen: the kernel family (gen_level).
-int occupancy_f64(int scheme, bool trans, bool mon, int block, int gen);
+int occupancy_f64(int scheme, bool trans, bool mon, int block, int gen, int ppt);
+// Particles per thread of the FP64 single-bunch kernel for a bunch of n on nsm SMs.
+int f64_particles_per_thread(bool trans, bool mon, int gen, int64_t n, int nsm);
 int occupancy_f32c(int scheme, bool trans, bool mon, int dtype, int block, int gen);
 int occupancy_perturn(int scheme, bool trans, bool mon, int dtype, int block, int gen);
 

@@ -57,7 +57,7 @@ __device__ __forceinline__ void run_f64_mode(double (&z)[f64::P], double (&d)[f6
             f64::long_turn_nl<SCHEME, MODE>(z, d, c, gw, c.dual_rf != 0);
             f64::transverse_gen(x, xp, y, yp, d, hx, hy, c, gw);
         } else {
-            f64::long_turn<SCHEME, MODE>(z, d, c, w, f64::RotateBeside<SCHEME>{x, xp, y, yp, hx, hy, c, w});
+            f64::long_turn<SCHEME, MODE>(z, d, c, w, f64::RotateBeside<SCHEME, f64::P>{x, xp, y, yp, hx, hy, c, w});
         }
         if (MON && J.mon) {
             if (--until == 0) {

@@ -32,9 +32,9 @@ using namespace f64;
 // The turn loop of one particle chunk (state in registers throughout).  GEN: the widened
 // map (slippage expansion, chromaticity, RK4), DUAL: with the second RF system; both
 // chosen once per launch.
-template <int SCHEME, bool TRANS, bool MON, int MODE, bool GEN, bool DUAL>
-__device__ __forceinline__ void turns(double (&z)[P], double (&d)[P], double (&x)[P],
-                                      double (&xp)[P], double (&y)[P], double (&yp)[P], bool hx,
+template <int SCHEME, bool TRANS, bool MON, int MODE, bool GEN, bool DUAL, int N>
+__device__ __forceinline__ void turns(double (&z)[N], double (&d)[N], double (&x)[N],
+                                      double (&xp)[N], double (&y)[N], double (&yp)[N], bool hx,
                                       bool hy, float cnt, const MapConsts& c, const TurnWeights& w,
                                       const MonitorArgs& m, int nturns, double* smem, int& parity)
 {
@@ -47,7 +47,7 @@ __device__ __forceinline__ void turns(double (&z)[P], double (&d)[P], double (&x
             if (TRANS) transverse_gen(x, xp, y, yp, d, hx, hy, c, gw);
         } else {
             if (TRANS)
-                long_turn<SCHEME, MODE>(z, d, c, w, RotateBeside<SCHEME>{x, xp, y, yp, hx, hy, c, w});
+                long_turn<SCHEME, MODE>(z, d, c, w, RotateBeside<SCHEME, N>{x, xp, y, yp, hx, hy, c, w});
             else
                 long_turn<SCHEME, MODE>(z, d, c, w, NoSideWork{});
         }
@@ -77,7 +77,7 @@ __device__ __forceinline__ void turns(double (&z)[P], double (&d)[P], double (&x
 #endif
 #define PHTL_F64_BOUNDS(S, G) __launch_bounds__(256, (G) ? PHTL_F64_GEN_MIN_BLOCKS : min_blocks_256<S>())
 #endif
-template <int SCHEME, bool TRANS, bool MON, bool GEN, bool DUAL = false>
+template <int SCHEME, bool TRANS, bool MON, bool GEN, bool DUAL = false, int N = P>
 __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
     k_track_f64(LaunchDesc L, MapConsts c, MonitorArgs m)
 {
@@ -92,19 +92,19 @@ __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
     const bool hx = TRANS && gx != nullptr;
     const bool hy = TRANS && gy != nullptr;
     const bool vec = L.vec != 0;
-    const int64_t chunk = static_cast<int64_t>(blockDim.x) * P;
+    const int64_t chunk = static_cast<int64_t>(blockDim.x) * N;
     const int64_t nchunks = (L.n + chunk - 1) / chunk;
     int parity = 0;
     TurnWeights w{};
     if (!GEN) w = turn_weights<SCHEME, TRANS>(c.dc, c.kw, c);
 
     for (int64_t ci = blockIdx.x; ci < nchunks; ci += gridDim.x) {
-        const int64_t base = ci * chunk + static_cast<int64_t>(threadIdx.x) * P;
-        double z[P], d[P], x[P], xp[P], y[P], yp[P];
+        const int64_t base = ci * chunk + static_cast<int64_t>(threadIdx.x) * N;
+        double z[N], d[N], x[N], xp[N], y[N], yp[N];
         load2(gz, base, L.n, vec, z);
         load2(gd, base, L.n, vec, d);
 #pragma unroll
-        for (int p = 0; p < P; ++p) x[p] = xp[p] = y[p] = yp[p] = 0.0;
+        for (int p = 0; p < N; ++p) x[p] = xp[p] = y[p] = yp[p] = 0.0;
         if (hx) {
             load2(gx, base, L.n, vec, x);
             load2(gxp, base, L.n, vec, xp);
@@ -114,7 +114,7 @@ __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
             load2(gyp, base, L.n, vec, yp);
         }
         const int64_t left = L.n - base;
-        const float cnt = left >= P ? static_cast<float>(P) : (left > 0 ? static_cast<float>(left) : 0.0f);
+        const float cnt = left >= N ? static_cast<float>(N) : (left > 0 ? static_cast<float>(left) : 0.0f);
 
         if (MON && m.rows && m.initial) {
             record<TRANS>(z, d, x, xp, y, yp, cnt, hx, hy, smem, parity, m.rows, 0);

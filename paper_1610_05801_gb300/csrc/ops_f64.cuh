@@ -1,6 +1,7 @@
 // FP64 per-particle operations shared by the FP64 kernels (single bunch and batched).
 //
-// One thread owns P = 2 particles.  The stage order of each scheme follows the readings
+// One thread owns P = 2 particles (1 in small bunches: the functions take their number N from the
+// arrays).  The stage order of each scheme follows the readings
 // of Sec. 1.1.2 stated in phtl.h; the transverse push is the Sec. 1.1.1 matrix.
 #pragma once
 
@@ -94,20 +95,20 @@ struct NoSideWork {
 };
 
 // The force of the main RF system per unit weight, sin(phi_s + k z) - sin(phi_s) or lin z in
-// rf_linear mode, of the thread's P particles.
-template <int MODE, class Side>
-__device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[P], double (&f)[P],
+// rf_linear mode, of the thread's N particles.
+template <int MODE, int N, class Side>
+__device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[N], double (&f)[N],
                                          const Side& side, int j)
 {
     if (MODE == kRfGeneral && c.linear) {
 #pragma unroll
-        for (int p = 0; p < P; ++p) f[p] = branch_product(c.lin, z[p]);
+        for (int p = 0; p < N; ++p) f[p] = branch_product(c.lin, z[p]);
         side(j);
         return;
     }
-    bool ok[P], all = true;
+    bool ok[N], all = true;
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         f[p] = MODE != kRfGeneral ? sin_kz_fixed(c.kap, z[p], ok[p])
                                   : sin_kz_phi_fixed(c.kap, z[p], c.uphis, ok[p]);
         all = all && ok[p];
@@ -115,38 +116,39 @@ __device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[P
     side(j);
     if (!all) {
 #pragma unroll
-        for (int p = 0; p < P; ++p)
+        for (int p = 0; p < N; ++p)
             if (!ok[p])
                 f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.uphis);
     }
     if (MODE == kRfGeneral) {
 #pragma unroll
-        for (int p = 0; p < P; ++p) f[p] -= c.sinphis;
+        for (int p = 0; p < N; ++p) f[p] -= c.sinphis;
     }
 }
 
 // Linear drift, ndc = -w eta C.
-__device__ __forceinline__ void drift_neg(double (&z)[P], const double (&d)[P], double ndc)
+template <int N>
+__device__ __forceinline__ void drift_neg(double (&z)[N], const double (&d)[N], double ndc)
 {
 #pragma unroll
-    for (int p = 0; p < P; ++p) z[p] = fma(ndc, d[p], z[p]);
+    for (int p = 0; p < N; ++p) z[p] = fma(ndc, d[p], z[p]);
 }
 
-template <int MODE, class Side>
-__device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], double kw,
+template <int MODE, int N, class Side>
+__device__ __forceinline__ void kick(const double (&z)[N], double (&d)[N], double kw,
                                      const MapConsts& c, const Side& side, int j)
 {
-    double f[P];
+    double f[N];
     rf_force<MODE>(c, z, f, side, j);
 #pragma unroll
-    for (int p = 0; p < P; ++p) d[p] = fma(kw, f[p], d[p]);
+    for (int p = 0; p < N; ++p) d[p] = fma(kw, f[p], d[p]);
 }
 
 // One turn of the scheme; stage order as in Sec. 1.1.2's readings (see phtl.h).
 // w: the drift (negated) and kick weights of this bunch's scheme, -w_i eta C and w_j A.
 // side: work beside the kicks' sines that touches neither z nor delta.
-template <int SCHEME, int MODE, class Side>
-__device__ __forceinline__ void long_turn(double (&z)[P], double (&d)[P], const MapConsts& c,
+template <int SCHEME, int MODE, int N, class Side>
+__device__ __forceinline__ void long_turn(double (&z)[N], double (&d)[N], const MapConsts& c,
                                           const TurnWeights& w, const Side& side)
 {
     if (SCHEME == PHTL_EULER_CROMER) {
@@ -169,12 +171,13 @@ __device__ __forceinline__ void long_turn(double (&z)[P], double (&d)[P], const 
 
 // Transverse push of one plane (Sec. 1.1.1 matrix).  With use_shear the rotation is
 // applied as three shears (3 DFMA instead of 2 DMUL + 2 DFMA); the same map up to rounding.
-__device__ __forceinline__ void rotate(double (&u)[P], double (&v)[P], const double (&m)[4],
+template <int N>
+__device__ __forceinline__ void rotate(double (&u)[N], double (&v)[N], const double (&m)[4],
                                        const double (&sh)[2], bool use_shear)
 {
     if (use_shear) {
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
+        for (int p = 0; p < N; ++p) {
             u[p] = fma(sh[0], v[p], u[p]);
             v[p] = fma(sh[1], u[p], v[p]);
             u[p] = fma(sh[0], v[p], u[p]);
@@ -182,7 +185,7 @@ __device__ __forceinline__ void rotate(double (&u)[P], double (&v)[P], const dou
         return;
     }
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         const double un = fma(m[1], v[p], m[0] * u[p]);
         const double vn = fma(m[3], v[p], m[2] * u[p]);
         u[p] = un;
@@ -192,13 +195,13 @@ __device__ __forceinline__ void rotate(double (&u)[P], double (&v)[P], const dou
 
 // The linear map's transverse push as the side work of a turn's kicks: both planes beside the
 // only kick, or x beside Ruth4's first and y beside its second.
-template <int SCHEME>
+template <int SCHEME, int N>
 struct RotateBeside {
     static constexpr int kYBeside = SCHEME == PHTL_RUTH4 ? 1 : 0;
-    double (&x)[P];
-    double (&xp)[P];
-    double (&y)[P];
-    double (&yp)[P];
+    double (&x)[N];
+    double (&xp)[N];
+    double (&y)[N];
+    double (&yp)[N];
     bool hx, hy;
     const MapConsts& c;
     const TurnWeights& w;
@@ -267,15 +270,15 @@ __device__ __forceinline__ GeneralWeights general_weights(const double* dc, cons
 
 // Drift with the slippage expansion: z -= (dc + g1 d + g2 d^2) d for this stage's
 // w eta(d) C (weights negated, see GeneralWeights).  Without the expansion the linear drift.
-template <int MODE>
-__device__ __forceinline__ void drift_nl(double (&z)[P], const double (&d)[P], const GeneralWeights& w, int i)
+template <int MODE, int N>
+__device__ __forceinline__ void drift_nl(double (&z)[N], const double (&d)[N], const GeneralWeights& w, int i)
 {
     if (MODE == kRfPlain) {
         drift_neg(z, d, w.dc[i]);
         return;
     }
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         const double e = fma(fma(w.g2[i], d[p], w.g1[i]), d[p], w.dc[i]);
         z[p] = fma(e, d[p], z[p]);
     }
@@ -286,9 +289,9 @@ __device__ __forceinline__ void drift_nl(double (&z)[P], const double (&d)[P], c
 // run together, before the particles they do not cover are mended.
 // `dual`: a compile-time constant in the single-bunch kernels, which have a variant without the
 // second system; the batched kernels pass the ring's flag.
-template <int MODE>
-__device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[P], double (&f)[P],
-                                          double (&g)[P], bool dual)
+template <int MODE, int N>
+__device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[N], double (&f)[N],
+                                          double (&g)[N], bool dual)
 {
     if (!dual) {
         rf_force<MODE>(c, z, f, NoSideWork{}, 0);
@@ -296,15 +299,15 @@ __device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[
     }
     if (MODE == kRfGeneral && c.linear) {
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
+        for (int p = 0; p < N; ++p) {
             f[p] = branch_product(c.lin, z[p]);
             g[p] = branch_product(c.lin2, z[p]);
         }
         return;
     }
-    bool ok[P], ok2[P], all = true;
+    bool ok[N], ok2[N], all = true;
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         f[p] = MODE != kRfGeneral ? sin_kz_fixed(c.kap, z[p], ok[p])
                                   : sin_kz_phi_fixed(c.kap, z[p], c.uphis, ok[p]);
         g[p] = sin_kz_phi_fixed(c.kap2, z[p], c.uphi2, ok2[p]);
@@ -312,14 +315,14 @@ __device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[
     }
     if (!all) {
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
+        for (int p = 0; p < N; ++p) {
             if (!ok[p])
                 f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.uphis);
             if (!ok2[p]) g[p] = sin_phi_rest(c.k2, c.kap2, z[p], c.phi2, c.uphi2);
         }
     }
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         if (MODE == kRfGeneral) f[p] -= c.sinphis;
         if (MODE != kRfPlain) g[p] -= c.sinphi2;
     }
@@ -327,14 +330,14 @@ __device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[
 
 // Kick of the widened map: the main RF system, then the second one when `dual` -- kw2: this
 // stage's w_j A2.
-template <int MODE>
-__device__ __forceinline__ void kick_gen(const double (&z)[P], double (&d)[P], double kw, double kw2,
+template <int MODE, int N>
+__device__ __forceinline__ void kick_gen(const double (&z)[N], double (&d)[N], double kw, double kw2,
                                          const MapConsts& c, bool dual)
 {
-    double f[P], g[P];
+    double f[N], g[N];
     rf_forces<MODE>(c, z, f, g, dual);
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         d[p] = fma(kw, f[p], d[p]);
         if (dual) d[p] = fma(kw2, g[p], d[p]);
     }
@@ -343,19 +346,19 @@ __device__ __forceinline__ void kick_gen(const double (&z)[P], double (&d)[P], d
 // Right-hand side of the smooth motion per turn (classic RK4's derivative):
 // dz/dn = -eta(d) C d = -(dc + g1 d + g2 d^2) d and dd/dn = kw F1(z) + kw2 F2(z), with
 // dc = eta0 C, g1 = eta1 C, g2 = eta2 C, kw = A, kw2 = A2.
-template <int MODE>
-__device__ __forceinline__ void rk4_rhs(const double (&z)[P], const double (&d)[P], const MapConsts& c,
-                                        const GeneralWeights& w, bool dual, double (&fz)[P],
-                                        double (&fd)[P])
+template <int MODE, int N>
+__device__ __forceinline__ void rk4_rhs(const double (&z)[N], const double (&d)[N], const MapConsts& c,
+                                        const GeneralWeights& w, bool dual, double (&fz)[N],
+                                        double (&fd)[N])
 {
     // the products are rounded on their own: the stage arguments and the weighted sum reuse
     // them, and an FMA contraction chosen differently where `dual` is a compile-time constant
     // than where it is not would break the bitwise agreement of the single-bunch and batched
     // kernels
-    double f[P], g[P];
+    double f[N], g[N];
     rf_forces<MODE>(c, z, f, g, dual);
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         const double e = MODE == kRfPlain ? w.dc[0] : fma(fma(w.g2[0], d[p], w.g1[0]), d[p], w.dc[0]);
         fz[p] = __fma_rn(e, d[p], w.mzero);
         fd[p] = __fma_rn(w.kw[0], f[p], w.mzero);
@@ -368,13 +371,13 @@ __device__ __forceinline__ void rk4_rhs(const double (&z)[P], const double (&d)[
 // The four stages are a loop that is not unrolled: with the sines of both RF systems in line
 // four times the turn's code did not fit the instruction cache (3.5 stalled cycles for
 // instructions per issue on the double-RF ring).
-template <int MODE>
-__device__ __forceinline__ void rk4_turn(double (&z)[P], double (&d)[P], const MapConsts& c,
+template <int MODE, int N>
+__device__ __forceinline__ void rk4_turn(double (&z)[N], double (&d)[N], const MapConsts& c,
                                          const GeneralWeights& w, bool dual)
 {
-    double a[P], b[P], kz[P], kd[P], sz[P], sd[P];
+    double a[N], b[N], kz[N], kd[N], sz[N], sd[N];
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         a[p] = integer_copy(z[p], w.zero);
         b[p] = integer_copy(d[p], w.zero);
         sz[p] = sd[p] = 0.0;
@@ -385,7 +388,7 @@ __device__ __forceinline__ void rk4_turn(double (&z)[P], double (&d)[P], const M
         if (st == 3) break;
         const double cs = st == 0 ? w.one : w.two, step = st == 2 ? w.one : w.half;
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
+        for (int p = 0; p < N; ++p) {
             sz[p] = fma(cs, kz[p], sz[p]);
             sd[p] = fma(cs, kd[p], sd[p]);
             a[p] = fma(step, kz[p], z[p]);
@@ -393,15 +396,15 @@ __device__ __forceinline__ void rk4_turn(double (&z)[P], double (&d)[P], const M
         }
     }
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         z[p] = fma(__fma_rn(kz[p], w.one, sz[p]), w.sixth, z[p]);
         d[p] = fma(__fma_rn(kd[p], w.one, sd[p]), w.sixth, d[p]);
     }
 }
 
 // One turn of the scheme with the slippage expansion and the second RF system.
-template <int SCHEME, int MODE>
-__device__ __forceinline__ void long_turn_nl(double (&z)[P], double (&d)[P], const MapConsts& c,
+template <int SCHEME, int MODE, int N>
+__device__ __forceinline__ void long_turn_nl(double (&z)[N], double (&d)[N], const MapConsts& c,
                                              const GeneralWeights& w, bool dual)
 {
     if (SCHEME == PHTL_RK4) {
@@ -426,25 +429,26 @@ __device__ __forceinline__ void long_turn_nl(double (&z)[P], double (&d)[P], con
 
 // Chromatic rotation of one plane: each particle turns by 2 pi (q + xi d) with its own d
 // (after the turn's longitudinal step).
-__device__ __forceinline__ void rotate_chroma(double (&u)[P], double (&v)[P], const double (&d)[P],
+template <int N>
+__device__ __forceinline__ void rotate_chroma(double (&u)[N], double (&v)[N], const double (&d)[N],
                                               const ChromaPlane& h, double q, double xi, double b,
                                               double ib, double mzero)
 {
-    double sb[P], sib[P], cs[P];
-    bool ok[P], all = h.on != 0;
+    double sb[N], sib[N], cs[N];
+    bool ok[N], all = h.on != 0;
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         chroma_fixed(h, d[p], sb[p], sib[p], cs[p], ok[p]);
         ok[p] = ok[p] && h.on != 0;
         all = all && ok[p];
     }
     if (!all) {
 #pragma unroll
-        for (int p = 0; p < P; ++p)
+        for (int p = 0; p < N; ++p)
             if (!ok[p]) chroma_rest(q, xi, b, ib, d[p], sb[p], sib[p], cs[p]);
     }
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         const double un = fma(sb[p], v[p], __fma_rn(cs[p], u[p], mzero));
         const double vn = fma(-sib[p], u[p], __fma_rn(cs[p], v[p], mzero));
         u[p] = un;
@@ -453,8 +457,9 @@ __device__ __forceinline__ void rotate_chroma(double (&u)[P], double (&v)[P], co
 }
 
 // The transverse step of the general loop: chromatic where xi != 0, else the one matrix.
-__device__ __forceinline__ void transverse_gen(double (&x)[P], double (&xp)[P], double (&y)[P],
-                                               double (&yp)[P], const double (&d)[P], bool hx,
+template <int N>
+__device__ __forceinline__ void transverse_gen(double (&x)[N], double (&xp)[N], double (&y)[N],
+                                               double (&yp)[N], const double (&d)[N], bool hx,
                                                bool hy, const MapConsts& c, const GeneralWeights& w)
 {
     if (hx) {
@@ -478,7 +483,8 @@ __device__ __forceinline__ void transverse_gen(double (&x)[P], double (&xp)[P], 
 //
 // The double-float sums before these took ~590 instructions per particle and record with both
 // planes (bit splits, TwoSum and Fast2Sum in every addition); these take ~390.
-constexpr int kMomentShift = P <= 2 ? 3 : 4;  // P X below 2^62
+template <int N>
+constexpr int kMomentShift = N <= 2 ? 3 : 4;  // N X below 2^62
 constexpr int kSumDrop = 4;                   // the warp adds (sum of X) 2^-4 ...
 constexpr int kProductDrop = 65;              // ... and (sum of X Y) 2^-65, below 2^63
 
@@ -487,21 +493,23 @@ struct PlaneExponents {
 };
 
 // High words without the sign: ordered as the magnitudes are.
-__device__ __forceinline__ int warp_exponent(const double (&a)[P])
+template <int N>
+__device__ __forceinline__ int warp_exponent(const double (&a)[N])
 {
     unsigned m = 0u;
 #pragma unroll
-    for (int p = 0; p < P; ++p) m = max(m, static_cast<unsigned>(__double2hiint(a[p])) & 0x7fffffffu);
+    for (int p = 0; p < N; ++p) m = max(m, static_cast<unsigned>(__double2hiint(a[p])) & 0x7fffffffu);
     return static_cast<int>(__reduce_max_sync(kFullMask, m) >> 20);
 }
 
 // |a| in units of 2^(E + kMomentShift - 1086), and the sign as a mask.
+template <int N>
 __device__ __forceinline__ uint64_t moment_magnitude(double a, int E, uint32_t& neg)
 {
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(a));
     neg = static_cast<uint32_t>(static_cast<int32_t>(hi) >> 31);
     const uint32_t e = (hi >> 20) & 0x7ffu;  // 0: zero (or subnormal) has no leading one, shift it out
-    return detail::shr_sat(detail::mantissa64(a), e != 0u ? static_cast<uint32_t>(E + kMomentShift) - e : 64u);
+    return detail::shr_sat(detail::mantissa64(a), e != 0u ? static_cast<uint32_t>(E + kMomentShift<N>) - e : 64u);
 }
 
 __device__ __forceinline__ int64_t moment_signed(uint64_t X, uint32_t neg)
@@ -512,16 +520,17 @@ __device__ __forceinline__ int64_t moment_signed(uint64_t X, uint32_t neg)
 
 // Sums of one plane (a, b) over the thread's particles: a, b (in 2^kSumDrop X), a^2, b^2 and ab
 // (in 2^kProductDrop X Y).
-__device__ __forceinline__ void pair_sums_fixed(const double (&a)[P], const double (&b)[P],
+template <int N>
+__device__ __forceinline__ void pair_sums_fixed(const double (&a)[N], const double (&b)[N],
                                                 PlaneExponents E, int64_t* f)
 {
     uint64_t aa = 0, aac = 0, bb = 0, bbc = 0;
     int64_t ab = 0, abc = 0;
     int64_t sa = 0, sb = 0;
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < N; ++p) {
         uint32_t na, nb;
-        const uint64_t A = moment_magnitude(a[p], E.a, na), B = moment_magnitude(b[p], E.b, nb);
+        const uint64_t A = moment_magnitude<N>(a[p], E.a, na), B = moment_magnitude<N>(b[p], E.b, nb);
         const uint32_t a1 = static_cast<uint32_t>(A >> 32), a0 = static_cast<uint32_t>(A);
         const uint32_t b1 = static_cast<uint32_t>(B >> 32), b0 = static_cast<uint32_t>(B);
         aa += static_cast<uint64_t>(a1) * a1;     // A^2 = aa 2^64 + 2 aac 2^32 + (below 2^64)
@@ -572,10 +581,10 @@ __device__ __forceinline__ double scaled_to_double(int64_t S, int x, uint32_t ne
 
 // Add this block's moment sums of the current turn into monitor row `row`.
 // smem: 2 * (blockDim.x / 32) * 16 doubles.
-template <bool TRANS>
-__device__ __forceinline__ void record(const double (&z)[P], const double (&d)[P],
-                                       const double (&x)[P], const double (&xp)[P],
-                                       const double (&y)[P], const double (&yp)[P],
+template <bool TRANS, int N>
+__device__ __forceinline__ void record(const double (&z)[N], const double (&d)[N],
+                                       const double (&x)[N], const double (&xp)[N],
+                                       const double (&y)[N], const double (&yp)[N],
                                        float cnt, bool hx, bool hy, double* smem, int parity,
                                        double* rows, int64_t row)
 {
@@ -614,8 +623,8 @@ __device__ __forceinline__ void record(const double (&z)[P], const double (&d)[P
     const int e1 = k == 1 || k == 3 ? Ef.b : Ef.a;
     const int e2 = k == 3 || k == 4 ? Ef.b : Ef.a;
     const int ex = field == 0 ? 0
-                   : k < 2    ? e1 + kMomentShift - 1086 + kSumDrop
-                              : e1 + e2 + 2 * (kMomentShift - 1086) + kProductDrop;
+                   : k < 2    ? e1 + kMomentShift<N> - 1086 + kSumDrop
+                              : e1 + e2 + 2 * (kMomentShift<N> - 1086) + kProductDrop;
     // squares truncated once more: a single particle's variance stays at or below zero
     double v = scaled_to_double(total, ex, k == 2 || k == 3 ? 0u : 1u);
     // Inf or NaN among the warp's values
@@ -642,34 +651,40 @@ __device__ __forceinline__ bool aligned16(const void* p)
     return (reinterpret_cast<uintptr_t>(p) & 15) == 0;
 }
 
+template <int N>
 __device__ __forceinline__ void load2(const double* __restrict__ g, int64_t base, int64_t n,
-                                      bool vec, double (&v)[P])
+                                      bool vec, double (&v)[N])
 {
-    if (vec && base + P <= n && aligned16(g + base)) {
+    if constexpr (N % 2 == 0) {
+        if (vec && base + N <= n && aligned16(g + base)) {
 #pragma unroll
-        for (int k = 0; k < P; k += 2) {
-            const double2 t = __ldcs(reinterpret_cast<const double2*>(g + base + k));
-            v[k] = t.x;
-            v[k + 1] = t.y;
+            for (int k = 0; k < N; k += 2) {
+                const double2 t = __ldcs(reinterpret_cast<const double2*>(g + base + k));
+                v[k] = t.x;
+                v[k + 1] = t.y;
+            }
+            return;
         }
-    } else {
-#pragma unroll
-        for (int p = 0; p < P; ++p) v[p] = (base + p < n) ? g[base + p] : 0.0;
     }
+#pragma unroll
+    for (int p = 0; p < N; ++p) v[p] = (base + p < n) ? g[base + p] : 0.0;
 }
 
+template <int N>
 __device__ __forceinline__ void store2(double* __restrict__ g, int64_t base, int64_t n,
-                                       bool vec, const double (&v)[P])
+                                       bool vec, const double (&v)[N])
 {
-    if (vec && base + P <= n && aligned16(g + base)) {
+    if constexpr (N % 2 == 0) {
+        if (vec && base + N <= n && aligned16(g + base)) {
 #pragma unroll
-        for (int k = 0; k < P; k += 2)
-            __stcs(reinterpret_cast<double2*>(g + base + k), make_double2(v[k], v[k + 1]));
-    } else {
-#pragma unroll
-        for (int p = 0; p < P; ++p)
-            if (base + p < n) g[base + p] = v[p];
+            for (int k = 0; k < N; k += 2)
+                __stcs(reinterpret_cast<double2*>(g + base + k), make_double2(v[k], v[k + 1]));
+            return;
+        }
     }
+#pragma unroll
+    for (int p = 0; p < N; ++p)
+        if (base + p < n) g[base + p] = v[p];
 }
 
 }  // namespace f64

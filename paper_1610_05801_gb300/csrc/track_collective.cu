@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256, 3)
                 else long_turn_nl<S, kRfGeneral>(z, d, c, gw, c.dual_rf != 0);
                 transverse_gen(x, xp, y, yp, d, hx, hy, c, gw);
             } else {
-                const RotateBeside<S> side{x, xp, y, yp, hx, hy, c, w};
+                const RotateBeside<S, P> side{x, xp, y, yp, hx, hy, c, w};
                 if (c.phis_zero) long_turn<S, kRfZero>(z, d, c, w, side);
                 else long_turn<S, kRfGeneral>(z, d, c, w, side);
             }

@@ -2,6 +2,7 @@
 // their selection, occupancy and launch, and the sine diagnostics.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "internal.h"
@@ -15,17 +16,18 @@ namespace {
 using namespace f64;
 
 template <int S, bool T, bool M>
-const void* kernel_ptr()
+const void* kernel_ptr(int ppt)
 {
-    return reinterpret_cast<const void*>(&kf64::k_track_f64<S, T, M, false>);
+    return ppt == 1 ? reinterpret_cast<const void*>(&kf64::k_track_f64<S, T, M, false, false, 1>)
+                    : reinterpret_cast<const void*>(&kf64::k_track_f64<S, T, M, false>);
 }
 
-const void* select_kernel(int scheme, bool trans, bool mon)
+const void* select_kernel(int scheme, bool trans, bool mon, int ppt)
 {
 #define PHTL_SEL(S)                                                              \
     if (scheme == S) {                                                           \
-        if (trans) return mon ? kernel_ptr<S, true, true>() : kernel_ptr<S, true, false>(); \
-        return mon ? kernel_ptr<S, false, true>() : kernel_ptr<S, false, false>();         \
+        if (trans) return mon ? kernel_ptr<S, true, true>(ppt) : kernel_ptr<S, true, false>(ppt); \
+        return mon ? kernel_ptr<S, false, true>(ppt) : kernel_ptr<S, false, false>(ppt);         \
     }
     PHTL_SEL(PHTL_EULER_CROMER)
     PHTL_SEL(PHTL_LEAPFROG)
@@ -36,10 +38,26 @@ const void* select_kernel(int scheme, bool trans, bool mon)
 
 }  // namespace
 
-int occupancy_f64(int scheme, bool trans, bool mon, int block, int gen)
+// Two particles a thread share the turn's instructions beyond the particles' own and keep the pipes
+// busy; one halves what a warp issues in a turn, which is what a bunch too small to fill the SMs
+// waits for.  The limits are where the two cross (warps per SM at two particles a thread; us per
+// turn, 1 against 2):
+//   no planes, no moments   1e4 particles leap-frog 0.46 / 0.75, Ruth4 1.13 / 1.87, Euler-Cromer 0.74 /
+//                           0.91; 2e5 1.31 / 1.46; 2.7e5 1.78 / 1.76
+//   no planes, moments      1e4 0.84 / 1.19; 6e4 1.32 / 1.40; 8e4 1.59 / 1.56
+//   planes                  1e4 0.95 / 1.20 (1.51 / 2.01 with moments); 3e4 1.24 / 1.25; 4.5e4 1.69 / 1.37
+// The general map's kernels always take two.
+int f64_particles_per_thread(bool trans, bool mon, int gen, int64_t n, int nsm)
+{
+    const double warps = static_cast<double>(n) / (32.0 * P * std::max(nsm, 1));
+    const double limit = trans ? 3.0 : (mon ? 7.0 : 24.0);
+    return gen == 0 && warps < limit ? 1 : P;
+}
+
+int occupancy_f64(int scheme, bool trans, bool mon, int block, int gen, int ppt)
 {
     const void* k = gen ? general_kernel_single(scheme, PHTL_F64, gen == 2)
-                        : select_kernel(scheme, trans, mon);
+                        : select_kernel(scheme, trans, mon, ppt);
     if (!k) return 0;
     int nb = 0;
     const size_t smem = mon ? 2u * (block / 32) * 16 * sizeof(double) : 0;
@@ -53,7 +71,7 @@ cudaError_t launch_track_f64(const LaunchDesc& L, const MapConsts& c, const Moni
     const bool trans = L.c[2] != nullptr || L.c[4] != nullptr;
     const bool mon = m.rows != nullptr;
     const void* k = c.general ? general_kernel_single(L.scheme, PHTL_F64, c.dual_rf != 0)
-                              : select_kernel(L.scheme, trans, mon);
+                              : select_kernel(L.scheme, trans, mon, L.ppt);
     if (!k) return cudaErrorInvalidValue;
     const size_t smem = mon ? 2u * (L.block / 32) * 16 * sizeof(double) : 0;
     LaunchDesc Lc = L;

@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256, PHTL_F64_RAMP_MIN_BLOCKS)
         for (int t = 0; t < L.nturns; ++t) {
             // the next turn's constants, loaded while this turn computes
             const Turn Tn = load_turn(prog + turn0 + (t + 1 < L.nturns ? t + 1 : t));
-            turn<S>(z, d, T, c, stage_weights<S>(prog + turn0 + t), unit, RotateBeside<S>{x, xp, y, yp, hx, hy, c, tw});
+            turn<S>(z, d, T, c, stage_weights<S>(prog + turn0 + t), unit, RotateBeside<S, P>{x, xp, y, yp, hx, hy, c, tw});
 #pragma unroll
             for (int p = 0; p < P; ++p) {
                 d[p] = __fma_rn(T.r, d[p], unit.mzero);

@@ -103,3 +103,35 @@ def test_moments_of_non_finite_values_are_nan():
     R.close()
     assert row[0] == 4 and np.all(np.isnan(row[[1, 3, 5]]))
     assert abs(row[2] - 2e-3) < 1e-18 and abs(row[4] - 6e-6) < 1e-20
+
+
+@pytest.mark.parametrize("planes, small, large", [(0, 4097, 240_001), (2, 4097, 60_001)])
+@pytest.mark.parametrize("stride", [0, 1])
+def test_small_bunches_track_as_inside_large_ones(planes, small, large, stride):
+    """Bunches below and above the size at which a thread takes two particles instead of one: the
+    same particles bitwise, and moments of the small bunch against its own coordinates' sums."""
+    ring = synth.ring(4.5e6, transverse=True)
+    rng = np.random.default_rng(7)
+    coords = [rng.normal(0, 0.15, large), rng.normal(0, 1e-3, large)]
+    for _ in range(planes):
+        coords += [rng.normal(0, 2e-3, large), rng.normal(0, 4e-5, large)]
+    out = []
+    for n in (small, large):
+        R = phtl.Ring(**ring)
+        bufs = [torch.tensor(a[:n], dtype=torch.float64, device=DEV) for a in coords]
+        mon = torch.zeros(26, phtl.MON_FIELDS, dtype=torch.float64, device=DEV)
+        if stride:
+            R.set_monitor(mon, stride=stride)
+        R.track(*bufs, *[None] * (6 - len(bufs)), turns=25, integrator="leapfrog")
+        out.append([b[:small].cpu().numpy() for b in bufs])
+        if stride and n == small:
+            row, a = mon.cpu().numpy()[25], out[0]
+            assert row[0] == n
+            for i in range(1 + planes):
+                u, v = a[2 * i], a[2 * i + 1]
+                want = [u.sum(), v.sum(), u @ u, v @ v, u @ v]
+                scale = [np.abs(u).sum(), np.abs(v).sum(), u @ u, v @ v, np.abs(u) @ np.abs(v)]
+                assert np.all(np.abs(row[1 + 5 * i:6 + 5 * i] - want) <= 1e-12 * np.array(scale))
+        R.close()
+    for u, v in zip(*out):
+        assert np.array_equal(u, v)
