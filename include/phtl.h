@@ -585,8 +585,8 @@ int phtl_get_stats(const phtl_handle* h, phtl_stats* out);
 int phtl_moments_from_sums(const double* row, double* out15);
 
 /* Diagnostic: y[i] = sine of x[i] on the device, for n device doubles, stream-ordered.
- * which = 0: the library's own FP64 sine used by the FP64 kick (Cody-Waite reduction
- * plus a fitted polynomial); which = 1: CUDA's sin(), for comparison; which = 2: the
+ * which = 0: the library's own sine in FP64 arithmetic (Cody-Waite reduction plus a
+ * fitted polynomial), which the FP64 kicks take beyond their fixed-point sine's range; which = 1: CUDA's sin(), for comparison; which = 2: the
  * double-float sine of the PHTL_F32C / PHTL_F32CD kicks, applied to x[i] truncated to
  * a float pair (48 bits) and returned as hi + lo.
  * Errors: PHTL_E_INVALID, PHTL_E_NODEVICE, PHTL_E_CUDA.                           */
@@ -594,8 +594,8 @@ int phtl_eval_sin(const double* x, double* y, int64_t n, int which, void* cuda_s
 
 /* Diagnostic: y[i] = sin(k * z[i]) for n device doubles, stream-ordered, through the
  * form the FP64 kick takes for phi_s = 0 (Sec. 1.1.2's kick with a stationary bucket):
- * the product k z is folded into the sine's argument reduction, so it is never rounded
- * on its own.  |k z| beyond ~1e5, Inf and NaN use which = 0 of phtl_eval_sin on the
+ * the phase k z as a fixed-point fraction of a turn, so it is never rounded to FP64, and
+ * a fixed-point sine.  |k z| beyond ~1e5, Inf and NaN use which = 0 of phtl_eval_sin on the
  * rounded product.  Errors: PHTL_E_INVALID (n < 0, null pointer with n > 0, k not
  * finite), PHTL_E_NODEVICE, PHTL_E_CUDA.                                           */
 int phtl_eval_sin_kz(double k, const double* z, double* y, int64_t n, void* cuda_stream);

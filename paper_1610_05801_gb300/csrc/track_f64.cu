@@ -104,9 +104,11 @@ __global__ void k_eval_sin_kz(double k, PhaseScale kap, const double* __restrict
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x)
     {
+        // kap is |k|'s: sin(k z) = sin(|k| (-z)) for a negative k
+        const double u = k < 0.0 ? -z[i] : z[i];
         bool ok;
-        const double s = sin_kz_fixed(kap, z[i], ok);
-        y[i] = ok ? s : sin_kz_rest(k, kap, z[i]);
+        const double s = sin_kz_fixed(kap, u, ok);
+        y[i] = ok ? s : sin_kz_rest(fabs(k), kap, u);
     }
 }
 
@@ -149,7 +151,7 @@ extern "C" int phtl_eval_sin_kz(double k, const double* z, double* y, int64_t n,
     if (n == 0) return PHTL_OK;
     const int block = 256;
     phtl::k_eval_sin_kz<<<phtl::eval_grid(n, block), block, 0, static_cast<cudaStream_t>(stream)>>>(
-        k, phtl::phase_scale(k), z, y, n);
+        k, phtl::phase_scale(std::fabs(k)), z, y, n);
     if (cudaGetLastError() != cudaSuccess) return PHTL_E_CUDA;
     return PHTL_OK;
 }

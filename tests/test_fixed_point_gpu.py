@@ -135,3 +135,18 @@ def test_small_bunches_track_as_inside_large_ones(planes, small, large, stride):
         R.close()
     for u, v in zip(*out):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("k", [2 * math.pi * 4620 / 6911.5, 1.0, 0.037])
+def test_sine_of_a_negative_wave_number(k):
+    """sin(-k z) = -sin(k z) bitwise, and within 2 units of 2^-53 of the exact sine, in the bucket, some
+    turns and many turns away."""
+    rng = np.random.default_rng(3)
+    ph = np.concatenate([rng.uniform(-3, 3, 3001), rng.uniform(-60, 60, 3001), rng.uniform(-9e4, 9e4, 3001)])
+    z = torch.tensor(ph / k, dtype=torch.float64, device=DEV)
+    a, b = phtl.eval_sin_kz(k, z).cpu().numpy(), phtl.eval_sin_kz(-k, z).cpu().numpy()
+    assert np.array_equal(a, -b)
+    want = _longdouble_sin_minus(k, z.cpu().numpy(), 0.0)
+    # the reference's own phase, in the host's long double (64 bits at least): half a unit of it
+    tol = 2 * 2.0 ** -53 + np.abs(ph) * float(np.finfo(np.longdouble).eps)
+    assert np.all(np.abs((a - want).astype(np.float64)) <= tol)
