@@ -130,7 +130,7 @@ int derive(const phtl_params& p, phtl_derived& d, MapConsts (&mc)[4])
         scheme_consts(d, s, c);
         c.k = d.k;
         c.kap = integer_phase(d.k, p.phi_s_rad);
-        c.uphis = phase_turns(p.phi_s_rad);
+        c.ophis = phase_offset(p.phi_s_rad);
         c.kq = quarter_phase(d.k, p.phi_s_rad);
         c.kq2 = quarter_phase(k2, p.phi2_rad);
         c.phis = p.phi_s_rad;
@@ -175,7 +175,7 @@ int derive(const phtl_params& p, phtl_derived& d, MapConsts (&mc)[4])
             scheme_weights(s, A2, d.etaC, dc2, c.kw2);
             c.k2 = k2;
             c.kap2 = integer_phase(k2, p.phi2_rad);
-            c.uphi2 = phase_turns(p.phi2_rad);
+            c.ophi2 = phase_offset(p.phi2_rad);
             c.phi2 = p.phi2_rad;
             c.sinphi2 = std::sin(p.phi2_rad);
             c.lin2 = cos_phi2 * k2;

@@ -53,7 +53,7 @@ int derive_programme(const phtl_params& p, const double* V, const double* p0, in
             if (!(std::fabs(x) < 1.0)) return PHTL_E_UNSTABLE;
             T.phis = eta > 0.0 ? std::asin(x) : kPi - std::asin(x);
             T.sinphis = std::sin(T.phis);
-            T.uphis = phase_turns(T.phis);
+            T.ophis = phase_offset(T.phis);
             const QuarterPhase q = quarter_phase(0.0, T.phis);
             T.phq_h = q.ph;
             T.phq_l = q.pl;

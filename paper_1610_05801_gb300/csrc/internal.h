@@ -80,6 +80,33 @@ inline uint64_t phase_turns(double phi)
     return phi < 0.0 ? 0 - u : u;
 }
 
+// The phase phi added to k z, phi / 2 pi = u 2^(-64 - g) turns modulo 1.  g = 0 from a quarter
+// radian on; below it u keeps all the bits of phi and |phi / 2 pi| < 2^(-g - 3), so that a small
+// sum k z + phi is exact relative to its larger term.  phi = 0: u = 0 and g beyond every shift.
+struct PhaseOffset {
+    int64_t u;
+    int32_t g;
+    int32_t pad_;
+};
+
+inline PhaseOffset phase_offset(double phi)
+{
+    PhaseOffset r{0, 1 << 20, 0};
+    int e = 0;
+    const double f = std::frexp(std::fabs(phi), &e);
+    if (f == 0.0) return r;
+    r.g = e < 0 ? -1 - e : 0;
+    if (r.g == 0) {
+        r.u = static_cast<int64_t>(phase_turns(phi));
+        return r;
+    }
+    // |phi| / 2 pi = v 2^(e - 130) with v < 2^127.4
+    const unsigned __int128 v = over_two_pi(static_cast<uint64_t>(std::ldexp(f, 53)) << 11);
+    const int64_t a = static_cast<int64_t>(v >> 67) + static_cast<int64_t>((v >> 66) & 1);
+    r.u = phi < 0.0 ? -a : a;
+    return r;
+}
+
 // The phase scale of sin(k z + phi): none where |phi| is beyond phase_turns().
 inline PhaseScale integer_phase(double k, double phi)
 {
@@ -181,7 +208,7 @@ struct MapConsts {
     int32_t linear;  // rf_linear flag
     int32_t pad2_;
     PhaseScale kap;  // k / 2 pi and phi_s / 2 pi of the integer phase
-    uint64_t uphis;
+    PhaseOffset ophis;
     // widened map: nonlinear slippage eta(d) = eta0 + eta1 d + eta2 d^2 and chromaticity
     int32_t general;             // eta1, eta2 or a chromaticity nonzero: general turn loop
     int32_t chroma_x, chroma_y;  // xi != 0 in that plane
@@ -203,7 +230,7 @@ struct MapConsts {
     double kw2[3];
     double k2, phi2, sinphi2, lin2;
     PhaseScale kap2;
-    uint64_t uphi2;
+    PhaseOffset ophi2;
     float kw2_hi[3], kw2_lo[3];
     float k2_hi, k2_lo, phi2_hi, phi2_lo, sinphi2_hi, sinphi2_lo, lin2_hi, lin2_lo;
 };
@@ -246,10 +273,10 @@ struct RampTurn {
     double w_ec[2];
     double w_lf[3];
     double w_r4[7];
-    uint64_t uphis;      // phi_s,n / 2 pi in 2^-64 turns
+    PhaseOffset ophis;   // phi_s,n of the integer phase
     float phq_h, phq_l;  // phi_s,n in quarter turns, modulo a whole turn
 };
-static_assert(sizeof(RampTurn) == 208, "RampTurn is 208 bytes");
+static_assert(sizeof(RampTurn) == 216, "RampTurn is 216 bytes");
 
 // Slicing grid and strength of the collective (wake) step.
 struct CollArgs {

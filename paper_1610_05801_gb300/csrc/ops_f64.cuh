@@ -109,8 +109,8 @@ __device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[N
     bool ok[N], all = true;
 #pragma unroll
     for (int p = 0; p < N; ++p) {
-        f[p] = MODE != kRfGeneral ? sin_kz_fixed(c.kap, z[p], ok[p])
-                                  : sin_kz_phi_fixed(c.kap, z[p], c.uphis, ok[p]);
+        f[p] = MODE != kRfGeneral ? sin_kz_fixed<false>(c.kap, z[p], ok[p])
+                                  : sin_kz_phi_fixed(c.kap, z[p], c.ophis, ok[p]);
         all = all && ok[p];
     }
     side(j);
@@ -118,7 +118,7 @@ __device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[N
 #pragma unroll
         for (int p = 0; p < N; ++p)
             if (!ok[p])
-                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.uphis);
+                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.ophis);
     }
     if (MODE == kRfGeneral) {
 #pragma unroll
@@ -308,17 +308,20 @@ __device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[
     bool ok[N], ok2[N], all = true;
 #pragma unroll
     for (int p = 0; p < N; ++p) {
-        f[p] = MODE != kRfGeneral ? sin_kz_fixed(c.kap, z[p], ok[p])
-                                  : sin_kz_phi_fixed(c.kap, z[p], c.uphis, ok[p]);
-        g[p] = sin_kz_phi_fixed(c.kap2, z[p], c.uphi2, ok2[p]);
+        f[p] = MODE != kRfGeneral ? sin_kz_fixed<false>(c.kap, z[p], ok[p])
+                                  : sin_kz_phi_fixed(c.kap, z[p], c.ophis, ok[p]);
+        g[p] = MODE == kRfPlain ? sin_kz_fixed<true>(c.kap2, z[p], ok2[p])
+                                : sin_kz_phi_fixed(c.kap2, z[p], c.ophi2, ok2[p]);
         all = all && ok[p] && ok2[p];
     }
     if (!all) {
 #pragma unroll
         for (int p = 0; p < N; ++p) {
             if (!ok[p])
-                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.uphis);
-            if (!ok2[p]) g[p] = sin_phi_rest(c.k2, c.kap2, z[p], c.phi2, c.uphi2);
+                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.ophis);
+            if (!ok2[p])
+                g[p] = MODE == kRfPlain ? sin_kz_rest(c.k2, c.kap2, z[p])
+                                        : sin_phi_rest(c.k2, c.kap2, z[p], c.phi2, c.ophi2);
         }
     }
 #pragma unroll

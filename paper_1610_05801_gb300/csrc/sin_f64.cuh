@@ -86,6 +86,12 @@ __device__ __forceinline__ uint64_t shr_sat(uint64_t a, uint32_t n)
     asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
     return r;
 }
+__device__ __forceinline__ int64_t sar_sat(int64_t a, uint32_t n)  // the sign for 64 and more
+{
+    int64_t r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
+    return r;
+}
 __device__ __forceinline__ uint64_t shl_sat(uint64_t a, uint32_t n)
 {
     uint64_t r;
@@ -134,17 +140,8 @@ __device__ __forceinline__ double fixed_to_double(uint64_t S, int x, uint32_t si
     return __hiloint2double(static_cast<int>(hi | (sign & 0x80000000u)), static_cast<int>(static_cast<uint32_t>(r)));
 }
 
-// sin(2 pi U), U in 2^-64 turns, with the sign flipped where bit 31 of `flip` is set.  ok is
-// cleared within 2^-31 of a zero, where the result does not fill the significand.
-__device__ __forceinline__ double sin_turns_fixed(uint64_t U, uint32_t flip, bool& ok)
-{
-    const uint64_t V = fold_half_turn(U << 1);
-    const uint64_t S = mulhi_trunc63(V, sin_poly_fixed(V));
-    ok = ok && (S >> 32) != 0u;
-    return fixed_to_double(S, 0, static_cast<uint32_t>(U >> 32) ^ flip);
-}
-
-// The same with every U valid: 0 at a zero of the sine, fewer significant bits next to one.
+// sin(2 pi U), U in 2^-64 turns, with the sign flipped where bit 31 of `flip` is set: 0 at a zero of
+// the sine, fewer significant bits next to one.
 __device__ __forceinline__ double sin_turns_any(uint64_t U, uint32_t flip)
 {
     const uint64_t V = fold_half_turn(U << 1);
@@ -219,11 +216,14 @@ static __device__ __noinline__ double sin_kz_rest(double k, PhaseScale kap, doub
     return detail::sin_turns_any(U, static_cast<uint32_t>(__double2hiint(z)));
 }
 
-// sin(k z + phi) where sin_kz_phi_fixed does not cover it, likewise.
-static __device__ __noinline__ double sin_phi_rest(double k, PhaseScale kap, double z, double phi, uint64_t uphi)
+// sin(k z + phi) where sin_kz_phi_fixed does not cover it, likewise.  A sum below 2^-7 is left to the
+// FP64 product and sine, which are exact relative to it (the phase in turns is exact to 2^-64).
+static __device__ __noinline__ double sin_phi_rest(double k, PhaseScale kap, double z, double phi, PhaseOffset o)
 {
+    const double x = fma(k, z, phi);
     uint64_t U;
-    if (!phase_of_turns(kap, z, U)) return sin_f64(fma(k, z, phi));
+    if ((__double2hiint(x) & 0x7fffffff) < 0x3f800000 || !phase_of_turns(kap, z, U)) return sin_f64(x);
+    const uint64_t uphi = static_cast<uint64_t>(detail::sar_sat(o.u, static_cast<uint32_t>(o.g)));
     return detail::sin_turns_any(__double2hiint(z) < 0 ? uphi - U : uphi + U, 0u);
 }
 
@@ -233,35 +233,48 @@ static __device__ __noinline__ double sin_phi_rest(double k, PhaseScale kap, dou
 
 // sin(k z) of a phase below one turn: k / 2 pi = kap.K 2^(959 - kap.cn), so that with the
 // significand M and the biased exponent e of z the phase is (M K 2^-64) 2^(-63 - n) turns,
-// n = cn - e (n >= 0 for every phase below half a turn).  Below a quarter turn (n >= 2) the product keeps all its bits as the last
-// factor, so the result is as exact relative to itself as to 1 however small z is.  Not
-// covered: z = 0, n < 0 (a particle that has left the bucket), |k z| below 2^-800, a phase within 1e-9 of a half turn, Inf and NaN.
+// n = cn - e (n >= 0 for every phase below half a turn, n >= -1 below a whole one).  Below a quarter
+// turn (n >= 2) the product keeps all its bits as the last factor, so the result is as exact relative
+// to itself as to 1 however small z is.  Not covered: z = 0, n < 0 (a particle that has left the
+// bucket; WIDE: n < -1, for the shorter wave of a second RF system, one instruction more), |k z| below
+// 2^-800, a phase within 1e-9 of a half turn, Inf and NaN.
+template <bool WIDE>
 __device__ __forceinline__ double sin_kz_fixed(PhaseScale kap, double z, bool& ok)
 {
     using namespace detail;
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(z));
-    const uint32_t n = static_cast<uint32_t>(kap.cn - static_cast<int>((hi >> 20) & 0x7ffu));
+    const int n = kap.cn - static_cast<int>((hi >> 20) & 0x7ffu);
     const uint64_t p = mulhi_trunc(mantissa64(z), kap.K);
-    const uint64_t W = shr_sat(p, n);                             // 2^-63 turns
+    // 2^-63 turns
+    const uint64_t W = WIDE ? shr_sat(p, static_cast<uint32_t>(n + 1)) << 1 : shr_sat(p, static_cast<uint32_t>(n));
     const uint64_t V = fold_half_turn(W << 2);
-    const bool small = n >= 2u;
+    const bool small = WIDE ? n >= 2 : static_cast<uint32_t>(n) >= 2u;
     const uint64_t S = mulhi_trunc63(small ? p : V, sin_poly_fixed(V));
-    ok = n <= 800u && (S >> 32) != 0u;
-    return fixed_to_double(S, small ? static_cast<int>(n) - 2 : 0, hi ^ static_cast<uint32_t>(W >> 31));
+    ok = static_cast<uint32_t>(WIDE ? n + 1 : n) <= 800u && (S >> 32) != 0u;
+    return fixed_to_double(S, small ? n - 2 : 0, hi ^ static_cast<uint32_t>(W >> 31));
 }
 
-// sin(k z + phi), phi as uphi in 2^-64 turns: the phases are added as fractions of a turn,
-// without rounding.  Not covered: n < -1 (never below one turn of k z), a denormal z, a total phase within
-// 1e-9 of a half turn, Inf and NaN.
-__device__ __forceinline__ double sin_kz_phi_fixed(PhaseScale kap, double z, uint64_t uphi, bool& ok)
+// sin(k z + phi), phi as a PhaseOffset.  The phases are added as integers in 2^(-64 - t) turns:
+// t = 0 adds fractions of a turn modulo 1; where both phases are small, t > 0 scales the sum up until
+// its larger term fills the word (k z below 2^-n turns takes t <= n - 3, phi takes t <= g: the sum
+// stays below a quarter turn of the scaled word, where the fold is the magnitude).  So the sum is exact
+// to 2^-59 of its larger term however small both are, as the FP64 fma(k, z, phi) is to 2^-53; with
+// t = 0 throughout it was exact to 2^-62 turns only, which a small k z or phi does not have bits for.
+// Not covered: n < -1 (never below one turn of k z), a sum that does not fill the significand (within
+// 2^-31 of a half turn, or of cancellation) or lies below 2^-800, Inf and NaN.
+__device__ __forceinline__ double sin_kz_phi_fixed(PhaseScale kap, double z, PhaseOffset o, bool& ok)
 {
     using namespace detail;
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(z));
-    const uint32_t e = (hi >> 20) & 0x7ffu;
-    const uint32_t n1 = static_cast<uint32_t>(kap.cn + 1 - static_cast<int>(e));  // n + 1: from n = -1 on
-    const uint64_t U = shr_sat(mulhi_trunc(mantissa64(z), kap.K), n1) << 2;
-    ok = n1 <= 2047u && (e != 0u || (hi << 1 | static_cast<uint32_t>(__double2loint(z))) == 0u);
-    return sin_turns_fixed(static_cast<int>(hi) < 0 ? uphi - U : uphi + U, 0u, ok);
+    const int n1 = kap.cn + 1 - static_cast<int>((hi >> 20) & 0x7ffu);  // n + 1: from n = -1 on
+    const int t = max(min(n1 - 4, o.g), 0);
+    const uint64_t U = shr_sat(mulhi_trunc(mantissa64(z), kap.K), static_cast<uint32_t>(n1 - t)) << 2;
+    const uint64_t uphi = static_cast<uint64_t>(sar_sat(o.u, static_cast<uint32_t>(o.g - t)));
+    const uint64_t W = static_cast<int>(hi) < 0 ? uphi - U : uphi + U;
+    const uint64_t V = fold_half_turn(W << 1);
+    const uint64_t S = mulhi_trunc63(V, sin_poly_fixed(shr_sat(V, static_cast<uint32_t>(t))));
+    ok = n1 >= 0 && t <= 800 && (S >> 32) != 0u;
+    return fixed_to_double(S, t, static_cast<uint32_t>(W >> 32));
 }
 
 // sin and cos of 2 pi a, a in turns (the chromatic phase advance): the fraction of a as 2^-64

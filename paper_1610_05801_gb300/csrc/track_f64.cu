@@ -107,7 +107,7 @@ __global__ void k_eval_sin_kz(double k, PhaseScale kap, const double* __restrict
         // kap is |k|'s: sin(k z) = sin(|k| (-z)) for a negative k
         const double u = k < 0.0 ? -z[i] : z[i];
         bool ok;
-        const double s = sin_kz_fixed(kap, u, ok);
+        const double s = sin_kz_fixed<false>(kap, u, ok);
         y[i] = ok ? s : sin_kz_rest(fabs(k), kap, u);
     }
 }

@@ -5,7 +5,7 @@
 // The same persistent structure as the fixed-machine kernels (Sec. 2.3: turn loop inside
 // the kernel, state in registers, grid-stride over particle chunks), but each turn reads
 // its constants -- eta_n C, A_n, phi_s,n, sin(phi_s,n), r_n = p0_n / p0_{n+1} -- from a
-// device table that the host derived in FP64 (208 bytes per turn, the same address for
+// device table that the host derived in FP64 (216 bytes per turn, the same address for
 // every thread, so the loads are L1 broadcasts).  The next turn's phase constants are
 // loaded while the current turn computes.  After the turn's stages and the transverse
 // rotation, delta and the slopes x', y' are re-expressed against the next turn's reference
@@ -29,7 +29,7 @@ using namespace f64;
 
 struct Turn {
     double phis, sinphis, lin, r;
-    uint64_t uphis;
+    PhaseOffset ophis;
 };
 
 // Sums and products as FMAs of registers, a + b = fma(a, 1, b) and a b = fma(a, b, -0) exactly:
@@ -45,7 +45,7 @@ __device__ __forceinline__ Turn load_turn(const RampTurn* __restrict__ p)
     t.sinphis = __ldg(&p->sinphis);
     t.lin = __ldg(&p->lin);
     t.r = __ldg(&p->r);
-    t.uphis = __ldg(reinterpret_cast<const unsigned long long*>(&p->uphis));
+    t.ophis = PhaseOffset{__ldg(reinterpret_cast<const long long*>(&p->ophis.u)), __ldg(&p->ophis.g), 0};
     return t;
 }
 
@@ -79,14 +79,14 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
     } else {
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            f[p] = sin_kz_phi_fixed(c.kap, z[p], T.uphis, ok[p]);
+            f[p] = sin_kz_phi_fixed(c.kap, z[p], T.ophis, ok[p]);
             all = all && ok[p];
         }
         side(j);
         if (!all) {
 #pragma unroll
             for (int p = 0; p < P; ++p)
-                if (!ok[p]) f[p] = sin_phi_rest(c.k, c.kap, z[p], T.phis, T.uphis);
+                if (!ok[p]) f[p] = sin_phi_rest(c.k, c.kap, z[p], T.phis, T.ophis);
         }
 #pragma unroll
         for (int p = 0; p < P; ++p) f[p] = __fma_rn(f[p], u.one, -T.sinphis);
