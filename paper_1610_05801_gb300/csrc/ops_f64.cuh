@@ -597,7 +597,9 @@ __device__ __forceinline__ void record(const double (&z)[N], const double (&d)[N
     const int field = lane >> kShift;  // the field whose total this lane ends up with
     int64_t f[NF];
     f[0] = static_cast<int64_t>(static_cast<int>(cnt));
-    PlaneExponents E{warp_exponent(z), warp_exponent(d)}, Ef = E;
+    PlaneExponents E{warp_exponent(z), warp_exponent(d)};
+    PlaneExponents Ef{0, 0};           // of this lane's field; an absent plane's sums are zeros
+    if (field < 6) Ef = E;
     int k = field - 1;                 // 0..4: a, b, a^2, b^2, ab of the plane Ef
     pair_sums_fixed(z, d, E, f + 1);
     if constexpr (TRANS) {
