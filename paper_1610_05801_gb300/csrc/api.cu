@@ -137,7 +137,6 @@ int derive(const phtl_params& p, phtl_derived& d, MapConsts (&mc)[4])
         c.sinphis = d.sin_phis;
         c.lin = d.cos_phis * d.k;
         c.linear = p.rf_linear != 0;
-        c.phis_zero = p.phi_s_rad == 0.0 && !p.rf_linear ? 1 : 0;
         for (int i = 0; i < 4; ++i) {
             c.mx[i] = d.mx[i];
             c.my[i] = d.my[i];
@@ -165,7 +164,11 @@ int derive(const phtl_params& p, phtl_derived& d, MapConsts (&mc)[4])
         c.chy = chroma_plane(c.qy, p.xi_y, p.beta_y_m);
         c.slip = p.eta1 != 0.0 || p.eta2 != 0.0 ? 1 : 0;
         c.phi2_zero = p.phi2_rad == 0.0 ? 1 : 0;
-        c.plain = c.phis_zero && !c.slip && (!dual || c.phi2_zero) ? 1 : 0;
+        c.phis_zero = p.phi_s_rad == 0.0 ? 1 : 0;
+        c.rf_mode = p.rf_linear                         ? kRfLinear
+                    : !c.phis_zero                      ? kRfGeneral
+                    : !c.slip && (!dual || c.phi2_zero) ? kRfPlain
+                                                        : kRfZero;
         c.chroma_x = p.xi_x != 0.0 ? 1 : 0;
         c.chroma_y = p.xi_y != 0.0 ? 1 : 0;
         // second RF system
@@ -393,17 +396,10 @@ cudaError_t launch_perturn(const LaunchDesc& L, const MapConsts& c, const Monito
     return dtype == PHTL_F64 ? launch_track_f64(L, c, m, s) : launch_track_f32c(L, c, m, dtype, s);
 }
 
-int occupancy_perturn(int scheme, bool trans, bool mon, int dtype, int block, int gen)
+int occupancy(const MapConsts& c, int dtype, int scheme, bool trans, bool mon, int block, int ppt)
 {
-    return dtype == PHTL_F64 ? occupancy_f64(scheme, trans, mon, block, gen, 0)
-                             : occupancy_f32c(scheme, trans, mon, dtype, block, gen);
-}
-
-int occupancy(int dtype, int scheme, bool trans, bool mon, int block, bool perturn, int gen, int ppt)
-{
-    if (perturn) return occupancy_perturn(scheme, trans, mon, dtype, block, gen);
-    if (dtype == PHTL_F64) return occupancy_f64(scheme, trans, mon, block, gen, ppt);
-    return occupancy_f32c(scheme, trans, mon, dtype, block, gen);
+    return dtype == PHTL_F64 ? occupancy_f64(c, scheme, trans, mon, block, ppt)
+                             : occupancy_f32c(scheme, trans, mon, dtype, block, gen_level(c));
 }
 
 int check_track_args(const phtl_handle* h, void* const* c, int64_t n, int64_t turns,
@@ -464,7 +460,7 @@ int enqueue_track(phtl_handle* h, void* const* c, int64_t n, int64_t turns, int 
     // FP32C buffers are [hi | comp]: the comp half is 16-byte aligned only if n % 4 == 0
     if (dtype != PHTL_F64 && (n * es) % 16 != 0) vec = false;
 
-    const int occ = occupancy(dtype, integrator, trans, mon, block, perturn, gen, ppt);
+    const int occ = occupancy(h->mc[integrator], dtype, integrator, trans, mon, block, ppt);
     if (occ <= 0) return PHTL_E_INVALID;
     const int64_t chunk = static_cast<int64_t>(block) * ppt;
     const int64_t nchunks = (n + chunk - 1) / chunk;

@@ -99,10 +99,10 @@ int coll_launch(phtl_handle* h, void* const* c, int64_t n, int integrator, int d
     // particles, 19.8 / 17.8 at 3e5, 25.5 / 26.2 at 6e5, 37.4 / 34.7 at 1e6, 63.4 / 64.5 at 2e6), 128 in
     // FP32 (25.8 / 26.7 at 1e6, 44.9 / 49.1 at 2e6)
     const int block = h->block > 0 ? h->block : (dtype == PHTL_F64 ? 256 : 128);
-    const int occ = dtype == PHTL_F64 ? occupancy_coll(integrator, h->mc[integrator].general != 0, block,
-                                                       h->coll.nslices)
-                                      : occupancy_coll_f32(integrator, dtype, h->mc[integrator].general != 0,
-                                                           block, h->coll.nslices);
+    const MapConsts& mc = h->mc[integrator];
+    const int occ = dtype == PHTL_F64 ? occupancy_coll(mc, integrator, block, h->coll.nslices)
+                                      : occupancy_coll_f32(integrator, dtype, mc.general != 0, block,
+                                                           h->coll.nslices);
     if (occ <= 0) return PHTL_E_INVALID;
     const int64_t chunk = static_cast<int64_t>(block) * particles_per_thread(dtype);
     const int64_t nchunks = (n + chunk - 1) / chunk;

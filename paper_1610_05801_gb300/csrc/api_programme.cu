@@ -179,7 +179,7 @@ int phtl_track_programme(phtl_handle* h, void* z, void* dp, void* x, void* xp, v
     for (int i = 0; i < 6; ++i)
         if (c[i] && (reinterpret_cast<uintptr_t>(c[i]) % 16) != 0) vec = false;
     if (dtype != PHTL_F64 && (n * 4) % 16 != 0) vec = false;
-    const int occ = occupancy_ramp(integrator, dtype, block);
+    const int occ = occupancy_ramp(h->mc[integrator], integrator, dtype, block);
     if (occ <= 0) return PHTL_E_INVALID;
     const int64_t chunk = static_cast<int64_t>(block) * ppt;
     const int64_t nchunks = (n + chunk - 1) / chunk;

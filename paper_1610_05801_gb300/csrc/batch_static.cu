@@ -134,7 +134,7 @@ extern "C" int phtl_batch_run_noalloc(phtl_handle* h, const phtl_job* jobs, int3
         g.mon = mon;
         g.mc = batch_consts(h, rk4);
         g.block = h->block > 0 ? h->block : 128;
-        if (occupancy_batched(dt, mon, g.block, g.mc.general != 0) <= 0) return PHTL_E_INVALID;
+        if (occupancy_batched(g.mc, dt, mon, g.block) <= 0) return PHTL_E_INVALID;
         g.T = h->tpl > 0 ? h->tpl : auto_turns_per_launch(dt, jobs[ord[0]].integrator, active);
         const int64_t per_tile = static_cast<int64_t>(g.block) * particles_per_thread(dt);
         JobDesc* G = host + used;

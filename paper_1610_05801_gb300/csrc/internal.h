@@ -179,6 +179,17 @@ inline QuarterPhase quarter_phase(double k, double phi)
     return q;
 }
 
+// What the turn loop's code leaves out:
+//   kRfGeneral  any phi_s;
+//   kRfZero     phi_s = 0: the kick is sin(k z), no subtraction;
+//   kRfPlain    kRfZero, a second RF system (if any) with phi2 = 0, no slippage expansion (the general
+//               map's FP64 kernels only; the others take it as kRfZero);
+//   kRfLinear   rf_linear: no sines.
+// The FP64 kernels are built once per mode and the launch picks one: with the modes as branches in one
+// kernel they shared its register budget, and rf_linear runs of the general map took up to 42 % longer
+// than before the integer sines (0.9 to 1.05 of that now).  In the FP32 kernels they stay branches.
+enum RfMode { kRfGeneral = 0, kRfZero = 1, kRfPlain = 2, kRfLinear = 3 };
+
 // Per-stage coefficients of one turn of the longitudinal map (Sec. 1.1.2 schemes),
 // pre-multiplied on the host in FP64:
 //   drift stage i:  z <- z - dc[i] * delta           dc[i] = w_i * eta * C
@@ -198,7 +209,7 @@ struct MapConsts {
     // p = beta tan(mu/2), q = -sin(mu)/beta (shear_* = 0: use the matrix instead)
     double shx[2], shy[2];
     int32_t shear_x, shear_y;
-    int32_t phis_zero;  // phi_s == 0 and not rf_linear: the kick is sin(k z)
+    int32_t phis_zero;  // phi_s == 0: the kick is sin(k z)
     // double-float (FP32 pair) copies for the FP32 paths: value = hi + lo
     float dc_hi[4], dc_lo[4];
     float kw_hi[3], kw_lo[3];
@@ -225,7 +236,7 @@ struct MapConsts {
     // kw2[j] = w_j * A2 (lin2 z in rf_linear mode)
     int32_t dual_rf;
     int32_t phi2_zero;
-    int32_t plain;  // phis_zero, phi2 = 0 where there is a second system, no slippage expansion
+    int32_t rf_mode;  // RfMode
     int32_t pad4_;
     double kw2[3];
     double k2, phi2, sinphi2, lin2;
@@ -471,7 +482,7 @@ cudaError_t launch_perturn(const LaunchDesc& L, const MapConsts& c, const Monito
 // (grid = the tiles of those jobs), or row-0 records only when T == 0.
 cudaError_t launch_batched(const JobDesc* jobs, int32_t njobs, const MapConsts& c, int dtype,
                            bool mon, int64_t t0, int32_t T, int grid, int block, cudaStream_t s);
-int occupancy_batched(int dtype, bool mon, int block, bool general);
+int occupancy_batched(const MapConsts& c, int dtype, bool mon, int block);
 int particles_per_thread(int dtype);
 
 // Which single-bunch kernel family a map needs: 0 the linear map's, 1 the widened map's,
@@ -480,17 +491,16 @@ inline int gen_level(const MapConsts& c) { return c.general ? (c.dual_rf ? 2 : 1
 
 // Resident blocks per SM of a kernel variant at a block size (0 = cannot launch);
 // gen: the kernel family (gen_level).
-int occupancy_f64(int scheme, bool trans, bool mon, int block, int gen, int ppt);
+int occupancy_f64(const MapConsts& c, int scheme, bool trans, bool mon, int block, int ppt);
 // Particles per thread of the FP64 single-bunch kernel for a bunch of n on nsm SMs.
 int f64_particles_per_thread(bool trans, bool mon, int gen, int64_t n, int nsm);
 int occupancy_f32c(int scheme, bool trans, bool mon, int dtype, int block, int gen);
-int occupancy_perturn(int scheme, bool trans, bool mon, int dtype, int block, int gen);
 
 // Ramp programme kernels (track_ramp.cu): turns [turn0, turn0 + L.nturns) of the
 // programme table prog (device memory), linear map only.
 cudaError_t launch_ramp(const LaunchDesc& L, const MapConsts& c, const MonitorArgs& m,
                         const RampTurn* prog, int64_t turn0, int dtype, cudaStream_t s);
-int occupancy_ramp(int scheme, int dtype, int block);
+int occupancy_ramp(const MapConsts& c, int scheme, int dtype, int block);
 
 // Collective step kernels (track_collective.cu): one turn (optionally the previous turn's
 // kick U first, a monitor row, the map, the slicing of the new z), and the per-slice wake
@@ -501,7 +511,7 @@ cudaError_t launch_coll_turn(const LaunchDesc& L, const MapConsts& c, const Coll
                              int64_t rec_row, bool kick, bool map, cudaStream_t s);
 cudaError_t launch_wake_potential(const unsigned* counts, const double* w, const CollArgs& A,
                                   double* V, double* U, float2* U2, unsigned* clear, cudaStream_t s);
-int occupancy_coll(int scheme, bool gen, int block, int nslices);  // gen: MapConsts::general
+int occupancy_coll(const MapConsts& c, int scheme, int block, int nslices);
 // The FP32-compensated turn kernel (track_collective_f32.cu): the same steps on float-pair
 // state, the kick read from U2 (U as hi + lo floats).
 cudaError_t launch_coll_turn_f32(const LaunchDesc& L, const MapConsts& c, const CollArgs& A,
@@ -513,11 +523,11 @@ int occupancy_coll_f32(int scheme, int dtype, bool gen, int block, int nslices);
 const void* coll_kernel_f32_lin(int scheme, int dtype);
 
 // Kernels of the widened map (track_general.cu, track_general_batched.cu).
-const void* general_kernel_single(int scheme, int dtype, bool dual);
-const void* general_kernel_single_rk4(int dtype);                   // track_general_rk4.cu
-const void* general_kernel_single_dual(int scheme, int dtype);      // track_general_dual.cu
+const void* general_kernel_single(int scheme, int dtype, bool dual, int mode);
+const void* general_kernel_single_rk4(int dtype, int mode);                   // track_general_rk4.cu
+const void* general_kernel_single_dual(int scheme, int dtype, int mode);      // track_general_dual.cu
 const void* general_kernel_single_dual_f32(int scheme, int dtype);  // track_general_dual_f32.cu
-const void* general_kernel_batched(int dtype);
+const void* general_kernel_batched(const MapConsts& c, int dtype);
 const void* general_kernel_batched_f32(int dtype);  // PHTL_F32CD, PHTL_F32CS
 
 }  // namespace phtl

@@ -38,8 +38,8 @@ __device__ __forceinline__ int find_job(const JobDesc* __restrict__ jobs, int nj
 }
 
 // ---------------------------------------------------------------------------------- FP64
-template <int SCHEME, bool MON, int MODE, bool GEN>
-__device__ __forceinline__ void run_f64_mode(double (&z)[f64::P], double (&d)[f64::P],
+template <int SCHEME, bool MON, int MODE, bool GEN, bool DUAL>
+__device__ __forceinline__ void run_f64(double (&z)[f64::P], double (&d)[f64::P],
                                         double (&x)[f64::P], double (&xp)[f64::P],
                                         double (&y)[f64::P], double (&yp)[f64::P], bool hx,
                                         bool hy, const MapConsts& c, const JobDesc& J,
@@ -54,7 +54,7 @@ __device__ __forceinline__ void run_f64_mode(double (&z)[f64::P], double (&d)[f6
     if (!GEN) w = f64::turn_weights<SCHEME, true>(J.dc, J.kw, c);
     for (int t = 0; t < nt; ++t) {
         if (GEN) {
-            f64::long_turn_nl<SCHEME, MODE>(z, d, c, gw, c.dual_rf != 0);
+            f64::long_turn_nl<SCHEME, MODE>(z, d, c, gw, DUAL);
             f64::transverse_gen(x, xp, y, yp, d, hx, hy, c, gw);
         } else {
             f64::long_turn<SCHEME, MODE>(z, d, c, w, f64::RotateBeside<SCHEME, f64::P>{x, xp, y, yp, hx, hy, c, w});
@@ -74,28 +74,12 @@ __device__ __forceinline__ void run_f64_mode(double (&z)[f64::P], double (&d)[f6
     }
 }
 
-template <int SCHEME, bool MON, bool GEN>
-__device__ __forceinline__ void run_f64(double (&z)[f64::P], double (&d)[f64::P],
-                                        double (&x)[f64::P], double (&xp)[f64::P],
-                                        double (&y)[f64::P], double (&yp)[f64::P], bool hx,
-                                        bool hy, const MapConsts& c, const JobDesc& J,
-                                        float cnt, int64_t t0, int nt, double* smem, int& parity)
-{
-    if (GEN && c.plain)
-        run_f64_mode<SCHEME, MON, f64::kRfPlain, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem,
-                                                      parity);
-    else if (c.phis_zero)
-        run_f64_mode<SCHEME, MON, f64::kRfZero, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem,
-                                                     parity);
-    else
-        run_f64_mode<SCHEME, MON, f64::kRfGeneral, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem,
-                                                        parity);
-}
-
 // GEN: the widened map (separate kernels chosen on the host; built with MON = true, the
-// per-job monitor pointer is checked at run time).
-template <bool MON, bool GEN>
-__global__ void __launch_bounds__(256, f64::kBatchedMinBlocks256) k_batched_f64(const JobDesc* __restrict__ jobs, int njobs,
+// per-job monitor pointer is checked at run time).  MODE: RfMode of the ring; DUAL (GEN only): with the
+// second RF system, whose sines cost a ring without one registers (80 a thread: Ruth4 on the widened map
+// took 20 % longer).
+template <bool MON, bool GEN, int MODE, bool DUAL>
+__global__ void __launch_bounds__(256, (f64::batched_min_blocks_256<GEN, MODE>())) k_batched_f64(const JobDesc* __restrict__ jobs, int njobs,
                                                      MapConsts c, int64_t t0, int T)
 {
     using namespace f64;
@@ -141,22 +125,22 @@ __global__ void __launch_bounds__(256, f64::kBatchedMinBlocks256) k_batched_f64(
     }
     if (GEN || mon) {
         if (J.scheme == PHTL_EULER_CROMER)
-            run_f64<PHTL_EULER_CROMER, true, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+            run_f64<PHTL_EULER_CROMER, true, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
         else if (J.scheme == PHTL_LEAPFROG)
-            run_f64<PHTL_LEAPFROG, true, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+            run_f64<PHTL_LEAPFROG, true, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
         else if (!GEN || J.scheme == PHTL_RUTH4)
-            run_f64<PHTL_RUTH4, true, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+            run_f64<PHTL_RUTH4, true, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
         else if constexpr (GEN)  // RK4 lives in the widened map's kernels only
-            run_f64<PHTL_RK4, true, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+            run_f64<PHTL_RK4, true, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
     } else {
         if (J.scheme == PHTL_EULER_CROMER)
-            run_f64<PHTL_EULER_CROMER, false, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+            run_f64<PHTL_EULER_CROMER, false, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
         else if (J.scheme == PHTL_LEAPFROG)
-            run_f64<PHTL_LEAPFROG, false, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+            run_f64<PHTL_LEAPFROG, false, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
         else if (!GEN || J.scheme == PHTL_RUTH4)
-            run_f64<PHTL_RUTH4, false, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+            run_f64<PHTL_RUTH4, false, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
         else if constexpr (GEN)  // RK4 lives in the widened map's kernels only
-            run_f64<PHTL_RK4, false, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
+            run_f64<PHTL_RK4, false, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
     }
     store2(gz, base, J.n, vec, z);
     store2(gd, base, J.n, vec, d);
@@ -224,7 +208,7 @@ __device__ __forceinline__ void run_f32c(f32c::DF (&z)[f32c::P], f32c::DF (&d)[f
                                          bool hy, const MapConsts& c, const JobDesc& J, float cnt,
                                          int64_t t0, int nt, double* smem, int& parity)
 {
-    if (c.phis_zero)
+    if (f32c::sine_only<DT>(c))
         run_f32c_zs<SCHEME, DT, MON, true, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
     else
         run_f32c_zs<SCHEME, DT, MON, false, GEN>(z, d, x, xp, y, yp, hx, hy, c, J, cnt, t0, nt, smem, parity);
@@ -301,6 +285,17 @@ __global__ void PHTL_F32C_BATCHED_BOUNDS(DT, GEN) k_batched_f32c(const JobDesc* 
         store4(g[4], base, J.n, vec, y);
         store4(g[5], base, J.n, vec, yp);
     }
+}
+
+// The FP64 kernels of a ring's mode (kRfPlain: the general map's only, kRfZero without it).
+template <bool MON, bool GEN, bool DUAL = false>
+const void* batched_f64(int mode)
+{
+    if (mode == kRfLinear) return reinterpret_cast<const void*>(&k_batched_f64<MON, GEN, kRfLinear, DUAL>);
+    if (mode == kRfGeneral) return reinterpret_cast<const void*>(&k_batched_f64<MON, GEN, kRfGeneral, DUAL>);
+    if constexpr (GEN)
+        if (mode == kRfPlain) return reinterpret_cast<const void*>(&k_batched_f64<MON, GEN, kRfPlain, DUAL>);
+    return reinterpret_cast<const void*>(&k_batched_f64<MON, GEN, kRfZero, DUAL>);
 }
 
 }  // namespace

@@ -118,7 +118,7 @@ __global__ void PHTL_COLL_F32_BOUNDS
         }
         if (map) {
             if constexpr (GEN) {
-                if (c.phis_zero)
+                if (sine_only<DT>(c))
                     long_turn_nl<S, DT, true>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo, c.kw2_hi,
                                               c.kw2_lo, g1h, g1l, g2h, g2l, c.dual_rf != 0);
                 else
@@ -126,7 +126,7 @@ __global__ void PHTL_COLL_F32_BOUNDS
                                                c.kw2_lo, g1h, g1l, g2h, g2l, c.dual_rf != 0);
                 transverse_gen<DT>(x, xp, y, yp, d, hx, hy, c);
             } else {
-                if (c.phis_zero) long_turn<S, DT, true>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
+                if (sine_only<DT>(c)) long_turn<S, DT, true>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
                 else long_turn<S, DT, false>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
                 if (hx) {
 #pragma unroll

@@ -111,7 +111,7 @@ __global__ void PHTL_F32C_TRACK_BOUNDS(SCHEME, DT, GEN) k_track_f32c(LaunchDesc 
             record<TRANS>(z, d, x, xp, y, yp, cnt, hx, hy, smem, parity, m.rows, 0);
             parity ^= 1;
         }
-        if (c.phis_zero)
+        if (sine_only<DT>(c))
             turns<SCHEME, DT, TRANS, MON, true, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, m,
                                                            L.nturns, smem, parity);
         else

@@ -77,7 +77,8 @@ __device__ __forceinline__ void turns(double (&z)[N], double (&d)[N], double (&x
 #endif
 #define PHTL_F64_BOUNDS(S, G) __launch_bounds__(256, (G) ? PHTL_F64_GEN_MIN_BLOCKS : min_blocks_256<S>())
 #endif
-template <int SCHEME, bool TRANS, bool MON, bool GEN, bool DUAL = false, int N = P>
+// MODE: RfMode.
+template <int SCHEME, bool TRANS, bool MON, bool GEN, bool DUAL, int N, int MODE>
 __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
     k_track_f64(LaunchDesc L, MapConsts c, MonitorArgs m)
 {
@@ -120,15 +121,8 @@ __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
             record<TRANS>(z, d, x, xp, y, yp, cnt, hx, hy, smem, parity, m.rows, 0);
             parity ^= 1;
         }
-        if (GEN && c.plain)
-            turns<SCHEME, TRANS, MON, kRfPlain, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
-                                                           L.nturns, smem, parity);
-        else if (c.phis_zero)
-            turns<SCHEME, TRANS, MON, kRfZero, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
-                                                          L.nturns, smem, parity);
-        else
-            turns<SCHEME, TRANS, MON, kRfGeneral, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m,
-                                                             L.nturns, smem, parity);
+        turns<SCHEME, TRANS, MON, MODE, GEN, DUAL>(z, d, x, xp, y, yp, hx, hy, cnt, c, w, m, L.nturns,
+                                                   smem, parity);
         store2(gz, base, L.n, vec, z);
         store2(gd, base, L.n, vec, d);
         if (hx) {
@@ -140,6 +134,20 @@ __global__ void PHTL_F64_BOUNDS(SCHEME, GEN)
             store2(gyp, base, L.n, vec, yp);
         }
     }
+}
+
+// The kernel of a launch's mode (kRfPlain: the general map only, kRfZero without it).
+template <int SCHEME, bool TRANS, bool MON, bool GEN, bool DUAL = false, int N = P>
+const void* track_kernel(int mode)
+{
+    if (mode == kRfLinear)
+        return reinterpret_cast<const void*>(&k_track_f64<SCHEME, TRANS, MON, GEN, DUAL, N, kRfLinear>);
+    if (mode == kRfGeneral)
+        return reinterpret_cast<const void*>(&k_track_f64<SCHEME, TRANS, MON, GEN, DUAL, N, kRfGeneral>);
+    if constexpr (GEN)
+        if (mode == kRfPlain)
+            return reinterpret_cast<const void*>(&k_track_f64<SCHEME, TRANS, MON, GEN, DUAL, N, kRfPlain>);
+    return reinterpret_cast<const void*>(&k_track_f64<SCHEME, TRANS, MON, GEN, DUAL, N, kRfZero>);
 }
 
 }  // namespace kf64

@@ -288,6 +288,15 @@ __device__ __forceinline__ void force_df(const QuarterPhase& q, float ph, float 
     }
 }
 
+// The turn loop without phi_s (ZS), chosen outside it.  rf_linear takes it too with PHTL_F32CS, and the other
+// one with the double-float types: what the branch inside the kick leaves of each runs faster there (Ruth4 on
+// the double-RF ring, 1000 particles, moments every turn: PHTL_F32CS 22 % with phi_s, PHTL_F32CD 38 % without).
+template <int DT>
+__device__ __forceinline__ bool sine_only(const MapConsts& c)
+{
+    return DT == PHTL_F32CS ? c.phis_zero != 0 : c.rf_mode == kRfZero || c.rf_mode == kRfPlain;
+}
+
 // kick: delta += kw * (sin(phi) - sin(phi_s)), kw = kh + kl (the FP64 weight as a pair);
 // ZS: phi_s == 0, no subtraction
 template <int DT, bool ZS>

@@ -35,7 +35,14 @@ static_assert(P % 2 == 0, "P must be even (128-bit loads of two doubles)");
 #ifndef PHTL_F64_BATCHED_MIN_BLOCKS
 #define PHTL_F64_BATCHED_MIN_BLOCKS 3  // mixed batch 2 % faster than at 2
 #endif
-constexpr int kBatchedMinBlocks256 = PHTL_F64_BATCHED_MIN_BLOCKS;
+// The general map's batched kernels hold four schemes and spill at 3 (80 registers); at 2 the widened
+// map runs 2 to 20 % faster (16 bunches, Ruth4 without planes 1.85 -> 1.57 ms, RK4 3.45 -> 3.06 ms), but
+// two sines without a phase or a slippage expansion 2 to 5 % slower (RK4 2.93 -> 3.09 ms).
+template <bool GEN, int MODE>
+constexpr int batched_min_blocks_256()
+{
+    return GEN && MODE != kRfPlain ? 2 : PHTL_F64_BATCHED_MIN_BLOCKS;
+}
 template <int SCHEME>
 constexpr int min_blocks_256()
 {
@@ -78,16 +85,6 @@ __device__ __forceinline__ TurnWeights turn_weights(const double* dc, const doub
     return w;
 }
 
-// a b for the rf_linear branches: out of line, or the compiler issues the product with every
-// kick under a predicate (an FP64 instruction, half a clock of the pipe, even when it is off).
-static __device__ __noinline__ double branch_product(double a, double b) { return a * b; }
-
-// What the turn loop's code leaves out, chosen once per launch:
-//   kRfGeneral  any phi_s, rf_linear;
-//   kRfZero     phi_s = 0 with the sine force: the kick is sin(k z), no subtraction;
-//   kRfPlain    kRfZero, a second RF system (if any) with phi2 = 0, no slippage expansion.
-enum RfMode { kRfGeneral = 0, kRfZero = 1, kRfPlain = 2 };
-
 // Work that a turn runs beside the sines of its kick j, in the same stretch of code without a
 // branch: the sines occupy the integer pipe and the transverse push the FP64 pipe.
 struct NoSideWork {
@@ -100,9 +97,9 @@ template <int MODE, int N, class Side>
 __device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[N], double (&f)[N],
                                          const Side& side, int j)
 {
-    if (MODE == kRfGeneral && c.linear) {
+    if (MODE == kRfLinear) {
 #pragma unroll
-        for (int p = 0; p < N; ++p) f[p] = branch_product(c.lin, z[p]);
+        for (int p = 0; p < N; ++p) f[p] = c.lin * z[p];
         side(j);
         return;
     }
@@ -297,11 +294,11 @@ __device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[
         rf_force<MODE>(c, z, f, NoSideWork{}, 0);
         return;
     }
-    if (MODE == kRfGeneral && c.linear) {
+    if (MODE == kRfLinear) {
 #pragma unroll
         for (int p = 0; p < N; ++p) {
-            f[p] = branch_product(c.lin, z[p]);
-            g[p] = branch_product(c.lin2, z[p]);
+            f[p] = c.lin * z[p];
+            g[p] = c.lin2 * z[p];
         }
         return;
     }
@@ -373,12 +370,37 @@ __device__ __forceinline__ void rk4_rhs(const double (&z)[N], const double (&d)[
 // and k2, k4 at the full step from k3, and the weighted sum (k1 + 2 k2 + 2 k3 + k4) / 6.
 // The four stages are a loop that is not unrolled: with the sines of both RF systems in line
 // four times the turn's code did not fit the instruction cache (3.5 stalled cycles for
-// instructions per issue on the double-RF ring).
+// instructions per issue on the double-RF ring).  rf_linear has no sines: in line, and two FP64
+// operations fewer.
 template <int MODE, int N>
 __device__ __forceinline__ void rk4_turn(double (&z)[N], double (&d)[N], const MapConsts& c,
                                          const GeneralWeights& w, bool dual)
 {
     double a[N], b[N], kz[N], kd[N], sz[N], sd[N];
+    if constexpr (MODE == kRfLinear) {
+        double k1z[N], k1d[N], k2z[N], k2d[N];
+        rk4_rhs<MODE>(z, d, c, w, dual, k1z, k1d);
+#pragma unroll
+        for (int p = 0; p < N; ++p) a[p] = fma(w.half, k1z[p], z[p]), b[p] = fma(w.half, k1d[p], d[p]);
+        rk4_rhs<MODE>(a, b, c, w, dual, k2z, k2d);
+#pragma unroll
+        for (int p = 0; p < N; ++p) a[p] = fma(w.half, k2z[p], z[p]), b[p] = fma(w.half, k2d[p], d[p]);
+        rk4_rhs<MODE>(a, b, c, w, dual, kz, kd);
+#pragma unroll
+        for (int p = 0; p < N; ++p) {
+            sz[p] = __fma_rn(k2z[p], w.one, kz[p]);
+            sd[p] = __fma_rn(k2d[p], w.one, kd[p]);
+            a[p] = __fma_rn(kz[p], w.one, z[p]);
+            b[p] = __fma_rn(kd[p], w.one, d[p]);
+        }
+        rk4_rhs<MODE>(a, b, c, w, dual, kz, kd);
+#pragma unroll
+        for (int p = 0; p < N; ++p) {
+            z[p] = fma(fma(w.two, sz[p], __fma_rn(k1z[p], w.one, kz[p])), w.sixth, z[p]);
+            d[p] = fma(fma(w.two, sd[p], __fma_rn(k1d[p], w.one, kd[p])), w.sixth, d[p]);
+        }
+        return;
+    }
 #pragma unroll
     for (int p = 0; p < N; ++p) {
         a[p] = integer_copy(z[p], w.zero);

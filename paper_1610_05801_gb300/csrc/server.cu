@@ -139,7 +139,7 @@ public:
     int64_t saturation(int dtype) const
     {
         const int g = dtype < 0 || dtype >= kNumDtypes ? 0 : dtype;
-        const int occ = std::max(1, occupancy_batched(g, true, block_[g], h_->mc[0].general != 0));
+        const int occ = std::max(1, occupancy_batched(h_->mc[0], g, true, block_[g]));
         const int64_t waves = cfg_.waves > 0 ? cfg_.waves : 8;
         return waves * occ * h_->nsm * block_[g] * particles_per_thread(g);
     }

@@ -8,11 +8,10 @@
 namespace phtl {
 namespace {
 
-const void* select_batched(int dtype, bool mon)
+const void* select_batched(const MapConsts& c, int dtype, bool mon)
 {
-    if (dtype == PHTL_F64)
-        return mon ? reinterpret_cast<const void*>(&k_batched_f64<true, false>)
-                   : reinterpret_cast<const void*>(&k_batched_f64<false, false>);
+    if (c.general) return general_kernel_batched(c, dtype);
+    if (dtype == PHTL_F64) return mon ? batched_f64<true, false>(c.rf_mode) : batched_f64<false, false>(c.rf_mode);
     // PHTL_F32C and PHTL_F32CD are the same arithmetic: one instantiation
     if (dtype == PHTL_F32C || dtype == PHTL_F32CD)
         return mon ? reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32CD, true, false>)
@@ -27,9 +26,9 @@ const void* select_batched(int dtype, bool mon)
 
 int particles_per_thread(int dtype) { return dtype == PHTL_F64 ? f64::P : f32c::P; }
 
-int occupancy_batched(int dtype, bool mon, int block, bool general)
+int occupancy_batched(const MapConsts& c, int dtype, bool mon, int block)
 {
-    const void* k = general ? general_kernel_batched(dtype) : select_batched(dtype, mon);
+    const void* k = select_batched(c, dtype, mon);
     if (!k) return 0;
     int nb = 0;
     const size_t smem = mon ? 2u * (block / 32) * 16 * sizeof(double) : 0;
@@ -40,7 +39,7 @@ int occupancy_batched(int dtype, bool mon, int block, bool general)
 cudaError_t launch_batched(const JobDesc* jobs, int32_t njobs, const MapConsts& c, int dtype,
                            bool mon, int64_t t0, int32_t T, int grid, int block, cudaStream_t s)
 {
-    const void* k = c.general ? general_kernel_batched(dtype) : select_batched(dtype, mon);
+    const void* k = select_batched(c, dtype, mon);
     if (!k) return cudaErrorInvalidValue;
     if (grid <= 0) return cudaSuccess;
     const size_t smem = mon ? 2u * (block / 32) * 16 * sizeof(double) : 0;

@@ -58,7 +58,8 @@ __device__ __forceinline__ int slice_of(double z, double z_lo, double inv_dz, in
 // otherwise the linear map's, which a ring without those terms gives bitwise the same result
 // with fewer FP64 operations (a drift is one FMA instead of three).
 // Shared memory: ns uint32 histogram bins, then the monitor's 2 * warps * 16 DF2.
-template <int S, bool GEN>
+// MODE: RfMode; DUAL (GEN only): with the second RF system.
+template <int S, bool GEN, int MODE, bool DUAL>
 __global__ void __launch_bounds__(256, 3)
     k_coll_turn(LaunchDesc L, MapConsts c, CollArgs A, const double* __restrict__ U,
                 unsigned* __restrict__ counts, uint16_t* __restrict__ slot,
@@ -116,13 +117,11 @@ __global__ void __launch_bounds__(256, 3)
         }
         if (map) {
             if constexpr (GEN) {
-                if (c.phis_zero) long_turn_nl<S, kRfZero>(z, d, c, gw, c.dual_rf != 0);
-                else long_turn_nl<S, kRfGeneral>(z, d, c, gw, c.dual_rf != 0);
+                long_turn_nl<S, MODE>(z, d, c, gw, DUAL);
                 transverse_gen(x, xp, y, yp, d, hx, hy, c, gw);
             } else {
                 const RotateBeside<S, P> side{x, xp, y, yp, hx, hy, c, w};
-                if (c.phis_zero) long_turn<S, kRfZero>(z, d, c, w, side);
-                else long_turn<S, kRfGeneral>(z, d, c, w, side);
+                long_turn<S, MODE>(z, d, c, w, side);
             }
         }
         if (counts) {
@@ -201,21 +200,32 @@ __global__ void __launch_bounds__(256)
     griddep_launch_dependents();
 }
 
-template <int S>
-const void* coll_kernel_s(bool gen)
+template <int S, bool GEN, bool DUAL>
+const void* coll_kernel_s(int mode)
 {
-    return gen ? reinterpret_cast<const void*>(&k_coll_turn<S, true>)
-               : reinterpret_cast<const void*>(&k_coll_turn<S, false>);
+    if (mode == kRfLinear) return reinterpret_cast<const void*>(&k_coll_turn<S, GEN, kRfLinear, DUAL>);
+    if (mode == kRfGeneral) return reinterpret_cast<const void*>(&k_coll_turn<S, GEN, kRfGeneral, DUAL>);
+    if constexpr (GEN)
+        if (mode == kRfPlain) return reinterpret_cast<const void*>(&k_coll_turn<S, GEN, kRfPlain, DUAL>);
+    return reinterpret_cast<const void*>(&k_coll_turn<S, GEN, kRfZero, DUAL>);
 }
 
 // The linear map's variant where the ring has no widened term (RK4 always takes the
 // widened map's code).
-const void* coll_kernel(int scheme, bool gen)
+const void* coll_kernel(const MapConsts& c, int scheme)
 {
-    if (scheme == PHTL_EULER_CROMER) return coll_kernel_s<PHTL_EULER_CROMER>(gen);
-    if (scheme == PHTL_LEAPFROG) return coll_kernel_s<PHTL_LEAPFROG>(gen);
-    if (scheme == PHTL_RUTH4) return coll_kernel_s<PHTL_RUTH4>(gen);
-    if (scheme == PHTL_RK4) return reinterpret_cast<const void*>(&k_coll_turn<PHTL_RK4, true>);
+    const bool gen = c.general != 0, dual = c.dual_rf != 0;
+    const int mode = c.rf_mode;
+#define PHTL_COLL(S)                                                                     \
+    if (scheme == S)                                                                     \
+        return dual ? coll_kernel_s<S, true, true>(mode)                                 \
+                    : (gen ? coll_kernel_s<S, true, false>(mode) : coll_kernel_s<S, false, false>(mode));
+    PHTL_COLL(PHTL_EULER_CROMER)
+    PHTL_COLL(PHTL_LEAPFROG)
+    PHTL_COLL(PHTL_RUTH4)
+#undef PHTL_COLL
+    if (scheme == PHTL_RK4)
+        return dual ? coll_kernel_s<PHTL_RK4, true, true>(mode) : coll_kernel_s<PHTL_RK4, true, false>(mode);
     return nullptr;
 }
 
@@ -226,9 +236,9 @@ size_t coll_smem(int block, int ns)
 
 }  // namespace
 
-int occupancy_coll(int scheme, bool gen, int block, int nslices)
+int occupancy_coll(const MapConsts& c, int scheme, int block, int nslices)
 {
-    const void* k = coll_kernel(scheme, gen);
+    const void* k = coll_kernel(c, scheme);
     if (!k) return 0;
     const size_t sm = coll_smem(block, nslices);
     if (sm > 48 * 1024 &&
@@ -246,7 +256,7 @@ cudaError_t launch_coll_turn(const LaunchDesc& L, const MapConsts& c, const Coll
                              const double* U, unsigned* counts, uint16_t* slot, double* mon_rows,
                              int64_t rec_row, bool kick, bool map, cudaStream_t s)
 {
-    const void* k = coll_kernel(L.scheme, c.general != 0);
+    const void* k = coll_kernel(c, L.scheme);
     if (!k) return cudaErrorInvalidValue;
     LaunchDesc Lc = L;
     MapConsts cc = c;

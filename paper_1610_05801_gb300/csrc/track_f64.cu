@@ -16,18 +16,19 @@ namespace {
 using namespace f64;
 
 template <int S, bool T, bool M>
-const void* kernel_ptr(int ppt)
+const void* kernel_ptr(int ppt, int mode)
 {
-    return ppt == 1 ? reinterpret_cast<const void*>(&kf64::k_track_f64<S, T, M, false, false, 1>)
-                    : reinterpret_cast<const void*>(&kf64::k_track_f64<S, T, M, false>);
+    return ppt == 1 ? kf64::track_kernel<S, T, M, false, false, 1>(mode) : kf64::track_kernel<S, T, M, false>(mode);
 }
 
-const void* select_kernel(int scheme, bool trans, bool mon, int ppt)
+const void* select_kernel(const MapConsts& c, int scheme, bool trans, bool mon, int ppt)
 {
-#define PHTL_SEL(S)                                                              \
-    if (scheme == S) {                                                           \
-        if (trans) return mon ? kernel_ptr<S, true, true>(ppt) : kernel_ptr<S, true, false>(ppt); \
-        return mon ? kernel_ptr<S, false, true>(ppt) : kernel_ptr<S, false, false>(ppt);         \
+    if (c.general) return general_kernel_single(scheme, PHTL_F64, c.dual_rf != 0, c.rf_mode);
+    const int mode = c.rf_mode;
+#define PHTL_SEL(S)                                                                                     \
+    if (scheme == S) {                                                                                  \
+        if (trans) return mon ? kernel_ptr<S, true, true>(ppt, mode) : kernel_ptr<S, true, false>(ppt, mode); \
+        return mon ? kernel_ptr<S, false, true>(ppt, mode) : kernel_ptr<S, false, false>(ppt, mode);    \
     }
     PHTL_SEL(PHTL_EULER_CROMER)
     PHTL_SEL(PHTL_LEAPFROG)
@@ -54,10 +55,9 @@ int f64_particles_per_thread(bool trans, bool mon, int gen, int64_t n, int nsm)
     return gen == 0 && warps < limit ? 1 : P;
 }
 
-int occupancy_f64(int scheme, bool trans, bool mon, int block, int gen, int ppt)
+int occupancy_f64(const MapConsts& c, int scheme, bool trans, bool mon, int block, int ppt)
 {
-    const void* k = gen ? general_kernel_single(scheme, PHTL_F64, gen == 2)
-                        : select_kernel(scheme, trans, mon, ppt);
+    const void* k = select_kernel(c, scheme, trans, mon, ppt);
     if (!k) return 0;
     int nb = 0;
     const size_t smem = mon ? 2u * (block / 32) * 16 * sizeof(double) : 0;
@@ -70,8 +70,7 @@ cudaError_t launch_track_f64(const LaunchDesc& L, const MapConsts& c, const Moni
 {
     const bool trans = L.c[2] != nullptr || L.c[4] != nullptr;
     const bool mon = m.rows != nullptr;
-    const void* k = c.general ? general_kernel_single(L.scheme, PHTL_F64, c.dual_rf != 0)
-                              : select_kernel(L.scheme, trans, mon, L.ppt);
+    const void* k = select_kernel(c, L.scheme, trans, mon, L.ppt);
     if (!k) return cudaErrorInvalidValue;
     const size_t smem = mon ? 2u * (L.block / 32) * 16 * sizeof(double) : 0;
     LaunchDesc Lc = L;

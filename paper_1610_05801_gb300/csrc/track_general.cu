@@ -12,23 +12,24 @@
 
 namespace phtl {
 
-const void* general_kernel_single(int scheme, int dtype, bool dual)
+// mode: RfMode, for the FP64 kernels
+const void* general_kernel_single(int scheme, int dtype, bool dual, int mode)
 {
-    if (dual) return general_kernel_single_dual(scheme, dtype);
-#define PHTL_GEN(S)                                                                          \
-    if (scheme == S) {                                                                       \
-        if (dtype == PHTL_F64) return reinterpret_cast<const void*>(&kf64::k_track_f64<S, true, true, true>); \
-        if (dtype == PHTL_F32C || dtype == PHTL_F32CD)                                       \
+    if (dual) return general_kernel_single_dual(scheme, dtype, mode);
+#define PHTL_GEN(S)                                                                                     \
+    if (scheme == S) {                                                                                  \
+        if (dtype == PHTL_F64) return kf64::track_kernel<S, true, true, true>(mode);                    \
+        if (dtype == PHTL_F32C || dtype == PHTL_F32CD)                                                  \
             return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32CD, true, true, true>); \
-        if (dtype == PHTL_F32CS)                                                             \
+        if (dtype == PHTL_F32CS)                                                                        \
             return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32CS, true, true, true>); \
-        return nullptr;                                                                      \
+        return nullptr;                                                                                 \
     }
     PHTL_GEN(PHTL_EULER_CROMER)
     PHTL_GEN(PHTL_LEAPFROG)
     PHTL_GEN(PHTL_RUTH4)
 #undef PHTL_GEN
-    if (scheme == PHTL_RK4) return general_kernel_single_rk4(dtype);
+    if (scheme == PHTL_RK4) return general_kernel_single_rk4(dtype, mode);
     return nullptr;
 }
 

@@ -10,10 +10,10 @@
 
 namespace phtl {
 
-const void* general_kernel_batched(int dtype)
+const void* general_kernel_batched(const MapConsts& c, int dtype)
 {
-    if (dtype == PHTL_F64) return reinterpret_cast<const void*>(&k_batched_f64<true, true>);
-    return general_kernel_batched_f32(dtype);
+    if (dtype != PHTL_F64) return general_kernel_batched_f32(dtype);
+    return c.dual_rf ? batched_f64<true, true, true>(c.rf_mode) : batched_f64<true, true>(c.rf_mode);
 }
 
 }  // namespace phtl

@@ -65,16 +65,17 @@ __device__ __forceinline__ void drift(double (&z)[P], const double (&d)[P], doub
     for (int p = 0; p < P; ++p) z[p] = fma(-dc, d[p], z[p]);
 }
 
-// delta += kw (sin(phi_s,n + k z) - sin(phi_s,n)), kw this stage's weight times A_n
-template <class Side>
+// delta += kw (sin(phi_s,n + k z) - sin(phi_s,n)), kw this stage's weight times A_n; LINEAR (rf_linear):
+// delta += kw lin_n z
+template <bool LINEAR, class Side>
 __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], double kw,
                                      const Turn& T, const MapConsts& c, const Unit& u, const Side& side, int j)
 {
     double f[P];
     bool ok[P], all = true;
-    if (c.linear) {
+    if (LINEAR) {
 #pragma unroll
-        for (int p = 0; p < P; ++p) f[p] = branch_product(T.lin, z[p]);
+        for (int p = 0; p < P; ++p) f[p] = __fma_rn(T.lin, z[p], u.mzero);
         side(j);
     } else {
 #pragma unroll
@@ -95,32 +96,63 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
     for (int p = 0; p < P; ++p) d[p] = fma(kw, f[p], d[p]);
 }
 
-template <int S, class Side>
+template <int S, bool LINEAR, class Side>
 __device__ __forceinline__ void turn(double (&z)[P], double (&d)[P], const Turn& T, const MapConsts& c,
                                      const double* __restrict__ w, const Unit& u, const Side& side)
 {
     if (S == PHTL_EULER_CROMER) {
-        kick(z, d, __ldg(w + 1), T, c, u, side, 0);
+        kick<LINEAR>(z, d, __ldg(w + 1), T, c, u, side, 0);
         drift(z, d, __ldg(w + 0));
     } else if (S == PHTL_LEAPFROG) {
         drift(z, d, __ldg(w + 0));
-        kick(z, d, __ldg(w + 2), T, c, u, side, 0);
+        kick<LINEAR>(z, d, __ldg(w + 2), T, c, u, side, 0);
         drift(z, d, __ldg(w + 1));
     } else {
         drift(z, d, __ldg(w + 0));
-        kick(z, d, __ldg(w + 4), T, c, u, side, 0);
+        kick<LINEAR>(z, d, __ldg(w + 4), T, c, u, side, 0);
         drift(z, d, __ldg(w + 1));
-        kick(z, d, __ldg(w + 5), T, c, u, side, 1);
+        kick<LINEAR>(z, d, __ldg(w + 5), T, c, u, side, 1);
         drift(z, d, __ldg(w + 2));
-        kick(z, d, __ldg(w + 6), T, c, u, side, 2);
+        kick<LINEAR>(z, d, __ldg(w + 6), T, c, u, side, 2);
         drift(z, d, __ldg(w + 3));
+    }
+}
+
+// The turn loop of one particle chunk, prog: the launch's first turn (LINEAR: rf_linear).
+template <int S, bool LINEAR>
+__device__ __forceinline__ void turns(double (&z)[P], double (&d)[P], double (&x)[P], double (&xp)[P], double (&y)[P],
+                                      double (&yp)[P], bool hx, bool hy, float cnt, const LaunchDesc& L,
+                                      const MapConsts& c, const MonitorArgs& m, const RampTurn* __restrict__ prog,
+                                      const Unit& unit, const TurnWeights& tw, double* smem, int& parity)
+{
+    int64_t until = m.until, row = m.row;
+    Turn T{};
+    if (L.nturns > 0) T = load_turn(prog);  // a launch reads its nturns entries only
+    for (int t = 0; t < L.nturns; ++t) {
+        // the next turn's constants, loaded while this turn computes
+        const Turn Tn = load_turn(prog + (t + 1 < L.nturns ? t + 1 : t));
+        turn<S, LINEAR>(z, d, T, c, stage_weights<S>(prog + t), unit,
+                        RotateBeside<S, P>{x, xp, y, yp, hx, hy, c, tw});
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            d[p] = __fma_rn(T.r, d[p], unit.mzero);
+            xp[p] = __fma_rn(T.r, xp[p], unit.mzero);
+            yp[p] = __fma_rn(T.r, yp[p], unit.mzero);
+        }
+        if (m.rows && --until == 0) {
+            record<true>(z, d, x, xp, y, yp, cnt, hx, hy, smem, parity, m.rows, row);
+            parity ^= 1;
+            ++row;
+            until = m.stride;
+        }
+        T = Tn;
     }
 }
 
 #ifndef PHTL_F64_RAMP_MIN_BLOCKS
 #define PHTL_F64_RAMP_MIN_BLOCKS 3  // 8 % faster than at 2 (leap-frog, both planes, moments)
 #endif
-template <int S>
+template <int S, bool LINEAR>
 __global__ void __launch_bounds__(256, PHTL_F64_RAMP_MIN_BLOCKS)
     k_ramp_f64(LaunchDesc L, MapConsts c, MonitorArgs m, const RampTurn* __restrict__ prog, int64_t turn0)
 {
@@ -162,27 +194,7 @@ __global__ void __launch_bounds__(256, PHTL_F64_RAMP_MIN_BLOCKS)
             record<true>(z, d, x, xp, y, yp, cnt, hx, hy, smem, parity, m.rows, 0);
             parity ^= 1;
         }
-        int64_t until = m.until, row = m.row;
-        Turn T{};
-        if (L.nturns > 0) T = load_turn(prog + turn0);  // a launch reads turns [turn0, turn0 + nturns) only
-        for (int t = 0; t < L.nturns; ++t) {
-            // the next turn's constants, loaded while this turn computes
-            const Turn Tn = load_turn(prog + turn0 + (t + 1 < L.nturns ? t + 1 : t));
-            turn<S>(z, d, T, c, stage_weights<S>(prog + turn0 + t), unit, RotateBeside<S, P>{x, xp, y, yp, hx, hy, c, tw});
-#pragma unroll
-            for (int p = 0; p < P; ++p) {
-                d[p] = __fma_rn(T.r, d[p], unit.mzero);
-                xp[p] = __fma_rn(T.r, xp[p], unit.mzero);
-                yp[p] = __fma_rn(T.r, yp[p], unit.mzero);
-            }
-            if (m.rows && --until == 0) {
-                record<true>(z, d, x, xp, y, yp, cnt, hx, hy, smem, parity, m.rows, row);
-                parity ^= 1;
-                ++row;
-                until = m.stride;
-            }
-            T = Tn;
-        }
+        turns<S, LINEAR>(z, d, x, xp, y, yp, hx, hy, cnt, L, c, m, prog + turn0, unit, tw, smem, parity);
         store2(g[0], base, L.n, vec, z);
         store2(g[1], base, L.n, vec, d);
         if (hx) {
@@ -386,20 +398,23 @@ __global__ void PHTL_F32C_RAMP_BOUNDS(S, DT)
 }  // namespace rf32
 
 template <int S>
-const void* ramp_kernel_s(int dtype)
+const void* ramp_kernel_s(int dtype, bool linear)
 {
-    if (dtype == PHTL_F64) return reinterpret_cast<const void*>(&rf64::k_ramp_f64<S>);
+    if (dtype == PHTL_F64)
+        return linear ? reinterpret_cast<const void*>(&rf64::k_ramp_f64<S, true>)
+                      : reinterpret_cast<const void*>(&rf64::k_ramp_f64<S, false>);
     // PHTL_F32C and PHTL_F32CD are the same arithmetic: one instantiation
     if (dtype == PHTL_F32C || dtype == PHTL_F32CD) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32CD>);
     if (dtype == PHTL_F32CS) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32CS>);
     return nullptr;
 }
 
-const void* ramp_kernel(int scheme, int dtype)
+const void* ramp_kernel(const MapConsts& c, int scheme, int dtype)
 {
-    if (scheme == PHTL_EULER_CROMER) return ramp_kernel_s<PHTL_EULER_CROMER>(dtype);
-    if (scheme == PHTL_LEAPFROG) return ramp_kernel_s<PHTL_LEAPFROG>(dtype);
-    if (scheme == PHTL_RUTH4) return ramp_kernel_s<PHTL_RUTH4>(dtype);
+    const bool linear = c.linear != 0;
+    if (scheme == PHTL_EULER_CROMER) return ramp_kernel_s<PHTL_EULER_CROMER>(dtype, linear);
+    if (scheme == PHTL_LEAPFROG) return ramp_kernel_s<PHTL_LEAPFROG>(dtype, linear);
+    if (scheme == PHTL_RUTH4) return ramp_kernel_s<PHTL_RUTH4>(dtype, linear);
     return nullptr;
 }
 
@@ -407,9 +422,9 @@ size_t ramp_smem(int block) { return 2u * (block / 32) * 16 * sizeof(double); }
 
 }  // namespace
 
-int occupancy_ramp(int scheme, int dtype, int block)
+int occupancy_ramp(const MapConsts& c, int scheme, int dtype, int block)
 {
-    const void* k = ramp_kernel(scheme, dtype);
+    const void* k = ramp_kernel(c, scheme, dtype);
     if (!k) return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, block, ramp_smem(block)) != cudaSuccess)
@@ -420,7 +435,7 @@ int occupancy_ramp(int scheme, int dtype, int block)
 cudaError_t launch_ramp(const LaunchDesc& L, const MapConsts& c, const MonitorArgs& m,
                         const RampTurn* prog, int64_t turn0, int dtype, cudaStream_t s)
 {
-    const void* k = ramp_kernel(L.scheme, dtype);
+    const void* k = ramp_kernel(c, L.scheme, dtype);
     if (!k) return cudaErrorInvalidValue;
     LaunchDesc Lc = L;
     MapConsts cc = c;
