@@ -115,7 +115,7 @@ __device__ __forceinline__ void rf_force(const MapConsts& c, const double (&z)[N
 #pragma unroll
         for (int p = 0; p < N; ++p)
             if (!ok[p])
-                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.ophis);
+                f[p] = sin_rest<MODE != kRfGeneral>(c.k, c.kap, z[p], c.phis, c.ophis);
     }
     if (MODE == kRfGeneral) {
 #pragma unroll
@@ -315,10 +315,8 @@ __device__ __forceinline__ void rf_forces(const MapConsts& c, const double (&z)[
 #pragma unroll
         for (int p = 0; p < N; ++p) {
             if (!ok[p])
-                f[p] = MODE != kRfGeneral ? sin_kz_rest(c.k, c.kap, z[p]) : sin_phi_rest(c.k, c.kap, z[p], c.phis, c.ophis);
-            if (!ok2[p])
-                g[p] = MODE == kRfPlain ? sin_kz_rest(c.k2, c.kap2, z[p])
-                                        : sin_phi_rest(c.k2, c.kap2, z[p], c.phi2, c.ophi2);
+                f[p] = sin_rest<MODE != kRfGeneral>(c.k, c.kap, z[p], c.phis, c.ophis);
+            if (!ok2[p]) g[p] = sin_rest<MODE == kRfPlain>(c.k2, c.kap2, z[p], c.phi2, c.ophi2);
         }
     }
 #pragma unroll

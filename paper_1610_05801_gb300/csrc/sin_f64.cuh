@@ -203,6 +203,11 @@ __device__ __forceinline__ bool phase_of_turns(PhaseScale kap, double z, uint64_
     return true;
 }
 
+__device__ __forceinline__ bool is_zero(double z)
+{
+    return (__double2hiint(z) << 1 | __double2loint(z)) == 0;
+}
+
 // sin(k z) where sin_kz_fixed does not cover it.  z = 0 (also the unused lanes of a ragged bunch)
 // is returned as it is; up to 2^14 turns (particles that have left the bucket, an unbunched beam)
 // the integer form with the longer phase; beyond it, close to zero and for Inf and NaN
@@ -210,7 +215,7 @@ __device__ __forceinline__ bool phase_of_turns(PhaseScale kap, double z, uint64_
 // kicks.
 static __device__ __noinline__ double sin_kz_rest(double k, PhaseScale kap, double z)
 {
-    if ((__double2hiint(z) << 1 | __double2loint(z)) == 0) return z;
+    if (is_zero(z)) return z;
     uint64_t U;
     if (!phase_of_turns(kap, z, U)) return sin_f64(k * z);
     return detail::sin_turns_any(U, static_cast<uint32_t>(__double2hiint(z)));
@@ -225,6 +230,16 @@ static __device__ __noinline__ double sin_phi_rest(double k, PhaseScale kap, dou
     if ((__double2hiint(x) & 0x7fffffff) < 0x3f800000 || !phase_of_turns(kap, z, U)) return sin_f64(x);
     const uint64_t uphi = static_cast<uint64_t>(detail::sar_sat(o.u, static_cast<uint32_t>(o.g)));
     return detail::sin_turns_any(__double2hiint(z) < 0 ? uphi - U : uphi + U, 0u);
+}
+
+// Either of the two where phi = 0 (ZERO) or not.  z = 0 with phi = 0 -- a particle at the centre, and the
+// lanes beyond the end of a bunch in its last warp, in every turn -- is answered without the call, whose
+// time the whole of a small bunch waits for.
+template <bool ZERO>
+__device__ __forceinline__ double sin_rest(double k, PhaseScale kap, double z, double phi, PhaseOffset o)
+{
+    if (is_zero(z) && (ZERO || o.u == 0)) return z;
+    return ZERO ? sin_kz_rest(k, kap, z) : sin_phi_rest(k, kap, z, phi, o);
 }
 
 // The kicks take the integer sine of all their particles first, without a branch in between

@@ -87,7 +87,7 @@ __device__ __forceinline__ void kick(const double (&z)[P], double (&d)[P], doubl
         if (!all) {
 #pragma unroll
             for (int p = 0; p < P; ++p)
-                if (!ok[p]) f[p] = sin_phi_rest(c.k, c.kap, z[p], T.phis, T.ophis);
+                if (!ok[p]) f[p] = sin_rest<false>(c.k, c.kap, z[p], T.phis, T.ophis);
         }
 #pragma unroll
         for (int p = 0; p < P; ++p) f[p] = __fma_rn(f[p], u.one, -T.sinphis);
