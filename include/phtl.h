@@ -88,10 +88,11 @@ enum { PHTL_EULER_CROMER = 0, PHTL_LEAPFROG = 1, PHTL_RUTH4 = 2, PHTL_RK4 = 3 };
  *               hi[i] + comp[i].  Increments are double-float products of the FP64
  *               coefficients (split into hi + lo floats) and the pair, added with
  *               TwoSum and renormalised with Fast2Sum.  The RF phase argument is formed
- *               in quarter turns from hi + comp and k 2/pi in three floats, reduced exactly
- *               and kept to 2^-47; the sine is the library's double-float sine (~2e-12
- *               absolute on the bucket).  No FP64 instruction on the path.
- *  PHTL_F32CD : the same arithmetic as PHTL_F32C (kept as a type of its own).
+ *               in FP64 from hi + comp; the sine is the library's double-float sine
+ *               (~2e-12 absolute on the bucket).
+ *  PHTL_F32CD : as PHTL_F32C, but the phase argument is formed in quarter turns from
+ *               hi + comp and k 2/pi in three floats, reduced exactly and kept to 2^-47:
+ *               no FP64 instruction on the path.
  *  PHTL_F32CS : FP32 increments (coefficients split into hi + lo, TwoSum accumulation),
  *               the phase rounded to FP32 and the SFU's sine (__sinf, absolute error
  *               ~2^-21 on [-pi, pi]): fastest, least accurate over long horizons.    */
@@ -587,8 +588,8 @@ int phtl_moments_from_sums(const double* row, double* out15);
 /* Diagnostic: y[i] = sine of x[i] on the device, for n device doubles, stream-ordered.
  * which = 0: the library's own sine in FP64 arithmetic (Cody-Waite reduction plus a
  * fitted polynomial), which the FP64 kicks take beyond their fixed-point sine's range; which = 1: CUDA's sin(), for comparison; which = 2: the
- * double-float sine of the PHTL_F32C / PHTL_F32CD kicks, applied to x[i] truncated to
- * a float pair (48 bits) and returned as hi + lo.
+ * double-float sine of the PHTL_F32CD kicks (PHTL_F32C's but for the phase), applied to
+ * x[i] truncated to a float pair (48 bits) and returned as hi + lo.
  * Errors: PHTL_E_INVALID, PHTL_E_NODEVICE, PHTL_E_CUDA.                           */
 int phtl_eval_sin(const double* x, double* y, int64_t n, int which, void* cuda_stream);
 

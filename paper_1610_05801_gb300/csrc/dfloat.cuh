@@ -71,6 +71,39 @@ __device__ __forceinline__ double widen_float_bits(float f)
                             static_cast<int>(m << 29));
 }
 
+// Cheaper forms of the two for the RF phase argument of the PHTL_F32C kernels (k z + phi formed in FP64
+// from a coordinate's two floats), where a term below 2^-126 in magnitude changes nothing.
+//
+// widen_float_phase: exact for normal floats and +-0 (a particle at z = 0 keeps the phase 0
+// exactly); subnormals become values of magnitude in [2^-127, 2^-126); Inf / NaN become
+// finite values of magnitude >= 2^128 (a lost particle's phase, which split_phase does not cover).
+__device__ __forceinline__ double widen_float_phase(float f)
+{
+    const unsigned u = __float_as_uint(f);
+    const unsigned mag = u & 0x7fffffffu;
+    const unsigned hi = mag != 0u ? (mag >> 3) + (896u << 20) : 0u;
+    return __hiloint2double(static_cast<int>((u & 0x80000000u) | hi), static_cast<int>(u << 29));
+}
+
+// split_phase: split_bits's high part; the low part is the remaining 29 bits rounded to
+// nearest (one integer-to-float conversion) instead of truncated, so
+// |x - (h + l)| <= 2^-48 |x|.  For 2^-74 <= |x| < 2^13; ok is cleared beyond, for 0, Inf and NaN
+// (without a branch, so that the phases of a thread's particles interleave).
+__device__ __forceinline__ DF2 split_phase(double x, bool& ok)
+{
+    const unsigned hi32 = static_cast<unsigned>(__double2hiint(x));
+    const unsigned lo32 = static_cast<unsigned>(__double2loint(x));
+    const unsigned e = (hi32 >> 20) & 0x7ffu;
+    ok = e - 949u <= 86u;
+    const unsigned sign = hi32 & 0x80000000u;
+    const unsigned t = (hi32 & 0x7fffffffu) - (896u << 20);  // FP32 biased exponent at bit 20
+    DF2 r;
+    r.h = __uint_as_float(sign | __funnelshift_l(lo32, t, 3));
+    const float m = __uint2float_rn(lo32 & 0x1fffffffu);      // the remaining bits, rounded
+    r.l = __fmul_rn(m, __uint_as_float(sign | ((e - 948u) << 23)));
+    return r;
+}
+
 __device__ __forceinline__ DF2 df_two_sum(float a, float b)
 {
     const float s = __fadd_rn(a, b);
@@ -151,6 +184,16 @@ __device__ __forceinline__ double df_to_double(DF2 a)
 __device__ __forceinline__ DF2 df_shfl_xor(DF2 a, int o)
 {
     return DF2{__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)};
+}
+
+// A launch constant held in a register.  An FP64 FMA whose operands all lie in registers takes
+// the pipe 0.50 clocks per lane and SM, one with an operand in the constant bank 0.59 (also
+// DADD and DMUL; measured), so the persistent kernels move the weights of their turn loop to
+// registers.  Through a shuffle, which the compiler does not fold back into the operand.
+__device__ __forceinline__ double in_register(double v)
+{
+    return __hiloint2double(__shfl_sync(0xffffffffu, __double2hiint(v), 0),
+                            __shfl_sync(0xffffffffu, __double2loint(v), 0));
 }
 
 }  // namespace phtl

@@ -169,13 +169,14 @@ __device__ __forceinline__ void run_f32c_zs(f32c::DF (&z)[f32c::P], f32c::DF (&d
     int64_t row = g0 / J.stride + 1;
     float g1h[4], g1l[4], g2h[4], g2l[4];
     if (GEN) slip_stages<SCHEME>(c, g1h, g1l, g2h, g2l);
+    const Waves wv = waves<DT>(c);
     for (int t = 0; t < nt; ++t) {
         if (GEN) {
-            long_turn_nl<SCHEME, DT, ZS>(z, d, c, J.dc_hi, J.dc_lo, J.kw_hi, J.kw_lo, J.kw2_hi,
+            long_turn_nl<SCHEME, DT, ZS>(z, d, c, wv, J.dc_hi, J.dc_lo, J.kw_hi, J.kw_lo, J.kw2_hi,
                                          J.kw2_lo, g1h, g1l, g2h, g2l, c.dual_rf != 0);
             transverse_gen<DT>(x, xp, y, yp, d, hx, hy, c);
         } else {
-            long_turn<SCHEME, DT, ZS>(z, d, c, J.dc_hi, J.dc_lo, J.kw_hi, J.kw_lo);
+            long_turn<SCHEME, DT, ZS>(z, d, c, wv, J.dc_hi, J.dc_lo, J.kw_hi, J.kw_lo);
             if (hx) {
 #pragma unroll
                 for (int p = 0; p < P; ++p) df_rotate(x[p], xp[p], c.mx_hi, c.mx_lo);

@@ -82,6 +82,7 @@ __global__ void PHTL_COLL_F32_BOUNDS
     int parity = 0;
     float g1h[4], g1l[4], g2h[4], g2l[4];
     if (GEN) slip_stages<S>(c, g1h, g1l, g2h, g2l);
+    const Waves wv{c.k, c.k2};  // one turn a chunk
     const int ns_hi = __double2hiint(static_cast<double>(A.nslices));
     for (int64_t ci = blockIdx.x; ci < nchunks; ci += gridDim.x) {
         const int64_t base = ci * chunk + static_cast<int64_t>(threadIdx.x) * P;
@@ -119,15 +120,15 @@ __global__ void PHTL_COLL_F32_BOUNDS
         if (map) {
             if constexpr (GEN) {
                 if (sine_only<DT>(c))
-                    long_turn_nl<S, DT, true>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo, c.kw2_hi,
+                    long_turn_nl<S, DT, true>(z, d, c, wv, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo, c.kw2_hi,
                                               c.kw2_lo, g1h, g1l, g2h, g2l, c.dual_rf != 0);
                 else
-                    long_turn_nl<S, DT, false>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo, c.kw2_hi,
+                    long_turn_nl<S, DT, false>(z, d, c, wv, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo, c.kw2_hi,
                                                c.kw2_lo, g1h, g1l, g2h, g2l, c.dual_rf != 0);
                 transverse_gen<DT>(x, xp, y, yp, d, hx, hy, c);
             } else {
-                if (sine_only<DT>(c)) long_turn<S, DT, true>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
-                else long_turn<S, DT, false>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
+                if (sine_only<DT>(c)) long_turn<S, DT, true>(z, d, c, wv, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
+                else long_turn<S, DT, false>(z, d, c, wv, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
                 if (hx) {
 #pragma unroll
                     for (int p = 0; p < P; ++p) df_rotate(x[p], xp[p], c.mx_hi, c.mx_lo);

@@ -6,8 +6,9 @@
 // registers), but every coordinate is an unevaluated sum hi + comp of two floats:
 //   - PHTL_F32C / PHTL_F32CD: each drift/kick increment is a double-float product of the
 //     FP64 weight (split into hi + lo) and the pair, added with Knuth's TwoSum and
-//     renormalised with Fast2Sum; the RF phase argument is formed from hi + comp in quarter
-//     turns and the sine is a double-float polynomial (sin_quarter_df, ~1e-12 absolute);
+//     renormalised with Fast2Sum; the RF phase argument is formed from hi + comp in FP64
+//     (PHTL_F32C) or in quarter turns in double-float arithmetic (PHTL_F32CD), and the sine is a
+//     double-float polynomial (sin_pair_poly, ~1e-12 absolute);
 //   - PHTL_F32CS: FP32 increments with split weights, the phase rounded to FP32 and the
 //     SFU's __sinf;
 //   - the transverse matrix (Sec. 1.1.1) is applied in double-float arithmetic (exact
@@ -15,9 +16,10 @@
 //   - per-turn moment sums are FP32 per thread and across the warp (<= 128 particles),
 //     then FP64 across warps and blocks.
 // Each thread owns P = 4 particles (one 128-bit load of hi and one of comp per
-// coordinate).  Issue bound: 127 instructions per particle and leap-frog turn, 0.99 clocks of an
-// SM's issue slots, 1.2 measured at 4e6 particles (213 instructions and 2.2 clocks before the
-// quarter-turn phase and with renormalised intermediate products).
+// coordinate).  Issue bound: PHTL_F32CD takes 127 instructions per particle and leap-frog turn, 0.99
+// clocks of an SM's issue slots, 1.2 measured at 4e6 particles (213 instructions and 2.2 clocks before
+// the quarter-turn phase and with renormalised intermediate products); PHTL_F32C's two FP64 FMAs take
+// the FP64 pipe 1.0 clocks beside it, 1.6 measured.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -42,13 +44,14 @@ __device__ __forceinline__ void turns(DF (&z)[P], DF (&d)[P], DF (&x)[P], DF (&x
     int64_t until = m.until, row = m.row;
     float g1h[4], g1l[4], g2h[4], g2l[4];
     if (GEN) slip_stages<SCHEME>(c, g1h, g1l, g2h, g2l);
+    const Waves wv = waves<DT>(c);
     for (int t = 0; t < nturns; ++t) {
         if (GEN) {
-            long_turn_nl<SCHEME, DT, ZS>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo, c.kw2_hi,
+            long_turn_nl<SCHEME, DT, ZS>(z, d, c, wv, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo, c.kw2_hi,
                                          c.kw2_lo, g1h, g1l, g2h, g2l, DUAL);
             if (TRANS) transverse_gen<DT>(x, xp, y, yp, d, hx, hy, c);
         } else {
-            long_turn<SCHEME, DT, ZS>(z, d, c, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
+            long_turn<SCHEME, DT, ZS>(z, d, c, wv, c.dc_hi, c.dc_lo, c.kw_hi, c.kw_lo);
             if (TRANS) {
                 if (hx) {
 #pragma unroll
@@ -75,7 +78,7 @@ __device__ __forceinline__ void turns(DF (&z)[P], DF (&d)[P], DF (&x)[P], DF (&x
 // true; planes and monitor are checked at run time); DUAL (GEN only): with the second RF
 // system.
 template <int SCHEME, int DT, bool TRANS, bool MON, bool GEN, bool DUAL = false>
-__global__ void PHTL_F32C_TRACK_BOUNDS(SCHEME, DT, GEN) k_track_f32c(LaunchDesc L, MapConsts c, MonitorArgs m)
+__global__ void PHTL_F32C_TRACK_BOUNDS(SCHEME, DT, GEN, TRANS) k_track_f32c(LaunchDesc L, MapConsts c, MonitorArgs m)
 {
     if (L.go && *L.go == 0) return;  // the call was cancelled before this launch
     extern __shared__ double smem[];

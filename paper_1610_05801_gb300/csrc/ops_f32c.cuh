@@ -16,18 +16,21 @@ namespace f32c {
 constexpr int P = 4;
 
 // Register budgets of the FP32-compensated kernels, as resident 256-thread blocks per SM asked
-// of the compiler, or as registers (PHTL_F32C and PHTL_F32CD run the PHTL_F32CD kernels, but for
-// the collective step).  The kernels are issue-bound; four particles' sines in
-// flight want registers more than the SM wants warps (1e6 particles and the benchmark's cases):
-//   - linear map: 2 blocks (at most 128 registers) for FP32C and FP32CD (leap-frog 3.7 % faster
-//     than at 64 or 80 registers, Ruth4 with planes and moments 4 %); 3 for FP32CS;
+// of the compiler, or as registers.  The kernels are issue-bound; four particles' sines in
+// flight want registers more than the SM wants warps (1e6 particles and the benchmark's cases),
+// unless they wait for FP64 phases (FP32C) with little else to do:
+//   - linear map: 2 blocks (at most 128 registers) for FP32C and FP32CD (FP32CD leap-frog 3.7 % faster
+//     than at 64 or 80 registers, Ruth4 with planes and moments 4 %; FP32C with planes and moments 4 to
+//     6 %); 4 (64 registers) for FP32C without planes (leap-frog, 4e6 particles, 20 turns: 397 us
+//     against 440 at 2 and 412 at 3; Ruth4, 6e5: 187, 223, 211); 3 for FP32CS;
 //   - widened map and RK4 / double RF (general kernels): 2 blocks for FP32C and FP32CD (widened
 //     leap-frog 5 % faster than at 3, RK4 on the double-RF ring 20 %), 3 for FP32CS;
 //   - batched kernels: 96 registers for FP32C and FP32CD (64 bunches, moments every turn: 7 %
 //     faster than at 80 or 128, 13 % than at 64; without launch bounds beside the cap, with which
 //     the compiler spills 288 bytes instead of 32 and the gain is lost), 80 for FP32CS; the widened
 //     map's: 128 for FP32C and FP32CD, 80 for FP32CS;
-//   - ramp programme: the compiler's choice (track_ramp.cu).
+//   - ramp programme: 2 blocks for FP32C (Ruth4 with planes and moments 20 % faster than the compiler's
+//     choice, 10 % than 3), the compiler's choice for the others (track_ramp.cu).
 // Build options PHTL_F32C_GEN_MIN_BLOCKS, PHTL_F32C_GEN_BATCHED_MIN_BLOCKS (general kernels) and
 // PHTL_F32C_MAXNREG (one register cap for all of them) override these, for measuring.
 constexpr int f32c_general_min_blocks(int scheme, int dtype)
@@ -38,9 +41,10 @@ constexpr int f32c_general_min_blocks(int scheme, int dtype)
     return (void)scheme, dtype == PHTL_F32CS ? 3 : 2;
 #endif
 }
-constexpr int f32c_track_min_blocks(int scheme, int dtype, bool general)
+constexpr int f32c_track_min_blocks(int scheme, int dtype, bool general, bool trans)
 {
-    return general ? f32c_general_min_blocks(scheme, dtype) : (dtype == PHTL_F32CS ? 3 : 2);
+    return general ? f32c_general_min_blocks(scheme, dtype)
+                   : (dtype == PHTL_F32CS ? 3 : (dtype == PHTL_F32C && !trans ? 4 : 2));
 }
 constexpr int f32c_batched_registers(int dtype, bool general)
 {
@@ -51,11 +55,11 @@ constexpr int f32c_batched_registers(int dtype, bool general)
 }
 #ifdef PHTL_F32C_MAXNREG
 #define PHTL_F32C_RAMP_BOUNDS(S, DT) __maxnreg__(PHTL_F32C_MAXNREG)
-#define PHTL_F32C_TRACK_BOUNDS(S, DT, G) __maxnreg__(PHTL_F32C_MAXNREG)
+#define PHTL_F32C_TRACK_BOUNDS(S, DT, G, T) __maxnreg__(PHTL_F32C_MAXNREG)
 #define PHTL_F32C_BATCHED_BOUNDS(DT, G) __maxnreg__(PHTL_F32C_MAXNREG)
 #else
-#define PHTL_F32C_RAMP_BOUNDS(S, DT) __launch_bounds__(256)
-#define PHTL_F32C_TRACK_BOUNDS(S, DT, G) __launch_bounds__(256, f32c::f32c_track_min_blocks(S, DT, G))
+#define PHTL_F32C_RAMP_BOUNDS(S, DT) __launch_bounds__(256, (DT) == PHTL_F32C ? 2 : 1)
+#define PHTL_F32C_TRACK_BOUNDS(S, DT, G, T) __launch_bounds__(256, f32c::f32c_track_min_blocks(S, DT, G, T))
 #define PHTL_F32C_BATCHED_BOUNDS(DT, G) __maxnreg__(f32c::f32c_batched_registers(DT, G))
 #endif
 constexpr float kTwoPiHi = 6.28318548202514648438f;     // float(2 pi)
@@ -151,45 +155,17 @@ struct DFC {
     __host__ __device__ constexpr DFC(double v) : h(static_cast<float>(v)), l(static_cast<float>(v - static_cast<double>(static_cast<float>(v)))) {}
 };
 
-// Double-float sine of k z + phi, absolute error ~1e-12 on the kick's range (a per-kick force
-// error far below what moves a particle's phase measurably in 1e6 turns).
-// The phase is formed in quarter turns, where its reduction is a subtraction of an integer: the
-// head product k.kh z.h less the nearest integer q is exact, and the product's error and the
-// cross terms (k in 72 bits) follow as one float, 2^-47 of the phase; r = pi/2 times that pair.
-// Then on |r| <= pi/4 one polynomial chosen per lane by the quadrant parity,
-// sin r = r + r^3 S(r^2), cos r = 1 - r^2/2 + r^4 C(r^2), with the coefficients of the FP64
-// sine (sin_f64.cuh): the two leading Horner steps in double-float, the four trailing terms
-// (|t^2 S_2| <= 8e-5, |t^2 C_2| <= 1e-5) in FP32: they set the accuracy (1.7e-13 rms).
-// Every double-float addition after the reduction adds a smaller term to a larger one
-// (Horner constant vs product, r vs r^3 S, 1 - t/2 vs r^4 C), so it uses Fast2Sum on the
-// heads, and neither products nor these sums are renormalised before the next operation (the
-// result is not either).  73 operations, where the radian form (FP64 or double-float phase,
-// Cody-Waite reduction, renormalised pairs) took 135.
-// ok is cleared at 6366 quarter turns (1e4 radians) and more, for Inf and NaN.
-template <bool ZS>
-__device__ __forceinline__ DF2 sin_quarter_df(const QuarterPhase& k, float ph, float pl, DF2 z, bool& ok)
+// sin(q pi/2 + r) for a pair |r| <= pi/4 (a hair more) and the low bits qi of q, absolute error ~1e-12
+// (a per-kick force error far below what moves a particle's phase measurably in 1e6 turns): one
+// polynomial chosen per lane by the quadrant parity, sin r = r + r^3 S(r^2), cos r = 1 - r^2/2 +
+// r^4 C(r^2), with the coefficients of the FP64 sine (sin_f64.cuh): the two leading Horner steps in
+// double-float, the four trailing terms (|t^2 S_2| <= 8e-5, |t^2 C_2| <= 1e-5) in FP32: they set the
+// accuracy (1.7e-13 rms).
+// Every double-float addition adds a smaller term to a larger one (Horner constant vs product, r vs
+// r^3 S, 1 - t/2 vs r^4 C), so it uses Fast2Sum on the heads, and neither products nor these sums are
+// renormalised before the next operation (the result is not either).
+__device__ __forceinline__ DF2 sin_pair_poly(DF2 r, int qi)
 {
-    float p = __fmul_rn(z.h, k.kh);
-    float c = __fmaf_rn(z.h, k.kh, -p);
-    c = __fmaf_rn(z.h, k.kl, c);
-    c = __fmaf_rn(z.h, k.km, c);
-    c = __fmaf_rn(z.l, k.kh, c);
-    if (!ZS) {
-        const DF2 s = df_two_sum(p, ph);
-        p = s.h;
-        c = __fadd_rn(__fadd_rn(c, pl), s.l);
-    }
-    ok = fabsf(p) < 6366.0f;
-    const float magic = 12582912.0f;
-    const float t0 = __fadd_rn(p, magic);
-    const int qi = __float_as_int(t0);
-    const float f = __fsub_rn(p, __fsub_rn(t0, magic));
-    // r = (f + c) pi/2, pi/2 = 1.57079637 - 4.37113883e-8 - 1.71512451e-15
-    const float rp = __fmul_rn(f, 1.5707963705062866f);
-    float re = __fmaf_rn(f, 1.5707963705062866f, -rp);
-    re = __fmaf_rn(f, -1.7151245100058819e-15f, re);
-    re = __fmaf_rn(f, -4.371138828673793e-08f, re);
-    const DF2 r = df_fast_two_sum(rp, __fmaf_rn(c, 1.5707963705062866f, re));
     DF2 t;
     t.h = __fmul_rn(r.h, r.h);
     t.l = __fmaf_rn(__fadd_rn(r.h, r.h), r.l, __fmaf_rn(r.h, r.h, -t.h));
@@ -214,8 +190,66 @@ __device__ __forceinline__ DF2 sin_quarter_df(const QuarterPhase& k, float ph, f
     return df_xor_sign(res, static_cast<unsigned>(qi & 2) << 30);      // quadrants 2, 3: -res
 }
 
-// sin(k z + phi) where sin_quarter_df does not cover it, in FP64.
-static __device__ __noinline__ DF2 sin_quarter_rest(double k, double phi, DF2 z)
+// The two forms of the phase k z + phi and its reduction.  ZS: phi == 0.
+//
+// PHTL_F32CD, in quarter turns, where the reduction is a subtraction of an integer: the head product
+// k.kh z.h less the nearest integer q is exact, and the product's error and the cross terms (k in 72
+// bits) follow as one float, 2^-47 of the phase; r = pi/2 times that pair.  73 operations with the
+// polynomial, where a phase in radians and renormalised pairs took 135.  ok is cleared at 1e4 radians and
+// more, for Inf and NaN.
+template <bool ZS>
+__device__ __forceinline__ DF2 sin_quarter_df(const QuarterPhase& k, float ph, float pl, DF2 z, bool& ok)
+{
+    float p = __fmul_rn(z.h, k.kh);
+    float c = __fmaf_rn(z.h, k.kh, -p);
+    c = __fmaf_rn(z.h, k.kl, c);
+    c = __fmaf_rn(z.h, k.km, c);
+    c = __fmaf_rn(z.l, k.kh, c);
+    if (!ZS) {
+        const DF2 s = df_two_sum(p, ph);
+        p = s.h;
+        c = __fadd_rn(__fadd_rn(c, pl), s.l);
+    }
+    ok = fabsf(p) < 6366.0f;  // quarter turns
+    const float magic = 12582912.0f;
+    const float t0 = __fadd_rn(p, magic);
+    const int qi = __float_as_int(t0);
+    const float f = __fsub_rn(p, __fsub_rn(t0, magic));
+    // r = (f + c) pi/2, pi/2 = 1.57079637 - 4.37113883e-8 - 1.71512451e-15
+    const float rp = __fmul_rn(f, 1.5707963705062866f);
+    float re = __fmaf_rn(f, 1.5707963705062866f, -rp);
+    re = __fmaf_rn(f, -1.7151245100058819e-15f, re);
+    re = __fmaf_rn(f, -4.371138828673793e-08f, re);
+    const DF2 r = df_fast_two_sum(rp, __fmaf_rn(c, 1.5707963705062866f, re));
+    return sin_pair_poly(r, qi);
+}
+
+// PHTL_F32C, in radians: formed in FP64 from hi and comp (two FMAs of registers) and split to 2^-48, less
+// q pi/2 (Cody-Waite, pi/2 = P1 + P2 + P3): q P1 is formed exactly, x.h - q P1 as a TwoSum pair, and
+// the small remainder in FP32.  At small phases, where nothing is subtracted, 1.6 times closer than the
+// quarter turns (6.8e-18 rms against 1.1e-17 for a bunch of 1 mm).  ok: see split_phase.
+// An FP64 FMA holds a warp's share of the pipe for 64 clocks, so eight of them (four particles) are what
+// a small bunch waits for: 1000 particles x 200 turns, leap-frog, 178 us against PHTL_F32CD's 82; 4e6
+// particles 1.32 of PHTL_F32CD's time.
+template <bool ZS>
+__device__ __forceinline__ DF2 sin_fp64_phase(double k, double phi, DF2 z, bool& ok)
+{
+    const double kc = __fma_rn(k, widen_float_phase(z.l), ZS ? 0.0 : phi);
+    const DF2 x = split_phase(__fma_rn(k, widen_float_phase(z.h), kc), ok);
+    const float magic = 12582912.0f;
+    const float t0 = __fmaf_rn(x.h, 0.6366197466850281f, magic);
+    const float q = __fsub_rn(t0, magic);
+    const float p1 = __fmul_rn(q, 1.5707963705062866f);
+    const float e1 = __fmaf_rn(q, 1.5707963705062866f, -p1);
+    const DF2 hd = df_two_sum(x.h, -p1);  // exact as a pair
+    float rest = __fadd_rn(__fsub_rn(x.l, e1), hd.l);
+    rest = __fmaf_rn(-q, -4.371138828673793e-08f, rest);
+    rest = __fmaf_rn(-q, -1.7151245100058819e-15f, rest);
+    return sin_pair_poly(df_fast_two_sum(hd.h, rest), __float_as_int(t0));
+}
+
+// sin(k z + phi) where neither covers it, in FP64.
+static __device__ __noinline__ DF2 sin_df_rest(double k, double phi, DF2 z)
 {
     return split_bits(sin_f64(fma(k, widen_bits(z.h) + widen_bits(z.l), phi)));
 }
@@ -226,7 +260,7 @@ __device__ __forceinline__ DF2 sin_df(DF2 x)
     constexpr QuarterPhase one{0.636619746685028076f, 2.5682552973194106e-08f, 2.93709547963155499e-16f, 0.0f, 0.0f};
     bool ok;
     const DF2 s = sin_quarter_df<true>(one, 0.0f, 0.0f, x, ok);
-    return ok ? s : sin_quarter_rest(1.0, 0.0, x);
+    return ok ? s : sin_df_rest(1.0, 0.0, x);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -264,23 +298,27 @@ __device__ __forceinline__ float sin_sfu(float x)
 
 // ---------------------------------------------------------------------------------------
 // Force of one RF system per unit weight of the thread's particles, sin(phi + k z) - sin(phi)
-// (ZS: phi == 0, no subtraction), in double-float: q, (ph, pl): the phase in quarter turns, k64
-// and phi64 for particles the quarter-turn form does not cover.  All sines first, so that the
-// particles' chains interleave.
-template <bool ZS, int N>
+// (ZS: phi == 0, no subtraction), in double-float: q, (ph, pl): the phase in quarter turns
+// (PHTL_F32CD), k64 and phi64: in FP64 (PHTL_F32C, and particles the forms do not cover).  All sines
+// first, so that the particles' chains interleave.
+template <int DT, bool ZS, int N>
 __device__ __forceinline__ void force_df(const QuarterPhase& q, float ph, float pl, double k64, double phi64,
                                          DF2 minus_sin_phi, const DF2 (&z)[N], DF2 (&f)[N])
 {
     bool ok[N], all = true;
 #pragma unroll
     for (int p = 0; p < N; ++p) {
-        f[p] = sin_quarter_df<ZS>(q, ph, pl, z[p], ok[p]);
+        f[p] = DT == PHTL_F32C ? sin_fp64_phase<ZS>(k64, phi64, z[p], ok[p])
+                               : sin_quarter_df<ZS>(q, ph, pl, z[p], ok[p]);
         all = all && ok[p];
     }
     if (!all) {
 #pragma unroll
         for (int p = 0; p < N; ++p)
-            if (!ok[p]) f[p] = sin_quarter_rest(k64, ZS ? 0.0 : phi64, z[p]);
+            if (!ok[p])  // split_phase leaves out z = 0 (also the lanes beyond a bunch's end): no call for it
+                f[p] = DT == PHTL_F32C && z[p].h == 0.0f && (ZS || phi64 == 0.0)
+                           ? z[p]
+                           : sin_df_rest(k64, ZS ? 0.0 : phi64, z[p]);
     }
     if (!ZS) {
 #pragma unroll
@@ -297,11 +335,24 @@ __device__ __forceinline__ bool sine_only(const MapConsts& c)
     return DT == PHTL_F32CS ? c.phis_zero != 0 : c.rf_mode == kRfZero || c.rf_mode == kRfPlain;
 }
 
+// k of both RF systems for the FP64 phases, in registers in the persistent kernels (an FP64 FMA with an operand
+// in the constant bank takes the pipe 0.59 clocks per lane and SM, one of registers 0.50).
+struct Waves {
+    double k, k2;
+};
+
+template <int DT>
+__device__ __forceinline__ Waves waves(const MapConsts& c)
+{
+    if (DT != PHTL_F32C) return Waves{c.k, c.k2};
+    return Waves{in_register(c.k), in_register(c.k2)};
+}
+
 // kick: delta += kw * (sin(phi) - sin(phi_s)), kw = kh + kl (the FP64 weight as a pair);
 // ZS: phi_s == 0, no subtraction
 template <int DT, bool ZS>
 __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], float kh, float kl,
-                                     const MapConsts& c)
+                                     const MapConsts& c, const Waves& wv)
 {
     if (DT == PHTL_F32CS) {
 #pragma unroll
@@ -324,7 +375,7 @@ __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], float kh, flo
 #pragma unroll
         for (int p = 0; p < P; ++p) f[p] = df_mul(DF2{c.lin_hi, c.lin_lo}, zz[p]);
     } else {
-        force_df<ZS>(c.kq, c.kq.ph, c.kq.pl, c.k, c.phis, DF2{-c.sinphis_hi, -c.sinphis_lo}, zz, f);
+        force_df<DT, ZS>(c.kq, c.kq.ph, c.kq.pl, wv.k, c.phis, DF2{-c.sinphis_hi, -c.sinphis_lo}, zz, f);
     }
 #pragma unroll
     for (int p = 0; p < P; ++p) acc2(d[p], df_mul_raw(DF2{kh, kl}, f[p]));
@@ -349,24 +400,24 @@ __device__ __forceinline__ void drift(DF (&z)[P], const DF (&d)[P], float dh, fl
 // hi + lo (the single-bunch kernel passes the MapConsts copies, the batched kernel the
 // job table's).
 template <int SCHEME, int DT, bool ZS>
-__device__ __forceinline__ void long_turn(DF (&z)[P], DF (&d)[P], const MapConsts& c,
+__device__ __forceinline__ void long_turn(DF (&z)[P], DF (&d)[P], const MapConsts& c, const Waves& wv,
                                           const float* dh, const float* dl, const float* kh,
                                           const float* kl)
 {
     if (SCHEME == PHTL_EULER_CROMER) {
-        kick<DT, ZS>(z, d, kh[0], kl[0], c);
+        kick<DT, ZS>(z, d, kh[0], kl[0], c, wv);
         drift<DT>(z, d, dh[0], dl[0]);
     } else if (SCHEME == PHTL_LEAPFROG) {
         drift<DT>(z, d, dh[0], dl[0]);
-        kick<DT, ZS>(z, d, kh[0], kl[0], c);
+        kick<DT, ZS>(z, d, kh[0], kl[0], c, wv);
         drift<DT>(z, d, dh[1], dl[1]);
     } else {
         drift<DT>(z, d, dh[0], dl[0]);
-        kick<DT, ZS>(z, d, kh[0], kl[0], c);
+        kick<DT, ZS>(z, d, kh[0], kl[0], c, wv);
         drift<DT>(z, d, dh[1], dl[1]);
-        kick<DT, ZS>(z, d, kh[1], kl[1], c);
+        kick<DT, ZS>(z, d, kh[1], kl[1], c, wv);
         drift<DT>(z, d, dh[2], dl[2]);
-        kick<DT, ZS>(z, d, kh[2], kl[2], c);
+        kick<DT, ZS>(z, d, kh[2], kl[2], c, wv);
         drift<DT>(z, d, dh[3], dl[3]);
     }
 }
@@ -398,16 +449,16 @@ __device__ __forceinline__ void drift_nl(DF (&z)[P], const DF (&d)[P], float dh,
 
 // Force of the second RF system per unit weight, sin(phi2 + k2 z) - sin(phi2) (rf_linear:
 // cos(phi2) k2 z), as a pair.
-template <int N>
-__device__ __forceinline__ void force2_df(const MapConsts& c, const DF2 (&z)[N], DF2 (&f)[N])
+template <int DT, int N>
+__device__ __forceinline__ void force2_df(const MapConsts& c, const Waves& wv, const DF2 (&z)[N], DF2 (&f)[N])
 {
     if (c.linear) {
 #pragma unroll
         for (int p = 0; p < N; ++p) f[p] = df_mul(DF2{c.lin2_hi, c.lin2_lo}, z[p]);
     } else if (c.phi2_zero) {
-        force_df<true>(c.kq2, 0.0f, 0.0f, c.k2, 0.0, DF2{0.0f, 0.0f}, z, f);
+        force_df<DT, true>(c.kq2, 0.0f, 0.0f, wv.k2, 0.0, DF2{0.0f, 0.0f}, z, f);
     } else {
-        force_df<false>(c.kq2, c.kq2.ph, c.kq2.pl, c.k2, c.phi2, DF2{-c.sinphi2_hi, -c.sinphi2_lo}, z, f);
+        force_df<DT, false>(c.kq2, c.kq2.ph, c.kq2.pl, wv.k2, c.phi2, DF2{-c.sinphi2_hi, -c.sinphi2_lo}, z, f);
     }
 }
 
@@ -420,13 +471,13 @@ __device__ __forceinline__ float force2_f(const MapConsts& c, DF2 z)
 }
 
 // Force of the main RF system per unit weight at a pair z (the bracket of kick()).
-template <bool ZS>
-__device__ __forceinline__ DF2 force1_df(const MapConsts& c, DF2 z)
+template <int DT, bool ZS>
+__device__ __forceinline__ DF2 force1_df(const MapConsts& c, const Waves& wv, DF2 z)
 {
     if (c.linear) return df_mul(DF2{c.lin_hi, c.lin_lo}, z);
     const DF2 zz[1] = {z};
     DF2 f[1];
-    force_df<ZS>(c.kq, c.kq.ph, c.kq.pl, c.k, c.phis, DF2{-c.sinphis_hi, -c.sinphis_lo}, zz, f);
+    force_df<DT, ZS>(c.kq, c.kq.ph, c.kq.pl, wv.k, c.phis, DF2{-c.sinphis_hi, -c.sinphis_lo}, zz, f);
     return f[0];
 }
 
@@ -442,9 +493,9 @@ __device__ __forceinline__ float force1_f(const MapConsts& c, DF2 z)
 // (k2h + k2l: this stage's w_j A2), each increment added on its own.
 template <int DT, bool ZS>
 __device__ __forceinline__ void kick_gen(const DF (&z)[P], DF (&d)[P], float kh, float kl, float k2h,
-                                         float k2l, const MapConsts& c, bool dual)
+                                         float k2l, const MapConsts& c, const Waves& wv, bool dual)
 {
-    kick<DT, ZS>(z, d, kh, kl, c);
+    kick<DT, ZS>(z, d, kh, kl, c, wv);
     if (!dual) return;
     if (DT == PHTL_F32CS) {
 #pragma unroll
@@ -457,7 +508,7 @@ __device__ __forceinline__ void kick_gen(const DF (&z)[P], DF (&d)[P], float kh,
     DF2 f[P], zz[P];
 #pragma unroll
     for (int p = 0; p < P; ++p) zz[p] = as2(z[p]);
-    force2_df(c, zz, f);
+    force2_df<DT>(c, wv, zz, f);
 #pragma unroll
     for (int p = 0; p < P; ++p) acc2(d[p], df_mul_raw(DF2{k2h, k2l}, f[p]));
 }
@@ -465,7 +516,7 @@ __device__ __forceinline__ void kick_gen(const DF (&z)[P], DF (&d)[P], float kh,
 // Right-hand side of the smooth motion per turn as pairs: dz/dn = -(dc + g1 d + g2 d^2) d,
 // dd/dn = kw F1(z) + kw2 F2(z) (dc = eta0 C, g1 = eta1 C, g2 = eta2 C, kw = A, kw2 = A2).
 template <int DT, bool ZS>
-__device__ __forceinline__ void rk4_rhs_df(DF2 z, DF2 d, const MapConsts& c, DF2 dc, DF2 g1, DF2 g2,
+__device__ __forceinline__ void rk4_rhs_df(DF2 z, DF2 d, const MapConsts& c, const Waves& wv, DF2 dc, DF2 g1, DF2 g2,
                                            DF2 kw, DF2 kw2, bool dual, DF2& fz, DF2& fd)
 {
     DF2 e = dc;
@@ -474,11 +525,11 @@ __device__ __forceinline__ void rk4_rhs_df(DF2 z, DF2 d, const MapConsts& c, DF2
         e = df_add(df_mul_raw(e, d), dc);
     }
     fz = neg2(df_mul(e, d));
-    fd = df_mul(kw, force1_df<ZS>(c, z));
+    fd = df_mul(kw, force1_df<DT, ZS>(c, wv, z));
     if (dual) {
         const DF2 zz[1] = {z};
         DF2 f[1];
-        force2_df(c, zz, f);
+        force2_df<DT>(c, wv, zz, f);
         fd = df_add(fd, df_mul_raw(kw2, f[0]));
     }
 }
@@ -490,7 +541,7 @@ __device__ __forceinline__ DF2 df_scale2(DF2 a, float s) { return DF2{s * a.h, s
 // PHTL_F32CS: the stages in FP32 (the state's comp folded into the stage arguments), the
 // weighted sum added with TwoSum.
 template <int DT, bool ZS>
-__device__ __forceinline__ void rk4_turn(DF (&z)[P], DF (&d)[P], const MapConsts& c, float dh,
+__device__ __forceinline__ void rk4_turn(DF (&z)[P], DF (&d)[P], const MapConsts& c, const Waves& wv, float dh,
                                          float dl, float kh, float kl, float k2h, float k2l,
                                          float g1h, float g1l, float g2h, float g2l, bool dual)
 {
@@ -525,7 +576,7 @@ __device__ __forceinline__ void rk4_turn(DF (&z)[P], DF (&d)[P], const MapConsts
             // instruction cache
 #pragma unroll 1
             for (int st = 0;; ++st) {
-                rk4_rhs_df<DT, ZS>(a, b, c, dc, g1, g2, kw, kw2, dual, kz, kd);
+                rk4_rhs_df<DT, ZS>(a, b, c, wv, dc, g1, g2, kw, kw2, dual, kz, kd);
                 if (st == 3) break;
                 const float cs = st == 0 ? 1.0f : 2.0f, step = st == 2 ? 1.0f : 0.5f;
                 sz = df_add(sz, df_scale2(kz, cs));
@@ -545,29 +596,29 @@ __device__ __forceinline__ void rk4_turn(DF (&z)[P], DF (&d)[P], const MapConsts
 // w_i eta2 C), second RF system (k2h, k2l: stage j's w_j A2) and, for RK4, the classic
 // Runge-Kutta step.
 template <int SCHEME, int DT, bool ZS>
-__device__ __forceinline__ void long_turn_nl(DF (&z)[P], DF (&d)[P], const MapConsts& c,
+__device__ __forceinline__ void long_turn_nl(DF (&z)[P], DF (&d)[P], const MapConsts& c, const Waves& wv,
                                              const float* dh, const float* dl, const float* kh,
                                              const float* kl, const float* k2h, const float* k2l,
                                              const float (&g1h)[4], const float (&g1l)[4],
                                              const float (&g2h)[4], const float (&g2l)[4], bool dual)
 {
     if (SCHEME == PHTL_RK4) {
-        rk4_turn<DT, ZS>(z, d, c, dh[0], dl[0], kh[0], kl[0], k2h[0], k2l[0], g1h[0], g1l[0],
+        rk4_turn<DT, ZS>(z, d, c, wv, dh[0], dl[0], kh[0], kl[0], k2h[0], k2l[0], g1h[0], g1l[0],
                          g2h[0], g2l[0], dual);
     } else if (SCHEME == PHTL_EULER_CROMER) {
-        kick_gen<DT, ZS>(z, d, kh[0], kl[0], k2h[0], k2l[0], c, dual);
+        kick_gen<DT, ZS>(z, d, kh[0], kl[0], k2h[0], k2l[0], c, wv, dual);
         drift_nl<DT>(z, d, dh[0], dl[0], g1h[0], g1l[0], g2h[0], g2l[0]);
     } else if (SCHEME == PHTL_LEAPFROG) {
         drift_nl<DT>(z, d, dh[0], dl[0], g1h[0], g1l[0], g2h[0], g2l[0]);
-        kick_gen<DT, ZS>(z, d, kh[0], kl[0], k2h[0], k2l[0], c, dual);
+        kick_gen<DT, ZS>(z, d, kh[0], kl[0], k2h[0], k2l[0], c, wv, dual);
         drift_nl<DT>(z, d, dh[1], dl[1], g1h[1], g1l[1], g2h[1], g2l[1]);
     } else {
         drift_nl<DT>(z, d, dh[0], dl[0], g1h[0], g1l[0], g2h[0], g2l[0]);
-        kick_gen<DT, ZS>(z, d, kh[0], kl[0], k2h[0], k2l[0], c, dual);
+        kick_gen<DT, ZS>(z, d, kh[0], kl[0], k2h[0], k2l[0], c, wv, dual);
         drift_nl<DT>(z, d, dh[1], dl[1], g1h[1], g1l[1], g2h[1], g2l[1]);
-        kick_gen<DT, ZS>(z, d, kh[1], kl[1], k2h[1], k2l[1], c, dual);
+        kick_gen<DT, ZS>(z, d, kh[1], kl[1], k2h[1], k2l[1], c, wv, dual);
         drift_nl<DT>(z, d, dh[2], dl[2], g1h[2], g1l[2], g2h[2], g2l[2]);
-        kick_gen<DT, ZS>(z, d, kh[2], kl[2], k2h[2], k2l[2], c, dual);
+        kick_gen<DT, ZS>(z, d, kh[2], kl[2], k2h[2], k2l[2], c, wv, dual);
         drift_nl<DT>(z, d, dh[3], dl[3], g1h[3], g1l[3], g2h[3], g2l[3]);
     }
 }

@@ -49,16 +49,6 @@ constexpr int min_blocks_256()
     return SCHEME == PHTL_RUTH4 ? PHTL_F64_MIN_BLOCKS_256_RUTH4 : PHTL_F64_MIN_BLOCKS_256;
 }
 
-// A launch constant held in a register.  An FP64 FMA whose operands all lie in registers takes
-// the pipe 0.50 clocks per lane and SM, one with an operand in the constant bank 0.59 (also
-// DADD and DMUL; measured), so the persistent kernels move the weights of their turn loop to
-// registers.  Through a shuffle, which the compiler does not fold back into the operand.
-__device__ __forceinline__ double in_register(double v)
-{
-    return __hiloint2double(__shfl_sync(kFullMask, __double2hiint(v), 0),
-                            __shfl_sync(kFullMask, __double2loint(v), 0));
-}
-
 // Weights of the linear map's turn loop (drifts, kicks, shears of the two planes).
 struct TurnWeights {
     double dc[4], kw[3], shx[2], shy[2];

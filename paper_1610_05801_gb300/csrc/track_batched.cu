@@ -12,8 +12,10 @@ const void* select_batched(const MapConsts& c, int dtype, bool mon)
 {
     if (c.general) return general_kernel_batched(c, dtype);
     if (dtype == PHTL_F64) return mon ? batched_f64<true, false>(c.rf_mode) : batched_f64<false, false>(c.rf_mode);
-    // PHTL_F32C and PHTL_F32CD are the same arithmetic: one instantiation
-    if (dtype == PHTL_F32C || dtype == PHTL_F32CD)
+    if (dtype == PHTL_F32C)
+        return mon ? reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32C, true, false>)
+                   : reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32C, false, false>);
+    if (dtype == PHTL_F32CD)
         return mon ? reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32CD, true, false>)
                    : reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32CD, false, false>);
     if (dtype == PHTL_F32CS)

@@ -27,8 +27,8 @@ const void* sel_tm(bool trans, bool mon)
 template <int S>
 const void* sel_d(int dtype, bool trans, bool mon)
 {
-    // PHTL_F32C and PHTL_F32CD are the same arithmetic: one instantiation
-    if (dtype == PHTL_F32C || dtype == PHTL_F32CD) return sel_tm<S, PHTL_F32CD>(trans, mon);
+    if (dtype == PHTL_F32C) return sel_tm<S, PHTL_F32C>(trans, mon);
+    if (dtype == PHTL_F32CD) return sel_tm<S, PHTL_F32CD>(trans, mon);
     if (dtype == PHTL_F32CS) return sel_tm<S, PHTL_F32CS>(trans, mon);
     return nullptr;
 }

@@ -19,7 +19,9 @@ const void* general_kernel_single(int scheme, int dtype, bool dual, int mode)
 #define PHTL_GEN(S)                                                                                     \
     if (scheme == S) {                                                                                  \
         if (dtype == PHTL_F64) return kf64::track_kernel<S, true, true, true>(mode);                    \
-        if (dtype == PHTL_F32C || dtype == PHTL_F32CD)                                                  \
+        if (dtype == PHTL_F32C)                                                                         \
+            return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32C, true, true, true>);  \
+        if (dtype == PHTL_F32CD)                                                                        \
             return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32CD, true, true, true>); \
         if (dtype == PHTL_F32CS)                                                                        \
             return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32CS, true, true, true>); \

@@ -12,6 +12,7 @@ namespace phtl {
 
 const void* general_kernel_batched(const MapConsts& c, int dtype)
 {
+    if (dtype == PHTL_F32C) return reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32C, true, true>);
     if (dtype != PHTL_F64) return general_kernel_batched_f32(dtype);
     return c.dual_rf ? batched_f64<true, true, true>(c.rf_mode) : batched_f64<true, true>(c.rf_mode);
 }

@@ -9,7 +9,7 @@ namespace phtl {
 
 const void* general_kernel_batched_f32(int dtype)
 {
-    if (dtype == PHTL_F32C || dtype == PHTL_F32CD) return reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32CD, true, true>);
+    if (dtype == PHTL_F32CD) return reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32CD, true, true>);
     if (dtype == PHTL_F32CS) return reinterpret_cast<const void*>(&k_batched_f32c<PHTL_F32CS, true, true>);
     return nullptr;
 }

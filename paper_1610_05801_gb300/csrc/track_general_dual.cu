@@ -5,16 +5,30 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "kernels_f32c.cuh"
 #include "kernels_f64.cuh"
 
 namespace phtl {
+namespace {
+
+template <int S>
+const void* dual_s(int dtype, int mode)
+{
+    if (dtype == PHTL_F64) return kf64::track_kernel<S, true, true, true, true>(mode);
+    if (dtype == PHTL_F32C)
+        return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32C, true, true, true, true>);
+    return nullptr;
+}
+
+}  // namespace
+
 const void* general_kernel_single_dual(int scheme, int dtype, int mode)
 {
-    if (dtype != PHTL_F64) return general_kernel_single_dual_f32(scheme, dtype);
-    if (scheme == PHTL_EULER_CROMER) return kf64::track_kernel<PHTL_EULER_CROMER, true, true, true, true>(mode);
-    if (scheme == PHTL_LEAPFROG) return kf64::track_kernel<PHTL_LEAPFROG, true, true, true, true>(mode);
-    if (scheme == PHTL_RUTH4) return kf64::track_kernel<PHTL_RUTH4, true, true, true, true>(mode);
-    if (scheme == PHTL_RK4) return kf64::track_kernel<PHTL_RK4, true, true, true, true>(mode);
+    if (dtype == PHTL_F32CD || dtype == PHTL_F32CS) return general_kernel_single_dual_f32(scheme, dtype);
+    if (scheme == PHTL_EULER_CROMER) return dual_s<PHTL_EULER_CROMER>(dtype, mode);
+    if (scheme == PHTL_LEAPFROG) return dual_s<PHTL_LEAPFROG>(dtype, mode);
+    if (scheme == PHTL_RUTH4) return dual_s<PHTL_RUTH4>(dtype, mode);
+    if (scheme == PHTL_RK4) return dual_s<PHTL_RK4>(dtype, mode);
     return nullptr;
 }
 

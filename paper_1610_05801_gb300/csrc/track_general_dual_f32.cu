@@ -11,7 +11,7 @@ namespace {
 template <int S>
 const void* dual_s(int dtype)
 {
-    if (dtype == PHTL_F32C || dtype == PHTL_F32CD)
+    if (dtype == PHTL_F32CD)
         return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32CD, true, true, true, true>);
     if (dtype == PHTL_F32CS)
         return reinterpret_cast<const void*>(&kf32::k_track_f32c<S, PHTL_F32CS, true, true, true, true>);

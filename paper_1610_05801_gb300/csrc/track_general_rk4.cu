@@ -12,7 +12,9 @@ namespace phtl {
 const void* general_kernel_single_rk4(int dtype, int mode)
 {
     if (dtype == PHTL_F64) return kf64::track_kernel<PHTL_RK4, true, true, true>(mode);
-    if (dtype == PHTL_F32C || dtype == PHTL_F32CD)
+    if (dtype == PHTL_F32C)
+        return reinterpret_cast<const void*>(&kf32::k_track_f32c<PHTL_RK4, PHTL_F32C, true, true, true>);
+    if (dtype == PHTL_F32CD)
         return reinterpret_cast<const void*>(&kf32::k_track_f32c<PHTL_RK4, PHTL_F32CD, true, true, true>);
     if (dtype == PHTL_F32CS)
         return reinterpret_cast<const void*>(&kf32::k_track_f32c<PHTL_RK4, PHTL_F32CS, true, true, true>);

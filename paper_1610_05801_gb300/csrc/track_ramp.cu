@@ -217,8 +217,8 @@ using namespace f32c;
 
 struct Turn {
     DF2 etaC, A, phis, sinphis, lin, r;
-    DF2 phq;        // phi_s,n in quarter turns
-    double phis64;  // for the particles that form does not cover
+    DF2 phq;        // phi_s,n in quarter turns (PHTL_F32CD)
+    double phis64;  // in FP64 (PHTL_F32C, and particles the forms do not cover)
 };
 
 template <int DT>
@@ -237,7 +237,7 @@ __device__ __forceinline__ Turn load_turn(const RampTurn* __restrict__ p)
 }
 
 // kick of weight w (a compile-time constant of the scheme): delta += w A_n (sin(phi_s,n +
-// k z) - sin(phi_s,n)), the phase in double-float quarter turns (PHTL_F32C, PHTL_F32CD) or
+// k z) - sin(phi_s,n)), the phase in FP64 (PHTL_F32C), in double-float quarter turns (PHTL_F32CD) or
 // rounded to FP32 for the SFU sine (PHTL_F32CS)
 template <int DT>
 __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], double w, const Turn& T,
@@ -266,8 +266,7 @@ __device__ __forceinline__ void kick(const DF (&z)[P], DF (&d)[P], double w, con
 #pragma unroll
         for (int p = 0; p < P; ++p) f[p] = df_mul(T.lin, zz[p]);
     } else {
-        force_df<false>(c.kq, T.phq.h, T.phq.l, c.k, T.phis64,
-                        neg2(T.sinphis), zz, f);
+        force_df<DT, false>(c.kq, T.phq.h, T.phq.l, c.k, T.phis64, neg2(T.sinphis), zz, f);
     }
 #pragma unroll
     for (int p = 0; p < P; ++p) acc2(d[p], df_mul_raw(kw, f[p]));
@@ -386,8 +385,8 @@ __device__ __forceinline__ void ramp_f32c_body(const LaunchDesc& L, const MapCon
     }
 }
 
-// The compiler's register choice: 3 resident 256-thread blocks per SM (80 registers) took 8 %
-// longer for FP32C / FP32CD (1e6 particles x 300 turns, leap-frog, both planes, moments every turn)
+// FP32CD: the compiler's register choice (3 resident 256-thread blocks per SM, 80 registers, took 8 %
+// longer: 1e6 particles x 300 turns, leap-frog, both planes, moments every turn); FP32C: 2 blocks
 template <int S, int DT>
 __global__ void PHTL_F32C_RAMP_BOUNDS(S, DT)
     k_ramp_f32c(LaunchDesc L, MapConsts c, MonitorArgs m, const RampTurn* __restrict__ prog, int64_t turn0)
@@ -403,8 +402,8 @@ const void* ramp_kernel_s(int dtype, bool linear)
     if (dtype == PHTL_F64)
         return linear ? reinterpret_cast<const void*>(&rf64::k_ramp_f64<S, true>)
                       : reinterpret_cast<const void*>(&rf64::k_ramp_f64<S, false>);
-    // PHTL_F32C and PHTL_F32CD are the same arithmetic: one instantiation
-    if (dtype == PHTL_F32C || dtype == PHTL_F32CD) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32CD>);
+    if (dtype == PHTL_F32C) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32C>);
+    if (dtype == PHTL_F32CD) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32CD>);
     if (dtype == PHTL_F32CS) return reinterpret_cast<const void*>(&rf32::k_ramp_f32c<S, PHTL_F32CS>);
     return nullptr;
 }
