@@ -176,16 +176,6 @@ __device__ __forceinline__ DF2 df_mul(DF2 a, DF2 b)
     return df_fast_two_sum(p, e);
 }
 
-__device__ __forceinline__ double df_to_double(DF2 a)
-{
-    return static_cast<double>(a.h) + static_cast<double>(a.l);
-}
-
-__device__ __forceinline__ DF2 df_shfl_xor(DF2 a, int o)
-{
-    return DF2{__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)};
-}
-
 // A launch constant held in a register.  An FP64 FMA whose operands all lie in registers takes
 // the pipe 0.50 clocks per lane and SM, one with an operand in the constant bank 0.59 (also
 // DADD and DMUL; measured), so the persistent kernels move the weights of their turn loop to

@@ -490,9 +490,11 @@ __device__ __forceinline__ void transverse_gen(double (&x)[N], double (&xp)[N], 
 // A coordinate's values are brought to the warp's common exponent E (the largest biased
 // exponent among its lanes) as 61-bit integers X, a = X 2^(E + kMomentShift - 1086): no bit of a
 // value within 2^-8 of the largest is lost.  The thread adds X, X^2 and X Y over its particles,
-// the warp the threads' sums as 64-bit integers, and each total is converted to FP64 once: sums
-// keep 2^-55 of the warp's largest term.  The squares are products of the magnitudes rounded
-// down, so a single particle's variance does not come out positive.
+// the warp the threads' sums as 64-bit integers, and each total is converted to FP64 once.  A
+// thread's sum is cut below 2^-56 of the warp's largest magnitude, one of products below 2^-55 of the
+// product of its coordinates' largest (up to 2.5 such units), so a warp's totals are within 2^-50.9
+// and 2^-48.6 of those.  The squares are products of the magnitudes rounded down, so a single
+// particle's variance does not come out positive.
 //
 // The double-float sums before these took ~590 instructions per particle and record with both
 // planes (bit splits, TwoSum and Fast2Sum in every addition); these take ~390.

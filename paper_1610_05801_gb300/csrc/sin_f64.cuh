@@ -334,7 +334,8 @@ __device__ __forceinline__ void chroma_fixed(const ChromaPlane& w, double d, dou
     using namespace detail;
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(d));
     const uint32_t e = (hi >> 20) & 0x7ffu;
-    // |xi d| = hi64(M K) 2^(e + xi.e - 1021) in 2^-64 turns; a turn or more is not covered
+    // |xi d| = hi64(M K) 2^(e + xi.e - 1021) in 2^-64 turns; every |xi d| below half a turn is covered, none
+    // from a turn on
     const uint32_t n = static_cast<uint32_t>(1022 - w.xi.e - static_cast<int>(e));
     const uint64_t A = shr_sat(mulhi_trunc(mantissa64(d), w.xi.K), n) << 1;
     ok = n <= 2047u && (e != 0u || (hi << 1 | static_cast<uint32_t>(__double2loint(d))) == 0u);

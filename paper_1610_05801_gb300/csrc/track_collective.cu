@@ -57,7 +57,7 @@ __device__ __forceinline__ int slice_of(double z, double z_lo, double inv_dz, in
 // GEN: the widened map's code (slippage expansion, chromaticity, second RF system, RK4);
 // otherwise the linear map's, which a ring without those terms gives bitwise the same result
 // with fewer FP64 operations (a drift is one FMA instead of three).
-// Shared memory: ns uint32 histogram bins, then the monitor's 2 * warps * 16 DF2.
+// Shared memory: ns uint32 histogram bins, then the monitor's 2 * warps * 16 doubles.
 // MODE: RfMode; DUAL (GEN only): with the second RF system.
 template <int S, bool GEN, int MODE, bool DUAL>
 __global__ void __launch_bounds__(256, 3)
