@@ -92,14 +92,30 @@ int phtl_set_wake(phtl_handle* h, const phtl_wake* wk)
 
 namespace {
 
-// Launch shape of the collective kernels for n particles (grid = resident capacity).
-int coll_launch(phtl_handle* h, void* const* c, int64_t n, int integrator, int dtype, LaunchDesc& L)
+// Threads a block where none are set.  Larger blocks share the slice histogram among more particles and
+// leave it to be added up by fewer, smaller ones fill the last round better and wait less for each other
+// in the moment sums.  us per turn at 128 / 256 threads, both planes, 512 slices, FP64, for 1e5, 3e5, 6e5,
+// 1e6 and 2e6 particles:
+//   leap-frog, no moments or every 10 turns   11.8/11.6  18.5/17.0  26.2/25.3  36.6/34.2   62.6/63.3
+//   leap-frog, moments every 3 turns          12.1/12.0  18.9/17.6  26.8/26.5  37.5/36.3   65.3/67.9
+//   leap-frog, moments every turn             12.7/13.3  20.3/19.5  28.5/29.9  40.0/42.9   73.1/81.4
+//   Ruth4, moments every 10 turns             13.2/12.8  20.6/20.7  30.8/31.6  43.0/43.7   77.7/79.6
+//   widened leap-frog, every 10 turns         15.3/15.6  23.8/25.8  37.4/40.0  55.0/55.6  101.7/103.4
+//   double-RF Ruth4, every 10 turns           17.4/18.7  25.9/29.1  40.6/44.0  61.8/62.7  114.7/117.7
+// so 256 for one kick on the linear map with rare moments, 128 otherwise; FP32: 128 (25.8 / 26.7 at 1e6,
+// 44.9 / 49.1 at 2e6).  mon_stride: 0 without moments.
+int coll_block(const MapConsts& mc, int integrator, int dtype, int64_t mon_stride)
 {
-    // 256 threads in FP64 (us per turn at 128 / 256, leap-frog, both planes, 512 slices: 12.5 / 12.1 at 1e5
-    // particles, 19.8 / 17.8 at 3e5, 25.5 / 26.2 at 6e5, 37.4 / 34.7 at 1e6, 63.4 / 64.5 at 2e6), 128 in
-    // FP32 (25.8 / 26.7 at 1e6, 44.9 / 49.1 at 2e6)
-    const int block = h->block > 0 ? h->block : (dtype == PHTL_F64 ? 256 : 128);
+    const bool light = !mc.general && (integrator == PHTL_EULER_CROMER || integrator == PHTL_LEAPFROG);
+    return dtype == PHTL_F64 && light && (mon_stride == 0 || mon_stride >= 3) ? 256 : 128;
+}
+
+// Launch shape of the collective kernels for n particles (grid = resident capacity).
+int coll_launch(phtl_handle* h, void* const* c, int64_t n, int integrator, int dtype, int64_t mon_stride,
+                LaunchDesc& L)
+{
     const MapConsts& mc = h->mc[integrator];
+    const int block = h->block > 0 ? h->block : coll_block(mc, integrator, dtype, mon_stride);
     const int occ = dtype == PHTL_F64 ? occupancy_coll(mc, integrator, block, h->coll.nslices)
                                       : occupancy_coll_f32(integrator, dtype, mc.general != 0, block,
                                                            h->coll.nslices);
@@ -196,7 +212,7 @@ int phtl_collective_kick(phtl_handle* h, void* z, void* dp, int64_t n, int dtype
         LaunchDesc L;
         const MapConsts& mc = h->mc[PHTL_LEAPFROG];
         rc = ensure_slots(h, n);
-        if (rc == PHTL_OK) rc = coll_launch(h, c, n, PHTL_LEAPFROG, dtype, L);
+        if (rc == PHTL_OK) rc = coll_launch(h, c, n, PHTL_LEAPFROG, dtype, 0, L);
         if (rc == PHTL_OK) rc = coll_turn(h, L, mc, cnt, nullptr, -1, false, false, dtype, s);
         if (rc == PHTL_OK) rc = coll_potential(h, cnt, nullptr, s);
         if (rc == PHTL_OK) rc = coll_turn(h, L, mc, nullptr, nullptr, -1, true, false, dtype, s);
@@ -232,7 +248,7 @@ int phtl_track_collective(phtl_handle* h, void* z, void* dp, void* x, void* xp, 
     rc = ensure_slots(h, n);
     if (rc != PHTL_OK) return rc;
     LaunchDesc L;
-    rc = coll_launch(h, c, n, integrator, dtype, L);
+    rc = coll_launch(h, c, n, integrator, dtype, mon ? stride : 0, L);
     if (rc != PHTL_OK) return rc;
     const int ns = h->coll.nslices;
     unsigned* cnt[2] = {h->wake_counts, h->wake_counts + ns};
