@@ -571,8 +571,7 @@ NCU_TRAFFIC_BYTES_PER_PARTICLE = {("f64", "ruth4", True, True): (144.729600e6 + 
 
 
 # FP64 flops per particle-turn of the kernels with the sines in FP64 arithmetic, from the same ncu
-# capture (what the present kernels execute is in EXECUTED_NOW below; this count is reported beside it
-# as the work of that form):
+# capture (what the present kernels execute is in EXECUTED_NOW below and replaces this count in the line):
 # (2 x DFMA + DMUL + DADD thread instructions per cycle) x cycles / particle-turns, i.e.
 # (2 x 225.068198 + 33.760230 + 0.474220) x 22.946400 ms x 2.044726 GHz / (3e6 x 88).
 # Fewer than the algorithmic count: for phi_s = 0 the kernel skips the phase addition and the
@@ -817,41 +816,45 @@ def issue_roofline(kname, key=None, pts=None, sm_mhz=None):
 # profiles/executed_counts_1e6x40.md): FP64 flops (2 DFMA + DMUL + DADD thread instructions) of the FP64
 # kernels, warp-instructions of the FP32 ones; keyed as above.
 EXECUTED_NOW = {
-    ("f64", "ruth4", True, True, "plain"): (2 * 520_000_000 + 40_466_944) / 4e7,
-    ("f64", "ruth4", True, True, "widened"): (2 * 920_012_240 + 2_002_720 + 82_000_000) / 4e7,
-    ("f64", "ruth4", True, True, "double_rf"): (2 * 640_000_000 + 42_000_000) / 4e7,
-    ("f64", "rk4", True, True, "double_rf"): (2 * 1_360_000_010 + 80_500_000) / 4e7,
-    ("f64", "ruth4", True, True, "ramp"): (2 * 520_000_010 + 120_000_002 + 120_000_000) / 4e7,
+    ("f64", "ruth4", True, True, "plain"): (2 * 520_000_000 + 466_944) / 4e7,
+    ("f64", "ruth4", True, True, "widened"): (2 * 920_000_000 + 2_000_000 + 2_000_000) / 4e7,
+    ("f64", "ruth4", True, True, "double_rf"): (2 * 640_000_000 + 2_000_000) / 4e7,
+    ("f64", "rk4", True, True, "double_rf"): (2 * 1_360_000_000 + 500_000) / 4e7,
+    ("f64", "ruth4", True, True, "ramp"): 2 * 760_000_010 / 4e7,
     ("f64", "leapfrog", False, True, "batched"): (2 * 2_402_150_400 + 41_724_852) / 799_999_200,
-    ("f64", "leapfrog", True, True, "collective"): (2 * 27_000_576 + 3_000_000 + 6_562_512) / 3e6,
+    ("f64", "leapfrog", True, True, "collective"): (2 * 27_002_880 + 3_000_000 + 6_656_320) / 3e6,
+    ("f32c", "leapfrog", True, True, False): 351369244 / 4e7,
+    ("f32c", "ruth4", True, True, False): 699995953 / 4e7,
+    ("f32c", "leapfrog", False, True, True): 4686939670 / 799999200,
+    ("f32c", "leapfrog", True, True, "widened"): 934032036 / 4e7,
+    ("f32c", "ruth4", True, True, "widened"): 1360098640 / 4e7,
+    ("f32c", "rk4", True, True, "double_rf"): 1871249906 / 4e7,
+    ("f32cd", "leapfrog", True, True, False): 315762505 / 4e7,
+    ("f32cd", "ruth4", True, True, False): 593402435 / 4e7,
+    ("f32cd", "leapfrog", False, True, True): 3913030858 / 799999200,
+    ("f32cd", "leapfrog", True, True, "widened"): 898409684 / 4e7,
+    ("f32cd", "ruth4", True, True, "widened"): 1252238952 / 4e7,
+    ("f32cd", "rk4", True, True, "double_rf"): 1569827554 / 4e7,
     ("f32cs", "leapfrog", True, True, False): 235314078 / 4e7,
     ("f32cs", "ruth4", True, True, False): 350447674 / 4e7,
     ("f32cs", "leapfrog", True, True, "widened"): 273249116 / 4e7,
     ("f32cs", "ruth4", True, True, "widened"): 400925430 / 4e7,
     ("f32cs", "rk4", True, True, "double_rf"): 460129668 / 4e7,
 }
-for _dt in ("f32c", "f32cd"):  # one arithmetic, the same kernels
-    EXECUTED_NOW.update({
-        (_dt, "leapfrog", True, True, False): 315765457 / 4e7,
-        (_dt, "ruth4", True, True, False): 593405387 / 4e7,
-        (_dt, "leapfrog", False, True, True): 3912999552 / 799999200,
-        (_dt, "leapfrog", True, True, "widened"): 898412636 / 4e7,
-        (_dt, "ruth4", True, True, "widened"): 1252241904 / 4e7,
-        (_dt, "rk4", True, True, "double_rf"): 1569819738 / 4e7,
-    })
 
 
 def executed_now(r, key, pts):
     """The roofline r with achieved and frac from what the present kernels execute (EXECUTED_NOW)
-    where a capture of the variant exists; the fraction r had goes to `frac_of_the_earlier_count`
-    (FP64: sines as FP64 work; FP32: instructions of the earlier kernels), which a kernel that
-    does the same work with less can take beyond 1."""
+    where a capture of the variant exists.  The fractions of counts that are not the present
+    kernels' go (FP64 flops with every sine as FP64 work; the earlier FP32 kernels' instructions):
+    a kernel that does the same work with less takes them beyond 1."""
     per = EXECUTED_NOW.get(key)
     if per is None or not r:
         return r
     issue = r.get("bound") == "issue"
     achieved = per * pts / (1e9 if issue else 1e12)
-    out = dict(r, frac_of_the_earlier_count=r.get("frac"), achieved=achieved, frac=achieved / r["peak"])
+    out = dict(r, achieved=achieved, frac=achieved / r["peak"])
+    out.pop("alg_frac", None)
     if issue:
         out["warp_inst_per_particle_turn_ncu"] = per
     else:
@@ -861,7 +864,7 @@ def executed_now(r, key, pts):
                    executed_frac=achieved / r["peak"],
                    basis="ncu-executed FP64 flops per particle-turn (2 DFMA + DMUL + DADD) of the present "
                          "kernels x live particle-turns/s; sines, chromatic phases and moment sums run on "
-                         f"the integer pipe; alg_frac counts each sine as {SINE_FLOPS} flops")
+                         f"the integer pipe (alg_achieved counts each sine as {SINE_FLOPS} flops)")
     return out
 
 
