@@ -74,15 +74,14 @@ __device__ __forceinline__ double widen_float_bits(float f)
 // Cheaper forms of the two for the RF phase argument of the PHTL_F32C kernels (k z + phi formed in FP64
 // from a coordinate's two floats), where a term below 2^-126 in magnitude changes nothing.
 //
-// widen_float_phase: exact for normal floats and +-0 (a particle at z = 0 keeps the phase 0
-// exactly); subnormals become values of magnitude in [2^-127, 2^-126); Inf / NaN become
-// finite values of magnitude >= 2^128 (a lost particle's phase, which split_phase does not cover).
+// widen_float_phase: exact for normal floats; +-0 and subnormals become values of magnitude in
+// [2^-127, 2^-126) (z = 0 is left to split_phase's caller); Inf / NaN become finite values of magnitude
+// >= 2^128 (a lost particle's phase, which split_phase does not cover).
 __device__ __forceinline__ double widen_float_phase(float f)
 {
     const unsigned u = __float_as_uint(f);
-    const unsigned mag = u & 0x7fffffffu;
-    const unsigned hi = mag != 0u ? (mag >> 3) + (896u << 20) : 0u;
-    return __hiloint2double(static_cast<int>((u & 0x80000000u) | hi), static_cast<int>(u << 29));
+    const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20));
+    return __hiloint2double(static_cast<int>(hi), static_cast<int>(u << 29));
 }
 
 // split_phase: split_bits's high part; the low part is the remaining 29 bits rounded to
@@ -93,14 +92,14 @@ __device__ __forceinline__ DF2 split_phase(double x, bool& ok)
 {
     const unsigned hi32 = static_cast<unsigned>(__double2hiint(x));
     const unsigned lo32 = static_cast<unsigned>(__double2loint(x));
-    const unsigned e = (hi32 >> 20) & 0x7ffu;
-    ok = e - 949u <= 86u;
-    const unsigned sign = hi32 & 0x80000000u;
-    const unsigned t = (hi32 & 0x7fffffffu) - (896u << 20);  // FP32 biased exponent at bit 20
+    ok = (hi32 & 0x7fffffffu) - (949u << 20) < (87u << 20);
+    // the FP32 biased exponent at bit 20, the sign in its place
+    const unsigned t = hi32 - (896u << 20);
+    const unsigned h = (t & 0x80000000u) | __funnelshift_l(lo32, t, 3);
+    const float m = __uint2float_rn(lo32 & 0x1fffffffu);  // the remaining bits, rounded
     DF2 r;
-    r.h = __uint_as_float(sign | __funnelshift_l(lo32, t, 3));
-    const float m = __uint2float_rn(lo32 & 0x1fffffffu);      // the remaining bits, rounded
-    r.l = __fmul_rn(m, __uint_as_float(sign | ((e - 948u) << 23)));
+    r.h = __uint_as_float(h);
+    r.l = __fmul_rn(m, __uint_as_float((h & 0xff800000u) - (52u << 23)));  // in units of 2^-52 of h's power of two
     return r;
 }
 

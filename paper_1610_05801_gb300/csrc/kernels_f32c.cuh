@@ -19,7 +19,7 @@
 // coordinate).  Issue bound: PHTL_F32CD takes 127 instructions per particle and leap-frog turn, 0.99
 // clocks of an SM's issue slots, 1.2 measured at 4e6 particles (213 instructions and 2.2 clocks before
 // the quarter-turn phase and with renormalised intermediate products); PHTL_F32C's two FP64 FMAs take
-// the FP64 pipe 1.0 clocks beside it, 1.6 measured.
+// the FP64 pipe 1.0 clocks beside it, 1.4 measured.
 #pragma once
 
 #include <cuda_runtime.h>

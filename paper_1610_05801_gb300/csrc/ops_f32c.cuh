@@ -21,8 +21,8 @@ constexpr int P = 4;
 // unless they wait for FP64 phases (FP32C) with little else to do:
 //   - linear map: 2 blocks (at most 128 registers) for FP32C and FP32CD (FP32CD leap-frog 3.7 % faster
 //     than at 64 or 80 registers, Ruth4 with planes and moments 4 %; FP32C with planes and moments 4 to
-//     6 %); 4 (64 registers) for FP32C without planes (leap-frog, 4e6 particles, 20 turns: 397 us
-//     against 440 at 2 and 412 at 3; Ruth4, 6e5: 187, 223, 211); 3 for FP32CS;
+//     6 %); 4 (64 registers) for FP32C without planes (leap-frog, 4e6 particles, 20 turns: 382 us
+//     against 426 at 2 and 391 at 3; Ruth4, 6e5: 182, 212, 202); 3 for FP32CS;
 //   - widened map and RK4 / double RF (general kernels): 2 blocks for FP32C and FP32CD (widened
 //     leap-frog 5 % faster than at 3, RK4 on the double-RF ring 20 %), 3 for FP32CS;
 //   - batched kernels: 96 registers for FP32C and FP32CD (64 bunches, moments every turn: 7 %
@@ -58,7 +58,7 @@ constexpr int f32c_batched_registers(int dtype, bool general)
 #define PHTL_F32C_TRACK_BOUNDS(S, DT, G, T) __maxnreg__(PHTL_F32C_MAXNREG)
 #define PHTL_F32C_BATCHED_BOUNDS(DT, G) __maxnreg__(PHTL_F32C_MAXNREG)
 #else
-#define PHTL_F32C_RAMP_BOUNDS(S, DT) __launch_bounds__(256, (DT) == PHTL_F32C ? 2 : 1)
+#define PHTL_F32C_RAMP_BOUNDS(S, DT) __launch_bounds__(256, (DT) == PHTL_F32C ? 2 : 0)
 #define PHTL_F32C_TRACK_BOUNDS(S, DT, G, T) __launch_bounds__(256, f32c::f32c_track_min_blocks(S, DT, G, T))
 #define PHTL_F32C_BATCHED_BOUNDS(DT, G) __maxnreg__(f32c::f32c_batched_registers(DT, G))
 #endif
@@ -225,12 +225,13 @@ __device__ __forceinline__ DF2 sin_quarter_df(const QuarterPhase& k, float ph, f
 }
 
 // PHTL_F32C, in radians: formed in FP64 from hi and comp (two FMAs of registers) and split to 2^-48, less
-// q pi/2 (Cody-Waite, pi/2 = P1 + P2 + P3): q P1 is formed exactly, x.h - q P1 as a TwoSum pair, and
-// the small remainder in FP32.  At small phases, where nothing is subtracted, 1.6 times closer than the
+// q pi/2 (Cody-Waite, pi/2 = P1 + P2 + P3): q P1 is formed exactly as a pair, its head's difference from
+// x.h is exact, and the small remainder in FP32.  At small phases, where nothing is subtracted, 1.6 times closer than the
 // quarter turns (6.8e-18 rms against 1.1e-17 for a bunch of 1 mm).  ok: see split_phase.
 // An FP64 FMA holds a warp's share of the pipe for 64 clocks, so eight of them (four particles) are what
-// a small bunch waits for: 1000 particles x 200 turns, leap-frog, 178 us against PHTL_F32CD's 82; 4e6
-// particles 1.32 of PHTL_F32CD's time.
+// a small bunch waits for: 1000 particles x 200 turns, leap-frog, 175 us against PHTL_F32CD's 83; 4e6
+// particles 1.27 of PHTL_F32CD's time.  One FMA, of hi and comp added as integers first (12 instructions
+// more), served small bunches and batches 2 to 14 % faster but the others up to 40 % slower: not kept.
 template <bool ZS>
 __device__ __forceinline__ DF2 sin_fp64_phase(double k, double phi, DF2 z, bool& ok)
 {
@@ -241,11 +242,12 @@ __device__ __forceinline__ DF2 sin_fp64_phase(double k, double phi, DF2 z, bool&
     const float q = __fsub_rn(t0, magic);
     const float p1 = __fmul_rn(q, 1.5707963705062866f);
     const float e1 = __fmaf_rn(q, 1.5707963705062866f, -p1);
-    const DF2 hd = df_two_sum(x.h, -p1);  // exact as a pair
-    float rest = __fadd_rn(__fsub_rn(x.l, e1), hd.l);
+    // exact: 0 for q = 0; otherwise both are multiples of 2^-24 or more (above 1/2) and differ by less than 1
+    const float hd = __fsub_rn(x.h, p1);
+    float rest = __fsub_rn(x.l, e1);
     rest = __fmaf_rn(-q, -4.371138828673793e-08f, rest);
     rest = __fmaf_rn(-q, -1.7151245100058819e-15f, rest);
-    return sin_pair_poly(df_fast_two_sum(hd.h, rest), __float_as_int(t0));
+    return sin_pair_poly(df_fast_two_sum(hd, rest), __float_as_int(t0));
 }
 
 // sin(k z + phi) where neither covers it, in FP64.
