@@ -318,7 +318,7 @@ __device__ __forceinline__ void force_df(const QuarterPhase& q, float ph, float 
 #pragma unroll
         for (int p = 0; p < N; ++p)
             if (!ok[p])  // split_phase leaves out z = 0 (also the lanes beyond a bunch's end): no call for it
-                f[p] = DT == PHTL_F32C && z[p].h == 0.0f && (ZS || phi64 == 0.0)
+                f[p] = DT == PHTL_F32C && z[p].h == 0.0f && z[p].l == 0.0f && (ZS || phi64 == 0.0)
                            ? z[p]
                            : sin_df_rest(k64, ZS ? 0.0 : phi64, z[p]);
     }

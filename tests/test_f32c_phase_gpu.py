@@ -53,3 +53,21 @@ def test_small_phase_kicks(path):
     rel = ((got - want) / want).astype(np.float64) / UNIT
     assert math.sqrt(float(np.mean(rel * rel))) <= 0.8
     assert float(np.max(np.abs(rel))) <= 8.0
+
+
+def test_tails_of_coordinates_whose_head_is_zero():
+    """Coordinates as a caller may hand them over, not normalised: hi = 0 and a compensation from 1e-36 to
+    1e-9, beside exact zeros.  sin(k z) is k z there, to the pairs' 8 2^-48 and FP32's smallest normal number."""
+    comp = np.concatenate([[0.0, -0.0], np.logspace(-36, -9, 28), -np.logspace(-36, -9, 28)]).astype(np.float32)
+    n = comp.size
+    d = oracle.load().derive(synth.ring(4.5e6, transverse=False))
+    R = phtl.Ring(**synth.ring(4.5e6, transverse=False))
+    bz = torch.tensor(np.concatenate([np.zeros(n, dtype=np.float32), comp]), device=DEV)
+    bd = torch.zeros_like(bz)
+    R.track(bz, bd, turns=1, integrator="euler_cromer", dtype="f32c")
+    torch.cuda.synchronize()
+    R.close()
+    got = phtl.join_f32c(bd.cpu().numpy())
+    want = d.A * d.k * comp.astype(np.float64)
+    assert np.all(np.abs(got - want) <= 8 * UNIT * np.abs(want) + 2.0 ** -126 * 1e-3)
+    assert np.all(got[:2] == 0.0)
