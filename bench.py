@@ -823,12 +823,12 @@ EXECUTED_NOW = {
     ("f64", "ruth4", True, True, "ramp"): 2 * 760_000_010 / 4e7,
     ("f64", "leapfrog", False, True, "batched"): (2 * 2_402_150_400 + 41_724_852) / 799_999_200,
     ("f64", "leapfrog", True, True, "collective"): (2 * 27_002_880 + 3_000_000 + 6_656_320) / 3e6,
-    ("f32c", "leapfrog", True, True, False): 351369244 / 4e7,
-    ("f32c", "ruth4", True, True, False): 699995953 / 4e7,
-    ("f32c", "leapfrog", False, True, True): 4686939670 / 799999200,
-    ("f32c", "leapfrog", True, True, "widened"): 934032036 / 4e7,
-    ("f32c", "ruth4", True, True, "widened"): 1360098640 / 4e7,
-    ("f32c", "rk4", True, True, "double_rf"): 1871249906 / 4e7,
+    ("f32c", "leapfrog", True, True, False): 341990044 / 4e7,
+    ("f32c", "ruth4", True, True, False): 670920433 / 4e7,
+    ("f32c", "leapfrog", False, True, True): 4486581270 / 799999200,
+    ("f32c", "leapfrog", True, True, "widened"): 924027556 / 4e7,
+    ("f32c", "ruth4", True, True, "widened"): 1331023120 / 4e7,
+    ("f32c", "rk4", True, True, "double_rf"): 1781522226 / 4e7,
     ("f32cd", "leapfrog", True, True, False): 315762505 / 4e7,
     ("f32cd", "ruth4", True, True, False): 593402435 / 4e7,
     ("f32cd", "leapfrog", False, True, True): 3913030858 / 799999200,
